@@ -254,6 +254,22 @@ BNN_API size_t bnn_output_prepared_bytes(int C, int H);
 BNN_API int bnn_output_prepare(const float* Wout, int ldw, int C, int H,
                                void* prepared, size_t prepared_bytes, void* stream);
 
+/* The top layer on packed activations with exact sums.  bnn_output_prepare_digits writes each class row once as
+ * fixed-point numbers of a power-of-two scale of its own, in three byte digits (about 23 bits relative to the row's
+ * largest weight; four digits, 31 bits, for the whole matrix when some row's largest weight exceeds 16 times the
+ * row's mean magnitude), in the order the tensor core reads them; bnn_output_layer_digits multiplies the digits
+ * with the activations' signs in integers, so that a logit is rounded once instead of at every step, and takes 3/4
+ * of the tensor-core passes of bnn_output_layer's fp16 terms:
+ *   |z - exact| <= H * 2^-23 * max_h |Wout[c][h]|  (2^-31 with four digits) + one fp32 rounding + the bias addition.
+ * act_values : bnn_act_values of Hp.  H <= 2^15 (larger: BNN_ERR_UNSUPPORTED; use bnn_output_layer).
+ * digits : device buffer, 256-byte aligned, at least bnn_output_digits_bytes(C, H) bytes.  In bnn_forward: the
+ * `Wp` of a BNN_LAYER_REAL_OUT layer. */
+BNN_API size_t bnn_output_digits_bytes(int C, int H);
+BNN_API int bnn_output_prepare_digits(const float* Wout, int ldw, int C, int H,
+                                      void* digits, size_t digits_bytes, void* stream);
+BNN_API int bnn_output_layer_digits(const uint32_t* Hp, int ldhp, const void* digits, const float* b, int act_values,
+                                    int M, int C, int H, float* logp, int ldo, int log_softmax, void* stream);
+
 /* ------------------------------------------------------------------------------------
  * Whole forward pass: the loops "for l = 1 to L" of Algorithms 1 and 2.
  */
@@ -269,7 +285,8 @@ typedef enum {
 typedef struct bnn_layer {
     int kind;
     int K, N;              /* fan-in, fan-out */
-    const uint32_t* Wp;    /* SIGNW, XNOR: packed weights [N][ldwp] */
+    const uint32_t* Wp;    /* SIGNW, XNOR: packed weights [N][ldwp]; REAL_OUT on packed activations:
+                              bnn_output_prepare_digits image of W (preferred to W_prepared), or NULL */
     int ldwp;
     const float* W;        /* REAL_OUT, REAL: fp32 weights [N][ldw] */
     int ldw;

@@ -102,6 +102,12 @@ def lib():
         L.bnn_signw_gemm_ws.argtypes = [C.c_void_p, C.c_int, C.c_void_p, C.c_int, C.c_int, C.c_int, C.c_int, C.c_void_p,
                                         C.c_int, C.POINTER(Epilogue), C.c_void_p, C.c_size_t, C.c_void_p]
         i, p = C.c_int, C.c_void_p
+        L.bnn_output_digits_bytes.argtypes = [i, i]
+        L.bnn_output_digits_bytes.restype = C.c_size_t
+        L.bnn_output_prepare_digits.argtypes = [p, i, i, i, p, C.c_size_t, p]
+        L.bnn_output_prepare_digits.restype = i
+        L.bnn_output_layer_digits.argtypes = [p, i, p, p, i, i, i, i, p, i, i, p]
+        L.bnn_output_layer_digits.restype = i
         L.bnn_pack_weights.argtypes = [p, i, i, i, p, i, i, p]
         L.bnn_binarize_pack.argtypes = [p, i, i, i, p, i, i, p]
         L.bnn_fold_thresholds.argtypes = [p, p, i, i, i, p, p, p]
@@ -335,6 +341,25 @@ def bnn_output_prepare(Wout, prepared):
     return prepared
 
 
+def bnn_output_digits_bytes(C_, H) -> int:
+    return int(lib().bnn_output_digits_bytes(int(C_), int(H)))
+
+
+def bnn_output_prepare_digits(Wout, digits):
+    c, h = Wout.shape
+    _check(lib().bnn_output_prepare_digits(_ptr(Wout, torch.float32), _ld(Wout), c, h, _ptr(digits),
+                                           digits.numel() * digits.element_size(), _stream()), "bnn_output_prepare_digits")
+    return digits
+
+
+def bnn_output_layer_digits(Hp, digits, b, logp, H, log_softmax=True, values=VALUES_PM1):
+    """The top layer on packed activations with the weights given as bnn_output_prepare_digits made them."""
+    _check(lib().bnn_output_layer_digits(_ptr(Hp, torch.int32), _ld(Hp), _ptr(digits), _ptr(b, torch.float32), values,
+                                         Hp.shape[0], logp.shape[1], H, _ptr(logp, torch.float32), _ld(logp),
+                                         int(log_softmax), _stream()), "bnn_output_layer_digits")
+    return logp
+
+
 def bnn_real_layer(Hf, W, bias, Y, act=ACT_SIGMOID, prepared=None, workspace=None):
     """Y = act(Hf W^T + bias) with real-valued weights; tensor cores with ``prepared`` and ``workspace``."""
     m, k = Hf.shape
@@ -395,6 +420,8 @@ class ModelDesc:
             a.kind, a.K, a.N, a.act = d["kind"], d["K"], d["N"], d.get("act", ACT_NONE)
             wp, w = d.get("Wp"), d.get("W")
             a.Wp, a.ldwp = _ptr(wp, torch.int32), (_ld(wp) if wp is not None else 0)
+            if d.get("W_digits") is not None:   # top layer: the digit image of W
+                a.Wp = _ptr(d["W_digits"])
             a.W, a.ldw = _ptr(w, torch.float32), (_ld(w) if w is not None else 0)
             a.W_prepared = _ptr(d.get("W_prepared"))
             a.scale, a.shift = _ptr(d.get("scale"), torch.float32), _ptr(d.get("shift"), torch.float32)
@@ -437,6 +464,7 @@ def bnn_forward_events(model: ModelDesc, X, logp, workspace, events, layer_out=N
 
 
 STATIC_WORKSPACE_BYTES = 8 << 20
+MAX_K_DIGITS = 1 << 15   # widest input of the kernels on byte digits
 
 
 def bnn_forward_static(model: ModelDesc, X, logp):

@@ -87,6 +87,7 @@ int validate_model(const bnn_model* model) {
                 if (l != L - 1) return BNN_ERR_UNSUPPORTED;
                 if (!y.W) return BNN_ERR_NULL;
                 if (y.ldw < y.K) return BNN_ERR_SHAPE;
+                if (reinterpret_cast<uintptr_t>(y.Wp) & 255u) return BNN_ERR_ALIGN;   // the digit image, or NULL
                 break;
             default:
                 return BNN_ERR_UNSUPPORTED;
@@ -370,7 +371,7 @@ static int output_layer_impl(const uint32_t* Hp, int ldhp, const float* Hf, int 
                              int M, int C, int H, float* logp, int ldo, int log_softmax,
                              int zo, void* workspace, size_t workspace_bytes, const float* log_prior,
                              int act, void* mid_event, void* stream, bool image_ready = false,
-                             int* done = nullptr) {
+                             int* done = nullptr, const void* digits = nullptr) {
     if (int rc = check_dims(M, C, H)) return rc;
     if (act != BNN_ACT_NONE && (Hp || log_softmax || (act != BNN_ACT_SIGMOID && act != BNN_ACT_HARDTANH)))
         return BNN_ERR_UNSUPPORTED;
@@ -394,10 +395,14 @@ static int output_layer_impl(const uint32_t* Hp, int ldhp, const float* Hf, int 
     int rc;
     // `done` (zeroed counters in the caller's workspace): the log-softmax kernel is launched right behind
     // the tensor-core kernel and takes each group of frames as soon as all its logits are stored
-    const bool follow = done && Hp && prepared && g_real_path != BNN_PATH_CUDA_CORE && log_softmax && !mid_event &&
+    const bool by_digits = Hp && digits && H <= kMaxKDigit && g_real_path != BNN_PATH_CUDA_CORE;
+    const bool by_halves = Hp && prepared && !by_digits && g_real_path != BNN_PATH_CUDA_CORE;
+    const bool follow = done && (by_digits || by_halves) && log_softmax && !mid_event &&
                         g_softmax_follow && log_softmax_can_follow(logp, ldo, C, log_prior) &&
-                        out_tc_more_than_one_wave(M, C);
-    if (Hp && prepared && g_real_path != BNN_PATH_CUDA_CORE)
+                        (by_digits ? out_digit_can_be_followed(M, C, H) : out_tc_more_than_one_wave(M, C));
+    if (by_digits)
+        rc = launch_out_digit(Hp, ldhp, digits, b, M, C, H, logp, ldo, zo, follow ? done : nullptr, (cudaStream_t)stream);
+    else if (by_halves)
         rc = launch_out_tc(Hp, ldhp, prepared, b, M, C, H, logp, ldo, zo, follow ? done : nullptr, (cudaStream_t)stream);
     else if (Hf && prepared && g_real_path != BNN_PATH_CUDA_CORE && workspace &&
              !(reinterpret_cast<uintptr_t>(workspace) & 255u) && workspace_bytes >= outf_image_bytes(M, H))
@@ -410,8 +415,9 @@ static int output_layer_impl(const uint32_t* Hp, int ldhp, const float* Hf, int 
     if (mid_event && cudaEventRecord((cudaEvent_t)mid_event, (cudaStream_t)stream) != cudaSuccess)
         return BNN_ERR_CUDA;
     if (follow)
-        return launch_log_softmax_rows_follow(logp, ldo, M, C, log_prior, done, out_tc_group_arrivals(C),
-                                              out_tc_group_rows(), (cudaStream_t)stream);
+        return launch_log_softmax_rows_follow(logp, ldo, M, C, log_prior,
+                                              by_digits ? out_digit_follow(digits, M, C, H, done) : out_tc_follow(C, done),
+                                              (cudaStream_t)stream);
     if (log_softmax) return launch_log_softmax_rows(logp, ldo, M, C, log_prior, (cudaStream_t)stream);
     return BNN_OK;
 }
@@ -453,6 +459,33 @@ int bnn_output_layer_ws(const float* Hf, int ldhf, const float* Wout, int ldw, c
                              log_softmax, 0, workspace, workspace_bytes, nullptr, BNN_ACT_NONE, nullptr, stream);
 }
 
+size_t bnn_output_digits_bytes(int C, int H) {
+    if (C < 1 || H < 1) return 0;
+    return out_digits_bytes(C, H);
+}
+
+int bnn_output_prepare_digits(const float* Wout, int ldw, int C, int H, void* digits, size_t digits_bytes, void* stream) {
+    if (!Wout || !digits) return BNN_ERR_NULL;
+    if (C < 1 || H < 1 || ldw < H) return BNN_ERR_SHAPE;
+    if (H > kMaxKDigit) return BNN_ERR_UNSUPPORTED;
+    if (digits_bytes < out_digits_bytes(C, H)) return BNN_ERR_WORKSPACE;
+    if (reinterpret_cast<uintptr_t>(digits) & 255u) return BNN_ERR_ALIGN;
+    return launch_out_prepare_digits(Wout, ldw, C, H, digits, (cudaStream_t)stream);
+}
+
+int bnn_output_layer_digits(const uint32_t* Hp, int ldhp, const void* digits, const float* b, int act_values,
+                            int M, int C, int H, float* logp, int ldo, int log_softmax, void* stream) {
+    if (!Hp || !digits || !logp) return BNN_ERR_NULL;
+    if (int rc = check_dims(M, C, H)) return rc;
+    if (ldo < C) return BNN_ERR_SHAPE;
+    if (H > kMaxKDigit || (act_values != BNN_VALUES_PM1 && act_values != BNN_VALUES_01)) return BNN_ERR_UNSUPPORTED;
+    if (int rc = check_packed(Hp, ldhp, H)) return rc;
+    if (reinterpret_cast<uintptr_t>(digits) & 255u) return BNN_ERR_ALIGN;
+    if (int rc = launch_out_digit(Hp, ldhp, digits, b, M, C, H, logp, ldo, act_values == BNN_VALUES_01, nullptr, (cudaStream_t)stream))
+        return rc;
+    return log_softmax ? launch_log_softmax_rows(logp, ldo, M, C, nullptr, (cudaStream_t)stream) : BNN_OK;
+}
+
 int bnn_output_layer01(const uint32_t* Hp, int ldhp, const float* Wout, int ldw, const float* b,
                        const void* prepared, int M, int C, int H, float* logp, int ldo,
                        int log_softmax, void* stream) {
@@ -479,7 +512,7 @@ static WorkspaceLayout workspace_layout(const bnn_model* model, int M) {
     }
     const size_t stack = round256(xnor_stack_sync_bytes(M, xnor_layers));
     const bool top = model->layers[model->n_layers - 1].kind == BNN_LAYER_REAL_OUT && model->n_layers > 1;
-    return WorkspaceLayout{round256(mx), stack, stack + (top ? round256(out_tc_done_bytes(M)) : 0)};
+    return WorkspaceLayout{round256(mx), stack, stack + (top ? round256(out_done_bytes(M)) : 0)};
 }
 
 size_t bnn_forward_min_workspace_bytes(const bnn_model* model, int M) {
@@ -562,8 +595,9 @@ int bnn_forward_events(const bnn_model* model, const float* X, int ldx, int M,
             any = stackable(model, l) && stackable(model, l + 1) && model->layers[l].N == model->layers[l].K &&
                   model->layers[l + 1].N == model->layers[l].N && model->layers[l + 1].K == model->layers[l].K;
         const bnn_layer& top = model->layers[L - 1];
-        if (g_softmax_follow && !events && lay.sync > lay.stack_sync && top.kind == BNN_LAYER_REAL_OUT && top.W_prepared &&
-            L > 1 && model->layers[L - 2].act == BNN_ACT_SIGN_PACK && out_tc_more_than_one_wave(M, top.N))
+        if (g_softmax_follow && !events && lay.sync > lay.stack_sync && top.kind == BNN_LAYER_REAL_OUT && L > 1 &&
+            model->layers[L - 2].act == BNN_ACT_SIGN_PACK &&
+            ((top.Wp && out_digit_can_be_followed(M, top.N, top.K)) || (top.W_prepared && out_tc_more_than_one_wave(M, top.N))))
             top_done = sync + lay.stack_sync / sizeof(int);
         clear_pending = any || top_done;
         // When the first layer splits its input into an image, that kernel clears them on its way (a memset
@@ -613,7 +647,7 @@ int bnn_forward_events(const bnn_model* model, const float* X, int ldx, int M,
                                        in_bits && model->act_values == BNN_VALUES_01,
                                        chain_in ? img + (size_t)chain_slot * img_half : img, chain_in ? img_half : img_bytes,
                                        model->log_prior, BNN_ACT_NONE, events ? events[L + 1] : nullptr, stream, chain_in,
-                                       in_bits ? top_done : nullptr);
+                                       in_bits ? top_done : nullptr, in_bits ? y.Wp : nullptr);
             if (rc) return rc;
             if (events && events[L] &&
                 cudaEventRecord((cudaEvent_t)events[L], (cudaStream_t)stream) != cudaSuccess)

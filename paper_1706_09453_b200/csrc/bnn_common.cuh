@@ -147,6 +147,9 @@ int launch_pipe_rate(int which, int repeat, void* scratch, size_t scratch_bytes,
 // Tensor map of a packed operand [rows][ceil(K/32) words] of pitch `ld` words: boxes of 16 words x
 // box_rows rows, 64-byte swizzle, zero fill outside the tensor.  False when the encoder fails.
 bool encode_packed_map(CUtensorMap* map, const uint32_t* base, int ld, int rows, int K, int box_rows);
+// Tensor map of a digit image (digit_gemm.cuh): `chunks` rows of `rows` x 16 bytes, boxes of box_rows x 16 bytes x
+// box_chunks rows, zero fill outside.  Elements are 8 bytes (a box may have at most 256 of them).
+bool encode_digit_map(CUtensorMap* map, const void* base, int rows, int chunks, int box_rows, int box_chunks);
 // Reads (synchronously) the word that a tensor-core kernel sets when a bounded wait ran out.
 int read_tc_status(int* out);
 // The same as a copy enqueued on `st` (dst: device or pinned host memory), and the reset of the word.
@@ -201,19 +204,32 @@ int launch_signw_img(const RealGemmArgs& a, int terms, void* workspace, bool ima
                      int* clear, int clear_words, cudaStream_t st);
 size_t out_prepared_bytes(int C, int H);
 int launch_out_prepare(const float* W, int ldw, int C, int H, void* prepared, cudaStream_t st);
-// `done` (optional, out_tc_done_bytes(M) zeroed bytes): one counter per out_tc_group_rows() frames, then
-// the row counter of the kernel that follows; every epilogue warp adds 1 to a group's counter once its
-// share of a tile of that group is stored; out_tc_group_arrivals(C) arrivals complete a group.
-// launch_log_softmax_rows_follow, launched right behind, consumes the groups in order.
-int out_tc_group_rows();
-int out_tc_group_arrivals(int C);
-size_t out_tc_done_bytes(int M);
+// A top-layer kernel that is followed by the log-softmax gets `done` (out_done_bytes(M) zeroed bytes): one counter
+// per group_rows frames, then the row counter of the kernel that follows; every epilogue warp adds 1 to a group's
+// counter once its share of a tile of that group is stored; `need` (need4 where flag is given and *flag is set)
+// arrivals complete a group.  launch_log_softmax_rows_follow, launched right behind, consumes the groups in order.
+struct FollowArgs {
+    int* done;
+    int need, need4;
+    const int* flag;
+    int group_rows;
+};
+constexpr int kFollowGroupRows = 256;    // the smallest group
+inline size_t out_done_bytes(int M) { return (size_t)(ceil_div(M, kFollowGroupRows) + 1) * sizeof(int); }
 bool out_tc_more_than_one_wave(int M, int C);
+FollowArgs out_tc_follow(int C, int* done);
 int launch_out_tc(const uint32_t* Hp, int ldhp, const void* prepared, const float* bias,
                   int M, int C, int H, float* Z, int ldz, int zo, int* done, cudaStream_t st);
+// The same on the byte-digit image of the weights (out_digit_tc.cu), for H <= kMaxKDigit (its integer sums).
+constexpr int kMaxKDigit = 1 << 15;
+size_t out_digits_bytes(int C, int H);
+int launch_out_prepare_digits(const float* W, int ldw, int C, int H, void* image, cudaStream_t st);
+bool out_digit_can_be_followed(int M, int C, int H);
+FollowArgs out_digit_follow(const void* image, int M, int C, int H, int* done);
+int launch_out_digit(const uint32_t* Hp, int ldhp, const void* image, const float* bias,
+                     int M, int C, int H, float* Z, int ldz, int zo, int* done, cudaStream_t st);
 bool log_softmax_can_follow(const float* Z, int ldz, int C, const float* prior);
-int launch_log_softmax_rows_follow(float* Z, int ldz, int M, int C, const float* prior, int* done, int need,
-                                   int group_rows, cudaStream_t st);
+int launch_log_softmax_rows_follow(float* Z, int ldz, int M, int C, const float* prior, const FollowArgs& f, cudaStream_t st);
 // The top layer on fp32 activations (finite, |a| < 65504) with both operands split into fp16
 // terms (out_gemm_f32_tc.cu): `workspace` holds outf_image_bytes(M, H) bytes, 256-byte aligned.
 size_t outf_image_bytes(int M, int H);

@@ -352,9 +352,10 @@ int launch_out_prepare(const float* W, int ldw, int C, int H, void* prepared, cu
     return launch_status();
 }
 
-int out_tc_group_rows() { return FN; }
-int out_tc_group_arrivals(int C) { return ceil_div(C, BC) * EPI_WARPS; }
-size_t out_tc_done_bytes(int M) { return (size_t)(ceil_div(M, FN) + 1) * sizeof(int); }
+FollowArgs out_tc_follow(int C, int* done) {
+    const int need = ceil_div(C, BC) * EPI_WARPS;
+    return FollowArgs{done, need, need, nullptr, FN};
+}
 // With no more tiles than SMs every tile ends at about the same time: nothing for a following kernel to
 // overlap with (measured: 1-2 % slower than two launches in a row on 256 frames).
 bool out_tc_more_than_one_wave(int M, int C) { return ceil_div(M, FN) * ceil_div(C, BC) > device_sm_count(); }

@@ -393,11 +393,13 @@ constexpr int kFollowRows = 2, kFollowThreads = 128;
 template <int V>
 __global__ void __launch_bounds__(kFollowThreads)
 log_softmax_rows_follow_kernel(float* __restrict__ Z, int ldz, int M, int C, const float* __restrict__ prior,
-                               int* __restrict__ done, int need, int group_rows, tc::TcStatus status) {
+                               FollowArgs follow, tc::TcStatus status) {
     constexpr int R = kFollowRows, NT = kFollowThreads;
     __shared__ float sm[2][R][NT / 32], ss[2][R][NT / 32];
     __shared__ int claim;
     const int c4 = C >> 2;
+    int* const done = follow.done;
+    const int group_rows = follow.group_rows, need = follow.flag && __ldg(follow.flag) ? follow.need4 : follow.need;
     int* next_row = done + ceil_div(M, group_rows);
     int pending = 0, ready_group = -1;   // thread 0: the claim in flight; the last group seen complete
     int par = 0;
@@ -453,16 +455,15 @@ bool log_softmax_can_follow(const float* Z, int ldz, int C, const float* prior) 
     return (C % 4 == 0) && (ldz % 4 == 0) && aligned16(Z) && C <= 128 * 4 * 8 && (!prior || aligned16(prior));
 }
 
-int launch_log_softmax_rows_follow(float* Z, int ldz, int M, int C, const float* prior, int* done, int need,
-                                   int group_rows, cudaStream_t st) {
+int launch_log_softmax_rows_follow(float* Z, int ldz, int M, int C, const float* prior, const FollowArgs& f, cudaStream_t st) {
     const int sms = device_sm_count();
     const tc::TcStatus status = tc_status();
     if (sms <= 0 || !status.word || !log_softmax_can_follow(Z, ldz, C, prior)) return BNN_ERR_CUDA;
-    if (group_rows % kFollowRows != 0) return BNN_ERR_UNSUPPORTED;
+    if (f.group_rows % kFollowRows != 0) return BNN_ERR_UNSUPPORTED;
     const int blocks = M < sms * 5 * kFollowRows ? ceil_div(M, kFollowRows) : sms * 5;
     const cudaError_t e = C <= kFollowThreads * 4 * 4
-        ? launch_pdl(log_softmax_rows_follow_kernel<4>, dim3(blocks), dim3(kFollowThreads), 0, st, Z, ldz, M, C, prior, done, need, group_rows, status)
-        : launch_pdl(log_softmax_rows_follow_kernel<8>, dim3(blocks), dim3(kFollowThreads), 0, st, Z, ldz, M, C, prior, done, need, group_rows, status);
+        ? launch_pdl(log_softmax_rows_follow_kernel<4>, dim3(blocks), dim3(kFollowThreads), 0, st, Z, ldz, M, C, prior, f, status)
+        : launch_pdl(log_softmax_rows_follow_kernel<8>, dim3(blocks), dim3(kFollowThreads), 0, st, Z, ldz, M, C, prior, f, status);
     return e == cudaSuccess ? launch_status() : BNN_ERR_CUDA;
 }
 

@@ -74,11 +74,17 @@ class DeviceNet:
                                    scale=sc, shift=sh,
                                    act=B.ACT_SIGMOID if last_sigmoid else B.ACT_SIGN_PACK))
         self.Wout, self.bout = to_dev(net.Wout, device), to_dev(net.bout, device)
-        self.Wout_prepared = torch.empty(B.bnn_output_prepared_bytes(cfg.classes, cfg.hidden),
-                                         dtype=torch.uint8, device=device)
-        B.bnn_output_prepare(self.Wout, self.Wout_prepared)
+        # weights of the top layer in the form its kernel reads (built once): byte digits for packed activations,
+        # fp16 terms for fp32 activations
+        self.Wout_prepared = self.Wout_digits = None
+        if layers[-1]["act"] == B.ACT_SIGN_PACK and cfg.hidden <= B.MAX_K_DIGITS:
+            self.Wout_digits = torch.empty(B.bnn_output_digits_bytes(cfg.classes, cfg.hidden), dtype=torch.uint8, device=device)
+            B.bnn_output_prepare_digits(self.Wout, self.Wout_digits)
+        else:
+            self.Wout_prepared = torch.empty(B.bnn_output_prepared_bytes(cfg.classes, cfg.hidden), dtype=torch.uint8, device=device)
+            B.bnn_output_prepare(self.Wout, self.Wout_prepared)
         layers.append(dict(kind=B.LAYER_REAL_OUT, K=cfg.hidden, N=cfg.classes, W=self.Wout,
-                           W_prepared=self.Wout_prepared, shift=self.bout))
+                           W_prepared=self.Wout_prepared, W_digits=self.Wout_digits, shift=self.bout))
         self.log_prior = to_dev(log_prior, device) if log_prior is not None else None
         self.desc = B.ModelDesc(layers, sign_mode, act_values, splice, self.log_prior)
         self._ws = None

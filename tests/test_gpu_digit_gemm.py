@@ -1,0 +1,51 @@
+"""Products of packed signs with real-valued rows as exact integer products of byte digits, at the sizes where the
+kernels can go wrong: edges of the 256-row x 64- (or 32-) column tiles, fan-ins around 32 / 128 / 256 positions, one
+row, several turns of the persistent grid, and rows that need a fourth digit."""
+import numpy as np
+import pytest
+
+from oracle import bnn_oracle as o
+from paper_1706_09453_b200 import workloads as wl
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def env():
+    import torch
+    assert torch.cuda.is_available()
+    from paper_1706_09453_b200 import build, binding, model
+    build.build()
+    return torch, binding, model
+
+
+@pytest.mark.parametrize("m,h,c", [(1, 1, 1), (1, 32, 33), (255, 127, 63), (256, 128, 64), (257, 129, 65), (128, 255, 31),
+                                   (129, 257, 97), (40, 2048, 3307), (2100, 300, 700), (513, 31, 193)])
+@pytest.mark.parametrize("outlier", [False, True])
+@pytest.mark.parametrize("values", [0, 1])
+def test_output_layer_digits(env, m, h, c, outlier, values):
+    torch, B, model = env
+    rng = np.random.default_rng(1000 * m + h + c)
+    hp = wl.make_bit_planes(m, h, 0.5, 7 + m + h, B.packed_pitch(h))
+    w = rng.normal(0, 1 / np.sqrt(h), (c, h)).astype(np.float32)
+    if outlier:      # one weight dwarfs the rest of its row: three digits would lose them
+        w[c // 2] *= np.float32(1e-5)
+        w[c // 2, h // 3] = 1.0
+    b = rng.normal(0, 0.1, c).astype(np.float32)
+    digits = torch.full((B.bnn_output_digits_bytes(c, h),), 255, dtype=torch.uint8, device="cuda:0")
+    B.bnn_output_prepare_digits(model.to_dev(w), digits)
+    z = torch.full((m, c + 1), 9.0, dtype=torch.float32, device="cuda:0")
+    B.bnn_output_layer_digits(model.to_dev(hp), digits, model.to_dev(b), z[:, :c], h, log_softmax=False, values=values)
+    a = np.unpackbits(hp.view(np.uint8), axis=1, bitorder="little")[:, :h].astype(np.float64)
+    want = (a if values else 2 * a - 1) @ w.astype(np.float64).T + b
+    # every weight is off by at most half a unit of its row's fixed-point scale: 2^-22 of the largest weight when three
+    # digits are taken (the library's criterion; the scale may lose a bit to the power of two), 2^-30 with four;
+    # then two roundings of the result and one of the bias addition
+    mx, sm = np.abs(w).max(1).astype(np.float64), np.abs(w).sum(1, dtype=np.float64)
+    four = bool((h * mx > 16 * sm).any())
+    assert four or not outlier or h < 64
+    bound = h * mx * (2.0 ** -30 if four else 2.0 ** -22) / 2 + 3 * 2.0 ** -24 * (np.abs(want) + np.abs(b))
+    got = z.cpu().numpy()
+    assert (np.abs(got[:, :c] - want) <= bound).all(), (np.abs(got[:, :c] - want) / bound).max()
+    np.testing.assert_array_equal(got[:, c], 9.0)
+    assert B.bnn_device_status() == 0
