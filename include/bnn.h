@@ -184,11 +184,13 @@ BNN_API int bnn_signw_gemm(const float* X, int ldx, const uint32_t* Wp, int ldwp
                    const bnn_epilogue* epi, void* stream);
 
 /* bnn_signw_gemm with scratch.  With `workspace` (device, 256-byte aligned, at least
- * bnn_signw_workspace_bytes(M, K) bytes) the real operand is split into its bf16 terms once
- * per call, into an image laid out in the order the tensor core reads it, and the GEMM streams
- * that image with bulk copies: 2-4x faster than bnn_signw_gemm on the tensor path.  Without
- * workspace (NULL, or too small) it behaves exactly like bnn_signw_gemm.  Same results within
- * the same bound.  The paper has no counterpart. */
+ * bnn_signw_workspace_bytes(M, K) bytes) the real operand is written once per call as an image laid out
+ * in the order the tensor core reads it, which the GEMM streams: 2-5x faster than bnn_signw_gemm on the tensor
+ * path.  With two terms (BNN_OPT_SIGNW_TERMS), K <= 2^15 and an activation other than SIGN_PACK the image holds every row of X as fixed-point numbers of a
+ * power-of-two scale of its own in three byte digits, and the sums are exact integers:
+ *   |y - exact| <= K * 2^-23 * max_k |x[m][k]| + one fp32 rounding (a row with an infinity or a NaN gives NaN);
+ * otherwise it holds bf16 terms, as bnn_signw_gemm.  Without workspace (NULL, or too small) it behaves exactly like
+ * bnn_signw_gemm.  The paper has no counterpart. */
 BNN_API size_t bnn_signw_workspace_bytes(int M, int K);
 BNN_API int bnn_signw_gemm_ws(const float* X, int ldx, const uint32_t* Wp, int ldwp,
                               int M, int N, int K, float* Y, int ldy,
@@ -331,7 +333,8 @@ typedef struct bnn_model {
  * follow one another, because each writes the next one's image while it reads its own) or of a
  * real-valued layer fed with fp32 activations (see bnn_output_layer_ws).
  * bnn_forward_min_workspace_bytes is the least it accepts (the two buffers and the counters;
- * sign-weight layers then split their activations inside the GEMM and hand on fp32 rows). */
+ * sign-weight layers then keep their image in the rows of logp until the top layer writes those -- if they are
+ * contiguous, ldo == C, and long enough -- or split their activations inside the GEMM, and hand on fp32 rows). */
 BNN_API size_t bnn_forward_workspace_bytes(const bnn_model* model, int M);
 BNN_API size_t bnn_forward_min_workspace_bytes(const bnn_model* model, int M);
 
@@ -396,7 +399,8 @@ BNN_API int bnn_forward_events(const bnn_model* model, const float* X, int ldx, 
  *                        tcgen05 with split bf16/fp16 operands.  AUTO = TENSOR.
  *   BNN_OPT_SIGNW_TERMS: 2 (default) or 3 bf16 terms for the real operand of bnn_signw_gemm
  *                        on the tensor path: |error| <= 2^-17 sum|x_i| with 2, fp32-exact
- *                        products with 3.
+ *                        products with 3.  With 2 and scratch, activations other than SIGN_PACK: byte digits, see
+ *                        bnn_signw_gemm_ws.
  *   BNN_OPT_XNOR_PREPARED: which kernel bnn_xnor_gemm_prepared (and bnn_forward on prepared
  *                        layers) runs for a fused Sign layer: BNN_PREPARED_STREAM reads the
  *                        weight image from L2 for every tile of frames; BNN_PREPARED_RESIDENT

@@ -331,7 +331,7 @@ static int signw_impl(const float* X, int ldx, const uint32_t* Wp, int ldwp,
     if (!a.Y && !a.out_bits && !out_image) return BNN_ERR_NULL;
     if (g_real_path != BNN_PATH_CUDA_CORE) {
         if (workspace && !(reinterpret_cast<uintptr_t>(workspace) & 255u) &&
-            workspace_bytes >= signw_image_bytes(M, K, g_signw_terms)) {
+            workspace_bytes >= signw_scratch_bytes(M, K, g_signw_terms, a.act)) {
             // the kernel that splits the activations can clear the caller's counters on its way
             const bool clears = clear && clear_words > 0 && !image_ready;
             if (cleared) *cleared = clears;
@@ -708,7 +708,9 @@ int bnn_forward_events(const bnn_model* model, const float* X, int ldx, int M,
             // split-activation image (two images alternate in the scratch beyond the activation buffers),
             // and as fp32 only where the caller asked to see them.
             const bnn_layer* nx = l + 1 < L ? &model->layers[l + 1] : nullptr;
-            const bool to_signw = nx && nx->kind == BNN_LAYER_SIGNW && !(small && nx->act == BNN_ACT_SIGN_PACK);
+            // (both must use the same form of image: see signw_by_digits)
+            const bool to_signw = nx && nx->kind == BNN_LAYER_SIGNW && !(small && nx->act == BNN_ACT_SIGN_PACK) &&
+                                  signw_by_digits(g_signw_terms, y.K, y.act) == signw_by_digits(g_signw_terms, nx->K, nx->act);
             const bool to_real = nx && (nx->kind == BNN_LAYER_REAL_OUT || nx->kind == BNN_LAYER_REAL) && nx->W_prepared;
             const bool chain_out = y.act != BNN_ACT_SIGN_PACK && (to_signw || to_real) &&
                                    g_real_path != BNN_PATH_CUDA_CORE && img_bytes >= 2 * img_half;
@@ -722,8 +724,20 @@ int bnn_forward_events(const bnn_model* model, const float* X, int ldx, int M,
                 out_ld = y.N;
             }
             bool cleared = false;
+            size_t img_in_bytes = chain_in || chain_out ? img_half : img_bytes;
+            if (!chain_in && !chain_out && !(l == 0 && splice_dim > 0) && ldo == model->layers[L - 1].N &&
+                img_in_bytes < signw_scratch_bytes(M, y.K, g_signw_terms, y.act)) {
+                // no room for the image in the workspace: the log-probabilities' own rows are free until the top
+                // layer writes them (contiguous rows only: what lies between rows is the caller's)
+                const uintptr_t base = (reinterpret_cast<uintptr_t>(logp) + 255) & ~uintptr_t(255);
+                const uintptr_t end = reinterpret_cast<uintptr_t>(logp + (size_t)M * ldo);
+                if (end > base && end - base >= signw_scratch_bytes(M, y.K, g_signw_terms, y.act)) {
+                    img_in = reinterpret_cast<char*>(base);
+                    img_in_bytes = end - base;
+                }
+            }
             rc = signw_impl(static_cast<const float*>(in), in_ld, y.Wp, y.ldwp, M, y.N, y.K,
-                            yf, y.N, &e, img_in, chain_in ? img_half : (chain_out ? img_half : img_bytes),
+                            yf, y.N, &e, img_in, img_in_bytes,
                             l == 0 ? splice_dim : 0, model->splice_left, stream, chain_in, img_out, to_real ? 1 : 0,
                             (l == 0 && clear_by_first) ? sync : nullptr, (int)(lay.sync / sizeof(int)), &cleared);
             if (l == 0 && clear_pending) {

@@ -91,6 +91,9 @@ int launch_xnor_popc(const uint32_t* Ap, int ldap, const uint32_t* Wp, int ldwp,
 
 // Tensor-core (tcgen05) XNOR GEMM; same contract as launch_xnor_popc.  K <= kMaxKTensor.
 constexpr int kMaxKTensor = 1 << 22;
+// Largest fan-in of the kernels on byte digits (digit_gemm.cuh): their 32-bit sums of 64 * 128 * K, and the joined
+// low digits of 256 * 128 * K, stay below 2^31, the high digits' sums of 128 * K within 2^22.
+constexpr int kMaxKDigit = 1 << 15;
 int launch_xnor_tc(const uint32_t* Ap, int ldap, const uint32_t* Wp, int ldwp, int M, int N,
                    int K, int32_t* C, int ldc, const int32_t* thr, const uint32_t* flip,
                    uint32_t* out_bits, int ldob, int zo, cudaStream_t st);
@@ -196,12 +199,23 @@ size_t signw_image_bytes(int M, int K, int terms);
 // image_ready: `workspace` already holds the image of a.Af's values (a.Af is not read then);
 // out_image (256-byte aligned, signw_image_bytes(M, N, terms) bytes) or nullptr: the outputs are also
 // written as the image of a following layer of this kind with fan-in N.
-// out_kind 0: that layer's own image (bf16 terms, blocks of 128 frames); 1: the image the real-valued
+// out_kind 0: that layer's own image (digits, or bf16 terms in blocks of 128 frames); 1: the image the real-valued
 // layer on fp32 activations reads (two fp16 terms, blocks of 256 frames, outf_image_bytes(M, N) bytes).
 // clear / clear_words (optional, only with image_ready == false): words the splitting kernel sets to zero on
 // its way -- bnn_forward's counters, which would otherwise need a memset of their own in front of it.
 int launch_signw_img(const RealGemmArgs& a, int terms, void* workspace, bool image_ready, void* out_image, int out_kind,
                      int* clear, int clear_words, cudaStream_t st);
+// The same with the activations as byte digits and exact integer sums (signw_digit_tc.cu): what launch_signw_img runs
+// with two terms for layers that hand on real values, unless the fan-in is beyond kMaxKDigit; its image is smaller
+// than signw_image_bytes(M, K, 2).
+inline bool signw_by_digits(int terms, int K, int act) { return terms == 2 && K <= kMaxKDigit && act != BNN_ACT_SIGN_PACK; }
+size_t signw_digit_bytes(int M, int K);
+// What the path actually taken needs: at most signw_image_bytes(M, K, terms).
+inline size_t signw_scratch_bytes(int M, int K, int terms, int act) {
+    return signw_by_digits(terms, K, act) ? signw_digit_bytes(M, K) : signw_image_bytes(M, K, terms);
+}
+int launch_signw_digit(const RealGemmArgs& a, void* workspace, bool image_ready, void* out_image, int out_kind,
+                       int* clear, int clear_words, cudaStream_t st);
 size_t out_prepared_bytes(int C, int H);
 int launch_out_prepare(const float* W, int ldw, int C, int H, void* prepared, cudaStream_t st);
 // A top-layer kernel that is followed by the log-softmax gets `done` (out_done_bytes(M) zeroed bytes): one counter
@@ -221,7 +235,6 @@ FollowArgs out_tc_follow(int C, int* done);
 int launch_out_tc(const uint32_t* Hp, int ldhp, const void* prepared, const float* bias,
                   int M, int C, int H, float* Z, int ldz, int zo, int* done, cudaStream_t st);
 // The same on the byte-digit image of the weights (out_digit_tc.cu), for H <= kMaxKDigit (its integer sums).
-constexpr int kMaxKDigit = 1 << 15;
 size_t out_digits_bytes(int C, int H);
 int launch_out_prepare_digits(const float* W, int ldw, int C, int H, void* image, cudaStream_t st);
 bool out_digit_can_be_followed(int M, int C, int H);

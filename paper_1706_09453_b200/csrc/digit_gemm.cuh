@@ -210,22 +210,18 @@ __device__ __forceinline__ void widen_bits(const Work& w, const uint32_t* __rest
     int s = 0;
     uint32_t ph = 1;
     const int total = total_tiles * blocks;
-    // A stage goes out in two stores: the first half is widened before the wait, the second while the first store is
-    // on its way, and the next stage's first half while the second is.
     uint4 cur = fetch(), nxt = fetch();
-    uint32_t lo[16], hi[16];
-    widen_bytes<ZO>(cur.x, lo);
-    widen_bytes<ZO>(cur.y, lo + 8);
+    uint32_t o[32];
+    auto widen = [&](const uint4& v) {
+        widen_bytes<ZO>(v.x, o); widen_bytes<ZO>(v.y, o + 8); widen_bytes<ZO>(v.z, o + 16); widen_bytes<ZO>(v.w, o + 24);
+    };
+    widen(cur);
     for (int it = 0; it < total; ++it) {
+        // what lies between a free slot and a full one is kept short: the row was widened before the wait
         if (!warp_wait(smem_u32(&bars->empty_a[2 * s + team]), ph, abort_flag, lane)) return;
-        tmem_st16(tdst + s * A_COLS, lo);
-        widen_bytes<ZO>(cur.z, hi);
-        widen_bytes<ZO>(cur.w, hi + 8);
-        tmem_st16(tdst + s * A_COLS + 16, hi);
+        tmem_st32(tdst + s * A_COLS, o);
         cur = nxt;
         nxt = fetch();
-        widen_bytes<ZO>(cur.x, lo);
-        widen_bytes<ZO>(cur.y, lo + 8);
         tmem_st_wait();
         tc_fence_before_sync();
         __syncwarp();
@@ -235,6 +231,7 @@ __device__ __forceinline__ void widen_bits(const Work& w, const uint32_t* __rest
             else mbar_arrive_cluster(peer_addr(bar, 0));
         }
         if (++s == a_stages) { s = 0; ph ^= 1u; }
+        widen(cur);
     }
 }
 
@@ -340,7 +337,12 @@ __device__ __forceinline__ void join_granule(const uint32_t (&d)[4][8], int nd, 
         }
     } else {
 #pragma unroll
-        for (int i = 0; i < 8; ++i) S[i] = fmaf((float)(int)d[2][i], 1024.0f, (float)((int)d[1][i] * 4 + ((int)d[0][i] >> 6)));
+        for (int i = 0; i < 8; ++i) {
+            // the high sum is below 2^22: adding 1.5 * 2^23 as an integer to its bits makes it a float without the
+            // conversion unit, which the other conversion of every output already keeps busy
+            const float high = __int_as_float(((int)d[2][i] >> 6) + 0x4B400000) - 12582912.0f;
+            S[i] = fmaf(high, 65536.0f, (float)((int)d[1][i] * 4 + ((int)d[0][i] >> 6)));
+        }
     }
 }
 // `n` consecutive granules, handed to `use(g, S)` one by one; with three digits the next one is on its way meanwhile.
@@ -368,24 +370,38 @@ __device__ __forceinline__ void granules(uint32_t taddr, int n, int nd, F use) {
     }
 }
 
-// Largest e (up to 140) such that mx * 2^e is a balanced number of nd digits: at most 127 * (65536 + 256 + 1) with
-// three, and somewhat below 127 * 2^24 with four.
+// 2^h for -126 <= h <= 127.
+__device__ __forceinline__ float power_of_two(int h) { return __int_as_float((127 + h) << 23); }
+// Largest e (up to 140) such that mx * 2^e is a balanced number of nd digits: at most 127 * (65536 + 256 + 1) =
+// 0x7F7F7F with three, and somewhat below 127 * 2^24 with four (2e9).  mx >= 0; its exponent and fraction fields
+// are compared with those of the limit.
 __device__ __forceinline__ int scale_exponent(float mx, int nd) {
-    if (!(mx > 0.f)) return 0;
-    int e = (nd == 4 ? 30 : 22) - ilogbf(mx);
-    if (scalbnf(mx, e) > (nd == 4 ? 2.0e9f : 8355711.0f)) --e;
+    const int bits = __float_as_int(mx);
+    if (bits == 0) return 0;
+    const int over = (bits & 0x7FFFFF) > (nd == 4 ? 7236393 : 0x7EFEFE) ? 1 : 0;     // 2e9 / 2^30, 0x7F7F7F / 2^22
+    const int e = (nd == 4 ? 30 : 22) + 127 - (bits >> 23) - over;
     return e > 140 ? 140 : e;
 }
 // 2^-e, or NaN for a row that holds an infinity or a NaN.
 __device__ __forceinline__ float inverse_scale(float mx, int nd) {
-    return mx < 3.5e38f ? scalbnf(1.0f, -scale_exponent(mx, nd)) : __int_as_float(0x7FC00000);
+    const int e = scale_exponent(mx, nd), h = e >> 1;
+    return __float_as_int(mx) < 0x7F800000 ? power_of_two(-h) * power_of_two(h - e) : __int_as_float(0x7FC00000);
 }
-__device__ __forceinline__ int fixed_point(float x, int e) { return __float2int_rn(scalbnf(x, e)); }
-// Next balanced digit of v.
-__device__ __forceinline__ int take_digit(int& v) {
-    const int d = (int)(signed char)(v & 255);
-    v = (v - d) >> 8;
-    return d;
+// x * 2^e rounded to an integer; 2^e comes as two powers of two (e may be beyond the exponent range of one).
+struct Scale {
+    float a, b;
+    __device__ __forceinline__ explicit Scale(int e) : a(power_of_two(e >> 1)), b(power_of_two(e - (e >> 1))) {}
+    __device__ __forceinline__ int fixed_point(float x) const { return __float2int_rn(x * a * b); }
+};
+// The balanced base-256 digits of v in the bytes of a word: the sum of 128 at every place turns them into ordinary
+// bytes (no borrows), and the exclusive or takes 128 off each byte again.
+__device__ __forceinline__ uint32_t digits3(int v) { return ((uint32_t)v + 0x00808080u) ^ 0x00808080u; }
+__device__ __forceinline__ uint32_t digits4(int v) { return ((uint32_t)v + 0x80808080u) ^ 0x80808080u; }
+// Bytes q of four words, in their order.
+template <int Q>
+__device__ __forceinline__ uint32_t gather_bytes(uint32_t a, uint32_t b, uint32_t c, uint32_t d) {
+    constexpr uint32_t lo = (uint32_t)Q | ((uint32_t)(4 + Q) << 4);
+    return __byte_perm(__byte_perm(a, b, lo), __byte_perm(c, d, lo), 0x5410);
 }
 
 // Digit rows per tile (192 or 96) for `a_rows` x `b_rows` outputs on `pairs` CTA pairs: the one with the least

@@ -82,21 +82,22 @@ __global__ void out_digits_kernel(const float* __restrict__ W, int ldw, int C, i
     const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= (long long)chunks * Cpad8) return;
     const int c = (int)(i % Cpad8), ch = (int)(i / Cpad8);
-    const int e = c < C ? digit::scale_exponent(mxs[c], nd) : 0;
+    const digit::Scale scale(c < C ? digit::scale_exponent(mxs[c], nd) : 0);
     if (ch == 0) scales[c] = c < C ? digit::inverse_scale(mxs[c], nd) : 0.f;
     uint32_t d[4][4];
 #pragma unroll
     for (int t = 0; t < 4; ++t) {
-#pragma unroll
-        for (int q = 0; q < 4; ++q) d[q][t] = 0u;
+        uint32_t v[4];
 #pragma unroll
         for (int j = 0; j < 4; ++j) {          // byte 4 t + j of the chunk
             const int k = (ch >> 1) * 32 + (ch & 1) * 4 + t + 8 * j;
-            int v = (c < C && k < H) ? digit::fixed_point(W[(size_t)c * ldw + k], e) : 0;
-#pragma unroll
-            for (int q = 0; q < 4; ++q)
-                if (q < nd) d[q][t] |= ((uint32_t)digit::take_digit(v) & 255u) << (8 * j);
+            const int n = (c < C && k < H) ? scale.fixed_point(W[(size_t)c * ldw + k]) : 0;
+            v[j] = nd == 4 ? digit::digits4(n) : digit::digits3(n);
         }
+        d[0][t] = digit::gather_bytes<0>(v[0], v[1], v[2], v[3]);
+        d[1][t] = digit::gather_bytes<1>(v[0], v[1], v[2], v[3]);
+        d[2][t] = digit::gather_bytes<2>(v[0], v[1], v[2], v[3]);
+        d[3][t] = digit::gather_bytes<3>(v[0], v[1], v[2], v[3]);
     }
     uint8_t* dst = img + ((size_t)ch * rows + (size_t)(c / digit::GRAN) * digit::GRAN * nd + c % digit::GRAN) * 16;
 #pragma unroll

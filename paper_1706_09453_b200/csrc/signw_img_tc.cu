@@ -1,5 +1,6 @@
 // Binary weights x real-valued activations on the tensor cores, with the activations split
-// ONCE per call into bf16 terms (instead of once per tile of units):
+// ONCE per call into bf16 terms (instead of once per tile of units).  Serves the layers with Sign units, and all
+// with three terms or a fan-in beyond kMaxKDigit; the others run on byte digits (signw_digit_tc.cu).
 //
 //   1. x_split_kernel writes x = x_hi + x_lo (+ x_lo2) as bf16 planes into a scratch "image"
 //      that is stored in exactly the order the MMA reads shared memory (a memory-bound pass:
@@ -589,6 +590,7 @@ size_t signw_image_bytes(int M, int K, int terms) {
 int launch_signw_img(const RealGemmArgs& r, int terms, void* workspace, bool image_ready, void* out_image, int out_kind,
                      int* clear, int clear_words, cudaStream_t st) {
     if (clear && image_ready) return BNN_ERR_UNSUPPORTED;   // no split kernel runs: nobody to clear the words
+    if (signw_by_digits(terms, r.K, r.act)) return launch_signw_digit(r, workspace, image_ready, out_image, out_kind, clear, clear_words, st);
     return terms == 3 ? launch_nt<3>(r, workspace, image_ready, out_image, out_kind, clear, clear_words, st)
                       : launch_nt<2>(r, workspace, image_ready, out_image, out_kind, clear, clear_words, st);
 }

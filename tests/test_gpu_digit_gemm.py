@@ -49,3 +49,56 @@ def test_output_layer_digits(env, m, h, c, outlier, values):
     assert (np.abs(got[:, :c] - want) <= bound).all(), (np.abs(got[:, :c] - want) / bound).max()
     np.testing.assert_array_equal(got[:, c], 9.0)
     assert B.bnn_device_status() == 0
+
+
+@pytest.mark.parametrize("m,n,k", [(1, 1, 1), (8, 33, 31), (7, 255, 32), (63, 256, 127), (64, 257, 128), (65, 31, 129),
+                                   (9, 300, 257), (33, 2048, 440), (300, 129, 1300), (1100, 520, 96)])
+@pytest.mark.parametrize("act", [0, 2, 3])
+def test_signw_gemm_digits(env, m, n, k, act):
+    torch, B, model = env
+    rng = np.random.default_rng(m + 10 * n + 100 * k)
+    x = (rng.standard_normal((m, k)) * 10.0 ** rng.uniform(-3, 3, (m, 1))).astype(np.float32)
+    x[m // 2, k // 2] = 1e-30                      # far below its row's scale
+    wp = wl.make_bit_planes(n, k, 0.5, 3 + m + n, B.packed_pitch(k))
+    sc = rng.uniform(-1.5, 1.5, n).astype(np.float32)
+    sh = rng.normal(0, 0.1, n).astype(np.float32)
+    ws = torch.full((B.bnn_signw_workspace_bytes(m, k),), 255, dtype=torch.uint8, device="cuda:0")
+    y = torch.full((m, n + 1), 9.0, dtype=torch.float32, device="cuda:0")
+    B.bnn_signw_gemm(model.to_dev(x), model.to_dev(wp), k, Y=y[:, :n], act=act, scale=model.to_dev(sc), shift=model.to_dev(sh),
+                     workspace=ws)
+    ref, _ = o.signw_gemm(x, wp, k)
+    mx = np.abs(x).max(1).astype(np.float64)[:, None]
+    pre = sc.astype(np.float64) * ref + sh
+    # every value is off by at most half a unit of its row's fixed-point scale (2^-22 of the largest); the sum, the
+    # scale and the affine round once each
+    bound = np.abs(sc) * (k * mx * 2.0 ** -22 / 2 + 2.0 ** -23 * np.abs(ref)) + 2.0 ** -23 * (np.abs(pre) + np.abs(sh))
+    got = y.cpu().numpy()
+    np.testing.assert_array_equal(got[:, n], 9.0)
+    if act == B.ACT_HARDTANH:
+        pre = np.clip(pre, -1, 1)
+    elif act == B.ACT_SIGMOID:
+        with np.errstate(over="ignore"):
+            pre, bound = 1 / (1 + np.exp(-pre)), bound / 4 + 2e-7
+    assert (np.abs(got[:, :n] - pre) <= bound).all(), (np.abs(got[:, :n] - pre) / bound).max()
+    assert B.bnn_device_status() == 0
+
+
+def test_signw_gemm_digits_rows_with_infinities_and_nans(env):
+    """Such a row gives NaN everywhere; its neighbours are untouched."""
+    torch, B, model = env
+    m, n, k = 20, 70, 50
+    rng = np.random.default_rng(5)
+    x = rng.standard_normal((m, k)).astype(np.float32)
+    clean = x.copy()
+    x[3, 7], x[11, 0] = np.inf, np.nan
+    wp = wl.make_bit_planes(n, k, 0.5, 8, B.packed_pitch(k))
+    out = []
+    for a in (clean, x):
+        ws = torch.empty(B.bnn_signw_workspace_bytes(m, k), dtype=torch.uint8, device="cuda:0")
+        y = torch.empty((m, n), dtype=torch.float32, device="cuda:0")
+        B.bnn_signw_gemm(model.to_dev(a), model.to_dev(wp), k, Y=y, workspace=ws)
+        out.append(y.cpu().numpy())
+    bad = np.zeros(m, bool)
+    bad[[3, 11]] = True
+    np.testing.assert_array_equal(out[0][~bad], out[1][~bad])
+    assert np.isnan(out[1][bad]).all()
