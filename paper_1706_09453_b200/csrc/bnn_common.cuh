@@ -110,7 +110,7 @@ int launch_xnor_res(const uint32_t* Ap, int ldap, const void* image, int M, int 
 // A run of consecutive fused Sign layers of one shape (N == K beyond the first) in ONE launch of that
 // kernel: layer l reads the bits layer l - 1 wrote (pitch ldob), layer 0 reads Ap.  `progress` points
 // to xnor_stack_sync_bytes(M, n_layers) bytes of ZEROED device memory (per frame tile and layer
-// boundary a counter of the unit tiles that have stored their bits).  `chained`: the launch is part of a
+// boundary a counter of the epilogue warps that have stored their bits).  `chained`: the launch is part of a
 // forward pass (programmatic dependent launch on the layer kernel before it).
 constexpr int kXnorStackMax = 8;
 struct XnorStackLayer {

@@ -245,22 +245,13 @@ __device__ __forceinline__ void mma_mxf4_ts(uint32_t tmem_d, uint32_t tmem_a, ui
         "tcgen05.mma.cta_group::1.kind::mxf4.block_scale.block32 [%0], [%1], %2, %3, [%5], [%6], p;\n\t}"
         ::"r"(tmem_d), "r"(tmem_a), "l"(db), "r"(idesc), "r"(accumulate), "r"(sfa), "r"(sfb) : "memory");
 }
-// The `_if` forms are executed by a whole, converged warp and take effect in the lanes whose `issue` is
-// non-zero (one lane): the instruction is predicated instead of sitting in a divergent branch, so the
-// loop around it stays warp-uniform and its bookkeeping (descriptors, slots, parities) can live in
-// uniform registers.  (Measured on B200: 5 % off the hidden-layer kernel's MMA loop against a loop
-// inside `if (lane == 0)`.)
-__device__ __forceinline__ void mma_mxf4_ts_if(uint32_t issue, uint32_t tmem_d, uint32_t tmem_a, uint64_t db, uint32_t idesc,
-                                               uint32_t sfa, uint32_t sfb, uint32_t accumulate) {
+// The same with B's descriptor as two words, so that stepping through a stage is 32-bit arithmetic.
+__device__ __forceinline__ void mma_mxf4_ts(uint32_t tmem_d, uint32_t tmem_a, uint32_t db_lo, uint32_t db_hi, uint32_t idesc,
+                                            uint32_t sfa, uint32_t sfb, uint32_t accumulate) {
     asm volatile(
-        "{\n\t.reg .pred p, q;\n\tsetp.ne.b32 p, %4, 0;\n\tsetp.ne.b32 q, %7, 0;\n\t"
-        "@q tcgen05.mma.cta_group::1.kind::mxf4.block_scale.block32 [%0], [%1], %2, %3, [%5], [%6], p;\n\t}"
-        ::"r"(tmem_d), "r"(tmem_a), "l"(db), "r"(idesc), "r"(accumulate), "r"(sfa), "r"(sfb), "r"(issue) : "memory");
-}
-__device__ __forceinline__ void mma_commit_if(uint32_t issue, uint32_t bar) {
-    asm volatile(
-        "{\n\t.reg .pred q;\n\tsetp.ne.b32 q, %1, 0;\n\t"
-        "@q tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n\t}" ::"r"(bar), "r"(issue) : "memory");
+        "{\n\t.reg .pred p;\n\t.reg .b64 b;\n\tsetp.ne.b32 p, %5, 0;\n\tmov.b64 b, {%2, %3};\n\t"
+        "tcgen05.mma.cta_group::1.kind::mxf4.block_scale.block32 [%0], [%1], b, %4, [%6], [%7], p;\n\t}"
+        ::"r"(tmem_d), "r"(tmem_a), "r"(db_lo), "r"(db_hi), "r"(idesc), "r"(accumulate), "r"(sfa), "r"(sfb) : "memory");
 }
 // Arrive on an mbarrier once every MMA issued so far by this thread has completed.
 __device__ __forceinline__ void mma_commit(uint32_t bar) {

@@ -13,18 +13,19 @@
 //
 // The image is the one xnor_gemm_img.cu describes: a tile of BN units is, per stage of 256
 // positions of K, eight contiguous runs of BN x 16 bytes, copied to offsets c * BN * 16 of the
-// stage's block (K-major core matrices).  BN = 192 while K <= 2048 and BN = 128 while
-// K <= 3072 keep the slice within 192 KB; other shapes are left to the streaming kernel.
+// stage's block (K-major core matrices).  BN is 192 while K <= 2048 and 128 while K <= 3072 for batches that fill the
+// SMs, which keeps the slice within 192 KB; 96 or 32 for smaller ones, where more unit tiles occupy more SMs and the
+// region holds the next layer's slice beside this one's (tile_units).  Other shapes are left to the streaming kernel.
 //
-// Roles in a CTA of 15 warps (one CTA per SM):
-//   warp 13      one thread issues the bulk copies of the weight slice (once) and the 2-D TMA
-//                tile loads of the packed frame rows (64 bytes per row = two stages) into a
-//                staging ring (64-byte swizzle, no multicast)
+// Roles in a CTA of 16 warps (one CTA per SM):
+//   warp 15      one thread issues the bulk copies of the weight slices, layer after layer
+//   warp 13      one thread issues the 2-D TMA tile loads of the packed frame rows (64 bytes per row = two stages)
+//                into a staging ring (64-byte swizzle, no multicast)
 //   warps 5-12   two teams of four warps widen the frame rows, thread = one row, 32 bytes ->
 //                128 bytes per stage, into tensor memory (the MMA reads its A operand from
 //                there); the teams take alternate stages
-//   warps 4, 14  issue the MMAs (4 per stage, K = 64 each) and the commits, one lane each; the two
-//                warps take a tile's stages in turn and accumulate into the same accumulator
+//   warps 4, 14  issue the MMAs (4 per stage, K = 64 each) and the commits; the two warps take a tile's stages in
+//                turn and accumulate into the same accumulator
 //   warps 0-3    epilogue: accumulator -> threshold -> repacked bits; two accumulators in
 //                tensor memory, so it overlaps the next tile's MMAs
 // Every wait is bounded; a wait that runs out sets the CTA's abort flag, all roles fall
@@ -33,13 +34,20 @@
 // A run of consecutive hidden layers of the same shape (the forward loop of Algorithm 2 over
 // l = 2 .. L-1) is ONE launch: the roles above loop over the layers.  Between layers nothing is
 // torn down; a CTA keeps its unit tile index and its frame tiles.  What a layer needs from the
-// one before it is tracked per frame tile: a counter in global memory that every CTA increments
-// (release) once its bits of that frame tile and layer are stored, and the thread that loads a
-// frame tile waits (acquire, bounded) until all unit tiles have arrived.  The weight slice of the
-// next layer replaces the current one stage by stage, each stage as soon as the last frame tile's
-// MMAs of that stage have completed, so the reload overlaps the tail of the layer.  (Measured on
-// B200: five launches of one layer each spent 6 us per layer between the end of one kernel and
-// the first MMA of the next.)
+// one before it is tracked per frame tile: a counter in global memory that every epilogue warp increments
+// (after a fence) once its bits of that frame tile and layer are stored, and the thread that loads a frame
+// tile waits (acquire, bounded) until the warps of all unit tiles have arrived.  The weight stages of the layers
+// follow one another round a ring of as many as fit, each slot refilled as soon as the last frame tile's MMAs that read it
+// have completed.  (Measured on B200: five launches of one layer each spent 6 us per layer between the end of one
+// kernel and the first MMA of the next.)
+//
+// What bounds it, measured on B200: 65536 frames x 3072 the widening of the frame rows (2 teams, about 430 clocks per
+// stage against 256 of MMA; five layers 1.18 ms, 1.51 before the issue from one elected lane and the lean producer
+// loop); 8192 x 2048 MMA (384 clocks per stage of 192 units), epilogue and the fill of a layer's pipeline in like parts
+// (five layers 76 us, 91 before); a layer of one frame tile per CTA the chain store - count - load - widen -
+// MMA - decide, about 7 us (731 frames 36 us, 50 before, when all tiles were 192 wide).
+#include <type_traits>
+
 #include "bnn_common.cuh"
 #include "tcgen05.cuh"
 #include "xnor_widen.cuh"
@@ -57,28 +65,33 @@ constexpr int B_REGION = 192 * 1024;                      // shared memory that 
 constexpr int EPI_WARPS = 4, MMA_WARP = 4, PROD_WARP0 = 5, A_WARPS = BM / 32, TEAMS = 2;
 constexpr int TMA_WARP = PROD_WARP0 + TEAMS * A_WARPS;
 constexpr int MMA_WARP2 = TMA_WARP + 1;                   // the second issuing warp
-constexpr int THREADS = (MMA_WARP2 + 1) * 32;             // 480
+constexpr int WEIGHT_WARP = MMA_WARP2 + 1;                // loads the weight stages
+constexpr int THREADS = (WEIGHT_WARP + 1) * 32;           // 512
 constexpr int GROUPS = 4;                                 // staging ring of the packed frame rows: groups of two stages
 constexpr int GROUP_BYTES = BM * 64;
 constexpr uint32_t A_COLS = ROW_BYTES / 4;                // 32-bit columns per A stage
 constexpr uint32_t SF_COLS = 32, TMEM_COLS = 512;
-constexpr int MAX_NKS = 16;
+constexpr int MAX_SLOTS = 48, MAX_A_BARS = 6;
 
 template <int BN> struct Cfg {
     static constexpr int B_BYTES = BN * ROW_BYTES;                 // one stage of the unit operand
-    static constexpr int NKS = B_REGION / B_BYTES;                 // stages that fit: 8 (BN 192), 12 (BN 128)
+    static constexpr int SLOTS = B_REGION / B_BYTES;               // weight stages that fit: 8 (BN 192), 12 (128), 16 (96), 48 (32)
     static constexpr int A_STAGES = (int)((TMEM_COLS - SF_COLS - 2 * BN) / A_COLS) > 6 ? 6 : (int)((TMEM_COLS - SF_COLS - 2 * BN) / A_COLS);
+    // A stage `it` of the CTA's sequence has barrier it % A_BARS, an even number, so that a barrier always belongs to the
+    // same team and issuing warp.  (A wait on a parity holds only for one who has seen every phase before it: with
+    // three barriers the warps would take turns on each, and the one ahead could take the phase before for its own.)
+    static constexpr int A_BARS = A_STAGES % 2 ? 2 * A_STAGES : A_STAGES;
     static constexpr uint32_t TMEM_A_COL = 2 * BN;                 // A stages start after the two accumulators
     static constexpr uint32_t TMEM_SF_COL = TMEM_A_COL + A_STAGES * A_COLS;
-    static_assert(NKS <= MAX_NKS && A_STAGES >= 3 && TMEM_SF_COL + SF_COLS <= TMEM_COLS, "tile configuration");
+    static_assert(SLOTS <= MAX_SLOTS && A_STAGES >= 3 && A_BARS <= MAX_A_BARS && TMEM_SF_COL + SF_COLS <= TMEM_COLS, "tile configuration");
 };
 
 constexpr int MAX_STACK = kXnorStackMax;
 
 struct Control {
-    int T[192];              // per unit: threshold + kMagicBits
+    float T[192];            // per unit: threshold
     uint32_t flipw[8];
-    uint64_t full_a[6], empty_a[6], full_b[MAX_NKS], b_free[MAX_NKS], acc_full[2], acc_empty[2];
+    uint64_t full_a[MAX_A_BARS], empty_a[MAX_A_BARS], full_b[MAX_SLOTS], b_free[MAX_SLOTS], acc_full[2], acc_empty[2];
     uint64_t group_full[GROUPS], group_empty[GROUPS];
     uint64_t started[2];
     uint32_t tmem_base;
@@ -114,12 +127,15 @@ struct ProducerArgs {
     int my_tiles, nks, kw;
     uint32_t tmask;
     int lane;
-    int zo;               // the frame operand's bits stand for (0,1) instead of (-1,+1)
 };
 
 // Producer of the frame operand: thread = row `r` of every tile of this CTA; team `team`
 // takes the stages it = team, team + TEAMS, ... of the CTA's sequence of (tile, stage) pairs.
-template <int A_STAGES>
+// Template arguments say what the loop has to deal with: code that is there for another case costs this one, though it is
+// not executed, where this role is the bottleneck (five 3072-wide layers of 65536 frames 1.50 ms with the case of an
+// odd number of stages behind a branch, 1.24 ms without it).
+// ODD: a row has an odd number of stages; ZO: bits stand for (0,1); RAGGED: the last stage has positions >= K.
+template <int A_STAGES, int A_BARS, bool ODD, bool ZO, bool RAGGED>
 __device__ __forceinline__ void produce_a(const ProducerArgs& a, int r, int team) {
     Control* ctl = a.ctl;
     const int total = a.my_tiles * a.nks;
@@ -129,7 +145,14 @@ __device__ __forceinline__ void produce_a(const ProducerArgs& a, int r, int team
     // this row inside a staging group: 64 bytes per row, 16-byte chunk c stored at c ^ ((r/2)%4)
     const uint32_t stg0 = a.smem_stage + r * 64;
     const uint32_t sw = (uint32_t)(r >> 1) & 3u;
-    const bool ragged = (a.kw % 8 != 0) || a.tmask != 0xFFFFFFFFu;   // last stage has positions >= K
+    // A group that holds a single stage, of the other team: every team sees every phase of a group's barriers.
+    auto visit = [&](int gidx) {
+        const int gslot = gidx % GROUPS;
+        if (!warp_wait(smem_u32(&ctl->group_full[gslot]), (uint32_t)((gidx / GROUPS) & 1), a.abort_flag, a.lane)) return false;
+        if (a.lane == 0) mbar_arrive(smem_u32(&ctl->group_empty[gslot]));
+        return true;
+    };
+    if (ODD && a.nks == 1 && team == 1 && total > 0 && !visit(0)) return;
     int ks = team, tl = 0;
     while (ks >= a.nks) { ks -= a.nks; ++tl; }
     for (int it = team; it < total; it += TEAMS) {
@@ -141,20 +164,21 @@ __device__ __forceinline__ void produce_a(const ProducerArgs& a, int r, int team
         const uint4 v0 = lds128u(src + (((2u * gi) ^ sw) << 4));
         const uint4 v1 = lds128u(src + (((2u * gi + 1u) ^ sw) << 4));
         const int s = it % A_STAGES;
-        if (!warp_wait(smem_u32(&ctl->empty_a[s]), (uint32_t)(((it / A_STAGES) & 1) ^ 1), a.abort_flag, a.lane)) break;
+        const int e = it + A_BARS - A_STAGES;          // the stage that had this slot; a fresh barrier passes parity 1
+        if (!warp_wait(smem_u32(&ctl->empty_a[e % A_BARS]), (uint32_t)(((e / A_BARS) & 1) ^ 1), a.abort_flag, a.lane)) break;
         const uint32_t w[8] = {v0.x, v0.y, v0.z, v0.w, v1.x, v1.y, v1.z, v1.w};
         // 32-bit column 4c + t of the stage = word t of chunk c: the byte order of the
         // K-major shared-memory layout of the other operand
         uint32_t wr[32];
-        if (a.zo) {
+        if (ZO) {
 #pragma unroll
             for (int c = 0; c < 8; ++c) {
                 const int g = 8 * ks + c;   // index of the word in the row
-                const uint32_t valid = (!ragged || g < a.kw - 1) ? 0xFFFFFFFFu : (g == a.kw - 1 ? a.tmask : 0u);
+                const uint32_t valid = (!RAGGED || g < a.kw - 1) ? 0xFFFFFFFFu : (g == a.kw - 1 ? a.tmask : 0u);
                 const uint4 o = widen01_masked(w[c], valid);
                 wr[4 * c] = o.x; wr[4 * c + 1] = o.y; wr[4 * c + 2] = o.z; wr[4 * c + 3] = o.w;
             }
-        } else if (ragged && ks == a.nks - 1) {
+        } else if (RAGGED && ks == a.nks - 1) {
 #pragma unroll
             for (int c = 0; c < 8; ++c) {
                 const int g = 8 * ks + c;   // index of the word in the row
@@ -174,14 +198,14 @@ __device__ __forceinline__ void produce_a(const ProducerArgs& a, int r, int team
         tc_fence_before_sync();
         __syncwarp();
         if (a.lane == 0) {
-            mbar_arrive(smem_u32(&ctl->full_a[s]));
+            mbar_arrive(smem_u32(&ctl->full_a[it % A_BARS]));
             // The staging slot is handed back only after the stores that consumed the loaded
             // words: a shared-memory load that has merely been issued does not hold back the
-            // TMA write that refills the slot.  A group counts one arrival per warp and stage;
-            // the last group of a row with an odd number of stages holds a single stage, whose
-            // consumers arrive twice.
+            // TMA write that refills the slot.  A group counts one arrival per warp of both teams.
             mbar_arrive(smem_u32(&ctl->group_empty[gslot]));
-            if (gi == 0 && ks == a.nks - 1) mbar_arrive(smem_u32(&ctl->group_empty[gslot]));
+        }
+        if (ODD && it + 1 < total && (a.nks == 1 || ks + 2 == a.nks)) {
+            if (!visit(gidx + 1)) break;
         }
         ks += TEAMS;
         while (ks >= a.nks) { ks -= a.nks; ++tl; }
@@ -238,7 +262,7 @@ xnor_res_kernel(const __grid_constant__ StackMaps maps, const __grid_constant__ 
     // kernel before it writes; it waits (pdl_wait, below) before it touches the frames.
     pdl_trigger();
 
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int warp = warp_index(), lane = threadIdx.x & 31;
     const int kw = words_for(K);
     const int nks = ceil_div(K, BK);
     const int m_tiles = ceil_div(M, BM), n_tiles = ceil_div(N, BN);
@@ -246,13 +270,13 @@ xnor_res_kernel(const __grid_constant__ StackMaps maps, const __grid_constant__ 
     const int nt = (int)blockIdx.x % n_tiles, n0 = nt * BN;
 
     if (threadIdx.x == 0) {
-        for (int s = 0; s < C::A_STAGES; ++s) {
+        for (int s = 0; s < C::A_BARS; ++s) {
             mbar_init(smem_u32(&ctl->full_a[s]), A_WARPS);
             mbar_init(smem_u32(&ctl->empty_a[s]), 1);
         }
-        for (int s = 0; s < MAX_NKS; ++s) {
+        for (int s = 0; s < C::SLOTS; ++s) {
             mbar_init(smem_u32(&ctl->full_b[s]), 1);   // the copying thread (+ bytes)
-            mbar_init(smem_u32(&ctl->b_free[s]), 1);   // the MMA thread's commit
+            mbar_init(smem_u32(&ctl->b_free[s]), 2);   // one commit of each issuing warp
         }
         for (int b = 0; b < 2; ++b) {
             mbar_init(smem_u32(&ctl->acc_full[b]), 2);       // one commit of each issuing warp
@@ -261,7 +285,7 @@ xnor_res_kernel(const __grid_constant__ StackMaps maps, const __grid_constant__ 
         }
         for (int b = 0; b < GROUPS; ++b) {
             mbar_init(smem_u32(&ctl->group_full[b]), 1);              // the issuing thread (+ bytes)
-            mbar_init(smem_u32(&ctl->group_empty[b]), 2 * A_WARPS);   // per stage of the group, every warp of its team
+            mbar_init(smem_u32(&ctl->group_empty[b]), 2 * A_WARPS);   // every warp of both teams
         }
         wait_state_init(&ctl->wait, g.status);
         mbar_init_fence();
@@ -287,126 +311,158 @@ xnor_res_kernel(const __grid_constant__ StackMaps maps, const __grid_constant__ 
     __syncthreads();
     tc_fence_after_sync();
 
-    if (warp == TMA_WARP) {
-        // ---------------- one thread: per layer the weight slice, then the staging ring of frame rows
+    if (warp == WEIGHT_WARP) {
+        // ---------------- one thread: the weight stages of all layers, in a ring of as many stages as fit.  The weights
+        // do not depend on the kernel before this one in the stream nor on other CTAs, so with narrow tiles the next
+        // layer's arrive while this one runs; a slot is overwritten once the MMAs of this CTA's last frame
+        // tile that read it have completed.
         if (lane == 0 && share.count > 0) {
-            const uint32_t stg = smem_u32(smem) + B_REGION;
-            const int ng = ceil_div(nks, 2);
             const size_t run = (size_t)xnor_image_npad(N) * 16;   // bytes between chunks of the image
-            int gc = 0;   // groups issued so far, over all layers: slot gc % GROUPS, < GROUPS ahead of its consumers
-            int gl = 0, gt = 0, gi = 0;   // the next group to issue: layer, index of the frame tile, group inside the tile
+            int slot = 0;
+            uint32_t ph = 1;      // parity to wait for on `b_free`: a fresh barrier passes parity 1
             bool ok = true;
-            auto issue_group = [&]() {
-                const int mt = share.first + gt * share.step;
-                if (gi == 0 && gl > 0) {
-                    // the frame tile's bits of the layer before: every unit tile's CTA has stored them
-                    ok = wait_counter(g.progress + (size_t)(gl - 1) * m_tiles + mt, n_tiles, abort_flag);
-                    if (!ok) return;
-                    asm volatile("fence.proxy.async;" ::: "memory");   // generic-proxy writes of other CTAs -> this thread's TMA reads
-                }
-                const int slot = gc % GROUPS;
-                if (gc >= GROUPS) {
-                    ok = mbar_wait_relaxed(smem_u32(&ctl->group_empty[slot]), (uint32_t)(((gc / GROUPS) - 1) & 1), abort_flag);
-                    if (!ok) return;
-                }
-                const uint32_t bar = smem_u32(&ctl->group_full[slot]);
-                mbar_arrive_expect_tx(bar, GROUP_BYTES);
-                tma_load_2d(stg + slot * GROUP_BYTES, &maps.m[gl], gi * 16, mt * BM, bar);
-                ++gc;
-                if (++gi == ng) { gi = 0; if (++gt == share.count) { gt = 0; ++gl; } }
-            };
             for (int l = 0; l < L && ok; ++l) {
-                // A later layer's first frame rows go into the staging ring before its weights: the
-                // producers widen them into tensor memory while the weight stages arrive.
-                if (l > 0)
-                    for (int i = 0; i < GROUPS && gl == l && ok; ++i) issue_group();
-                if (!ok) break;
-                // The weights do not depend on the kernel before this one in the stream (layer 0) nor on
-                // other CTAs (later layers).  A stage of the previous layer's slice is overwritten once
-                // the MMAs of this CTA's last frame tile that read it have completed.
                 const uint8_t* src = g.layer[l].img + (size_t)n0 * 16;
-                for (int ks = 0; ks < nks && ok; ++ks) {
-                    if (l > 0) ok = mbar_wait(smem_u32(&ctl->b_free[ks]), (uint32_t)((l - 1) & 1), abort_flag);
+                for (int ks = 0; ks < nks; ++ks) {
+                    ok = mbar_wait(smem_u32(&ctl->b_free[slot]), ph, abort_flag);
                     if (!ok) break;
-                    const uint32_t bar = smem_u32(&ctl->full_b[ks]);
+                    const uint32_t bar = smem_u32(&ctl->full_b[slot]);
                     mbar_arrive_expect_tx(bar, C::B_BYTES);
 #pragma unroll
                     for (int c = 0; c < 8; ++c)
-                        bulk_g2s(smem_u32(smem + ks * C::B_BYTES + c * (BN * 16)), src + (size_t)(ks * 8 + c) * run, BN * 16, bar);
+                        bulk_g2s(smem_u32(smem + slot * C::B_BYTES + c * (BN * 16)), src + (size_t)(ks * 8 + c) * run, BN * 16, bar);
+                    if (++slot == C::SLOTS) { slot = 0; ph ^= 1u; }
                 }
-                if (!ok) break;
-                // the frames of layer 0 are the previous kernel's output: wait until that kernel has
-                // completed and its writes are visible (returns at once when there is no such dependency)
-                if (l == 0) pdl_wait();
-                while (gl == l && ok) issue_group();
             }
+        }
+        __syncwarp();
+    } else if (warp == TMA_WARP) {
+        // ---------------- one thread: the staging ring of frame rows
+        if (lane == 0 && share.count > 0) {
+            const uint32_t stg = smem_u32(smem) + B_REGION;
+            const int ng = ceil_div(nks, 2);
+            int gc = 0;   // groups issued so far, over all layers: slot gc % GROUPS, < GROUPS ahead of its consumers
+            bool ok = true;
+            // the frames of layer 0 are the previous kernel's output: wait until that kernel has
+            // completed and its writes are visible (returns at once when there is no such dependency)
+            pdl_wait();
+            for (int l = 0; l < L && ok; ++l)
+                for (int t = 0; t < share.count && ok; ++t) {
+                    const int mt = share.first + t * share.step;
+                    if (l > 0) {
+                        // the frame tile's bits of the layer before: every unit tile's CTA has stored them
+                        ok = wait_counter(g.progress + (size_t)(l - 1) * m_tiles + mt, n_tiles * EPI_WARPS, abort_flag);
+                        if (!ok) break;
+                        asm volatile("fence.proxy.async;" ::: "memory");   // generic-proxy writes of other CTAs -> this thread's TMA reads
+                    }
+                    for (int gi = 0; gi < ng; ++gi, ++gc) {
+                        const int slot = gc % GROUPS;
+                        if (gc >= GROUPS) {
+                            ok = mbar_wait_relaxed(smem_u32(&ctl->group_empty[slot]), (uint32_t)(((gc / GROUPS) - 1) & 1), abort_flag);
+                            if (!ok) break;
+                        }
+                        const uint32_t bar = smem_u32(&ctl->group_full[slot]);
+                        mbar_arrive_expect_tx(bar, GROUP_BYTES);
+                        tma_load_2d(stg + slot * GROUP_BYTES, &maps.m[l], gi * 16, mt * BM, bar);
+                    }
+                }
         }
         __syncwarp();
     } else if (warp >= PROD_WARP0 && warp < TMA_WARP) {
         // the layers follow one another in the producers' sequence of (tile, stage) pairs
-        ProducerArgs pa{smem_u32(smem) + B_REGION, tmem + C::TMEM_A_COL, ctl, abort_flag, L * share.count, nks, kw, tail_mask(K), lane, zo};
-        produce_a<C::A_STAGES>(pa, (warp & 3) * 32 + lane, (warp - PROD_WARP0) / A_WARPS);
+        ProducerArgs pa{smem_u32(smem) + B_REGION, tmem + C::TMEM_A_COL, ctl, abort_flag, L * share.count, nks, kw, tail_mask(K), lane};
+        const int row = (warp & 3) * 32 + lane, team = (warp - PROD_WARP0) / A_WARPS;
+        const bool ragged = (kw % 8 != 0) || pa.tmask != 0xFFFFFFFFu;   // last stage has positions >= K
+        auto go = [&](auto odd, auto zero_one) {
+            constexpr bool ODD = decltype(odd)::value, ZO = decltype(zero_one)::value;
+            if (ragged) produce_a<C::A_STAGES, C::A_BARS, ODD, ZO, true>(pa, row, team);
+            else produce_a<C::A_STAGES, C::A_BARS, ODD, ZO, false>(pa, row, team);
+        };
+        using T = std::true_type;
+        using F = std::false_type;
+        if (nks & 1) zo ? go(T{}, T{}) : go(T{}, F{});
+        else zo ? go(F{}, T{}) : go(F{}, F{});
     } else if (warp == MMA_WARP || warp == MMA_WARP2) {
-        // ---------------- MMA issue: two warps, one issuing lane each; the warps stay converged and the
-        // MMAs and commits are predicated on lane 0.  A tile's stages go to the two warps in turn, and both
+        // ---------------- MMA issue: two converged warps.  A tile's stages go to the two warps in turn, and both
         // accumulate into the tile's accumulator: the sums are exact integers (|sum| <= K < 2^24), so the
         // order of the accumulations does not matter.  Only the stage that overwrites the accumulator has
-        // to come first: warp 0 commits its first MMA of a tile to `started`, and warp 1 waits for that
-        // before its first MMA of the tile.  (Measured on B200: what an issuing thread does between MMAs
-        // -- polls, commits, bookkeeping -- is time the tensor pipe idles; with two issuers one thread's
-        // waits overlap the other's MMAs.  2 % off the WSJ-scale step against one issuer that takes the
-        // stages in pairs; two issuers taking pairs, and a deeper ring of narrower tiles, gained less.)
+        // to come first: the warp that takes it commits it to `started`, and the other one waits for that
+        // before its first MMA of the tile (the same one for every tile of an accumulator, whether nks is even or odd).  (Measured on B200: what an issuing warp does between MMAs
+        // -- polls, commits, bookkeeping -- is time the tensor pipe idles unless the other warp fills it.  The four MMAs of
+        // a stage go out together from one elected lane, see elect_one: five 3072-wide layers of 65536 frames 1.53 ->
+        // 1.35 ms against MMAs predicated on lane 0.)
         {
             const int w = warp == MMA_WARP ? 0 : 1;
-            const uint32_t issue = lane == 0;
             constexpr uint32_t idesc = instr_desc_mxf4(BM, BN);
             const uint32_t sfa = tmem + C::TMEM_SF_COL, sfb = tmem + C::TMEM_SF_COL + SF_COLS / 2;
-            const uint64_t desc0 = smem_desc_kmajor(smem_u32(smem), BN * 16, 128);
+            const uint64_t desc = smem_desc_kmajor(smem_u32(smem), BN * 16, 128);
+            const uint32_t desc_lo = (uint32_t)desc, desc_hi = (uint32_t)(desc >> 32);
             constexpr uint32_t kStepJ = (2 * BN * 16) >> 4, kStepS = C::B_BYTES >> 4;
             const uint32_t tmem_a = tmem + C::TMEM_A_COL;
             bool ok = true;
             int tl = 0;          // tiles so far, over all layers
-            int it_base = 0;     // stages before this tile, over all layers
+            int sa = w, ba = w;  // slot of the A ring and barrier of this warp's next stage, and that barrier's parity
+            uint32_t pa = 0;
+            int slot0 = 0;       // slot of the layer's first weight stage; its stages follow round the ring
+            uint32_t pb0 = 0;    // parity of `full` there
+            int turn = w;        // this warp's first stage of the tile: stages go to the two warps in turn, across tiles
             for (int l = 0; l < L && ok; ++l) {
-                const uint32_t pb = (uint32_t)(l & 1);   // a layer's weight stages arrive once and then stay
-                for (int t = 0; t < share.count && ok; ++t, ++tl, it_base += nks) {
-                    const bool first = t == 0;
-                    const bool hand_over = t == share.count - 1 && l + 1 < L;   // the next layer's slice follows
+                // A layer's weight stages arrive once and then stay; the last tile hands back a slot that is to be
+                // refilled.  Both warps see every phase of these barriers, whoever takes the stage.
+                const int later = (L - 1 - l) * nks;
+                for (int t = 0; t < share.count && ok; ++t, ++tl) {
+                    const bool first = t == 0, last = t == share.count - 1;
                     const int b = tl & 1;
-                    ok = mbar_wait(smem_u32(&ctl->acc_empty[b]), (uint32_t)(((tl >> 1) & 1) ^ 1), abort_flag);
+                    ok = warp_wait(smem_u32(&ctl->acc_empty[b]), (uint32_t)(((tl >> 1) & 1) ^ 1), abort_flag, lane);
                     if (!ok) break;
                     tc_fence_after_sync();
                     const uint32_t d = tmem + (uint32_t)(b * BN);
-                    for (int ks = w; ks < nks; ks += 2) {
-                        const int it = it_base + ks;             // this stage in the CTA's sequence: slot and parity of the A ring
-                        const int sa = it % C::A_STAGES;
-                        const uint32_t pa = (uint32_t)((it / C::A_STAGES) & 1);
-                        ok = (!first || mbar_wait(smem_u32(&ctl->full_b[ks]), pb, abort_flag)) &&
-                             mbar_wait(smem_u32(&ctl->full_a[sa]), pa, abort_flag) &&
-                             (ks != 1 || mbar_wait(smem_u32(&ctl->started[b]), (uint32_t)((tl >> 1) & 1), abort_flag));
+                    for (int ks = first || last ? 0 : turn; ks < nks; ++ks) {
+                        int slot = slot0 + ks;
+                        const uint32_t wrapped = slot >= C::SLOTS ? 1u : 0u;
+                        if (wrapped) slot -= C::SLOTS;
+                        const bool hand_over = last && later + nks - ks > C::SLOTS;
+                        if (first) {
+                            ok = warp_wait(smem_u32(&ctl->full_b[slot]), pb0 ^ wrapped, abort_flag, lane);
+                            if (!ok) break;
+                        }
+                        if ((ks & 1) != turn) {
+                            if (hand_over && elect_one()) mma_commit(smem_u32(&ctl->b_free[slot]));
+                            continue;
+                        }
+                        ok = warp_wait(smem_u32(&ctl->full_a[ba]), pa, abort_flag, lane) &&
+                             (ks != 1 || warp_wait(smem_u32(&ctl->started[b]), (uint32_t)((tl >> 1) & 1), abort_flag, lane));
                         if (!ok) break;
                         tc_fence_after_sync();
-                        // descriptor of stage ks, chunk pair 0; the address field (16-byte units) of the others is
-                        // reached by plain additions: the whole region lies below 2^14 * 16 bytes
-                        const uint64_t db = desc0 + (uint64_t)((uint32_t)ks * kStepS);
+                        // the address field (16-byte units) is advanced by plain additions: the whole region lies
+                        // below 2^14 * 16 bytes.  An MMA takes 64 positions of K = 32 bytes: 8 columns of A, two
+                        // 16-byte chunks of B
+                        const uint32_t db = desc_lo + (uint32_t)slot * kStepS;
                         const uint32_t ta = tmem_a + sa * A_COLS;
-#pragma unroll
-                        for (int j = 0; j < BK / 64; ++j) {  // 64 positions of K = 32 bytes: 8 columns of A, two 16-byte chunks of B
-                            mma_mxf4_ts_if(issue, d, ta + 8 * j, db + j * kStepJ, idesc, sfa, sfb, (ks | j) != 0);
-                            if (j == 0 && ks == 0) mma_commit_if(issue, smem_u32(&ctl->started[b]));
+                        if (elect_one()) {
+                            mma_mxf4_ts(d, ta, db, desc_hi, idesc, sfa, sfb, ks != 0);
+                            if (ks == 0) mma_commit(smem_u32(&ctl->started[b]));
+                            mma_mxf4_ts(d, ta + 8, db + kStepJ, desc_hi, idesc, sfa, sfb, 1u);
+                            mma_mxf4_ts(d, ta + 16, db + 2 * kStepJ, desc_hi, idesc, sfa, sfb, 1u);
+                            mma_mxf4_ts(d, ta + 24, db + 3 * kStepJ, desc_hi, idesc, sfa, sfb, 1u);
+                            mma_commit(smem_u32(&ctl->empty_a[ba]));
+                            if (hand_over) mma_commit(smem_u32(&ctl->b_free[slot]));
                         }
-                        mma_commit_if(issue, smem_u32(&ctl->empty_a[sa]));
-                        if (hand_over) mma_commit_if(issue, smem_u32(&ctl->b_free[ks]));
+                        if ((sa += 2) >= C::A_STAGES) sa -= C::A_STAGES;
+                        if ((ba += 2) >= C::A_BARS) { ba -= C::A_BARS; pa ^= 1u; }
+                        if (!(first || last)) ++ks;      // the next one is the other warp's
                     }
-                    if (ok) mma_commit_if(issue, smem_u32(&ctl->acc_full[b]));
+                    if (ok && elect_one()) mma_commit(smem_u32(&ctl->acc_full[b]));
+                    turn ^= nks & 1;
                 }
+                slot0 += nks;
+                if (slot0 >= C::SLOTS) { slot0 -= C::SLOTS; pb0 ^= 1u; }
             }
         }
         __syncwarp();
     } else {
         // ---------------- epilogue: 128 threads, thread = one frame (TMEM lane)
         const int row_in_tile = warp * 32 + lane;
-        const float magic = __int_as_float(kMagicBits);
         bool ok = true;
         int tl = 0;              // tiles so far, over all layers
         for (int l = 0; l < L && ok; ++l) {
@@ -419,7 +475,7 @@ xnor_res_kernel(const __grid_constant__ StackMaps maps, const __grid_constant__ 
 #pragma unroll
             for (int h = 0; h < 2; ++h) {
                 const int nl = row_in_tile + h * 128, n = n0 + nl;
-                if (nl < BN) ctl->T[nl] = kMagicBits + (n < N ? thr[n] : 0);
+                if (nl < BN) ctl->T[nl] = n < N ? (float)thr[n] : 0.0f;
             }
             if (row_in_tile < BN / 32) {
                 const int wi = (n0 >> 5) + row_in_tile;
@@ -437,49 +493,56 @@ xnor_res_kernel(const __grid_constant__ StackMaps maps, const __grid_constant__ 
                 const uint32_t taddr = tmem + ((uint32_t)(warp * 32) << 16) + (uint32_t)(b * BN);
                 const int nw = words_for(N), w0 = n0 >> 5;
                 uint32_t* dst = out_bits + (size_t)(m < M ? m : 0) * ldob + w0;
-                const bool whole = w0 + BN / 32 <= nw;   // rows are 16-byte aligned and BN/32 is even: 8-byte stores
+                uint32_t acc[32], held = 0u;
+                tmem_ld32(taddr, acc);
 #pragma unroll
-                for (int gp = 0; gp < BN / 64; ++gp) {
-                    uint32_t pair[2];
+                for (int gq = 0; gq < BN / 32; ++gq) {
+                    tmem_ld_wait();
+                    // The accumulator holds the integer dot product as a float, and so does T the threshold: the
+                    // sign of their difference is the decision.  The sign bits are shifted in from the top, the last
+                    // element first, so element j ends up in bit j, inverted; four chains of eight, joined at the end
+                    uint32_t part[4] = {0u, 0u, 0u, 0u};
 #pragma unroll
-                    for (int h = 0; h < 2; ++h) {
-                        const int gq = 2 * gp + h;
-                        uint32_t acc[32];
-                        tmem_ld32(taddr + gq * 32, acc);
-                        tmem_ld_wait();
-                        // The accumulator holds the integer dot product as a float; adding 1.5 * 2^23
-                        // leaves that integer, offset by kMagicBits, in the bit pattern of the sum.
-                        // bit = (dot - thr >= 0); the sign bits are shifted in from the top, element 31
-                        // first, so element j ends up in bit j, inverted.
-                        uint32_t wd = 0u;
+                    for (int j = 7; j >= 0; --j)
 #pragma unroll
-                        for (int j = 31; j >= 0; --j)
-                            wd = __funnelshift_l((uint32_t)(__float_as_int(__uint_as_float(acc[j]) + magic) - ctl->T[gq * 32 + j]), wd, 1);
-                        wd = ~wd ^ ctl->flipw[gq];
-                        const int valid = N - (n0 + gq * 32);  // columns of this word that exist
-                        if (valid < 32) wd = valid > 0 ? (wd & ((1u << valid) - 1u)) : 0u;
-                        pair[h] = wd;
+                        for (int c = 0; c < 4; ++c)
+                            part[c] = __funnelshift_l(__float_as_uint(__uint_as_float(acc[8 * c + j]) - ctl->T[gq * 32 + 8 * c + j]), part[c], 1);
+                    if (gq + 1 < BN / 32) {
+                        tmem_ld32(taddr + (gq + 1) * 32, acc);
+                    } else {
+                        // the accumulator is read: the MMA warps may start the tile after the next on it
+                        tc_fence_before_sync();
+                        __syncwarp();
+                        if (lane == 0) mbar_arrive(smem_u32(&ctl->acc_empty[b]));
                     }
-                    if (m < M) {
-                        if (whole) {
-                            reinterpret_cast<uint2*>(dst)[gp] = make_uint2(pair[0], pair[1]);
+                    uint32_t wd = __byte_perm(__byte_perm(part[0], part[1], 0x0040), __byte_perm(part[2], part[3], 0x0040), 0x5410);
+                    wd = ~wd ^ ctl->flipw[gq];
+                    const int valid = N - (n0 + gq * 32);  // columns of this word that exist
+                    if (valid < 32) wd = valid > 0 ? (wd & ((1u << valid) - 1u)) : 0u;
+                    if (BN % 64 == 0) {      // rows are 16-byte aligned and BN / 32 is even: 8-byte stores
+                        if (gq & 1) {
+                            if (m < M) {
+                                if (w0 + gq < nw) *reinterpret_cast<uint2*>(dst + gq - 1) = make_uint2(held, wd);
+                                else if (w0 + gq - 1 < nw) dst[gq - 1] = held;
+                            }
                         } else {
-                            if (w0 + 2 * gp < nw) dst[2 * gp] = pair[0];
-                            if (w0 + 2 * gp + 1 < nw) dst[2 * gp + 1] = pair[1];
+                            held = wd;
                         }
+                    } else if (m < M && w0 + gq < nw) {
+                        dst[gq] = wd;
                     }
                 }
-                tc_fence_before_sync();
-                __syncwarp();
-                if (lane == 0) mbar_arrive(smem_u32(&ctl->acc_empty[b]));
                 if (l + 1 < L) {
-                    // this CTA's share of frame tile mt is stored: tell the CTAs that read it in the next layer
-                    __threadfence();
-                    epi_bar_sync();
-                    if (threadIdx.x == 0) {
+                    // this warp's share of frame tile mt is stored: tell the CTAs that read it in the next layer.  The
+                    // fence (about 1200 clocks) covers what the lanes stored before the warp barrier; no barrier
+                    // over the four warps, and the count itself needs no second fence.
+                    __syncwarp();
+                    if (lane == 0) {
+                        __threadfence();
                         asm volatile("fence.proxy.async;" ::: "memory");
-                        asm volatile("red.release.gpu.global.add.s32 [%0], 1;" ::"l"(g.progress + (size_t)l * m_tiles + mt) : "memory");
+                        asm volatile("red.relaxed.gpu.global.add.s32 [%0], 1;" ::"l"(g.progress + (size_t)l * m_tiles + mt) : "memory");
                     }
+                    __syncwarp();
                 }
             }
         }
@@ -528,20 +591,35 @@ int launch_bn(const uint32_t* Ap, int ldap, const XnorStackLayer* layers, int n_
 
 }  // namespace
 
-// Units per tile for a layer of this shape, or 0 when the kernel does not apply: the slice of
-// a tile must fit the shared-memory region, and every unit tile needs a CTA of its own.
-static int tile_units(int N, int K, int sm_count) {
-    const int nks = ceil_div(K, BK);
-    const int bn = nks <= Cfg<192>::NKS ? 192 : (nks <= Cfg<128>::NKS ? 128 : 0);
-    if (bn == 0 || ceil_div(N, bn) > sm_count) return 0;
-    return bn;
+// Units per tile for a layer of this shape, or 0 when the kernel does not apply: the stages of a layer must fit the
+// shared-memory region, and every unit tile needs a CTA of its own.  Of the tiles that fit the one with the least estimated
+// time per layer: the stages of the busiest CTA's frame tiles (clocks as measured), and where the region does not hold the
+// next layer's weights beside this one's what their reload adds.  Wide tiles win for large batches (fewer, fuller MMAs),
+// narrow ones where there are too few frame tiles for all SMs.  Measured on B200, four 2048-wide layers, microseconds with
+// 192 / 128 / 96 / 32 units: 100 frames 29.5 / 27.3 / 27.0 / 25.5, 731 frames 30.4 / 28.5 / 28.8 / 33.5, 2000 frames
+// 35.4 / 33.8 / 37.3 / 71, 4000 frames 43 / 47 / 62 / 128.
+static int tile_units(int M, int N, int K, int sm_count) {
+    const int nks = ceil_div(K, BK), m_tiles = ceil_div(M, BM);
+    if (nks > Cfg<128>::SLOTS) return 0;
+    struct Candidate { int bn, slots, stage; };
+    const Candidate all[] = {{192, Cfg<192>::SLOTS, 480}, {128, Cfg<128>::SLOTS, 460}, {96, Cfg<96>::SLOTS, 450}, {32, Cfg<32>::SLOTS, 400}};
+    int best = 0;
+    long long best_cost = 0;
+    for (const Candidate& c : all) {
+        const int n_tiles = ceil_div(N, c.bn);
+        if (nks > c.slots || n_tiles > sm_count) continue;
+        const int peers = sm_count / n_tiles;
+        const long long cost = (long long)ceil_div(m_tiles, peers) * nks * c.stage + (2 * nks <= c.slots ? 0 : c.bn * nks * 2 / 3);
+        if (best == 0 || cost < best_cost) { best = c.bn; best_cost = cost; }
+    }
+    return best;
 }
 
 static int sm_count_of_device() { return device_sm_count(); }
 
 bool xnor_res_applicable(int N, int K) {
     const int sms = sm_count_of_device();
-    return sms > 0 && tile_units(N, K, sms) != 0;
+    return sms > 0 && tile_units(BM, N, K, sms) != 0;
 }
 
 size_t xnor_stack_sync_bytes(int M, int n_layers) {
@@ -553,9 +631,11 @@ int launch_xnor_stack(const uint32_t* Ap, int ldap, const XnorStackLayer* layers
     const int sms = sm_count_of_device();
     if (sms <= 0) return BNN_ERR_CUDA;
     if (n_layers < 1 || n_layers > kXnorStackMax || (n_layers > 1 && (N != K || !progress))) return BNN_ERR_UNSUPPORTED;
-    const int bn = tile_units(N, K, sms);
+    const int bn = tile_units(M, N, K, sms);
     if (bn == 192) return launch_bn<192>(Ap, ldap, layers, n_layers, M, N, K, ldob, zo, progress, chained, sms, st);
     if (bn == 128) return launch_bn<128>(Ap, ldap, layers, n_layers, M, N, K, ldob, zo, progress, chained, sms, st);
+    if (bn == 96) return launch_bn<96>(Ap, ldap, layers, n_layers, M, N, K, ldob, zo, progress, chained, sms, st);
+    if (bn == 32) return launch_bn<32>(Ap, ldap, layers, n_layers, M, N, K, ldob, zo, progress, chained, sms, st);
     return BNN_ERR_UNSUPPORTED;
 }
 

@@ -1,0 +1,50 @@
+"""The run of binary hidden layers with resident weights, over the tile widths it chooses from (by frames and layer
+size), even and odd numbers of stages of 256 positions, rings of weight stages that wrap inside a layer, ragged last stages
+and tiles: the bits of every layer against those of the kernel that streams the weights, one launch per layer."""
+import dataclasses
+
+import pytest
+
+from paper_1706_09453_b200 import workloads as wl
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def env():
+    import torch
+    assert torch.cuda.is_available()
+    from paper_1706_09453_b200 import build, binding, model
+    build.build()
+    return torch, binding, model
+
+
+@pytest.mark.parametrize("hidden,frames,values", [
+    (2048, 33, 0), (2048, 129, 1),       # 32 units a tile
+    (2048, 731, 0), (700, 300, 1),       # 96
+    (2048, 1100, 0), (3072, 2500, 0),    # 128
+    (2048, 5000, 1), (1800, 4500, 0),    # 192
+    (200, 4000, 0), (1300, 900, 1), (2300, 200, 0), (1290, 9000, 0),   # 1, 6, 9 and 6 stages, ragged
+    (1100, 9000, 1), (1100, 150, 0), (520, 12000, 0),                  # 5 and 3 stages, several frame tiles a block
+])
+def test_resident_run_equals_streamed_layers(env, hidden, frames, values):
+    torch, B, model = env
+    cfg = dataclasses.replace(wl.CONFIGS["tiny"], hidden=hidden, n_hidden=6, classes=64)
+    dn = model.DeviceNet(wl.make_model(cfg), act_values=values)
+    X = model.to_dev(wl.make_frames(cfg, frames))
+
+    def layers(kind):
+        prev = B.bnn_set_option(B.OPT_XNOR_PREPARED, kind)
+        try:
+            outs = dn.layer_out_buffers(frames)
+            dn.forward(X, layer_out=outs)
+            torch.cuda.synchronize()
+            return outs
+        finally:
+            B.bnn_set_option(B.OPT_XNOR_PREPARED, prev)
+
+    want, words = layers(B.PREPARED_STREAM), (hidden + 31) // 32
+    for _ in range(3):
+        for l, (a, b) in enumerate(zip(layers(B.PREPARED_RESIDENT), want)):
+            assert torch.equal(a[:, :words], b[:, :words]), "hidden layer %d" % (l + 1)
+    assert B.bnn_device_status() == 0
