@@ -150,6 +150,9 @@ int launch_pipe_rate(int which, int repeat, void* scratch, size_t scratch_bytes,
 // Tensor map of a packed operand [rows][ceil(K/32) words] of pitch `ld` words: boxes of 16 words x
 // box_rows rows, 64-byte swizzle, zero fill outside the tensor.  False when the encoder fails.
 bool encode_packed_map(CUtensorMap* map, const uint32_t* base, int ld, int rows, int K, int box_rows);
+// Tensor map of an int32 result [rows][cols] with pitch ld (a multiple of 4, base 16-byte aligned), for tile stores of
+// 32 rows x 32 columns; 128-byte swizzle.
+bool encode_int32_map(CUtensorMap* map, int32_t* base, int ld, int rows, int cols);
 // Tensor map of a digit image (digit_gemm.cuh): `chunks` rows of `rows` x 16 bytes, boxes of box_rows x 16 bytes x
 // box_chunks rows, zero fill outside.  Elements are 8 bytes (a box may have at most 256 of them).
 bool encode_digit_map(CUtensorMap* map, const void* base, int rows, int chunks, int box_rows, int box_chunks);

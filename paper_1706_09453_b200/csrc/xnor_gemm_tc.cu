@@ -19,17 +19,22 @@
 // w holds, in nibble i, bit 4i + t of w:   ((w << (3 - t)) & 0x88888888) ^ 0xAAAAAAAA
 // (sign bit = NOT the input bit, exponent field = 01).
 //
-// Roles in a CTA of 16 warps (persistent, one CTA per SM, tiles of 128 frames x 192 units):
-//   warp 15      one thread issues 2-D TMA tile loads of the packed rows (64 bytes per row =
+// Roles in a CTA of 27 warps (persistent, one CTA per SM, tiles of 128 frames x 192 units):
+//   warp 26      one thread issues 2-D TMA tile loads of the packed rows (64 bytes per row =
 //                two stages) into a staging ring (64-byte swizzle, no multicast)
-//   warps 5-8    widen the frame rows, thread = one row, 32 bytes -> 128 bytes per stage,
-//                written to tensor memory (the MMA reads its A operand from there)
-//   warps 9-14   widen the unit rows the same way into shared memory, two stages per iteration
-//   warp 4       one thread issues the MMAs (4 per stage, K = 64 each) and the commits
+//   warps 6-13   two teams widen the frame rows, thread = one row, 32 bytes -> 128 bytes per stage,
+//                written to tensor memory (the MMA reads its A operand from there); they take alternate stages
+//   warps 14-25  two teams widen the unit rows the same way into shared memory, two stages per iteration
+//   warps 4, 5   issue the MMAs (4 per stage, K = 64 each) and the commits; the two warps take the stages in turn
 //   warps 0-3    epilogue: accumulator -> Sign/threshold -> repacked bits (or int32 output);
 //                two accumulators in tensor memory, so it overlaps the next tile's MMAs
 // Every wait is bounded; a wait that runs out sets the CTA's abort flag, all roles fall
 // through to the common teardown and the device status word is set.
+//
+// What bounds it, measured on B200: the widening (two teams per operand; a stage takes about 720 clocks against 384
+// of MMA; with one team per operand, one issuing thread and the int32 tile written out by the epilogue warps it took
+// about 1000).  65536 x 4096 x 4096, int32 out, 646 -> 490 us; 4096 x 2048 x 4096 31 -> 26 us (its tiles have 8
+// stages, so the int32 epilogue counts there).
 #include "bnn_common.cuh"
 #include "tcgen05.cuh"
 #include "xnor_widen.cuh"
@@ -45,26 +50,30 @@ constexpr int BK = 256;                                   // bits of K per stage
 constexpr int ROW_BYTES = BK / 2;                         // widened bytes per row and stage (128)
 constexpr int B_BYTES = BN * ROW_BYTES, STAGE_BYTES = B_BYTES;   // only the unit operand lives in shared memory
 constexpr int A_STAGES = 3, B_STAGES = 4;               // rings of the frame operand (tensor memory) and the unit operand
-constexpr int EPI_WARPS = 4, MMA_WARP = 4, PROD_WARP0 = 5, A_WARPS = BM / 32, B_WARPS = BN / 32;
-constexpr int PROD_WARPS = A_WARPS + B_WARPS;
+// A stage `it` of the CTA's sequence has barrier it % A_BARS, an even number, so that a barrier always belongs to the same
+// team and issuing warp (a wait on a parity holds only for one who has seen every phase before it).
+constexpr int A_BARS = 2 * A_STAGES;
+static_assert(B_STAGES % 2 == 0, "a stage of units always belongs to the same issuing warp");
+constexpr int EPI_WARPS = 4, MMA_WARP = 4, MMA_WARP2 = 5, PROD_WARP0 = 6, TEAMS = 2, A_WARPS = BM / 32, B_WARPS = BN / 32;
+constexpr int PROD_WARPS = TEAMS * (A_WARPS + B_WARPS);
 constexpr int TMA_WARP = PROD_WARP0 + PROD_WARPS;
-constexpr int THREADS = (TMA_WARP + 1) * 32;              // 512
-constexpr int GROUPS = 4;                                 // staging ring: groups of two stages
+constexpr int THREADS = (TMA_WARP + 1) * 32;              // 864
+constexpr int GROUPS = 4;                                 // staging ring: groups of two stages (an odd last stage has an empty partner)
 constexpr int GA_BYTES = BM * 64, GB_BYTES = BN * 64, GROUP_BYTES = GA_BYTES + GB_BYTES;
 constexpr uint32_t TMEM_A_COL = 2 * BN;                   // A stages start after the two accumulators
 constexpr uint32_t A_COLS = ROW_BYTES / 4;                // 32-bit columns per A stage
 constexpr uint32_t TMEM_SF_COL = TMEM_A_COL + A_STAGES * A_COLS, SF_COLS = 32;   // block scales: 16 columns per operand
 constexpr uint32_t TMEM_COLS = 512;
 
-// With int32 output each epilogue warp needs two staging blocks of 32 rows x 128 bytes.
+// With int32 output each epilogue warp needs two staging blocks of 32 rows x 128 bytes (1024-byte aligned).
 template <bool STORE_C> struct Cfg {
-    static constexpr int CSTAGE_BYTES = STORE_C ? EPI_WARPS * 2 * 32 * 36 * 4 : 0;
+    static constexpr int CSTAGE_BYTES = STORE_C ? EPI_WARPS * 2 * 32 * 128 : 0;
 };
 
 struct Control {
     int T[BN];               // per unit: threshold + kMagicBits (Sign epilogue only)
     uint32_t flipw[BN / 32];
-    uint64_t full_a[A_STAGES], empty_a[A_STAGES], full_b[B_STAGES], empty_b[B_STAGES], acc_full[2], acc_empty[2];
+    uint64_t full_a[A_BARS], empty_a[A_BARS], full_b[B_STAGES], empty_b[B_STAGES], acc_full[2], acc_empty[2], started[2];
     uint64_t group_full[GROUPS], group_empty[GROUPS];
     uint32_t tmem_base;
     WaitState wait;
@@ -74,7 +83,6 @@ template <bool STORE_C> constexpr int smem_bytes() {
 }
 static_assert(smem_bytes<false>() <= 232448 && smem_bytes<true>() <= 232448, "shared memory of one CTA");
 static_assert(TMEM_SF_COL + SF_COLS <= TMEM_COLS, "tensor memory columns");
-static_assert(sizeof(Control) % 16 == 0, "the int32 staging blocks follow the control block");
 
 struct ProducerArgs {
     uint32_t smem;        // shared-space address of stage 0
@@ -84,21 +92,21 @@ struct ProducerArgs {
     int tiles, nks, kw;
     uint32_t tmask;
     int lane;
-    int zo;               // the frame operand's bits stand for (0,1) instead of (-1,+1)
 };
 
 // The eight 16-byte chunks of one widened row and stage; `ks` is the stage's index in the row.
-template <bool FRAMES>
-__device__ __forceinline__ void widen_stage(const ProducerArgs& a, bool ragged, int ks, const uint4& v0, const uint4& v1, uint4 (&o)[8]) {
+// ZO: the row's bits stand for (0,1) instead of (-1,+1); RAGGED: the last stage has positions >= K.
+template <bool ZO, bool RAGGED>
+__device__ __forceinline__ void widen_stage(const ProducerArgs& a, int ks, const uint4& v0, const uint4& v1, uint4 (&o)[8]) {
     const uint32_t w[8] = {v0.x, v0.y, v0.z, v0.w, v1.x, v1.y, v1.z, v1.w};
-    if (FRAMES && a.zo) {
+    if (ZO) {
 #pragma unroll
         for (int c = 0; c < 8; ++c) {
             const int g = 8 * ks + c;   // index of the word in the row
-            const uint32_t valid = (!ragged || g < a.kw - 1) ? 0xFFFFFFFFu : (g == a.kw - 1 ? a.tmask : 0u);
+            const uint32_t valid = (!RAGGED || g < a.kw - 1) ? 0xFFFFFFFFu : (g == a.kw - 1 ? a.tmask : 0u);
             o[c] = widen01_masked(w[c], valid);
         }
-    } else if (ragged && ks == a.nks - 1) {
+    } else if (RAGGED && ks == a.nks - 1) {
 #pragma unroll
         for (int c = 0; c < 8; ++c) {
             const int g = 8 * ks + c;   // index of the word in the row
@@ -111,31 +119,32 @@ __device__ __forceinline__ void widen_stage(const ProducerArgs& a, bool ragged, 
     }
 }
 
-// Producer of the frame operand: thread = row `r` of every tile of this CTA, one stage per
-// iteration, widened rows written to tensor memory (ring of A_STAGES stages).
-__device__ __forceinline__ void produce_a(const ProducerArgs& a, int r) {
+// Producer of the frame operand: thread = row `r` of every tile of this CTA; team `team` takes one of the two stages of every
+// group, widened rows written to tensor memory.
+// Template arguments say what the loops of the producers have to deal with: code that is there for another case costs this
+// one, though it is not executed.
+template <bool ZO, bool RAGGED>
+__device__ __forceinline__ void produce_a(const ProducerArgs& a, int r, int team) {
     Control* ctl = a.ctl;
     const int my_tiles = (a.tiles - 1 - (int)blockIdx.x) / (int)gridDim.x + 1;
-    const int total = my_tiles * a.nks;
+    const int ng = ceil_div(a.nks, 2), total = 2 * my_tiles * ng;
     // TMEM lane of this thread's frame row: a warp may only touch lanes 32*(warp%4)..+31
     const uint32_t tdst0 = a.tmem + ((uint32_t)(r & ~31) << 16) + TMEM_A_COL;
     // this row inside a staging group: 64 bytes per row, 16-byte chunk c stored at c ^ ((r/2)%4)
-    const uint32_t stg0 = a.smem + B_STAGES * STAGE_BYTES + r * 64;
     const uint32_t sw = (uint32_t)(r >> 1) & 3u;
-    const bool ragged = (a.kw % 8 != 0) || a.tmask != 0xFFFFFFFFu;   // last stage has positions >= K
-    int gslot = 0;
-    uint32_t gph = 0;
-    int ks = 0, s = 0;
-    uint32_t ph = 1;  // parity to wait for on `empty`: a fresh barrier passes parity 1
-    for (int it = 0; it < total; ++it) {
-        const uint32_t gi = (uint32_t)ks & 1u;   // stage inside its group of two
-        if (gi == 0 && !warp_wait(smem_u32(&ctl->group_full[gslot]), gph, a.abort_flag, a.lane)) break;
+    const uint32_t stg0 = a.smem + B_STAGES * STAGE_BYTES + r * 64 + (((2u * team) ^ (sw & 2u)) << 4);
+    const uint32_t lo = (sw & 1u) << 4;
+    int ks = team;
+    for (int it = team; it < total; it += TEAMS) {
+        const int g = it >> 1, gslot = g % GROUPS;
+        if (!warp_wait(smem_u32(&ctl->group_full[gslot]), (uint32_t)((g / GROUPS) & 1), a.abort_flag, a.lane)) break;
         const uint32_t src = stg0 + gslot * GROUP_BYTES;
-        const uint4 v0 = lds128u(src + (((2u * gi) ^ sw) << 4));
-        const uint4 v1 = lds128u(src + (((2u * gi + 1u) ^ sw) << 4));
-        if (!warp_wait(smem_u32(&ctl->empty_a[s]), ph, a.abort_flag, a.lane)) break;
+        const uint4 v0 = lds128u(src + lo), v1 = lds128u(src + (lo ^ 16u));
+        const int s = it % A_STAGES;
+        const int e = it + A_BARS - A_STAGES;          // the stage that had this slot; a fresh barrier passes parity 1
+        if (!warp_wait(smem_u32(&ctl->empty_a[e % A_BARS]), (uint32_t)(((e / A_BARS) & 1) ^ 1), a.abort_flag, a.lane)) break;
         uint4 o[8];
-        widen_stage<true>(a, ragged, ks, v0, v1, o);
+        widen_stage<ZO, RAGGED>(a, ks, v0, v1, o);
         // 32-bit column 4c + t of the stage = word t of chunk c: the byte order of the
         // K-major shared-memory layout of the other operand
         uint32_t wr[32];
@@ -145,89 +154,82 @@ __device__ __forceinline__ void produce_a(const ProducerArgs& a, int r) {
         tmem_st_wait();
         tc_fence_before_sync();
         __syncwarp();
-        if (a.lane == 0) mbar_arrive(smem_u32(&ctl->full_a[s]));
-        // The staging slot is handed back only here, after the stores that consumed the loaded
-        // words: a shared-memory load that has merely been issued does not hold back the TMA
-        // write that refills the slot (that write belongs to the async proxy; only the data
-        // dependency proves that the load has read its bytes).
-        if (gi == 1 || ks == a.nks - 1) {
-            if (a.lane == 0) mbar_arrive(smem_u32(&ctl->group_empty[gslot]));
-            if (++gslot == GROUPS) { gslot = 0; gph ^= 1u; }
+        if (a.lane == 0) {
+            mbar_arrive(smem_u32(&ctl->full_a[it % A_BARS]));
+            // The staging slot is handed back only here, after the stores that consumed the loaded
+            // words: a shared-memory load that has merely been issued does not hold back the TMA
+            // write that refills the slot (that write belongs to the async proxy; only the data
+            // dependency proves that the load has read its bytes).
+            mbar_arrive(smem_u32(&ctl->group_empty[gslot]));
         }
-        if (++s == A_STAGES) { s = 0; ph ^= 1u; }
-        if (++ks == a.nks) ks = 0;
+        ks += TEAMS;
+        if (ks >= 2 * ng) ks = team;
     }
 }
 
-// Producer of the unit operand: thread = row `r`, one staging group (two stages) per
-// iteration, so the fixed costs of an iteration (group wait, proxy fence, warp barrier,
-// release) are paid once per two stages; widened rows go to shared memory (ring of B_STAGES).
-__device__ __forceinline__ void produce_b(const ProducerArgs& a, int r) {
+// Producer of the unit operand: thread = row `r`; the teams take the staging groups in turn, two stages per
+// iteration, so the fixed costs of an iteration (group wait, proxy fence, warp barrier, release) are paid once per
+// two stages; widened rows go to shared memory, each team to its half of the ring.
+template <bool RAGGED>
+__device__ __forceinline__ void produce_b(const ProducerArgs& a, int r, int team) {
     Control* ctl = a.ctl;
     const int my_tiles = (a.tiles - 1 - (int)blockIdx.x) / (int)gridDim.x + 1;
-    const int ng = ceil_div(a.nks, 2);
-    const int total = my_tiles * ng;
-    const uint32_t dst0 = a.smem + r * 16;
+    const int ng = ceil_div(a.nks, 2), total = my_tiles * ng;
+    const int s = 2 * team;
+    const uint32_t dst0 = a.smem + s * STAGE_BYTES + r * 16;
     const uint32_t stg0 = a.smem + B_STAGES * STAGE_BYTES + GA_BYTES + r * 64;
     const uint32_t sw = (uint32_t)(r >> 1) & 3u;
-    const bool ragged = (a.kw % 8 != 0) || a.tmask != 0xFFFFFFFFu;
-    int gslot = 0;
-    uint32_t gph = 0;
-    int kg = 0, s = 0;
     uint32_t ph = 1;
-    for (int g = 0; g < total; ++g) {
-        const bool two = 2 * kg + 1 < a.nks;   // the last group of a row may hold a single stage
-        if (!warp_wait(smem_u32(&ctl->group_full[gslot]), gph, a.abort_flag, a.lane)) break;
+    int kg = team;
+    for (int g = team; g < total; g += TEAMS) {
+        while (kg >= ng) kg -= ng;
+        const int gslot = g % GROUPS;
+        if (!warp_wait(smem_u32(&ctl->group_full[gslot]), (uint32_t)((g / GROUPS) & 1), a.abort_flag, a.lane)) break;
         const uint32_t src = stg0 + gslot * GROUP_BYTES;
         const uint4 v0 = lds128u(src + ((0u ^ sw) << 4)), v1 = lds128u(src + ((1u ^ sw) << 4));
         const uint4 v2 = lds128u(src + ((2u ^ sw) << 4)), v3 = lds128u(src + ((3u ^ sw) << 4));
-        const int s2 = s + 1 == B_STAGES ? 0 : s + 1;
-        const uint32_t ph2 = s + 1 == B_STAGES ? ph ^ 1u : ph;
         if (!warp_wait(smem_u32(&ctl->empty_b[s]), ph, a.abort_flag, a.lane)) break;
         uint4 o[8];
-        widen_stage<false>(a, ragged, 2 * kg, v0, v1, o);
+        widen_stage<false, RAGGED>(a, 2 * kg, v0, v1, o);
 #pragma unroll
-        for (int c = 0; c < 8; ++c) sts128(dst0 + s * STAGE_BYTES + c * (BN * 16), o[c].x, o[c].y, o[c].z, o[c].w);
-        if (two) {
-            if (!warp_wait(smem_u32(&ctl->empty_b[s2]), ph2, a.abort_flag, a.lane)) break;
-            widen_stage<false>(a, ragged, 2 * kg + 1, v2, v3, o);
+        for (int c = 0; c < 8; ++c) sts128(dst0 + c * (BN * 16), o[c].x, o[c].y, o[c].z, o[c].w);
+        if (!warp_wait(smem_u32(&ctl->empty_b[s + 1]), ph, a.abort_flag, a.lane)) break;
+        widen_stage<false, RAGGED>(a, 2 * kg + 1, v2, v3, o);
 #pragma unroll
-            for (int c = 0; c < 8; ++c) sts128(dst0 + s2 * STAGE_BYTES + c * (BN * 16), o[c].x, o[c].y, o[c].z, o[c].w);
-        }
+        for (int c = 0; c < 8; ++c) sts128(dst0 + STAGE_BYTES + c * (BN * 16), o[c].x, o[c].y, o[c].z, o[c].w);
         fence_proxy_async_smem();
         __syncwarp();
         if (a.lane == 0) {
             mbar_arrive(smem_u32(&ctl->full_b[s]));
-            if (two) mbar_arrive(smem_u32(&ctl->full_b[s2]));
+            mbar_arrive(smem_u32(&ctl->full_b[s + 1]));
             mbar_arrive(smem_u32(&ctl->group_empty[gslot]));   // after the stores that consumed the loaded words (see produce_a)
         }
-        if (++gslot == GROUPS) { gslot = 0; gph ^= 1u; }
-        if (two) { s = s2; ph = ph2; }
-        if (++s == B_STAGES) { s = 0; ph ^= 1u; }
-        if (++kg == ng) kg = 0;
+        ph ^= 1u;
+        kg += TEAMS;
     }
 }
 
 template <bool STORE_C, bool SIGN_PACK>
 __global__ void __launch_bounds__(THREADS, 1)
 xnor_tc_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CUtensorMap mapB,
+                const __grid_constant__ CUtensorMap mapC, int tma_c,
                 int M, int N, int K, int32_t* __restrict__ C, int ldc,
                 const int32_t* __restrict__ thr, const uint32_t* __restrict__ flip,
                 uint32_t* __restrict__ out_bits, int ldob, int zo, TcStatus status) {
     extern __shared__ uint8_t smem_raw[];
     uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
-    Control* ctl = reinterpret_cast<Control*>(smem + B_STAGES * STAGE_BYTES + GROUPS * GROUP_BYTES);
-    int (*cstage)[2][32][36] = reinterpret_cast<int (*)[2][32][36]>(reinterpret_cast<uint8_t*>(ctl) + sizeof(Control));
+    const uint32_t cstage = smem_u32(smem) + B_STAGES * STAGE_BYTES + GROUPS * GROUP_BYTES;
+    Control* ctl = reinterpret_cast<Control*>(smem + B_STAGES * STAGE_BYTES + GROUPS * GROUP_BYTES + Cfg<STORE_C>::CSTAGE_BYTES);
     volatile int* abort_flag = &ctl->wait.abort;
 
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int warp = warp_index(), lane = threadIdx.x & 31;
     const int kw = words_for(K);
     const int nks = ceil_div(K, BK);
     const int m_tiles = ceil_div(M, BM), n_tiles = ceil_div(N, BN);
     const int tiles = m_tiles * n_tiles;
 
     if (threadIdx.x == 0) {
-        for (int s = 0; s < A_STAGES; ++s) {
+        for (int s = 0; s < A_BARS; ++s) {
             mbar_init(smem_u32(&ctl->full_a[s]), A_WARPS);
             mbar_init(smem_u32(&ctl->empty_a[s]), 1);
         }
@@ -236,12 +238,13 @@ xnor_tc_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_constant__
             mbar_init(smem_u32(&ctl->empty_b[s]), 1);
         }
         for (int b = 0; b < 2; ++b) {
-            mbar_init(smem_u32(&ctl->acc_full[b]), 1);
+            mbar_init(smem_u32(&ctl->acc_full[b]), 2);       // one commit of each issuing warp
+            mbar_init(smem_u32(&ctl->started[b]), 1);
             mbar_init(smem_u32(&ctl->acc_empty[b]), EPI_WARPS);
         }
         for (int b = 0; b < GROUPS; ++b) {
             mbar_init(smem_u32(&ctl->group_full[b]), 1);            // the issuing thread (+ bytes)
-            mbar_init(smem_u32(&ctl->group_empty[b]), PROD_WARPS);  // every producer warp has read it
+            mbar_init(smem_u32(&ctl->group_empty[b]), TEAMS * A_WARPS + B_WARPS);  // every warp that reads it
         }
         wait_state_init(&ctl->wait, status);
         mbar_init_fence();
@@ -268,7 +271,8 @@ xnor_tc_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_constant__
     tc_fence_after_sync();
 
     if (warp >= PROD_WARP0) {
-        ProducerArgs pa{smem_u32(smem), tmem, ctl, abort_flag, tiles, nks, kw, tail_mask(K), lane, zo};
+        ProducerArgs pa{smem_u32(smem), tmem, ctl, abort_flag, tiles, nks, kw, tail_mask(K), lane};
+        const bool ragged = (kw % 8 != 0) || pa.tmask != 0xFFFFFFFFu;   // the last stage has positions >= K
         if (warp == TMA_WARP) {
             // ---------------- one thread feeds the staging ring, a group of two stages at a time
             if (lane == 0) {
@@ -292,65 +296,63 @@ xnor_tc_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_constant__
                 }
             }
             __syncwarp();
-        } else if (warp < PROD_WARP0 + A_WARPS) {
-            produce_a(pa, (warp & 3) * 32 + lane);
+        } else if (warp < PROD_WARP0 + TEAMS * A_WARPS) {
+            const int row = (warp & 3) * 32 + lane, team = (warp - PROD_WARP0) / A_WARPS;
+            if (zo) ragged ? produce_a<true, true>(pa, row, team) : produce_a<true, false>(pa, row, team);
+            else ragged ? produce_a<false, true>(pa, row, team) : produce_a<false, false>(pa, row, team);
         } else {
-            produce_b(pa, (warp - PROD_WARP0 - A_WARPS) * 32 + lane);
+            const int pw = warp - PROD_WARP0 - TEAMS * A_WARPS, team = pw / B_WARPS, row = (pw - team * B_WARPS) * 32 + lane;
+            ragged ? produce_b<true>(pa, row, team) : produce_b<false>(pa, row, team);
         }
-    } else if (warp == MMA_WARP) {
-        // ---------------- MMA issue: one thread.  Two stages per iteration: whatever this thread
-        // does between two MMAs (polls, commits, bookkeeping) is time the tensor pipe idles, so
-        // the waits of two stages are taken together and their eight MMAs issued back to back.
-        if (lane == 0) {
-            constexpr uint32_t idesc = instr_desc_mxf4(BM, BN);
-            const uint32_t sfa = tmem + TMEM_SF_COL, sfb = tmem + TMEM_SF_COL + SF_COLS / 2;
-            const uint32_t smem0 = smem_u32(smem);
-            int sa = 0, sb = 0;        // ring slots and the parities their `full` barriers show next
-            uint32_t pa = 0, pb = 0;
-            int tl = 0;
-            bool ok = true;
-            auto issue = [&](uint32_t d, int slot_a, int slot_b, bool first) {
-                const uint32_t b0 = smem0 + slot_b * STAGE_BYTES;
-                const uint32_t ta = tmem + TMEM_A_COL + slot_a * A_COLS;
-#pragma unroll
-                for (int j = 0; j < BK / 64; ++j) {   // 64 positions of K = 32 bytes: 8 columns of A, two 16-byte chunks of B
-                    const uint64_t db = smem_desc_kmajor(b0 + 2 * j * (BN * 16), BN * 16, 128);
-                    mma_mxf4_ts(d, ta + 8 * j, db, idesc, sfa, sfb, !(first && j == 0));
-                }
-                mma_commit(smem_u32(&ctl->empty_a[slot_a]));
-                mma_commit(smem_u32(&ctl->empty_b[slot_b]));
-            };
-            for (int tile = blockIdx.x; tile < tiles && ok; tile += gridDim.x, ++tl) {
-                const int b = tl & 1;
-                ok = mbar_wait(smem_u32(&ctl->acc_empty[b]), (uint32_t)(((tl >> 1) & 1) ^ 1), abort_flag);
+    } else if (warp == MMA_WARP || warp == MMA_WARP2) {
+        // ---------------- MMA issue: two converged warps, which take the CTA's stages in turn and accumulate into the
+        // same accumulator (the sums are exact integers, so their order does not matter; only the stage that
+        // overwrites the accumulator has to come first, see `started`).  What an issuing warp does besides its
+        // MMAs (waits, commits) is time the tensor pipe idles unless the other warp fills it.
+        const int w = warp - MMA_WARP;
+        constexpr uint32_t idesc = instr_desc_mxf4(BM, BN);
+        const uint32_t sfa = tmem + TMEM_SF_COL, sfb = tmem + TMEM_SF_COL + SF_COLS / 2;
+        const uint64_t desc = smem_desc_kmajor(smem_u32(smem), BN * 16, 128);
+        const uint32_t desc_lo = (uint32_t)desc, desc_hi = (uint32_t)(desc >> 32);
+        constexpr uint32_t kStepJ = (2 * BN * 16) >> 4, kStepS = STAGE_BYTES >> 4;
+        int sa = w, ba = w, sb = w;     // this warp's next stage: slot of the A ring, its barrier, slot of the B ring
+        uint32_t pa = 0, pb = 0;        // ... and the parities the `full` barriers show next
+        int tl = 0;
+        bool ok = true;
+        for (int tile = blockIdx.x; tile < tiles && ok; tile += gridDim.x, ++tl) {
+            const int b = tl & 1;
+            ok = warp_wait(smem_u32(&ctl->acc_empty[b]), (uint32_t)(((tl >> 1) & 1) ^ 1), abort_flag, lane);
+            if (!ok) break;
+            tc_fence_after_sync();
+            const uint32_t d = tmem + (uint32_t)(b * BN);
+            for (int ks = w; ks < 2 * ceil_div(nks, 2); ks += 2) {
+                ok = warp_wait(smem_u32(&ctl->full_b[sb]), pb, abort_flag, lane) && warp_wait(smem_u32(&ctl->full_a[ba]), pa, abort_flag, lane) &&
+                     (ks != 1 || warp_wait(smem_u32(&ctl->started[b]), (uint32_t)((tl >> 1) & 1), abort_flag, lane));
                 if (!ok) break;
                 tc_fence_after_sync();
-                const uint32_t d = tmem + (uint32_t)(b * BN);
-                int ks = 0;
-                for (; ks + 1 < nks; ks += 2) {
-                    const int sa2 = sa + 1 == A_STAGES ? 0 : sa + 1, sb2 = sb + 1 == B_STAGES ? 0 : sb + 1;
-                    const uint32_t pa2 = sa + 1 == A_STAGES ? pa ^ 1u : pa, pb2 = sb + 1 == B_STAGES ? pb ^ 1u : pb;
-                    ok = mbar_wait(smem_u32(&ctl->full_b[sb]), pb, abort_flag) && mbar_wait(smem_u32(&ctl->full_b[sb2]), pb2, abort_flag) &&
-                         mbar_wait(smem_u32(&ctl->full_a[sa]), pa, abort_flag) && mbar_wait(smem_u32(&ctl->full_a[sa2]), pa2, abort_flag);
-                    if (!ok) break;
-                    tc_fence_after_sync();
-                    issue(d, sa, sb, ks == 0);
-                    issue(d, sa2, sb2, false);
-                    sa = sa2; pa = pa2; sb = sb2; pb = pb2;
-                    if (++sa == A_STAGES) { sa = 0; pa ^= 1u; }
-                    if (++sb == B_STAGES) { sb = 0; pb ^= 1u; }
-                }
-                if (ok && ks < nks) {   // odd number of stages: the last one alone
-                    ok = mbar_wait(smem_u32(&ctl->full_b[sb]), pb, abort_flag) && mbar_wait(smem_u32(&ctl->full_a[sa]), pa, abort_flag);
-                    if (ok) {
-                        tc_fence_after_sync();
-                        issue(d, sa, sb, ks == 0);
-                        if (++sa == A_STAGES) { sa = 0; pa ^= 1u; }
-                        if (++sb == B_STAGES) { sb = 0; pb ^= 1u; }
+                // the address field (16-byte units) is advanced by plain additions: the ring lies below 2^14 * 16
+                // bytes.  An MMA takes 64 positions of K = 32 bytes: 8 columns of A, two 16-byte chunks of B
+                const uint32_t db = desc_lo + (uint32_t)sb * kStepS;
+                const uint32_t ta = tmem + TMEM_A_COL + sa * A_COLS;
+                if (ks == nks) {        // the empty partner of an odd last stage
+                    if (elect_one()) {
+                        mma_commit(smem_u32(&ctl->empty_a[ba]));
+                        mma_commit(smem_u32(&ctl->empty_b[sb]));
                     }
+                } else if (elect_one()) {
+                    mma_mxf4_ts(d, ta, db, desc_hi, idesc, sfa, sfb, ks != 0);
+                    if (ks == 0) mma_commit(smem_u32(&ctl->started[b]));
+                    mma_mxf4_ts(d, ta + 8, db + kStepJ, desc_hi, idesc, sfa, sfb, 1u);
+                    mma_mxf4_ts(d, ta + 16, db + 2 * kStepJ, desc_hi, idesc, sfa, sfb, 1u);
+                    mma_mxf4_ts(d, ta + 24, db + 3 * kStepJ, desc_hi, idesc, sfa, sfb, 1u);
+                    mma_commit(smem_u32(&ctl->empty_a[ba]));
+                    mma_commit(smem_u32(&ctl->empty_b[sb]));
                 }
-                if (ok) mma_commit(smem_u32(&ctl->acc_full[b]));
+                if ((sa += 2) >= A_STAGES) sa -= A_STAGES;
+                if ((ba += 2) >= A_BARS) { ba -= A_BARS; pa ^= 1u; }
+                if ((sb += 2) >= B_STAGES) { sb -= B_STAGES; pb ^= 1u; }
             }
+            if (ok && elect_one()) mma_commit(smem_u32(&ctl->acc_full[b]));
         }
         __syncwarp();
     } else {
@@ -387,6 +389,12 @@ xnor_tc_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_constant__
                 uint32_t acc[32];
                 tmem_ld32(taddr + g * 32, acc);
                 tmem_ld_wait();
+                if (g + 1 == BN / 32) {
+                    // the accumulator is read: the MMA warps may start the tile after the next on it
+                    tc_fence_before_sync();
+                    __syncwarp();
+                    if (lane == 0) mbar_arrive(smem_u32(&ctl->acc_empty[b]));
+                }
                 const int nb = n0 + g * 32;
                 // The accumulator holds the integer dot product as a float; adding 1.5 * 2^23
                 // leaves that integer, offset by kMagicBits, in the bit pattern of the sum.
@@ -394,36 +402,49 @@ xnor_tc_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_constant__
 #pragma unroll
                 for (int j = 0; j < 32; ++j) q[j] = __float_as_int(__uint_as_float(acc[j]) + magic);
                 if (STORE_C) {
-                    // Each thread parks its 32 integers (128 bytes of one output row) in shared
-                    // memory; the warp then writes the 32 x 128-byte block with 16-byte stores in
-                    // which 8 consecutive lanes cover one row: every store instruction writes four
-                    // whole 128-byte lines.
-                    const bool vec_ok = (ldc % 4 == 0) && ((reinterpret_cast<uintptr_t>(C) & 15) == 0) && nb + 31 < N;
-                    if (vec_ok) {
-                        int (*blk)[36] = cstage[warp][g & 1];
-                        const uint32_t row_smem = smem_u32(&blk[lane][0]);
+                    // Each thread parks its 32 integers (128 bytes of one output row) in shared memory, 16-byte
+                    // chunk i at i ^ (row % 8).  One thread then has the 32 x 128-byte block stored, which goes on while
+                    // the warp turns to the next 32 columns.  (Measured on B200: written by the warp with 16-byte stores,
+                    // 8 lanes to a row, the epilogue took as long as 16 stages of MMAs.)
+                    // A tile store clips a row to 16 bytes, not to elements, and wants an aligned pitch.  Elsewhere the
+                    // warp writes the block a row at a time, and each row from the 32-byte sector its first
+                    // column lies in (from the block before) to the one of its last column, which is left to the next
+                    // block: every store but those at the tile's edges then covers whole sectors.  (4096 x 2048 x
+                    // 4095, microseconds: a thread a row 102, rows of 32 columns 68, whole sectors 57; 4096 columns 29.)
+                    const bool whole = tma_c && (nb + 31 < N || N % 4 == 0);
+                    const uint32_t blk = cstage + (uint32_t)((warp * 2 + (g & 1)) * 4096);
+                    if (lane == 0) bulk_wait_read<1>();      // the block's store of two rounds ago has read it
+                    __syncwarp();
 #pragma unroll
-                        for (int i = 0; i < 8; ++i)
-                            sts128(row_smem + 16 * i, (uint32_t)(q[4 * i] - kMagicBits), (uint32_t)(q[4 * i + 1] - kMagicBits),
-                                   (uint32_t)(q[4 * i + 2] - kMagicBits), (uint32_t)(q[4 * i + 3] - kMagicBits));
-                        __syncwarp();
-                        const int rr = lane >> 3, qq = lane & 7;
-                        const int mrow0 = m0 + warp * 32;
-#pragma unroll
-                        for (int i = 0; i < 8; ++i) {
-                            const int row = 4 * i + rr;
-                            const int4 v = *reinterpret_cast<const int4*>(&blk[row][4 * qq]);
-                            if (mrow0 + row < M)
-                                *reinterpret_cast<int4*>(C + (size_t)(mrow0 + row) * ldc + nb + 4 * qq) = v;
+                    for (int i = 0; i < 8; ++i)
+                        sts128(blk + lane * 128 + ((i ^ (lane & 7)) << 4), (uint32_t)(q[4 * i] - kMagicBits), (uint32_t)(q[4 * i + 1] - kMagicBits),
+                               (uint32_t)(q[4 * i + 2] - kMagicBits), (uint32_t)(q[4 * i + 3] - kMagicBits));
+                    if (whole) fence_proxy_async_smem();
+                    __syncwarp();
+                    if (whole) {
+                        if (lane == 0 && nb < N && m0 + warp * 32 < M) tma_store_2d(&mapC, nb, m0 + warp * 32, blk);
+                    } else if (nb < N) {
+                        const int rows = M - (m0 + warp * 32) < 32 ? M - (m0 + warp * 32) : 32;
+                        const bool tail = g + 1 == BN / 32 || nb + 32 >= N;     // the last block of the tile's row
+                        int32_t* dst = C + (size_t)(m0 + warp * 32) * ldc + nb;
+                        uint32_t at = (uint32_t)(reinterpret_cast<uintptr_t>(dst) >> 2);   // in words; its low bits count
+                        const uint32_t both = cstage + (uint32_t)(warp * 8192);
+#pragma unroll 4
+                        for (int r = 0; r < rows; ++r, dst += ldc, at += (uint32_t)ldc) {
+                            const int back = g == 0 ? 0 : (int)(at & 7u);       // columns of the block before that this store takes along
+                            const int lead = (int)(at & 7u) - back;             // the tile's first block starts inside a sector
+                            const int col = lane - back - lead;                 // from -7 to 31
+                            const uint32_t buf = both + (uint32_t)(((g & 1) ^ (col < 0)) * 4096) + r * 128;
+                            const uint32_t v = lds32u(buf + ((((uint32_t)col >> 2) & 7u) ^ ((uint32_t)r & 7u)) * 16 + (col & 3) * 4);
+                            if (col >= -back && nb + col < N) dst[col] = (int32_t)v;
+                            if (tail) {
+                                const int rest = col + 32;                      // the columns that stay over
+                                const uint32_t t = lds32u(both + (uint32_t)((g & 1) * 4096) + r * 128 + ((((uint32_t)rest >> 2) & 7u) ^ ((uint32_t)r & 7u)) * 16 + (rest & 3) * 4);
+                                if (rest < 32 && nb + rest < N) dst[rest] = (int32_t)t;
+                            }
                         }
-                        // the buffer is written again two blocks later: by then every lane has passed
-                        // the __syncwarp of the next block, i.e. has finished reading this one
-                    } else if (m < M) {
-                        int32_t* dst = C + (size_t)m * ldc + nb;
-#pragma unroll
-                        for (int j = 0; j < 32; ++j)
-                            if (nb + j < N) dst[j] = q[j] - kMagicBits;
                     }
+                    if (lane == 0) bulk_commit();            // (an empty group keeps the count)
                 }
                 if (SIGN_PACK) {
                     // bit = (dot - thr >= 0); the sign bits are shifted in from the top, element 31
@@ -437,9 +458,6 @@ xnor_tc_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_constant__
                     if (valid < 32) words[g] = valid > 0 ? (words[g] & ((1u << valid) - 1u)) : 0u;
                 }
             }
-            tc_fence_before_sync();
-            __syncwarp();
-            if (lane == 0) mbar_arrive(smem_u32(&ctl->acc_empty[b]));
             if (SIGN_PACK && m < M) {
                 const int nw = words_for(N), w0 = n0 >> 5;
                 uint32_t* dst = out_bits + (size_t)m * ldob + w0;
@@ -454,6 +472,7 @@ xnor_tc_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_constant__
                 }
             }
         }
+        if (STORE_C && lane == 0) bulk_wait<0>();
     }
 
     // ---------------- teardown: every thread arrives here, also after an aborted wait
@@ -483,7 +502,10 @@ int launch_variant(const uint32_t* Ap, int ldap, const uint32_t* Wp, int ldwp, i
     CUtensorMap mapA, mapB;
     if (!encode_packed_map(&mapA, Ap, ldap, M, K, BM) || !encode_packed_map(&mapB, Wp, ldwp, N, K, BN))
         return BNN_ERR_CUDA;
-    kern<<<grid, THREADS, SMEM, st>>>(mapA, mapB, M, N, K, C, ldc, thr, flip, out_bits, ldob, zo, status);
+    const int tma_c = C && ldc % 4 == 0 && (reinterpret_cast<uintptr_t>(C) & 15) == 0;
+    CUtensorMap mapC{};
+    if (tma_c && !encode_int32_map(&mapC, C, ldc, M, N)) return BNN_ERR_CUDA;
+    kern<<<grid, THREADS, SMEM, st>>>(mapA, mapB, mapC, tma_c, M, N, K, C, ldc, thr, flip, out_bits, ldob, zo, status);
     return launch_status();
 }
 
