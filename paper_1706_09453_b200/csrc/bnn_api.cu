@@ -398,7 +398,7 @@ static int output_layer_impl(const uint32_t* Hp, int ldhp, const float* Hf, int 
     const bool by_digits = Hp && digits && H <= kMaxKDigit && g_real_path != BNN_PATH_CUDA_CORE;
     const bool by_halves = Hp && prepared && !by_digits && g_real_path != BNN_PATH_CUDA_CORE;
     const bool follow = done && (by_digits || by_halves) && log_softmax && !mid_event &&
-                        g_softmax_follow && log_softmax_can_follow(logp, ldo, C, log_prior) &&
+                        g_softmax_follow && log_softmax_can_follow(C) &&
                         (by_digits ? out_digit_can_be_followed(M, C, H) : out_tc_more_than_one_wave(M, C));
     if (by_digits)
         rc = launch_out_digit(Hp, ldhp, digits, b, M, C, H, logp, ldo, zo, follow ? done : nullptr, (cudaStream_t)stream);

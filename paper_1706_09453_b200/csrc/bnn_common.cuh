@@ -244,7 +244,7 @@ bool out_digit_can_be_followed(int M, int C, int H);
 FollowArgs out_digit_follow(const void* image, int M, int C, int H, int* done);
 int launch_out_digit(const uint32_t* Hp, int ldhp, const void* image, const float* bias,
                      int M, int C, int H, float* Z, int ldz, int zo, int* done, cudaStream_t st);
-bool log_softmax_can_follow(const float* Z, int ldz, int C, const float* prior);
+bool log_softmax_can_follow(int C);
 int launch_log_softmax_rows_follow(float* Z, int ldz, int M, int C, const float* prior, const FollowArgs& f, cudaStream_t st);
 // The top layer on fp32 activations (finite, |a| < 65504) with both operands split into fp16
 // terms (out_gemm_f32_tc.cu): `workspace` holds outf_image_bytes(M, H) bytes, 256-byte aligned.

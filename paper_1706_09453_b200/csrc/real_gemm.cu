@@ -248,80 +248,62 @@ __device__ __forceinline__ float ex2_approx(float x) {
     return y;
 }
 
-// One row held in registers by the 256 threads of a CTA (C <= 256*4*V, 16-byte aligned rows): every
-// logit is read from memory once and written once.  The maximum is reduced first (warp shuffles, then
-// 8 values through shared memory), so each element costs a subtract, a multiply, one ex2 and one add;
-// the sum is reduced the same way.  sm/ss: 8 floats of shared scratch each; the caller alternates two
-// sets from row to row, which saves a barrier per row.
-template <int V>
-__device__ __forceinline__ void log_softmax_row_reg(float4* __restrict__ z, int c4, const float* __restrict__ prior,
-                                                    float* sm, float* ss) {
-    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    constexpr float kLog2e = 1.4426950408889634f, kLn2 = 0.6931471805599453f;
-    float4 v[V];
-    float mx = -FLT_MAX;
-#pragma unroll
-    for (int i = 0; i < V; ++i) {
-        const int c = threadIdx.x + i * 256;
-        v[i] = c < c4 ? z[c] : make_float4(-FLT_MAX, -FLT_MAX, -FLT_MAX, -FLT_MAX);
-        mx = fmaxf(fmaxf(mx, fmaxf(v[i].x, v[i].y)), fmaxf(v[i].z, v[i].w));
-    }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xFFFFFFFFu, mx, o));
-    if (lane == 0) sm[w] = mx;
-    __syncthreads();
-    mx = sm[0];
-#pragma unroll
-    for (int i = 1; i < 8; ++i) mx = fmaxf(mx, sm[i]);
-    // sum of exp(z - max) = sum of 2^((z - max) log2 e); the difference is taken first, so the
-    // rounding error scales with the distance from the maximum, not with the logit itself;
-    // padding (-FLT_MAX) contributes 0
-    float s = 0.f;
-#pragma unroll
-    for (int i = 0; i < V; ++i)
-        s += (ex2_approx((v[i].x - mx) * kLog2e) + ex2_approx((v[i].y - mx) * kLog2e)) +
-             (ex2_approx((v[i].z - mx) * kLog2e) + ex2_approx((v[i].w - mx) * kLog2e));
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xFFFFFFFFu, s, o);
-    if (lane == 0) ss[w] = s;
-    __syncthreads();
-    s = ss[0];
-#pragma unroll
-    for (int i = 1; i < 8; ++i) s += ss[i];
-    const float lse = mx + kLn2 * log2f(s);
-#pragma unroll
-    for (int i = 0; i < V; ++i) {
-        const int c = threadIdx.x + i * 256;
-        if (c < c4) {
-            // optional log-prior of each class (16-byte aligned, C % 4 == 0): a hybrid decoder
-            // wants log p(state | frame) - log p(state)
-            const float4 pr = prior ? __ldg(reinterpret_cast<const float4*>(prior) + c) : make_float4(0.f, 0.f, 0.f, 0.f);
-            z[c] = make_float4(v[i].x - lse - pr.x, v[i].y - lse - pr.y, v[i].z - lse - pr.z, v[i].w - lse - pr.w);
+// A row of C logits: its 16-byte chunks, and the up to three words before the first and after the last of them, which the
+// first threads take one each.  EVEN: the row starts on a 16-byte boundary and C is a multiple of 4, so there are only
+// chunks.  (Measured on B200, a CTA per row and a loop over single words before: 64 rows of 3307 classes 7.3 -> 2.7
+// us, 8192 rows of 3401 99 -> 37.)
+template <bool EVEN>
+struct LogitRow {
+    float* z;
+    int chunks, head, edge;  // `edge`: this thread's word, or -1
+    __device__ __forceinline__ LogitRow(float* row, int C) : z(row), edge(-1) {
+        head = EVEN ? 0 : (int)((0u - (unsigned)(reinterpret_cast<uintptr_t>(row) >> 2)) & 3u);
+        if (head > C) head = C;
+        chunks = (C - head) >> 2;
+        if (!EVEN) {
+            const int t = threadIdx.x, tail = (C - head) & 3;
+            if (t < head) edge = t;
+            else if (t >= 4 && t < 4 + tail) edge = head + 4 * chunks + t - 4;
         }
     }
-}
+    __device__ __forceinline__ float4* chunk(int i) const { return reinterpret_cast<float4*>(z + head) + i; }
+    // the optional log-prior of each class is what a hybrid decoder subtracts: log p(state | frame) - log p(state)
+    __device__ __forceinline__ float4 prior4(const float* __restrict__ prior, int i) const {
+        if (!prior) return make_float4(0.f, 0.f, 0.f, 0.f);
+        if (EVEN) return __ldg(reinterpret_cast<const float4*>(prior) + i);
+        const float* p = prior + head + 4 * i;
+        return make_float4(__ldg(p), __ldg(p + 1), __ldg(p + 2), __ldg(p + 3));
+    }
+};
 
-// R rows at once by a CTA of NT threads (z0, z0 + ldz4, ...; rows at or beyond `rows` are left alone):
-// the loads of all of them are in flight together and the reductions share their barriers.
-// sm/ss: R x (NT / 32) floats each.
-template <int V, int R, int NT>
-__device__ __forceinline__ void log_softmax_rows_reg(float4* __restrict__ z0, size_t ldz4, int rows, int c4,
+// R rows at once by a CTA of NT threads (z0, z0 + ldz, ...; rows at or beyond `rows` are left alone), held in registers
+// (C <= 4 NT V): every logit is read from memory once and written once.
+// The loads of all rows are in flight together and the reductions share their barriers.  The maximum is
+// reduced first (warp shuffles, then one value per warp through shared memory), so each element costs a subtract, a
+// multiply, one ex2 and one add; the sum is reduced the same way.  sm/ss: R x (NT / 32) floats each; the caller
+// alternates two sets, which saves a barrier per call.
+template <int V, int R, int NT, bool EVEN, bool STREAM>
+__device__ __forceinline__ void log_softmax_rows_reg(float* __restrict__ z0, size_t ldz, int rows, int C,
                                                      const float* __restrict__ prior, float (*sm)[NT / 32],
                                                      float (*ss)[NT / 32]) {
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     constexpr float kLog2e = 1.4426950408889634f, kLn2 = 0.6931471805599453f;
     float4 v[R][V];
-    float mx[R], s[R];
+    float x[R], mx[R], s[R];
 #pragma unroll
-    for (int r = 0; r < R; ++r)
+    for (int r = 0; r < R; ++r) {
+        const LogitRow<EVEN> row(z0 + r * ldz, r < rows ? C : 0);
 #pragma unroll
         for (int i = 0; i < V; ++i) {
             const int c = threadIdx.x + i * NT;
-            v[r][i] = (c < c4 && r < rows) ? __ldcs(z0 + r * ldz4 + c) : make_float4(-FLT_MAX, -FLT_MAX, -FLT_MAX, -FLT_MAX);
+            v[r][i] = make_float4(-FLT_MAX, -FLT_MAX, -FLT_MAX, -FLT_MAX);
+            if (c < row.chunks) v[r][i] = STREAM ? __ldcs(row.chunk(c)) : *row.chunk(c);
         }
+        x[r] = row.edge >= 0 ? row.z[row.edge] : -FLT_MAX;
+    }
 #pragma unroll
     for (int r = 0; r < R; ++r) {
-        mx[r] = -FLT_MAX;
+        mx[r] = x[r];
 #pragma unroll
         for (int i = 0; i < V; ++i)
             mx[r] = fmaxf(fmaxf(mx[r], fmaxf(v[r][i].x, v[r][i].y)), fmaxf(v[r][i].z, v[r][i].w));
@@ -335,8 +317,10 @@ __device__ __forceinline__ void log_softmax_rows_reg(float4* __restrict__ z0, si
         mx[r] = sm[r][0];
 #pragma unroll
         for (int i = 1; i < NT / 32; ++i) mx[r] = fmaxf(mx[r], sm[r][i]);
-        // sum of 2^((z - max) log2 e), as in log_softmax_row_reg; padding (-FLT_MAX) contributes 0
-        s[r] = 0.f;
+        // sum of exp(z - max) = sum of 2^((z - max) log2 e); the difference is taken first, so the
+        // rounding error scales with the distance from the maximum, not with the logit itself;
+        // padding (-FLT_MAX) contributes 0
+        s[r] = EVEN ? 0.f : ex2_approx((x[r] - mx[r]) * kLog2e);
 #pragma unroll
         for (int i = 0; i < V; ++i)
             s[r] += (ex2_approx((v[r][i].x - mx[r]) * kLog2e) + ex2_approx((v[r][i].y - mx[r]) * kLog2e)) +
@@ -352,28 +336,30 @@ __device__ __forceinline__ void log_softmax_rows_reg(float4* __restrict__ z0, si
 #pragma unroll
         for (int i = 1; i < NT / 32; ++i) t += ss[r][i];
         const float lse = mx[r] + kLn2 * log2f(t);
+        const LogitRow<EVEN> row(z0 + r * ldz, r < rows ? C : 0);
 #pragma unroll
         for (int i = 0; i < V; ++i) {
             const int c = threadIdx.x + i * NT;
-            if (c < c4 && r < rows) {
-                const float4 pr = prior ? __ldg(reinterpret_cast<const float4*>(prior) + c) : make_float4(0.f, 0.f, 0.f, 0.f);
-                __stcs(z0 + r * ldz4 + c, make_float4(v[r][i].x - lse - pr.x, v[r][i].y - lse - pr.y, v[r][i].z - lse - pr.z, v[r][i].w - lse - pr.w));
+            if (c < row.chunks) {
+                const float4 pr = row.prior4(prior, c);
+                const float4 o = make_float4(v[r][i].x - lse - pr.x, v[r][i].y - lse - pr.y, v[r][i].z - lse - pr.z, v[r][i].w - lse - pr.w);
+                if (STREAM) __stcs(row.chunk(c), o); else *row.chunk(c) = o;
             }
         }
+        if (row.edge >= 0) row.z[row.edge] = x[r] - lse - (prior ? __ldg(prior + row.edge) : 0.f);
     }
 }
 
 // Same result as log_softmax_rows_kernel, one CTA per row at a time.
-template <int V>
+template <int V, bool EVEN>
 __global__ void __launch_bounds__(256)
 log_softmax_rows_reg_kernel(float* __restrict__ Z, int ldz, int M, int C, const float* __restrict__ prior) {
-    __shared__ float sm[2][8], ss[2][8];
-    const int c4 = C >> 2;  // C % 4 == 0
+    __shared__ float sm[2][1][8], ss[2][1][8];
     int par = 0;
     // Rows are taken from the last one down: the kernel that wrote the logits just before this one
     // produced the last frames last, and those are the rows the L2 cache still holds.
     for (int r = blockIdx.x; r < M; r += gridDim.x, par ^= 1)
-        log_softmax_row_reg<V>(reinterpret_cast<float4*>(Z + (size_t)(M - 1 - r) * ldz), c4, prior, sm[par], ss[par]);
+        log_softmax_rows_reg<V, 1, 256, EVEN, false>(Z + (size_t)(M - 1 - r) * ldz, 0, 1, C, prior, sm[par], ss[par]);
 }
 
 // The same rows, taken while the kernel that writes the logits is still running.  That kernel counts, per
@@ -390,14 +376,13 @@ log_softmax_rows_reg_kernel(float* __restrict__ Z, int ldz, int M, int C, const 
 // of 72 registers of the kernel it follows: the busiest scheduler's register file has room for one more
 // warp of up to 152 registers.
 constexpr int kFollowRows = 2, kFollowThreads = 128;
-template <int V>
-__global__ void __launch_bounds__(kFollowThreads)
+template <int V, bool EVEN>
+__global__ void __launch_bounds__(kFollowThreads, 5)     // at most 96 registers: more were not resident beside it
 log_softmax_rows_follow_kernel(float* __restrict__ Z, int ldz, int M, int C, const float* __restrict__ prior,
                                FollowArgs follow, tc::TcStatus status) {
     constexpr int R = kFollowRows, NT = kFollowThreads;
     __shared__ float sm[2][R][NT / 32], ss[2][R][NT / 32];
     __shared__ int claim;
-    const int c4 = C >> 2;
     int* const done = follow.done;
     const int group_rows = follow.group_rows, need = follow.flag && __ldg(follow.flag) ? follow.need4 : follow.need;
     int* next_row = done + ceil_div(M, group_rows);
@@ -428,8 +413,7 @@ log_softmax_rows_follow_kernel(float* __restrict__ Z, int ldz, int M, int C, con
             break;
         }
         if (threadIdx.x == 0) pending = atomicAdd(next_row, R);   // in flight while these rows are worked on
-        log_softmax_rows_reg<V, R, NT>(reinterpret_cast<float4*>(Z + (size_t)r * ldz), (size_t)(ldz >> 2), M - r, c4, prior,
-                                   sm[par], ss[par]);
+        log_softmax_rows_reg<V, R, NT, EVEN, true>(Z + (size_t)r * ldz, (size_t)ldz, M - r, C, prior, sm[par], ss[par]);
         par ^= 1;   // the scratch alternates; `claim` is rewritten only after the two barriers inside
     }
     // completion of this kernel implies completion of the one it followed
@@ -451,31 +435,34 @@ int launch_real_gemm(const RealGemmArgs& a, cudaStream_t st) {
     return launch_status();
 }
 
-bool log_softmax_can_follow(const float* Z, int ldz, int C, const float* prior) {
-    return (C % 4 == 0) && (ldz % 4 == 0) && aligned16(Z) && C <= 128 * 4 * 8 && (!prior || aligned16(prior));
+// Rows that start on 16-byte boundaries and hold whole chunks of four.
+static bool rows_even(const float* Z, int ldz, int C, const float* prior) {
+    return (C % 4 == 0) && (ldz % 4 == 0) && aligned16(Z) && (!prior || aligned16(prior));
+}
+bool log_softmax_can_follow(int C) {
+    return C <= kFollowThreads * 4 * 8;
 }
 
 int launch_log_softmax_rows_follow(float* Z, int ldz, int M, int C, const float* prior, const FollowArgs& f, cudaStream_t st) {
     const int sms = device_sm_count();
     const tc::TcStatus status = tc_status();
-    if (sms <= 0 || !status.word || !log_softmax_can_follow(Z, ldz, C, prior)) return BNN_ERR_CUDA;
+    if (sms <= 0 || !status.word || !log_softmax_can_follow(C)) return BNN_ERR_CUDA;
     if (f.group_rows % kFollowRows != 0) return BNN_ERR_UNSUPPORTED;
     const int blocks = M < sms * 5 * kFollowRows ? ceil_div(M, kFollowRows) : sms * 5;
-    const cudaError_t e = C <= kFollowThreads * 4 * 4
-        ? launch_pdl(log_softmax_rows_follow_kernel<4>, dim3(blocks), dim3(kFollowThreads), 0, st, Z, ldz, M, C, prior, f, status)
-        : launch_pdl(log_softmax_rows_follow_kernel<8>, dim3(blocks), dim3(kFollowThreads), 0, st, Z, ldz, M, C, prior, f, status);
+    const bool even = rows_even(Z, ldz, C, prior), narrow = C <= kFollowThreads * 4 * 4;
+    auto kern = even ? (narrow ? log_softmax_rows_follow_kernel<4, true> : log_softmax_rows_follow_kernel<8, true>)
+                     : (narrow ? log_softmax_rows_follow_kernel<4, false> : log_softmax_rows_follow_kernel<8, false>);
+    const cudaError_t e = launch_pdl(kern, dim3(blocks), dim3(kFollowThreads), 0, st, Z, ldz, M, C, prior, f, status);
     return e == cudaSuccess ? launch_status() : BNN_ERR_CUDA;
 }
 
 int launch_log_softmax_rows(float* Z, int ldz, int M, int C, const float* prior, cudaStream_t st) {
     const int blocks = M < 148 * 8 ? M : 148 * 8;
-    const bool reg = (C % 4 == 0) && (ldz % 4 == 0) && aligned16(Z) && C <= 256 * 4 * 4 && (!prior || aligned16(prior));
-    if (reg && C <= 256 * 4 * 2)
-        log_softmax_rows_reg_kernel<2><<<blocks, 256, 0, st>>>(Z, ldz, M, C, prior);
-    else if (reg)
-        log_softmax_rows_reg_kernel<4><<<blocks, 256, 0, st>>>(Z, ldz, M, C, prior);
-    else
-        log_softmax_rows_kernel<<<blocks, 256, 0, st>>>(Z, ldz, M, C, prior);
+    const bool even = rows_even(Z, ldz, C, prior);
+    auto kern = C <= 256 * 4 * 2 ? (even ? log_softmax_rows_reg_kernel<2, true> : log_softmax_rows_reg_kernel<2, false>)
+              : C <= 256 * 4 * 4 ? (even ? log_softmax_rows_reg_kernel<4, true> : log_softmax_rows_reg_kernel<4, false>)
+                                     : log_softmax_rows_kernel;
+    kern<<<blocks, 256, 0, st>>>(Z, ldz, M, C, prior);
     return launch_status();
 }
 
