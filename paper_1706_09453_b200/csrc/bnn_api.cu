@@ -589,20 +589,28 @@ int bnn_forward_events(const bnn_model* model, const float* X, int ldx, int M,
     // The same goes for the counters on which the log-softmax follows the top layer's kernel.
     int* top_done = nullptr;
     bool clear_pending = false, clear_by_first = false;
-    if (!small && lay.sync > 0) {
+    // a layer that can be part of a run of the small-batch kernel
+    auto in_small_run = [&](int l) {
+        const bnn_layer& y = model->layers[l];
+        return y.kind == BNN_LAYER_XNOR && y.act == BNN_ACT_SIGN_PACK && small_fits_bits(y.K) && small_xnor_can_run(y.N);
+    };
+    const bool small_first = small && model->layers[0].kind == BNN_LAYER_SIGNW && model->layers[0].act == BNN_ACT_SIGN_PACK &&
+                             splice_dim == 0 && small_fits_real(model->layers[0].K);
+    if (lay.sync > 0) {
         bool any = false;
         for (int l = 0; g_xnor_stack && l + 1 < L && !any; ++l)
-            any = stackable(model, l) && stackable(model, l + 1) && model->layers[l].N == model->layers[l].K &&
+            any = (small ? !events && in_small_run(l) && in_small_run(l + 1) : stackable(model, l) && stackable(model, l + 1)) &&
+                  model->layers[l].N == model->layers[l].K &&
                   model->layers[l + 1].N == model->layers[l].N && model->layers[l + 1].K == model->layers[l].K;
         const bnn_layer& top = model->layers[L - 1];
-        if (g_softmax_follow && !events && lay.sync > lay.stack_sync && top.kind == BNN_LAYER_REAL_OUT && L > 1 &&
+        if (!small && g_softmax_follow && !events && lay.sync > lay.stack_sync && top.kind == BNN_LAYER_REAL_OUT && L > 1 &&
             model->layers[L - 2].act == BNN_ACT_SIGN_PACK &&
             ((top.Wp && out_digit_can_be_followed(M, top.N, top.K)) || (top.W_prepared && out_tc_more_than_one_wave(M, top.N))))
             top_done = sync + lay.stack_sync / sizeof(int);
         clear_pending = any || top_done;
-        // When the first layer splits its input into an image, that kernel clears them on its way (a memset
+        // When the first layer splits its input into an image, or is the small-batch kernel, that kernel clears them on its way (a memset
         // node of its own costs about 4 us per step in a replayed graph); otherwise a memset does.
-        clear_by_first = clear_pending && model->layers[0].kind == BNN_LAYER_SIGNW && g_real_path != BNN_PATH_CUDA_CORE;
+        clear_by_first = clear_pending && (small_first || (model->layers[0].kind == BNN_LAYER_SIGNW && g_real_path != BNN_PATH_CUDA_CORE));
         if (clear_pending && !clear_by_first) {
             if (cudaMemsetAsync(sync, 0, lay.sync, (cudaStream_t)stream) != cudaSuccess) return BNN_ERR_CUDA;
             clear_pending = false;
@@ -627,7 +635,10 @@ int bnn_forward_events(const bnn_model* model, const float* X, int ldx, int M,
         if (events && events[l] &&
             cudaEventRecord((cudaEvent_t)events[l], (cudaStream_t)stream) != cudaSuccess)
             return BNN_ERR_CUDA;
-        if (y.kind == BNN_LAYER_REAL_OUT && small && in_bits && small_fits_out(y.K)) {
+        // (With more than four frames the digit kernel is the faster one: 2048 -> 3307, 8 frames 10 us against 20, 3 frames
+        // 10 against 9; 1024 -> 2000, 8 frames 7 against 9.)
+        if (y.kind == BNN_LAYER_REAL_OUT && small && in_bits && small_fits_out(y.K) &&
+            (M <= 4 || !y.Wp || y.K > kMaxKDigit || g_real_path == BNN_PATH_CUDA_CORE)) {
             if (int rc = check_packed(in, in_ld, y.K)) return rc;
             if (int rc = launch_small_out(static_cast<const uint32_t*>(in), in_ld, y.W, y.ldw, y.shift, M, y.N, y.K,
                                           logp, ldo, zo01, (cudaStream_t)stream)) return rc;
@@ -684,6 +695,28 @@ int bnn_forward_events(const bnn_model* model, const float* X, int ldx, int M,
                 continue;
             }
         }
+        // The same for a handful of frames (small_batch.cu), which needs no prepared weights.
+        if (small && y.kind == BNN_LAYER_XNOR && y.act == BNN_ACT_SIGN_PACK && small_fits_bits(y.K)) {
+            XnorSmallLayer sl[kXnorStackMax];
+            int n = 0;
+            do {
+                const bnn_layer& z = model->layers[l + n];
+                void* o = (layer_out && layer_out[l + n]) ? layer_out[l + n] : buf[(l + n) & 1];
+                sl[n++] = XnorSmallLayer{z.Wp, z.ldwp, z.thr, z.flip, static_cast<uint32_t*>(o)};
+            } while (g_xnor_stack && !events && y.N == y.K && n < kXnorStackMax && l + n < L && in_small_run(l) && in_small_run(l + n) &&
+                     model->layers[l + n].N == y.N && model->layers[l + n].K == y.K);
+            if (int rc = check_packed(in, in_ld, y.K)) return rc;
+            const int ldob = bnn_packed_pitch(y.N);
+            if (int rc = launch_small_xnor(static_cast<const uint32_t*>(in), in_ld, sl, n, M, y.N, y.K, ldob, zo01, sync + sync_used,
+                                           (cudaStream_t)stream))
+                return rc;
+            sync_used += n - 1;
+            in = sl[n - 1].out_bits;
+            in_ld = ldob;
+            in_bits = true;
+            l += n - 1;
+            continue;
+        }
         void* out = (layer_out && layer_out[l]) ? layer_out[l] : buf[l & 1];
         bnn_epilogue e{};
         e.act = y.act;
@@ -692,13 +725,11 @@ int bnn_forward_events(const bnn_model* model, const float* X, int ldx, int M,
         if (small && y.act == BNN_ACT_SIGN_PACK && y.kind == BNN_LAYER_SIGNW && !(l == 0 && splice_dim > 0) &&
             small_fits_real(y.K)) {
             const int ldob = bnn_packed_pitch(y.N);
+            const bool clears = l == 0 && clear_pending;
             rc = launch_small_signw(static_cast<const float*>(in), in_ld, y.Wp, y.ldwp, M, y.N, y.K, y.scale, y.shift,
-                                    model->sign_mode, static_cast<uint32_t*>(out), ldob, (cudaStream_t)stream);
-            in_ld = ldob;
-        } else if (small && y.act == BNN_ACT_SIGN_PACK && y.kind == BNN_LAYER_XNOR && small_fits_bits(y.K)) {
-            const int ldob = bnn_packed_pitch(y.N);
-            rc = launch_small_xnor(static_cast<const uint32_t*>(in), in_ld, y.Wp, y.ldwp, M, y.N, y.K, y.thr, y.flip,
-                                   static_cast<uint32_t*>(out), ldob, zo01, (cudaStream_t)stream);
+                                    model->sign_mode, static_cast<uint32_t*>(out), ldob, sync, clears ? (int)(lay.sync / sizeof(int)) : 0,
+                                    (cudaStream_t)stream);
+            if (clears) clear_pending = false;
             in_ld = ldob;
         } else if (y.kind == BNN_LAYER_SIGNW) {
             e.scale = y.scale; e.shift = y.shift;

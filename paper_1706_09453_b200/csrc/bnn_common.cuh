@@ -138,10 +138,19 @@ inline bool small_fits_bits(int K) { return (size_t)kSmallBatchMax * words_for(K
 inline bool small_fits_out(int H) { return (size_t)words_for(H) * 32 * sizeof(uint16_t) <= kSmallSmemMax; }
 int launch_small_signw(const float* X, int ldx, const uint32_t* Wp, int ldwp, int M, int N, int K,
                        const float* scale, const float* shift, int sign_mode,
-                       uint32_t* out_bits, int ldob, cudaStream_t st);
-int launch_small_xnor(const uint32_t* Ap, int ldap, const uint32_t* Wp, int ldwp, int M, int N, int K,
-                      const int32_t* thr, const uint32_t* flip, uint32_t* out_bits, int ldob, int zo,
-                      cudaStream_t st);
+                       uint32_t* out_bits, int ldob, int* clear, int n_clear, cudaStream_t st);
+// A run of layers of one shape (N == K beyond the first) in one launch: layer l reads the bits layer l - 1 wrote (pitch
+// ldob).  `arrived`: n_layers - 1 counters that are zero once the kernels before it in the stream have completed.
+struct XnorSmallLayer {
+    const uint32_t* Wp;
+    int ldwp;
+    const int32_t* thr;
+    const uint32_t* flip;
+    uint32_t* out_bits;
+};
+bool small_xnor_can_run(int N);   // more than one layer: every CTA of the launch needs an SM of its own
+int launch_small_xnor(const uint32_t* Ap, int ldap, const XnorSmallLayer* layers, int n_layers, int M, int N, int K,
+                      int ldob, int zo, int* arrived, cudaStream_t st);
 int launch_small_out(const uint32_t* Hp, int ldhp, const float* W, int ldw, const float* bias,
                      int M, int C, int H, float* Z, int ldz, int zo, cudaStream_t st);
 // Pipe micro-benchmarks (pipe_rates.cu).
