@@ -18,9 +18,12 @@
 // a CTA tile is 128 classes x 256 frames with two accumulators, so the epilogue of one tile
 // overlaps the MMAs of the next.  A pipeline stage (32 positions of K) is two bulk copies:
 // 16 KB of the weight image and 32 KB of the activation image; nothing is widened on chip.
-//   warp 5       one thread issues the bulk copies
-//   warp 4       one thread issues the MMAs (6 per stage) and the commits
-//   warps 0-3    epilogue: z = acc * 2^-e + b, 32 consecutive classes of a frame per warp store
+//   warp 17      one thread issues the bulk copies
+//   warp 16      one thread issues the MMAs (6 per stage) and the commits
+//   warps 0-15   epilogue: f(acc * 2^-e + b), 32 consecutive classes of a frame per warp store; warp w takes the
+//                lanes of quarter w % 4 and 64 of the tile's frames.  (A Sigmoid is about 40 instructions, so a layer
+//                of short rows is bound by the epilogue: 8192 x 440 -> 2048 with Sigmoid 114 us with four warps, 44 us with
+//                sixteen; 8192 x 2048 -> 3400 without, 198 us, is bound by the MMAs: three passes at half-precision rate.)
 // Every wait is bounded; a wait that runs out sets the CTA's abort flag, all roles fall
 // through to the common teardown and the device status word is set.
 #include <cuda_fp16.h>
@@ -43,7 +46,8 @@ constexpr int B_PLANE = FN * BK * 2;        // 16 KB per activation term
 constexpr int B_BYTES = 2 * B_PLANE;
 constexpr int STAGE_BYTES = A_BYTES + B_BYTES;   // 48 KB
 constexpr int STAGES = 4;
-constexpr int EPI_WARPS = 4, MMA_WARP = 4, TMA_WARP = 5;
+constexpr int EPI_WARPS = 16, MMA_WARP = EPI_WARPS, TMA_WARP = MMA_WARP + 1;
+constexpr int EPI_FRAMES = FN / (EPI_WARPS / 4);   // frames of a tile per epilogue warp
 constexpr int THREADS = (TMA_WARP + 1) * 32;
 constexpr uint32_t TMEM_COLS = 512;
 
@@ -60,66 +64,74 @@ __device__ __forceinline__ void bulk_g2s(uint32_t dst, const void* src, uint32_t
                  ::"r"(dst), "l"(src), "r"(bytes), "r"(bar) : "memory");
 }
 
-// ---- split: one CTA per (tile of 256 frames, stage): thread = frame row ---------------------
+// ---- split: thread = one 16-byte chunk of a frame row ---------------------------------------
 // Block (ft, ks) of the image: [term 0..1][chunk c = 2 j + cc][row 0..255][16 bytes], where
 // chunk (j, cc) holds, in element e, position k = 32 ks + 8 j + (pos >> 1) + 16 (pos & 1),
-// pos = 8 cc + e: the order of the prepared weight image, so both operands agree on k.
+// pos = 8 cc + e: the order of the prepared weight image, so both operands agree on k.  In other words element
+// e of chunk c is position 4 c + (e >> 1) + 16 (e & 1): a chunk is two groups of four consecutive positions.
+// Four lanes cover the 128 bytes of a row, a warp eight rows.  (Measured on B200, a thread with the 32 positions of a
+// row before: 8192 x 2048 of int32 with Sigmoid 48 -> 37 us,
+// of which the Sigmoids are most.)
 // FROM_I32: the activations are Sigmoid(fma(scale[h], d, shift[h])) of integer dot products d (a binary
 // layer with Sigmoid units, Section 3.2 / Table 2), evaluated here instead of in a pass of their own.
-template <bool FROM_I32>
-__global__ void __launch_bounds__(FN)
-h_split_kernel(const void* __restrict__ src, int ldh, int M, int H, int nks, uint8_t* __restrict__ img,
-               const float* __restrict__ scale, const float* __restrict__ shift) {
-    const int ft = blockIdx.x / nks, ks = blockIdx.x % nks;
-    const int row = threadIdx.x, m = ft * FN + row;
-    float v[BK];
-    const bool vec = (ldh % 4 == 0) && ((reinterpret_cast<uintptr_t>(src) & 15) == 0) && ks * BK + BK <= H;
-    if (m < M && vec) {
-        const uint4* p = reinterpret_cast<const uint4*>(static_cast<const uint32_t*>(src) + (size_t)m * ldh + ks * BK);
-#pragma unroll
-        for (int q = 0; q < BK / 4; ++q) {
-            const uint4 t = __ldg(p + q);
-            v[4 * q] = __uint_as_float(t.x); v[4 * q + 1] = __uint_as_float(t.y);
-            v[4 * q + 2] = __uint_as_float(t.z); v[4 * q + 3] = __uint_as_float(t.w);
-        }
+// p[k0 .. k0 + 3] and p[k0 + 16 .. k0 + 19]; `other` beyond H or without p.
+__device__ __forceinline__ void load8(const float* __restrict__ p, int k0, int H, float other, float (&o)[8]) {
+    if (p && (reinterpret_cast<uintptr_t>(p) & 15) == 0 && k0 + 20 <= H) {
+        const float4 a = __ldg(reinterpret_cast<const float4*>(p + k0)), b = __ldg(reinterpret_cast<const float4*>(p + k0 + 16));
+        o[0] = a.x; o[1] = a.y; o[2] = a.z; o[3] = a.w; o[4] = b.x; o[5] = b.y; o[6] = b.z; o[7] = b.w;
     } else {
 #pragma unroll
-        for (int k = 0; k < BK; ++k) {
-            const int kk = ks * BK + k;
-            v[k] = (m < M && kk < H) ? __uint_as_float(__ldg(static_cast<const uint32_t*>(src) + (size_t)m * ldh + kk)) : 0.f;
+        for (int i = 0; i < 8; ++i) {
+            const int k = k0 + (i & 3) + (i >> 2) * 16;
+            o[i] = p && k < H ? __ldg(p + k) : other;
+        }
+    }
+}
+constexpr int SPLIT_THREADS = 256, SPLIT_ROWS = SPLIT_THREADS / 4;
+template <bool FROM_I32>
+__global__ void __launch_bounds__(SPLIT_THREADS)
+h_split_kernel(const void* __restrict__ src, int ldh, int M, int H, int nks, uint8_t* __restrict__ img,
+               const float* __restrict__ scale, const float* __restrict__ shift) {
+    const int ks = (int)blockIdx.x % nks, rb = (int)blockIdx.x / nks;      // rb: block of SPLIT_ROWS rows
+    const int c = threadIdx.x & 3, m = rb * SPLIT_ROWS + ((int)threadIdx.x >> 2);
+    const int ft = m / FN, row = m % FN, k0 = ks * BK + 4 * c;
+    float v[8];              // positions k0 .. k0 + 3, k0 + 16 .. k0 + 19
+    const uint32_t* p = static_cast<const uint32_t*>(src) + (size_t)m * ldh + k0;
+    const bool vec = (ldh % 4 == 0) && ((reinterpret_cast<uintptr_t>(src) & 15) == 0) && k0 + 20 <= H;
+    if (m < M && vec) {
+        const uint4 a = __ldg(reinterpret_cast<const uint4*>(p)), b = __ldg(reinterpret_cast<const uint4*>(p + 16));
+        v[0] = __uint_as_float(a.x); v[1] = __uint_as_float(a.y); v[2] = __uint_as_float(a.z); v[3] = __uint_as_float(a.w);
+        v[4] = __uint_as_float(b.x); v[5] = __uint_as_float(b.y); v[6] = __uint_as_float(b.z); v[7] = __uint_as_float(b.w);
+    } else {
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+            const int k = (i & 3) + (i >> 2) * 16;
+            v[i] = (m < M && k0 + k < H) ? __uint_as_float(__ldg(p + k)) : 0.f;
         }
     }
     if (FROM_I32) {
+        float sc[8], sh[8];
+        load8(scale, k0, H, 1.0f, sc);
+        load8(shift, k0, H, 0.0f, sh);
 #pragma unroll
-        for (int k = 0; k < BK; ++k) {
-            const int kk = ks * BK + k;
-            if (m < M && kk < H) {
-                const float d = (float)__float_as_int(v[k]);
-                const float y = fmaf(scale ? __ldg(scale + kk) : 1.0f, d, shift ? __ldg(shift + kk) : 0.0f);
-                v[k] = 1.0f / (1.0f + expf(-y));
-            } else {
-                v[k] = 0.f;
-            }
+        for (int i = 0; i < 8; ++i) {
+            const float d = (float)__float_as_int(v[i]);
+            const float y = fmaf(sc[i], d, sh[i]);
+            v[i] = (m < M && k0 + (i & 3) + (i >> 2) * 16 < H) ? 1.0f / (1.0f + expf(-y)) : 0.f;
         }
     }
-    uint8_t* blk = img + ((size_t)ft * nks + ks) * B_BYTES;
+    uint32_t hi[4], lo[4];
 #pragma unroll
-    for (int c = 0; c < 4; ++c) {
-        const int j = c >> 1, cc = c & 1;
-        uint32_t hi[4], lo[4];
-#pragma unroll
-        for (int e = 0; e < 8; ++e) {
-            const int pos = cc * 8 + e;
-            const float x = v[8 * j + (pos >> 1) + 16 * (pos & 1)];
-            const __half h1 = __float2half_rn(x);
-            const __half h2 = __float2half_rn(x - __half2float(h1));
-            const uint32_t b1 = __half_as_ushort(h1), b2 = __half_as_ushort(h2);
-            if (e & 1) { hi[e >> 1] |= b1 << 16; lo[e >> 1] |= b2 << 16; }
-            else { hi[e >> 1] = b1; lo[e >> 1] = b2; }
-        }
-        *reinterpret_cast<uint4*>(blk + (size_t)(c * FN + row) * 16) = make_uint4(hi[0], hi[1], hi[2], hi[3]);
-        *reinterpret_cast<uint4*>(blk + B_PLANE + (size_t)(c * FN + row) * 16) = make_uint4(lo[0], lo[1], lo[2], lo[3]);
+    for (int i = 0; i < 4; ++i) {      // elements 2 i and 2 i + 1
+        const __half2 h1 = __floats2half2_rn(v[i], v[i + 4]);
+        const float2 f1 = __half22float2(h1);
+        const __half2 h2 = __floats2half2_rn(v[i] - f1.x, v[i + 4] - f1.y);
+        hi[i] = *reinterpret_cast<const uint32_t*>(&h1);
+        lo[i] = *reinterpret_cast<const uint32_t*>(&h2);
     }
+    uint8_t* dst = img + ((size_t)ft * nks + ks) * B_BYTES + (size_t)(c * FN + row) * 16;
+    *reinterpret_cast<uint4*>(dst) = make_uint4(hi[0], hi[1], hi[2], hi[3]);
+    *reinterpret_cast<uint4*>(dst + B_PLANE) = make_uint4(lo[0], lo[1], lo[2], lo[3]);
 }
 
 // ---- the GEMM ---------------------------------------------------------------------------
@@ -132,7 +144,7 @@ outf_tc_kernel(const uint8_t* __restrict__ himg, const uint8_t* __restrict__ wim
     Control* ctl = reinterpret_cast<Control*>(smem + STAGES * STAGE_BYTES);
     volatile int* abort_flag = &ctl->wait.abort;
 
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int warp = warp_index(), lane = threadIdx.x & 31;
     const int nks = ceil_div(H, BK);
     const int c_tiles = ceil_div(C, BC), f_tiles = ceil_div(M, FN);
     const int tiles = c_tiles * f_tiles;
@@ -218,22 +230,23 @@ outf_tc_kernel(const uint8_t* __restrict__ himg, const uint8_t* __restrict__ wim
         __syncwarp();
     } else {
         // ---------------- epilogue: thread = one class (TMEM lane), columns = frames
-        const int row_in_tile = warp * 32 + lane;
+        const int row_in_tile = (warp & 3) * 32 + lane;
+        const int col0 = (warp >> 2) * EPI_FRAMES;
         int tl = 0;
         bool ok = true;
         for (int tile = blockIdx.x; tile < tiles && ok; tile += gridDim.x, ++tl) {
             const int c = (tile % c_tiles) * BC + row_in_tile;
-            const int f0 = (tile / c_tiles) * FN;
+            const int f0 = (tile / c_tiles) * FN + col0;
             const float scl = rs[c];                       // rs is padded to whole tiles
             const float bia = (bias && c < C) ? bias[c] : 0.f;
             const int b = tl & 1;
-            ok = epi_all(warp_wait_relaxed(smem_u32(&ctl->acc_full[b]), (uint32_t)((tl >> 1) & 1), abort_flag, lane));
+            ok = warp_wait_relaxed(smem_u32(&ctl->acc_full[b]), (uint32_t)((tl >> 1) & 1), abort_flag, lane);
             if (!ok) break;
             tc_fence_after_sync();
-            const uint32_t taddr = tmem + ((uint32_t)(warp * 32) << 16) + (uint32_t)(b * FN);
+            const uint32_t taddr = tmem + ((uint32_t)((warp & 3) * 32) << 16) + (uint32_t)(b * FN + col0);
 #pragma unroll 1
-            for (int gi = 0; gi < FN / 32; ++gi) {
-                if (f0 + gi * 32 >= M) break;              // uniform over the CTA
+            for (int gi = 0; gi < EPI_FRAMES / 32; ++gi) {
+                if (f0 + gi * 32 >= M) break;              // uniform over the warp
                 uint32_t acc[32];
                 tmem_ld32(taddr + gi * 32, acc);
                 tmem_ld_wait();
@@ -282,7 +295,7 @@ int launch_outf_tc(const float* Hf, int ldhf, const void* prepared, const float*
     const TcStatus status = tc_status();
     if (!status.word) return BNN_ERR_CUDA;
     if (!image_ready)   // (else the layer that produced the activations wrote the image itself)
-        h_split_kernel<false><<<ft * hs, FN, 0, st>>>(Hf, ldhf, M, H, hs, himg, nullptr, nullptr);
+        h_split_kernel<false><<<ft * hs * (FN / SPLIT_ROWS), SPLIT_THREADS, 0, st>>>(Hf, ldhf, M, H, hs, himg, nullptr, nullptr);
     const int tiles = ct * ft;
     outf_tc_kernel<<<tiles < sms ? tiles : sms, THREADS, SMEM_BYTES, st>>>(himg, wimg, rs, bias, M, C, H, Z, ldz, act, status);
     return launch_status();
@@ -292,7 +305,7 @@ int launch_outf_tc(const float* Hf, int ldhf, const void* prepared, const float*
 int launch_outf_image_from_i32(const int32_t* D, int ldd, const float* scale, const float* shift, int M, int H,
                                void* image, cudaStream_t st) {
     const int hs = ceil_div(H, BK), ft = ceil_div(M, FN);
-    h_split_kernel<true><<<ft * hs, FN, 0, st>>>(D, ldd, M, H, hs, static_cast<uint8_t*>(image), scale, shift);
+    h_split_kernel<true><<<ft * hs * (FN / SPLIT_ROWS), SPLIT_THREADS, 0, st>>>(D, ldd, M, H, hs, static_cast<uint8_t*>(image), scale, shift);
     return launch_status();
 }
 
