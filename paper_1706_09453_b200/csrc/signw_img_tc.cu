@@ -10,7 +10,11 @@
 //      bf16 on chip, one MMA per term accumulates in fp32 in tensor memory.
 //
 // Frames are on the M side (TMEM lane = frame), units on the N side.  A CTA tile is 128 frames
-// x 512 units (two 256-column accumulators fed by the same activation stage).  The epilogue
+// x 512 units (two 256-column accumulators fed by the same activation stage), or, for layers that hand on nothing but
+// bits and batches that would leave SMs idle, 256 or 128 units (one accumulator, double buffered; the sums are the same
+// bit for bit).  A layer of 440 -> 2048 is one wave of such tiles up to 1152 or 2304 frames.  Measured on
+// B200, after the split pass, 64 / 731 / 2000 / 3000 frames: 14.9 / 14.8 / 15.5 / 15.9 us with 512 units, 10.5 / 10.2 /
+// 10.6 / 17.3 with 256, 9.0 / 9.2 / 14.4 / 20.2 with 128.  The epilogue
 // thread owns a frame: per-unit affine (one fma), then Sign + pack (16 words per row and
 // tile) and/or fp32 stores of 128 contiguous bytes.  When the layer that consumes the outputs is
 // again of this kind (a network with binary weights and real activations, Algorithm 1), the
@@ -33,23 +37,24 @@ namespace {
 using namespace tc;
 
 constexpr int BM = 128;           // frames per tile
-constexpr int UN = 512;           // units per tile (2 x 256)
 constexpr int BK = 32;            // k per stage
 constexpr int A_PLANE = BM * BK * 2;        // 8 KB per bf16 term
-constexpr int B_BYTES = UN * BK * 2;        // 32 KB
 constexpr int MMA_WARP = 4, PROD_WARP0 = 5, PROD_WARPS = 8, EPI_WARPS = 4;
 constexpr int THREADS = (PROD_WARP0 + PROD_WARPS) * 32;
 constexpr uint32_t TMEM_COLS = 512;
 
-template <int NT> struct Cfg {
-    static constexpr int A_BYTES = NT * A_PLANE;
+// UN: units per tile
+template <int NT, int UN> struct Cfg {
+    static constexpr int SUBS = UN == 512 ? 2 : 1, SUB = UN / SUBS;      // accumulators a tile is spread over, their columns
+    static constexpr int A_BYTES = NT * A_PLANE, B_BYTES = UN * BK * 2;
     static constexpr int STAGE_BYTES = A_BYTES + B_BYTES;
-    static constexpr int STAGES = NT == 2 ? 4 : 3;
+    static constexpr int STAGES = UN == 512 ? (NT == 2 ? 4 : 3) : UN == 256 ? 5 : 7;
 };
+constexpr int MAX_UN = 512, MAX_STAGES = 7;
 
 struct Control {
-    float sc[UN], sh[UN];
-    uint64_t full[4], empty[4], acc_full, acc_empty[2];
+    float sc[MAX_UN], sh[MAX_UN];
+    uint64_t full[MAX_STAGES], empty[MAX_STAGES], acc_full[2], acc_empty[2];
     uint32_t tmem_base;
     WaitState wait;
 };
@@ -184,8 +189,8 @@ __device__ __forceinline__ float activate(float v) {
     return v;
 }
 
-// Epilogue of one 256-column accumulator for a layer that hands on nothing but bits.
-template <bool ZERO_NEG>
+// Epilogue of one accumulator of COLS columns for a layer that hands on nothing but bits.
+template <bool ZERO_NEG, int COLS>
 __device__ __forceinline__ void epilogue_bits(uint32_t taddr, const float* sc, const float* sh, int cols_left,
                                               uint32_t* dst, int words_left, bool row_ok) {
     // (loads of columns beyond the layer's last unit stay inside the accumulator; their bits are
@@ -193,7 +198,7 @@ __device__ __forceinline__ void epilogue_bits(uint32_t taddr, const float* sc, c
     uint32_t a0[16], a1[16];
     tmem_ld16(taddr, a0);
 #pragma unroll 1
-    for (int q4 = 0; q4 < 2; ++q4) {              // 128 columns = four words = one 16-byte store
+    for (int q4 = 0; q4 < COLS / 128; ++q4) {              // 128 columns = four words = one 16-byte store
         if (q4 * 128 >= cols_left) break;         // uniform over the CTA
         uint32_t words[4];
 #pragma unroll
@@ -203,7 +208,7 @@ __device__ __forceinline__ void epilogue_bits(uint32_t taddr, const float* sc, c
             tmem_ld16(taddr + c + 16, a1);
             uint32_t wd = sign_bits16<ZERO_NEG>(a0, sc + c, sh + c);
             tmem_ld_wait();
-            if (c + 32 < 256) tmem_ld16(taddr + c + 32, a0);
+            if (c + 32 < COLS) tmem_ld16(taddr + c + 32, a0);
             wd |= sign_bits16<ZERO_NEG>(a1, sc + c + 16, sh + c + 16) << 16;
             const int valid = cols_left - c;
             words[gq] = valid >= 32 ? wd : (valid > 0 ? (wd & ((1u << valid) - 1u)) : 0u);
@@ -327,15 +332,15 @@ struct Args {
     TcStatus status;
 };
 
-template <int NT>
+template <int NT, int UN>
 __global__ void __launch_bounds__(THREADS, 1) signw_img_kernel(Args g) {
-    using C = Cfg<NT>;
+    using C = Cfg<NT, UN>;
     extern __shared__ uint8_t smem_raw[];
     uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 127) & ~uintptr_t(127));
     Control* ctl = reinterpret_cast<Control*>(smem + C::STAGES * C::STAGE_BYTES);
     volatile int* abort_flag = &ctl->wait.abort;
 
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int warp = warp_index(), lane = threadIdx.x & 31;
     const int M = g.M, N = g.N;
     const int nks = ceil_div(g.K, BK);
     const int m_tiles = ceil_div(M, BM), n_tiles = ceil_div(N, UN);
@@ -346,7 +351,8 @@ __global__ void __launch_bounds__(THREADS, 1) signw_img_kernel(Args g) {
             mbar_init(smem_u32(&ctl->full[s]), PROD_WARPS);
             mbar_init(smem_u32(&ctl->empty[s]), 1);
         }
-        mbar_init(smem_u32(&ctl->acc_full), 1);
+        mbar_init(smem_u32(&ctl->acc_full[0]), 1);
+        mbar_init(smem_u32(&ctl->acc_full[1]), 1);
         mbar_init(smem_u32(&ctl->acc_empty[0]), EPI_WARPS);
         mbar_init(smem_u32(&ctl->acc_empty[1]), EPI_WARPS);
         wait_state_init(&ctl->wait, g.status);
@@ -362,37 +368,40 @@ __global__ void __launch_bounds__(THREADS, 1) signw_img_kernel(Args g) {
     const uint32_t tmem = ctl->tmem_base;
 
     if (warp >= PROD_WARP0) {
-        // ---------------- producers: thread p widens packed weight rows p and p+256 of the unit
-        // tile; the first producer thread also starts the bulk copy of the activation stage.
+        // ---------------- producers: thread p widens packed weight rows p and p + 256 of a tile of 512 units, row p of
+        // one of 256, half of row p % 128 of one of 128; the first producer thread also starts the bulk copy of the
+        // activation stage.
         const int p = threadIdx.x - PROD_WARP0 * 32;  // 0..255
+        constexpr int ROWS = UN == 512 ? 2 : 1, CHUNKS = UN == 128 ? 2 : 4;
+        const int prow = p & (UN < 256 ? UN - 1 : 255), chunk0 = UN == 128 ? (p >> 7) * 2 : 0;
         const int my_tiles = (tiles - 1 - (int)blockIdx.x) / (int)gridDim.x + 1;
         const int total = my_tiles * nks;
         // Packed rows are read 16 bytes (4 stages) at a time, one group ahead of use.  Bits at
         // positions >= K may hold anything: the activation image is zero there.
         const int ngroups = ceil_div(nks, 4);
         int pf_g = 0, pf_tile = blockIdx.x, pf_left = my_tiles;
-        auto fetch = [&](uint4 (&o)[2]) {
-            o[0] = make_uint4(0u, 0u, 0u, 0u);
-            o[1] = o[0];
+        auto fetch = [&](uint4 (&o)[ROWS]) {
+#pragma unroll
+            for (int q = 0; q < ROWS; ++q) o[q] = make_uint4(0u, 0u, 0u, 0u);
             if (pf_left == 0) return;
             const int n0 = (pf_tile / m_tiles) * UN;
 #pragma unroll
-            for (int q = 0; q < 2; ++q) {
-                const int n = n0 + p + 256 * q;
+            for (int q = 0; q < ROWS; ++q) {
+                const int n = n0 + prow + 256 * q;
                 if (n < N) o[q] = ldg_nc_u4(reinterpret_cast<const uint4*>(g.Wp + (size_t)n * g.ldwp) + pf_g);
             }
             if (++pf_g == ngroups) { pf_g = 0; pf_tile += gridDim.x; --pf_left; }
         };
-        uint4 grp[2], nxt[2];
+        uint4 grp[ROWS], nxt[ROWS];
         fetch(grp);
         fetch(nxt);
         int ks = 0, tile = blockIdx.x, s = 0;
         uint32_t ph = 1;  // parity to wait for on `empty`: a fresh barrier passes parity 1
         for (int it = 0; it < total; ++it) {
             const int sub = ks & 3;
-            uint32_t cur[2];
+            uint32_t cur[ROWS];
 #pragma unroll
-            for (int q = 0; q < 2; ++q)
+            for (int q = 0; q < ROWS; ++q)
                 cur[q] = sub == 0 ? grp[q].x : sub == 1 ? grp[q].y : sub == 2 ? grp[q].z : grp[q].w;
             if (!warp_wait(smem_u32(&ctl->empty[s]), ph, abort_flag, lane)) break;
             const uint32_t st = smem_u32(smem) + s * C::STAGE_BYTES;
@@ -405,14 +414,14 @@ __global__ void __launch_bounds__(THREADS, 1) signw_img_kernel(Args g) {
                 bulk_g2s(st, g.img + ((size_t)mt * nks + ks) * C::A_BYTES, C::A_BYTES, smem_u32(&ctl->full[s]));
             }
 #pragma unroll
-            for (int q = 0; q < 2; ++q) {
-                const uint32_t nw = ~cur[q];
-                uint32_t wv[16];
+            for (int q = 0; q < ROWS; ++q) {
+                const uint32_t nw = ~cur[q] << (CHUNKS == 2 ? 8 - 4 * chunk0 : 0);     // the second half's bits are 8 higher
+                uint32_t wv[4 * CHUNKS];
 #pragma unroll
-                for (int t = 0; t < 16; ++t) wv[t] = ((nw << (15 - t)) & 0x80008000u) | 0x3F803F80u;
+                for (int t = 0; t < 4 * CHUNKS; ++t) wv[t] = ((nw << (4 * CHUNKS - 1 - t)) & 0x80008000u) | 0x3F803F80u;
 #pragma unroll
-                for (int c = 0; c < 4; ++c)
-                    sts128(st + C::A_BYTES + (c * UN + p + 256 * q) * 16, wv[4 * c], wv[4 * c + 1], wv[4 * c + 2], wv[4 * c + 3]);
+                for (int c = 0; c < CHUNKS; ++c)
+                    sts128(st + C::A_BYTES + ((chunk0 + c) * UN + prow + 256 * q) * 16, wv[4 * c], wv[4 * c + 1], wv[4 * c + 2], wv[4 * c + 3]);
             }
             fence_proxy_async_smem();
             __syncwarp();
@@ -420,11 +429,45 @@ __global__ void __launch_bounds__(THREADS, 1) signw_img_kernel(Args g) {
             if (++s == C::STAGES) { s = 0; ph ^= 1u; }
             ++ks;
             if ((ks & 3) == 0 || ks == nks) {   // group used up: take the prefetched one
-                grp[0] = nxt[0]; grp[1] = nxt[1];
+#pragma unroll
+                for (int q = 0; q < ROWS; ++q) grp[q] = nxt[q];
                 fetch(nxt);
             }
             if (ks == nks) { ks = 0; tile += gridDim.x; }
         }
+    } else if (UN != 512 && warp == MMA_WARP) {
+        // ---------------- MMA issue, one accumulator per tile, two in turn: a converged warp, the MMAs of a stage
+        // from one elected lane
+        constexpr uint32_t idesc = instr_desc(kAccF32, kFmtBF16, kFmtBF16, BM, C::SUB);
+        const uint64_t da0 = smem_desc_kmajor(smem_u32(smem), BM * 16, 128), db0 = smem_desc_kmajor(smem_u32(smem) + C::A_BYTES, UN * 16, 128);
+        int s = 0, tl = 0;
+        uint32_t ph = 0;
+        bool ok = true;
+        for (int tile = blockIdx.x; tile < tiles && ok; tile += gridDim.x, ++tl) {
+            const int b = tl & 1;
+            ok = warp_wait(smem_u32(&ctl->acc_empty[b]), (uint32_t)(((tl >> 1) & 1) ^ 1), abort_flag, lane);
+            if (!ok) break;
+            tc_fence_after_sync();
+            for (int ks = 0; ks < nks; ++ks) {
+                ok = warp_wait(smem_u32(&ctl->full[s]), ph, abort_flag, lane);
+                if (!ok) break;
+                tc_fence_after_sync();
+                // the address field (16-byte units) is advanced by plain additions: the ring lies below 2^14 * 16 bytes
+                const uint64_t da = da0 + (uint64_t)(s * (C::STAGE_BYTES >> 4)), db = db0 + (uint64_t)(s * (C::STAGE_BYTES >> 4));
+                if (elect_one()) {
+#pragma unroll
+                    for (int j = 0; j < 2; ++j)
+#pragma unroll
+                        for (int q = 0; q < NT; ++q)
+                            mma_f16(tmem + b * C::SUB, da + (uint64_t)((q * A_PLANE + 2 * j * (BM * 16)) >> 4), db + (uint64_t)((2 * j * (UN * 16)) >> 4),
+                                    idesc, (ks | j | q) != 0);
+                    mma_commit(smem_u32(&ctl->empty[s]));
+                }
+                if (++s == C::STAGES) { s = 0; ph ^= 1u; }
+            }
+            if (ok && elect_one()) mma_commit(smem_u32(&ctl->acc_full[b]));
+        }
+        __syncwarp();
     } else if (warp == MMA_WARP) {
         if (lane == 0) {
             constexpr uint32_t idesc = instr_desc(kAccF32, kFmtBF16, kFmtBF16, BM, 256);
@@ -479,7 +522,7 @@ __global__ void __launch_bounds__(THREADS, 1) signw_img_kernel(Args g) {
                     issue(s, 1, ks);
                     mma_commit(smem_u32(&ctl->empty[s]));
                 }
-                if (ok) mma_commit(smem_u32(&ctl->acc_full));
+                if (ok) mma_commit(smem_u32(&ctl->acc_full[0]));
             }
         }
         __syncwarp();
@@ -502,7 +545,21 @@ __global__ void __launch_bounds__(THREADS, 1) signw_img_kernel(Args g) {
                 ctl->sh[nl] = (g.shift && n < N) ? g.shift[n] : 0.0f;
             }
             epi_bar_sync();
-            ok = epi_all(warp_wait(smem_u32(&ctl->acc_full), (uint32_t)(tl & 1), abort_flag, lane));
+            if constexpr (UN != 512) {
+                const int b = tl & 1;
+                ok = epi_all(warp_wait(smem_u32(&ctl->acc_full[b]), (uint32_t)((tl >> 1) & 1), abort_flag, lane));
+                if (!ok) break;
+                tc_fence_after_sync();
+                const uint32_t taddr = tmem + ((uint32_t)(warp * 32) << 16) + (uint32_t)(b * C::SUB);
+                uint32_t* bits = g.out_bits + (size_t)(m < M ? m : 0) * g.ldob + (n0 >> 5);
+                if (g.sign_mode == kSignZeroNeg) epilogue_bits<true, C::SUB>(taddr, ctl->sc, ctl->sh, N - n0, bits, nw - (n0 >> 5), m < M);
+                else epilogue_bits<false, C::SUB>(taddr, ctl->sc, ctl->sh, N - n0, bits, nw - (n0 >> 5), m < M);
+                tc_fence_before_sync();
+                __syncwarp();
+                if (lane == 0) mbar_arrive(smem_u32(&ctl->acc_empty[b]));
+                continue;
+            }
+            ok = epi_all(warp_wait(smem_u32(&ctl->acc_full[0]), (uint32_t)(tl & 1), abort_flag, lane));
             if (!ok) break;
             tc_fence_after_sync();
 #pragma unroll 1
@@ -528,8 +585,8 @@ __global__ void __launch_bounds__(THREADS, 1) signw_img_kernel(Args g) {
                         }
                     }
                     if (pack && !g.Y) {
-                        if (g.sign_mode == kSignZeroNeg) epilogue_bits<true>(taddr, sc, sh, left, bits, nw - w0, m < M);
-                        else epilogue_bits<false>(taddr, sc, sh, left, bits, nw - w0, m < M);
+                        if (g.sign_mode == kSignZeroNeg) epilogue_bits<true, 256>(taddr, sc, sh, left, bits, nw - w0, m < M);
+                        else epilogue_bits<false, 256>(taddr, sc, sh, left, bits, nw - w0, m < M);
                     } else if (pack) {
                         epilogue_real<BNN_ACT_SIGN_PACK, NT>(taddr, sc, sh, left, y, vy, bits, nw - w0, m < M, g.sign_mode, ImageOut{nullptr, 0u, 0u, 0u, false});
                     } else if (g.act == BNN_ACT_HARDTANH) {
@@ -558,27 +615,56 @@ __global__ void __launch_bounds__(THREADS, 1) signw_img_kernel(Args g) {
     if (threadIdx.x == 0 && ctl->wait.abort) atomicExch(g.status.word, 1);
 }
 
+template <int NT, int UN>
+int launch_gemm(const Args& a, int mt, int sms, cudaStream_t st) {
+    using C = Cfg<NT, UN>;
+    constexpr int SMEM = C::STAGES * C::STAGE_BYTES + (int)sizeof(Control) + 128;
+    static_assert(SMEM <= 232448, "shared memory of one CTA");
+    if (!ensure_dynamic_smem(reinterpret_cast<const void*>(signw_img_kernel<NT, UN>), SMEM)) return BNN_ERR_CUDA;
+    const int tiles = mt * ceil_div(a.N, UN);
+    if (launch_pdl(signw_img_kernel<NT, UN>, dim3(tiles < sms ? tiles : sms), dim3(THREADS), SMEM, st, a) != cudaSuccess)
+        return BNN_ERR_CUDA;
+    return launch_status();
+}
+
+// Units per tile for two terms and a layer that hands on nothing but bits: the least clocks of the busiest CTA, from what a
+// stage takes (as measured; bound by the MMAs at 512 units, by the widening at 128) and, with a single tile, its epilogue.
+int tile_units(int mt, int N, int nks, int sms) {
+    struct Candidate { int un, stage, ends; };
+    const Candidate all[] = {{512, 1040, 3500}, {256, 560, 2500}, {128, 400, 1800}};
+    int best = 512;
+    long long best_cost = 0;
+    for (const Candidate& c : all) {
+        const int turns = ceil_div(mt * ceil_div(N, c.un), sms);
+        const long long cost = (long long)turns * nks * c.stage + c.ends;
+        if (best_cost == 0 || cost < best_cost) { best = c.un; best_cost = cost; }
+    }
+    return best;
+}
+
 template <int NT>
 int launch_nt(const RealGemmArgs& r, void* workspace, bool image_ready, void* out_image, int out_kind, int* clear,
               int clear_words, cudaStream_t st) {
-    using C = Cfg<NT>;
-    constexpr int SMEM = C::STAGES * C::STAGE_BYTES + (int)sizeof(Control) + 128;
     const int sms = device_sm_count();
-    if (sms <= 0 || !ensure_dynamic_smem(reinterpret_cast<const void*>(signw_img_kernel<NT>), SMEM)) return BNN_ERR_CUDA;
+    if (sms <= 0) return BNN_ERR_CUDA;
     const int nks = ceil_div(r.K, BK), mt = ceil_div(r.M, BM);
     uint8_t* img = static_cast<uint8_t*>(workspace);
+    Args a{static_cast<uint8_t*>(out_image), ceil_div(r.N, BK), out_kind, img, r.Bb, r.ldb, r.M, r.N, r.K, r.scale, r.shift, r.act, r.sign_mode, r.Y, r.ldy, r.out_bits, r.ldob,
+           tc_status()};
+    if (!a.status.word) return BNN_ERR_CUDA;
     // (when the kernel before this one in the stream already wrote the image -- the layer that produced
     // these activations -- there is nothing to split)
     if (!image_ready)
         x_split_kernel<NT><<<mt * nks, 256, 0, st>>>(r.Af, r.lda, r.M, r.K, nks, img, r.splice_dim, r.splice_left, clear,
                                                      clear ? clear_words : 0);
-    Args a{static_cast<uint8_t*>(out_image), ceil_div(r.N, BK), out_kind, img, r.Bb, r.ldb, r.M, r.N, r.K, r.scale, r.shift, r.act, r.sign_mode, r.Y, r.ldy, r.out_bits, r.ldob,
-           tc_status()};
-    if (!a.status.word) return BNN_ERR_CUDA;
-    const int tiles = mt * ceil_div(r.N, UN);
-    if (launch_pdl(signw_img_kernel<NT>, dim3(tiles < sms ? tiles : sms), dim3(THREADS), SMEM, st, a) != cudaSuccess)
-        return BNN_ERR_CUDA;
-    return launch_status();
+    if constexpr (NT == 2) {
+        if (r.act == BNN_ACT_SIGN_PACK && r.out_bits && !r.Y && !out_image) {
+            const int un = tile_units(mt, r.N, nks, sms);
+            if (un == 256) return launch_gemm<NT, 256>(a, mt, sms, st);
+            if (un == 128) return launch_gemm<NT, 128>(a, mt, sms, st);
+        }
+    }
+    return launch_gemm<NT, 512>(a, mt, sms, st);
 }
 
 }  // namespace
