@@ -267,16 +267,22 @@ def layer_table(cfg, frames, peaks, sm_mhz, xnor_path="tensor", real_path="tenso
             # (a sign-weight layer fed by another one finds its split-activation image written by that
             # layer's epilogue: no split launch of its own)
             chained = l > 0 and not mixed
-            rows.append(dict(name="signw_%d" % (l + 1), kernel="signw_img_kernel" if chained else "x_split_kernel+signw_img_kernel",
-                             work=work, unit="TFLOP/s", bound="tensor", peak=peaks["bf16"], passes=2))
+            if cfg.act == 1:
+                rows.append(dict(name="signw_%d" % (l + 1), kernel="x_split_kernel+signw_img_kernel",
+                                 work=work, unit="TFLOP/s", bound="tensor", peak=peaks["bf16"], passes=2))
+            else:
+                # three byte digits of the activations, exact integer MMAs at twice the half-precision rate
+                rows.append(dict(name="signw_%d" % (l + 1), kernel="signw_digit_kernel" if chained else "x_digits_kernel+signw_digit_kernel",
+                                 work=work, unit="TFLOP/s", bound="tensor", peak=2.0 * peaks["bf16"], passes=3))
         else:
             rows.append(dict(name="signw_%d" % (l + 1), kernel="real_gemm_kernel", work=work, unit="TFLOP/s",
                              bound="alu", peak=fp32_peak))
         k = cfg.hidden
     owork = 2.0 * frames * cfg.classes * cfg.hidden
     if real_path == "tensor" and cfg.act == 1 and not mixed:
-        rows.append(dict(name="output_gemm", kernel="out_tc_kernel", work=owork, unit="TFLOP/s", bound="tensor",
-                         peak=peaks["bf16"], passes=2))
+        # three byte digits of the weights, exact integer MMAs at twice the half-precision rate
+        rows.append(dict(name="output_gemm", kernel="out_digit_kernel", work=owork, unit="TFLOP/s", bound="tensor",
+                         peak=2.0 * peaks["bf16"], passes=3))
     elif real_path == "tensor":
         # fp32 activations: both operands in two fp16 terms, three MMAs per step
         # (its fp16 activation image comes from the epilogue of the layer before: no split launch)
@@ -294,7 +300,7 @@ def layer_table(cfg, frames, peaks, sm_mhz, xnor_path="tensor", real_path="tenso
             elif r["name"].startswith("xnor"):
                 r.update(kernel="small_xnor_kernel", bound="alu", peak=popc_peak)
                 r.pop("smem_bytes", None)
-            elif r["name"] == "output_gemm":
+            elif r["name"] == "output_gemm" and frames <= 4:
                 r.update(kernel="small_out_kernel", bound="hbm", unit="GB/s", peak=peaks["hbm_gbs"], scale=1e9, passes=1,
                          work=4.0 * cfg.classes * cfg.hidden + 4.0 * frames * cfg.classes)
     # log-softmax: one read and one write of the [frames][classes] fp32 matrix
@@ -589,7 +595,7 @@ def run_ours(args):
         "ms_per_step": total_ms / K, "higher_is_better": True, "scaling": "weak", "vs_baseline": None,
         "dtype": "%s (hidden layers) + %s (first and top layer)"
                  % ("e2m1 (mxf4) tensor-core MMA, f32 accumulate, exact" if args.xnor_path != "popc" else "int32 popcount",
-                    "split bf16/fp16 tensor-core MMA, f32 accumulate" if args.real_path == "tensor" else "f32"),
+                    "split bf16 tensor-core MMA, f32 accumulate / byte digits, s32 accumulate, exact" if args.real_path == "tensor" else "f32"),
         "device_status": B.bnn_device_status(), "data": "synthetic",
         "config": {"workload": workload_name(cfg, frames), "frames_per_gpu": frames,
                    "launch": "host launches" if args.no_graph else "one captured CUDA graph per step (a single bnn_forward call each)", "l2": "inputs/outputs rotate over %d buffer sets (%.0f MB > 2 x L2); weights stay hot"
