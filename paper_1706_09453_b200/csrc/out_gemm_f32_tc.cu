@@ -95,6 +95,8 @@ template <bool FROM_I32>
 __global__ void __launch_bounds__(SPLIT_THREADS)
 h_split_kernel(const void* __restrict__ src, int ldh, int M, int H, int nks, uint8_t* __restrict__ img,
                const float* __restrict__ scale, const float* __restrict__ shift) {
+    pdl_trigger();
+    pdl_wait();
     const int ks = (int)blockIdx.x % nks, rb = (int)blockIdx.x / nks;      // rb: block of SPLIT_ROWS rows
     const int c = threadIdx.x & 3, m = rb * SPLIT_ROWS + ((int)threadIdx.x >> 2);
     const int ft = m / IMG, row = m % IMG, k0 = ks * BK + 4 * c;
@@ -189,6 +191,8 @@ outf_tc_kernel(const uint8_t* __restrict__ himg, const uint8_t* __restrict__ wim
     __syncthreads();
     tc_fence_after_sync();
     const uint32_t tmem = ctl->tmem_base;
+    pdl_trigger();
+    pdl_wait();      // the set-up above overlaps the end of the kernel before this one
 
     if (warp == TMA_WARP) {
         // ---------------- a warp streams both images, a lane per copy (one thread takes about 100 clocks for each); class
@@ -363,13 +367,15 @@ static int launch_gemm(const uint8_t* himg, const uint8_t* wimg, const float* rs
     cfg.blockDim = dim3(THREADS);
     cfg.dynamicSmemBytes = SMEM;
     cfg.stream = st;
-    cudaLaunchAttribute attr;
-    attr.id = cudaLaunchAttributeClusterDimension;
-    attr.val.clusterDim.x = SPLIT;
-    attr.val.clusterDim.y = 1;
-    attr.val.clusterDim.z = 1;
-    cfg.attrs = &attr;
-    cfg.numAttrs = SPLIT > 1 ? 1 : 0;
+    cudaLaunchAttribute attr[2];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    attr[1].id = cudaLaunchAttributeClusterDimension;
+    attr[1].val.clusterDim.x = SPLIT;
+    attr[1].val.clusterDim.y = 1;
+    attr[1].val.clusterDim.z = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = SPLIT > 1 ? 2 : 1;
     if (cudaLaunchKernelEx(&cfg, kern, himg, wimg, rs, bias, M, C, H, Z, ldz, act, status) != cudaSuccess) return BNN_ERR_CUDA;
     return launch_status();
 }
@@ -391,7 +397,9 @@ int launch_outf_tc(const float* Hf, int ldhf, const void* prepared, const float*
     const float* rs = reinterpret_cast<const float*>(wimg + (size_t)ct * hs * A_BYTES);
     uint8_t* himg = static_cast<uint8_t*>(workspace);
     if (!image_ready)   // (else the layer that produced the activations wrote the image itself)
-        h_split_kernel<false><<<ceil_div(M, IMG) * hs * (IMG / SPLIT_ROWS), SPLIT_THREADS, 0, st>>>(Hf, ldhf, M, H, hs, himg, nullptr, nullptr);
+        if (launch_pdl(h_split_kernel<false>, dim3(ceil_div(M, IMG) * hs * (IMG / SPLIT_ROWS)), dim3(SPLIT_THREADS), 0, st, Hf, ldhf, M, H, hs, himg,
+                       nullptr, nullptr) != cudaSuccess)
+            return BNN_ERR_CUDA;
     const Tiling t = tiling(M, C, hs, act, sms);
     if (t.frames == 64) return launch_split<64>(t.split, himg, wimg, rs, bias, M, C, H, Z, ldz, act, sms, st);
     if (t.frames == 128) return launch_split<128>(t.split, himg, wimg, rs, bias, M, C, H, Z, ldz, act, sms, st);
@@ -402,7 +410,9 @@ int launch_outf_tc(const float* Hf, int ldhf, const void* prepared, const float*
 int launch_outf_image_from_i32(const int32_t* D, int ldd, const float* scale, const float* shift, int M, int H,
                                void* image, cudaStream_t st) {
     const int hs = ceil_div(H, BK), ft = ceil_div(M, IMG);
-    h_split_kernel<true><<<ft * hs * (IMG / SPLIT_ROWS), SPLIT_THREADS, 0, st>>>(D, ldd, M, H, hs, static_cast<uint8_t*>(image), scale, shift);
+    if (launch_pdl(h_split_kernel<true>, dim3(ft * hs * (IMG / SPLIT_ROWS)), dim3(SPLIT_THREADS), 0, st, D, ldd, M, H, hs, static_cast<uint8_t*>(image),
+                   scale, shift) != cudaSuccess)
+        return BNN_ERR_CUDA;
     return launch_status();
 }
 

@@ -228,6 +228,7 @@ __device__ __forceinline__ float block_logsumexp(float mx, float s, float* sm, f
 __global__ void __launch_bounds__(256)
 log_softmax_rows_kernel(float* __restrict__ Z, int ldz, int M, int C, const float* __restrict__ prior) {
     __shared__ float sm[8], ss[8];
+    pdl_wait();
     for (int row = blockIdx.x; row < M; row += gridDim.x) {
         float* z = Z + (size_t)row * ldz;
         float mx = -FLT_MAX, s = 0.f;
@@ -356,6 +357,7 @@ __global__ void __launch_bounds__(256)
 log_softmax_rows_reg_kernel(float* __restrict__ Z, int ldz, int M, int C, const float* __restrict__ prior) {
     __shared__ float sm[2][1][8], ss[2][1][8];
     int par = 0;
+    pdl_wait();
     // Rows are taken from the last one down: the kernel that wrote the logits just before this one
     // produced the last frames last, and those are the rows the L2 cache still holds.
     for (int r = blockIdx.x; r < M; r += gridDim.x, par ^= 1)
@@ -462,8 +464,7 @@ int launch_log_softmax_rows(float* Z, int ldz, int M, int C, const float* prior,
     auto kern = C <= 256 * 4 * 2 ? (even ? log_softmax_rows_reg_kernel<2, true> : log_softmax_rows_reg_kernel<2, false>)
               : C <= 256 * 4 * 4 ? (even ? log_softmax_rows_reg_kernel<4, true> : log_softmax_rows_reg_kernel<4, false>)
                                      : log_softmax_rows_kernel;
-    kern<<<blocks, 256, 0, st>>>(Z, ldz, M, C, prior);
-    return launch_status();
+    return launch_pdl(kern, dim3(blocks), dim3(256), 0, st, Z, ldz, M, C, prior) == cudaSuccess ? launch_status() : BNN_ERR_CUDA;
 }
 
 }  // namespace bnn
