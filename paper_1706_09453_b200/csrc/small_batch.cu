@@ -20,8 +20,8 @@
 // weights are in registers when that opens.
 // The per-frame partial sums of a unit are reduced all at once, each step halving
 // the number of frames a lane is responsible for (31 shuffles for 16 frames instead of 80) in the same tree.
-// Measured on B200, 440 -> 6 x 2048 -> 3307, a launch per layer and 32 units a block before: one frame 44 -> 31 us (the
-// host's four launches take 25), 16 frames 85 -> 45 (run of five layers 31 -> 18 us of kernel time and four launches less,
+// Measured on B200, 440 -> 6 x 2048 -> 3307, a launch per layer and 32 units a block before: one frame 44 -> 29 us (the
+// host's four launches take 20 to 25), 16 frames 85 -> 41 (run of five layers 31 -> 18 us of kernel time and four launches less,
 // first layer 12 -> 6; the rest from the top layer, which takes the digit kernel beyond four frames).  The top
 // layer's kernel is launched plainly: started under the run it takes from the run what it gains (3 frames 37 us against 33).
 #include "bnn_common.cuh"

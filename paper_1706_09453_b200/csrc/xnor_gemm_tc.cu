@@ -33,7 +33,7 @@
 //
 // What bounds it, measured on B200: the widening (two teams per operand; a stage takes about 720 clocks against 384
 // of MMA; with one team per operand, one issuing thread and the int32 tile written out by the epilogue warps it took
-// about 1000).  65536 x 4096 x 4096, int32 out, 646 -> 490 us; 4096 x 2048 x 4096 31 -> 26 us (its tiles have 8
+// about 1000).  65536 x 4096 x 4096, int32 out, 647 -> 472 us; 4096 x 2048 x 4096 31 -> 23 us (its tiles have 8
 // stages, so the int32 epilogue counts there).
 #include "bnn_common.cuh"
 #include "tcgen05.cuh"
