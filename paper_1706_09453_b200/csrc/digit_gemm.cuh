@@ -266,9 +266,13 @@ __device__ __forceinline__ void issue(const Work& w, uint32_t ring, Bars* bars, 
         const uint32_t d = tmem + (uint32_t)(b * w.n);
         for (int kb = 0; kb < blocks; ++kb) {
             if ((kb & 1) == which) {
-                if (!warp_wait_both(smem_u32(&bars->full_b[sb]), pb, smem_u32(&bars->full_a[2 * sa]), pa, abort_flag)) return;
-                // only the MMA that overwrites the accumulator has to come first
+                // The MMA that overwrites the accumulator has to come first.  This wait also stands before those for the
+                // stage, because a wait on a parity holds only for one who knows that the phase before it is over.  With
+                // an odd number of stages per tile the other warp takes two in a row, the last of a tile and the first
+                // of the next; when there are two slots the former had this stage's.  `started` says that the other
+                // warp has issued the latter, so it has found the former full.
                 if (kb == 1 && !warp_wait(smem_u32(&bars->started[b]), (uint32_t)((tl >> 1) & 1), abort_flag, 0)) return;
+                if (!warp_wait_both(smem_u32(&bars->full_b[sb]), pb, smem_u32(&bars->full_a[2 * sa]), pa, abort_flag)) return;
                 tc_fence_after_sync();
                 // the address field (16-byte units) is advanced by plain additions: the ring lies below 2^14 * 16 bytes
                 const uint32_t db = desc_lo + (uint32_t)sb * stage16;

@@ -102,3 +102,74 @@ def test_signw_gemm_digits_rows_with_infinities_and_nans(env):
     bad[[3, 11]] = True
     np.testing.assert_array_equal(out[0][~bad], out[1][~bad])
     assert np.isnan(out[1][bad]).all()
+
+
+# Several turns of the persistent grid on wide tiles with an odd number of 256-position stages per tile, where the two issuing
+# warps change places from tile to tile and the two slots of widened bits with them; the last stage short or whole.
+@pytest.mark.parametrize("m,h,c", [(8192, 1100, 3400), (6000, 520, 2000), (8192, 2100, 1500), (4096, 768, 3307)])
+@pytest.mark.parametrize("outlier", [False, True])
+@pytest.mark.parametrize("values", [0, 1])
+def test_output_layer_digits_many_tiles(env, m, h, c, outlier, values):
+    torch, B, model = env
+    rng = np.random.default_rng(m + h + c)
+    hp = wl.make_bit_planes(m, h, 0.5, 7 + m + h, B.packed_pitch(h))
+    w = rng.normal(0, 1 / np.sqrt(h), (c, h)).astype(np.float32)
+    if outlier:
+        w[c // 2] *= np.float32(1e-5)
+        w[c // 2, h // 3] = 1.0
+    digits = torch.empty(B.bnn_output_digits_bytes(c, h), dtype=torch.uint8, device="cuda:0")
+    wd = model.to_dev(w)
+    B.bnn_output_prepare_digits(wd, digits)
+    a = torch.from_numpy(np.unpackbits(hp.view(np.uint8), axis=1, bitorder="little")[:, :h]).cuda().double()
+    want = (a if values else 2 * a - 1) @ wd.double().T
+    # as above: half a unit of the row's scale per weight, then two roundings of the result
+    bound = h * wd.abs().amax(1).double() * (2.0 ** -30 if outlier else 2.0 ** -22) / 2 + 2.0 ** -23 * want.abs()
+    z = torch.empty((m, c), dtype=torch.float32, device="cuda:0")
+    hpd = model.to_dev(hp)
+    for _ in range(4):
+        z.fill_(9.0)
+        B.bnn_output_layer_digits(hpd, digits, None, z, h, log_softmax=False, values=values)
+        assert bool(((z.double() - want).abs() <= bound).all()), float(((z.double() - want).abs() / bound).max())
+    assert B.bnn_device_status() == 0
+
+
+@pytest.mark.parametrize("m,n,k", [(8192, 2048, 600), (6000, 2048, 1100), (5001, 2500, 2100)])
+def test_signw_gemm_digits_many_tiles(env, m, n, k):
+    torch, B, model = env
+    x = torch.randn((m, k), generator=torch.Generator("cuda:0").manual_seed(m + n + k), device="cuda:0")
+    wp = wl.make_bit_planes(n, k, 0.5, 3 + m + n, B.packed_pitch(k))
+    w = 2 * torch.from_numpy(np.unpackbits(wp.view(np.uint8), axis=1, bitorder="little")[:, :k]).cuda().double() - 1
+    want = x.double() @ w.T
+    bound = k * x.abs().amax(1).double()[:, None] * 2.0 ** -22 / 2 + 2.0 ** -23 * want.abs()     # as above
+    ws = torch.empty(B.bnn_signw_workspace_bytes(m, k), dtype=torch.uint8, device="cuda:0")
+    y = torch.empty((m, n), dtype=torch.float32, device="cuda:0")
+    wd = model.to_dev(wp)
+    for _ in range(4):
+        y.fill_(9.0)
+        B.bnn_signw_gemm(x, wd, k, Y=y, workspace=ws)
+        assert bool(((y.double() - want).abs() <= bound).all()), float(((y.double() - want).abs() / bound).max())
+    assert B.bnn_device_status() == 0
+
+
+def test_chained_digit_layers_many_tiles(env):
+    """Layers of 1100 units with binary weights only, each against double precision on the activations it was given."""
+    torch, B, model = env
+    cfg = wl.Config("chained", 3, 6000, 600, 1100, 4, 300, wl.ACT_HARDTANH, True)
+    net = wl.make_model(cfg)
+    dn = model.DeviceNet(net)
+    x = model.to_dev(wl.make_frames(cfg, cfg.frames))
+    outs = dn.layer_out_buffers(cfg.frames)
+    for _ in range(4):
+        dn.forward(x, layer_out=outs)
+        below = x
+        for l in range(cfg.n_hidden):
+            w = torch.from_numpy(np.where(np.asarray(net.W[l]) < 0, -1.0, 1.0)).cuda()
+            sc, sh = (torch.from_numpy(np.array(v, dtype=np.float64)).cuda() for v in (net.scale[l], net.shift[l]))
+            dot = below.double() @ w.T
+            # half a unit of the scale per value: 2^-22 of the frame's largest in the first layer, of 1 behind a hardtanh
+            unit = below.abs().amax(1).double()[:, None] if l == 0 else 1.0
+            bound = sc.abs() * (w.shape[1] * unit * 2.0 ** -22 / 2 + 2.0 ** -23 * dot.abs()) + 2.0 ** -23 * (sc * dot + sh).abs()
+            err = (outs[l].double() - (sc * dot + sh).clamp(-1, 1)).abs()
+            assert bool((err <= bound).all()), (l, float((err / bound).max()))
+            below = outs[l]
+    assert B.bnn_device_status() == 0
