@@ -89,7 +89,7 @@ template <int BN> struct Cfg {
 constexpr int MAX_STACK = kXnorStackMax;
 
 struct Control {
-    float T[192];            // per unit: threshold
+    float T[192];            // per unit: threshold less 1/2
     uint32_t flipw[8];
     uint64_t full_a[MAX_A_BARS], empty_a[MAX_A_BARS], full_b[MAX_SLOTS], b_free[MAX_SLOTS], acc_full[2], acc_empty[2];
     uint64_t group_full[GROUPS], group_empty[GROUPS];
@@ -475,7 +475,9 @@ xnor_res_kernel(const __grid_constant__ StackMaps maps, const __grid_constant__ 
 #pragma unroll
             for (int h = 0; h < 2; ++h) {
                 const int nl = row_in_tile + h * 128, n = n0 + nl;
-                if (nl < BN) ctl->T[nl] = n < N ? (float)thr[n] : 0.0f;
+                // half-way between two sums: exact for every threshold a sum can meet, and no difference is a zero
+                // (whose sign would depend on that of a sum of zeros)
+                if (nl < BN) ctl->T[nl] = n < N ? (float)thr[n] - 0.5f : 0.0f;
             }
             if (row_in_tile < BN / 32) {
                 const int wi = (n0 >> 5) + row_in_tile;
@@ -498,7 +500,7 @@ xnor_res_kernel(const __grid_constant__ StackMaps maps, const __grid_constant__ 
 #pragma unroll
                 for (int gq = 0; gq < BN / 32; ++gq) {
                     tmem_ld_wait();
-                    // The accumulator holds the integer dot product as a float, and so does T the threshold: the
+                    // The accumulator holds the integer dot product as a float, T the threshold less 1/2: the
                     // sign of their difference is the decision.  The sign bits are shifted in from the top, the last
                     // element first, so element j ends up in bit j, inverted; four chains of eight, joined at the end
                     uint32_t part[4] = {0u, 0u, 0u, 0u};

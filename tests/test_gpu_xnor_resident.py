@@ -48,3 +48,25 @@ def test_resident_run_equals_streamed_layers(env, hidden, frames, values):
         for l, (a, b) in enumerate(zip(layers(B.PREPARED_RESIDENT), want)):
             assert torch.equal(a[:, :words], b[:, :words]), "hidden layer %d" % (l + 1)
     assert B.bnn_device_status() == 0
+
+
+@pytest.mark.parametrize("k,n", [(256, 33), (512, 700), (2048, 2048), (3072, 256)])
+def test_resident_layer_decides_sums_of_zeros(env, k, n):
+    """(0,1) frames without a one on -1 weights: every product is a zero, and the sum 0 meets thresholds around it."""
+    torch, B, model = env
+    m = 200
+    hp = torch.zeros((m, B.packed_pitch(k)), dtype=torch.int32, device="cuda:0")
+    wp = torch.zeros((n, B.packed_pitch(k)), dtype=torch.int32, device="cuda:0")
+    img = torch.empty(B.bnn_xnor_prepared_bytes(n, k), dtype=torch.uint8, device="cuda:0")
+    B.bnn_xnor_prepare(wp, k, img)
+    thr = (torch.arange(n, device="cuda:0", dtype=torch.int32) % 3 - 1)
+    flip = torch.zeros((n + 31) // 32, dtype=torch.int32, device="cuda:0")
+    out = torch.full((m, B.packed_pitch(n)), -1, dtype=torch.int32, device="cuda:0")
+    prev = B.bnn_set_option(B.OPT_XNOR_PREPARED, B.PREPARED_RESIDENT)
+    try:
+        B.bnn_gemm01(hp, None, k, N=n, prepared=img, thr=thr, flip=flip, out_bits=out)
+    finally:
+        B.bnn_set_option(B.OPT_XNOR_PREPARED, prev)
+    bits = (out.unsqueeze(2) >> torch.arange(32, device="cuda:0", dtype=torch.int32)) & 1
+    want = (thr <= 0).int().expand(m, n)
+    assert torch.equal(bits.reshape(m, -1)[:, :n], want)
