@@ -189,7 +189,9 @@ BNN_API int bnn_signw_gemm(const float* X, int ldx, const uint32_t* Wp, int ldwp
  * path.  With two terms (BNN_OPT_SIGNW_TERMS), K <= 2^15 and an activation other than SIGN_PACK the image holds every row of X as fixed-point numbers of a
  * power-of-two scale of its own in three byte digits, and the sums are exact integers:
  *   |y - exact| <= K * 2^-23 * max_k |x[m][k]| + one fp32 rounding (a row with an infinity or a NaN gives NaN);
- * otherwise it holds bf16 terms, as bnn_signw_gemm.  Without workspace (NULL, or too small) it behaves exactly like
+ * otherwise it holds bf16 terms, as bnn_signw_gemm.  Inside bnn_forward a layer writes the image of the next one of its kind
+ * before a frame's largest output is known; max |x| is then replaced by a bound on it, min(1, max |scale| *
+ * sqrt(K) |x'|_2 + max |shift|) for hardtanh units on inputs x', and likewise for Sigmoid.  Without workspace (NULL, or too small) it behaves exactly like
  * bnn_signw_gemm.  The paper has no counterpart. */
 BNN_API size_t bnn_signw_workspace_bytes(int M, int K);
 BNN_API int bnn_signw_gemm_ws(const float* X, int ldx, const uint32_t* Wp, int ldwp,

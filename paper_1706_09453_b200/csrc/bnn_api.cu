@@ -302,8 +302,8 @@ static int signw_impl(const float* X, int ldx, const uint32_t* Wp, int ldwp,
                       int M, int N, int K, float* Y, int ldy,
                       const bnn_epilogue* epi, void* workspace, size_t workspace_bytes,
                       int splice_dim, int splice_left, void* stream,
-                      bool image_ready = false, void* out_image = nullptr, int out_kind = 0,
-                      int* clear = nullptr, int clear_words = 0, bool* cleared = nullptr) {
+                      bool image_ready = false, void* out_image = nullptr, int out_kind = 0, int pos = 0,
+                      const bnn_layer* next = nullptr, int* clear = nullptr, int clear_words = 0, bool* cleared = nullptr) {
     if (cleared) *cleared = false;
     if (int rc = check_dims(M, N, K)) return rc;
     if (!X && !image_ready) return BNN_ERR_NULL;
@@ -329,13 +329,14 @@ static int signw_impl(const float* X, int ldx, const uint32_t* Wp, int ldwp,
         }
     }
     if (!a.Y && !a.out_bits && !out_image) return BNN_ERR_NULL;
+    if (next) { a.next_scale = next->scale; a.next_shift = next->shift; a.next_N = next->N; }
     if (g_real_path != BNN_PATH_CUDA_CORE) {
         if (workspace && !(reinterpret_cast<uintptr_t>(workspace) & 255u) &&
             workspace_bytes >= signw_scratch_bytes(M, K, g_signw_terms, a.act)) {
             // the kernel that splits the activations can clear the caller's counters on its way
             const bool clears = clear && clear_words > 0 && !image_ready;
             if (cleared) *cleared = clears;
-            return launch_signw_img(a, g_signw_terms, workspace, image_ready, out_image, out_kind,
+            return launch_signw_img(a, g_signw_terms, workspace, image_ready, out_image, out_kind, pos,
                                     clears ? clear : nullptr, clears ? clear_words : 0, (cudaStream_t)stream);
         }
         if (splice_dim > 0 || image_ready || out_image) return BNN_ERR_WORKSPACE;
@@ -617,7 +618,7 @@ int bnn_forward_events(const bnn_model* model, const float* X, int ldx, int M,
         }
     }
     bool chain_in = false;   // the layer before wrote this layer's split-activation image (slot chain_slot)
-    int chain_slot = 0;
+    int chain_slot = 0, chain_pos = 0;      // chain_pos: sign-weight layers of the chain so far
     size_t img_half = 0;     // bytes of one of the two alternating images: the largest any sign-weight layer reads
     for (int l = 0; l < L; ++l)
         if (model->layers[l].kind == BNN_LAYER_SIGNW) {
@@ -769,7 +770,7 @@ int bnn_forward_events(const bnn_model* model, const float* X, int ldx, int M,
             }
             rc = signw_impl(static_cast<const float*>(in), in_ld, y.Wp, y.ldwp, M, y.N, y.K,
                             yf, y.N, &e, img_in, img_in_bytes,
-                            l == 0 ? splice_dim : 0, model->splice_left, stream, chain_in, img_out, to_real ? 1 : 0,
+                            l == 0 ? splice_dim : 0, model->splice_left, stream, chain_in, img_out, to_real ? 1 : 0, chain_in ? chain_pos : 0, to_signw ? nx : nullptr,
                             (l == 0 && clear_by_first) ? sync : nullptr, (int)(lay.sync / sizeof(int)), &cleared);
             if (l == 0 && clear_pending) {
                 // the layer took another kernel than the one that clears the counters: clear them now
@@ -779,6 +780,7 @@ int bnn_forward_events(const bnn_model* model, const float* X, int ldx, int M,
             }
             in_ld = out_ld;
             if (chain_out) chain_slot = (chain_in ? chain_slot : 0) ^ 1;
+            chain_pos = chain_in ? chain_pos + 1 : 1;
             chain_in = chain_out;
         } else if (y.kind == BNN_LAYER_REAL) {
             if (l == 0 && splice_dim > 0) return BNN_ERR_UNSUPPORTED;

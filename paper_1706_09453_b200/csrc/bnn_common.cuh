@@ -201,6 +201,9 @@ struct RealGemmArgs {
     int ldy;
     uint32_t* out_bits;   // packed out [M][ldob] or nullptr
     int ldob;
+    const float* next_scale;   // [next_N] or nullptr: of the sign-weight layer that reads the outputs as its image
+    const float* next_shift;
+    int next_N;
 };
 int launch_real_gemm(const RealGemmArgs& a, cudaStream_t st);
 // Tensor-core versions: +-1 weights x real input (A fp32, B bits; `terms` bf16 terms), and
@@ -216,7 +219,9 @@ size_t signw_image_bytes(int M, int K, int terms);
 // layer on fp32 activations reads (two fp16 terms, blocks of 256 frames, outf_image_bytes(M, N) bytes).
 // clear / clear_words (optional, only with image_ready == false): words the splitting kernel sets to zero on
 // its way -- bnn_forward's counters, which would otherwise need a memset of their own in front of it.
-int launch_signw_img(const RealGemmArgs& a, int terms, void* workspace, bool image_ready, void* out_image, int out_kind,
+// pos: how many layers of the chain came before this one (0 when image_ready == false).  A chain of layers that hand one
+// another digits alternates between two places of signw_image_bytes(M, the largest fan-in, 2) bytes.
+int launch_signw_img(const RealGemmArgs& a, int terms, void* workspace, bool image_ready, void* out_image, int out_kind, int pos,
                      int* clear, int clear_words, cudaStream_t st);
 // The same with the activations as byte digits and exact integer sums (signw_digit_tc.cu): what launch_signw_img runs
 // with two terms for layers that hand on real values, unless the fan-in is beyond kMaxKDigit; its image is smaller
@@ -227,7 +232,7 @@ size_t signw_digit_bytes(int M, int K);
 inline size_t signw_scratch_bytes(int M, int K, int terms, int act) {
     return signw_by_digits(terms, K, act) ? signw_digit_bytes(M, K) : signw_image_bytes(M, K, terms);
 }
-int launch_signw_digit(const RealGemmArgs& a, void* workspace, bool image_ready, void* out_image, int out_kind,
+int launch_signw_digit(const RealGemmArgs& a, void* workspace, bool image_ready, void* out_image, int out_kind, int pos,
                        int* clear, int clear_words, cudaStream_t st);
 size_t out_prepared_bytes(int C, int H);
 int launch_out_prepare(const float* W, int ldw, int C, int H, void* prepared, cudaStream_t st);

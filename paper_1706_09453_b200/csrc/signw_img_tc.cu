@@ -673,10 +673,10 @@ size_t signw_image_bytes(int M, int K, int terms) {
     return (size_t)ceil_div(M, BM) * ceil_div(K, BK) * (terms == 3 ? 3 : 2) * A_PLANE;
 }
 
-int launch_signw_img(const RealGemmArgs& r, int terms, void* workspace, bool image_ready, void* out_image, int out_kind,
+int launch_signw_img(const RealGemmArgs& r, int terms, void* workspace, bool image_ready, void* out_image, int out_kind, int pos,
                      int* clear, int clear_words, cudaStream_t st) {
     if (clear && image_ready) return BNN_ERR_UNSUPPORTED;   // no split kernel runs: nobody to clear the words
-    if (signw_by_digits(terms, r.K, r.act)) return launch_signw_digit(r, workspace, image_ready, out_image, out_kind, clear, clear_words, st);
+    if (signw_by_digits(terms, r.K, r.act)) return launch_signw_digit(r, workspace, image_ready, out_image, out_kind, pos, clear, clear_words, st);
     return terms == 3 ? launch_nt<3>(r, workspace, image_ready, out_image, out_kind, clear, clear_words, st)
                       : launch_nt<2>(r, workspace, image_ready, out_image, out_kind, clear, clear_words, st);
 }

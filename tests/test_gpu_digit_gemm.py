@@ -173,3 +173,62 @@ def test_chained_digit_layers_many_tiles(env):
             assert bool((err <= bound).all()), (l, float((err / bound).max()))
             below = outs[l]
     assert B.bnn_device_status() == 0
+
+
+def _chain(torch, B, model, widths, alphas, shift, act, classes=70, seed=0):
+    """A network of layers with binary weights only: widths[0] inputs, one Sigmoid or hardtanh layer per further width."""
+    g = torch.Generator("cuda:0").manual_seed(seed)
+    layers, plain = [], []
+    for l, (k, n) in enumerate(zip(widths, widths[1:])):
+        w = torch.randn((n, k), generator=g, device="cuda:0")
+        wp = model.packed_empty(n, k)
+        B.bnn_pack_weights(w, wp)
+        sc = torch.full((n,), alphas[l], device="cuda:0") * (0.5 + torch.rand((n,), generator=g, device="cuda:0"))
+        sh = torch.full((n,), shift, device="cuda:0") * (0.5 + torch.rand((n,), generator=g, device="cuda:0"))
+        layers.append(dict(kind=B.LAYER_SIGNW, K=k, N=n, Wp=wp, scale=sc, shift=sh, act=act))
+        plain.append((torch.where(w < 0, -1.0, 1.0).double(), sc, sh))
+    w = torch.randn((classes, widths[-1]), generator=g, device="cuda:0")
+    img = torch.empty(B.bnn_output_prepared_bytes(classes, widths[-1]), dtype=torch.uint8, device="cuda:0")
+    B.bnn_output_prepare(w, img)
+    layers.append(dict(kind=B.LAYER_REAL_OUT, K=widths[-1], N=classes, W=w, W_prepared=img))
+    return B.ModelDesc(layers), plain
+
+
+@pytest.mark.parametrize("widths", [[440, 1024, 1024, 1024, 1024, 1024], [200, 700, 96, 1100, 64, 300]])
+@pytest.mark.parametrize("act,alpha,shift", [(2, 0.001, 0.0), (2, 1e-5, 1e-4), (2, 0.05, 0.1), (3, 0.05, -7.0), (3, 0.5, -30.0)])
+@pytest.mark.parametrize("frames", [3, 700])
+def test_chained_layers_of_small_activations(env, widths, act, alpha, shift, frames):
+    """Every layer against double precision on the activations it was given, however small these are; twice, with what the first
+    pass left in the workspace."""
+    torch, B, model = env
+    desc, plain = _chain(torch, B, model, widths, [alpha] * (len(widths) - 1), shift, act)
+    x = torch.randn((frames, widths[0]), generator=torch.Generator("cuda:0").manual_seed(1), device="cuda:0")
+    x[1] *= 1e-3                                                    # one frame far below the others
+    ws = torch.full((desc.workspace_bytes(frames),), 255, dtype=torch.uint8, device="cuda:0")
+    for _ in range(2):
+        outs = [torch.empty((frames, n), device="cuda:0") for n in widths[1:]]
+        logp = torch.empty((frames, 70), device="cuda:0")
+        B.bnn_forward(desc, x, logp, ws, outs)
+        # a value is off by at most half a unit of its frame's scale, and the scale is the finest power of two at which the
+        # bound below stays within 0x7F7F7F
+        below, top = x.double(), x.abs().amax(1).double()
+        for l, ((w, sc, sh), y) in enumerate(zip(plain, outs)):
+            k = w.shape[1]
+            off = k * top[:, None] / 0x7F7F7F
+            dot = below @ w.T
+            pre = sc.double() * dot + sh.double()
+            want = pre.clamp(-1, 1) if act == B.ACT_HARDTANH else torch.sigmoid(pre)
+            tol = sc.abs() * (off + 2.0 ** -22 * dot.abs()) + 2.0 ** -23 * (pre.abs() + sh.abs())
+            if act == B.ACT_SIGMOID:     # its slope is at most its value, and within tol the value changes by a factor e^tol;
+                # expf(-pre) is infinite where the value is below the normal numbers
+                tol = want * torch.expm1(tol) + 2.0 ** -21 * want + 2.0 ** -126
+            err = (y.double() - want).abs()
+            assert bool((err <= tol).all()), float((err / tol).max())
+            # the bound from which the next scale is chosen: sum |x| itself in the first layer, sqrt(k) |x|_2 in the others; it
+            # is counted in high digits, 65536 units each, rounded at both ends
+            d = below.abs().sum(1) if l == 0 else k ** 0.5 * below.norm(dim=1)
+            d = sc.abs().max().double() * (d * 1.002 + 2 * 65536 * k * 2 * top / 0x7F7F7F)
+            top = torch.exp(d + sh.max() + 1e-6 * (d + sh.abs().max())) if act == B.ACT_SIGMOID else d + sh.abs().max()
+            top = (top * 1.0001).clamp(max=1.0)
+            below = y.double()
+    assert B.bnn_device_status() == 0
