@@ -48,7 +48,8 @@ static_assert(SMEM_BYTES <= 232448, "shared memory of one CTA");
 
 // Image of M frames of K values: [K / 16][3 ceil8(M)][16 bytes], then 2^-e per frame.  The images that layers of a chain hand
 // one another start with what the next scales are chosen from: the UnitBounds of the layer that reads the image, and two
-// arrays of a word per frame, the sum of the squares of the frame's high digits (at most 2^29).  Whoever writes the image
+// arrays of a word per frame, the sum of the squares of the frame's high digits (at most 2^29) and, in the top bit, whether an
+// output is a NaN, which has no digits: the reader then takes the frame's scale for a NaN.  Whoever writes the image
 // adds to one array; its reader clears the other one, for the image that is written in the same place next
 // (launch_signw_digit).  There is room: the digits leave 32 bytes or more a frame of what bf16 terms take.
 struct Image {
@@ -100,11 +101,11 @@ struct UnitBounds {
     __device__ __forceinline__ void store(uint8_t* img) const { *reinterpret_cast<uint4*>(img) = make_uint4(scale, shift, top_shift, 0u); }
     // Exponent of the scale of a frame whose inputs' magnitudes add up to at most `sum`.  (Up to 100: beyond, 2^-e leaves the
     // range of numbers that keep their precision.)
-    __device__ __forceinline__ int exponent(float sum, int act) const {
+    __device__ __forceinline__ int exponent(float sum, bool sigmoid) const {
         const float d = __uint_as_float(scale) * sum, sh = __uint_as_float(shift);
         const float top = __uint_as_float(top_shift & kTop ? top_shift & ~kTop : ~top_shift);
         // roundings of the sums, the affine and the activation stay far below the margins
-        float b = act == BNN_ACT_SIGMOID ? expf(d + top + 1e-6f * (d + sh)) : d + sh;
+        float b = sigmoid ? expf(d + top + 1e-6f * (d + sh)) : d + sh;
         b *= 1.0001f;
         const int e = digit::scale_exponent(max(scale, shift) < kInf && b < 1.0f ? b : 1.0f, 3);
         return e > 100 ? 100 : e;
@@ -142,6 +143,13 @@ struct Frames {
         return make_float4(at(m, k), at(m, k + 1), at(m, k + 2), at(m, k + 3));
     }
 };
+
+// A NaN among a layer's outputs is handed on as the number below all others, of which the high digit alone is not zero.  The
+// outputs of Sigmoid units are not negative, so their high digits with the top bit set are NaNs, and a part of a frame's
+// sum of squares (at most 8 * 4 * 127^2 together) is replaced by one that shows in the sum.
+constexpr float kNaNDigits = -8388608.0f;
+constexpr int kNaNSquare = 1 << 27;
+constexpr uint32_t kNaNOutput = 0x80000000u;     // in a frame's sum
 
 // At least sum_k |v| * 2^-e, given 2^-e and the sum of the squares of the high digits (|v| <= 65536 |high| + 32896).
 __device__ __forceinline__ float magnitude_bound(float inv_scale, uint32_t squares, int K) {
@@ -249,11 +257,11 @@ struct Args {
     const uint32_t* Wp; int ldwp;
     const uint8_t* img;
     const float* in_scales;      // 2^-e per frame
-    const uint32_t* in_sums;     // per frame, where the layer hands on digits
+    const uint32_t* in_sums;     // per frame, in the image of a chain
     uint32_t* spare_sums;        // to be cleared, or nullptr
     const float* scale; const float* shift;
     Affine next;                 // of the layer that reads the digits handed on
-    int act;                     // NONE, HARDTANH or SIGMOID
+    int hardtanh;                // (not SIGMOID) 0: no activation
     int K;
     float* Y; int ldy;
     uint8_t* img_out;            // image of the layer that consumes the outputs, or nullptr
@@ -261,6 +269,9 @@ struct Args {
     uint32_t* out_sums;          // of that image (digits)
 };
 
+// (What is handed on is no template argument: the layers of a network then run the same code, which the SMs still hold from one
+// launch to the next; 517 frames, six layers, 100.2 us, with a kernel per kind 101.6.)
+template <bool SIGMOID>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(digit::THREADS, 1)
 signw_digit_kernel(const __grid_constant__ CUtensorMap map, const __grid_constant__ digit::Work w, const __grid_constant__ Args g,
                    TcStatus status) {
@@ -270,9 +281,9 @@ signw_digit_kernel(const __grid_constant__ CUtensorMap map, const __grid_constan
     digit::Bars* bars = reinterpret_cast<digit::Bars*>(staging + digit::EPI_WARPS * STAGING);
     volatile int* abort_flag = &bars->wait.abort;
     const int warp = warp_index(), lane = threadIdx.x & 31, rank = (int)cluster_rank();
+    const bool digits_out = g.img_out && g.img_out_kind == 0;
     const uint32_t ring = smem_u32(smem);
     const uint32_t tmem = digit::set_up(bars, status, warp);
-    const bool digits_out = g.img_out && g.img_out_kind == 0;
 
     if (warp >= digit::PROD_WARP0) {
         digit::widen_bits<false>(w, g.Wp, g.ldwp, bars, tmem, rank, warp, lane);
@@ -320,11 +331,12 @@ signw_digit_kernel(const __grid_constant__ CUtensorMap map, const __grid_constan
             {
                 const int f = f0 + lane;
                 const bool one = n0 == 0 && f < M && lane < ng * digit::GRAN;     // of all warps that work on a frame
-                const float r = f < M ? __ldcg(g.in_scales + f) : 0.f;
-                float o = 0.f;
+                float r = f < M ? __ldcg(g.in_scales + f) : 0.f, o = 0.f;
+                const uint32_t word = g.in_sums && f < M ? __ldcg(g.in_sums + f) : 0u;
+                if (word & kNaNOutput) r = __int_as_float(0x7FC00000);
                 rs[lane] = r;
                 if (digits_out) {
-                    const int e = bounds.exponent(f < M ? magnitude_bound(r, __ldcg(g.in_sums + f), g.K) : 0.f, g.act);
+                    const int e = bounds.exponent(magnitude_bound(r, word & ~kNaNOutput, g.K), SIGMOID);
                     o = digit::power_of_two(e);
                     os[lane] = o;
                     if (one) {
@@ -358,12 +370,12 @@ signw_digit_kernel(const __grid_constant__ CUtensorMap map, const __grid_constan
 #pragma unroll
                         for (int i = 0; i < 8; ++i) y[i] = fmaf(sc, S[i] * r[i], sh);
                     }
-                    if (g.act == BNN_ACT_HARDTANH) {
-#pragma unroll
-                        for (int i = 0; i < 8; ++i) y[i] = fminf(fmaxf(y[i], -1.0f), 1.0f);
-                    } else if (g.act == BNN_ACT_SIGMOID) {
+                    if (SIGMOID) {
 #pragma unroll
                         for (int i = 0; i < 8; ++i) y[i] = 1.0f / (1.0f + expf(-y[i]));
+                    } else if (g.hardtanh) {
+#pragma unroll
+                        for (int i = 0; i < 8; ++i) y[i] = fminf(fmaxf(y[i], -1.0f), 1.0f);
                     }
                     const int f = f0 + gi * digit::GRAN;
                     if (g.Y && unit) {
@@ -386,7 +398,10 @@ signw_digit_kernel(const __grid_constant__ CUtensorMap map, const __grid_constan
                             for (int i = 0; i < 8; ++i) y[i] *= o[i];
                         }
 #pragma unroll
-                        for (int i = 0; i < 8; ++i) v[i] = unit ? digit::digits3(__float2int_rn(y[i])) : 0u;
+                        for (int i = 0; i < 8; ++i) {
+                            if (SIGMOID) y[i] = fmaxf(y[i], kNaNDigits);      // (a hardtanh unit gives -1 for a NaN)
+                            v[i] = unit ? digit::digits3(__float2int_rn(y[i])) : 0u;
+                        }
                         uint8_t* dst = g.img_out + im.digits + ((size_t)(2 * (n0 >> 5) + ((lane >> 2) & 1)) * im.rows + (size_t)(f / digit::GRAN) * 24 + (lane >> 3)) * 16 + (lane & 3) * 4;
 #pragma unroll
                         for (int h = 0; h < 2; ++h)
@@ -398,7 +413,7 @@ signw_digit_kernel(const __grid_constant__ CUtensorMap map, const __grid_constan
                                 x = __byte_perm(x, __shfl_xor_sync(0xFFFFFFFFu, x, 16), sel16);
                                 x = __byte_perm(x, __shfl_xor_sync(0xFFFFFFFFu, x, 8), sel8);
                                 *reinterpret_cast<uint32_t*>(dst + (q * 8 + h * 4) * 16) = x;
-                                if (q == 2) squares[gi * 64 + h * 32 + lane] = __dp4a((int)x, (int)x, 0);     // frame 4 h + lane / 8
+                                if (q == 2) squares[gi * 64 + h * 32 + lane] = SIGMOID && (x & 0x80808080u) ? kNaNSquare : __dp4a((int)x, (int)x, 0);     // frame 4 h + lane / 8
                             }
                     } else if (g.img_out && !digits_out) {
 #pragma unroll
@@ -412,12 +427,15 @@ signw_digit_kernel(const __grid_constant__ CUtensorMap map, const __grid_constan
                     }
                 });
             digit::release_acc(bars, b, lane);
-            if (any && digits_out) {
+            if (digits_out && any) {
                 // of the eight parts of a frame's sum
                 __syncwarp();
                 const int4 a = reinterpret_cast<const int4*>(squares)[2 * lane], c = reinterpret_cast<const int4*>(squares)[2 * lane + 1];
-                if (lane < ng * digit::GRAN && f0 + lane < M)
-                    atomicAdd(g.out_sums + f0 + lane, (uint32_t)((a.x + a.y) + (a.z + a.w) + (c.x + c.y) + (c.z + c.w)));
+                const int sum = (a.x + a.y) + (a.z + a.w) + (c.x + c.y) + (c.z + c.w);
+                if (lane < ng * digit::GRAN && f0 + lane < M) {
+                    if (sum >= kNaNSquare) atomicOr(g.out_sums + f0 + lane, kNaNOutput);
+                    else atomicAdd(g.out_sums + f0 + lane, (uint32_t)sum);
+                }
             }
             if (any && g.img_out && !digits_out) {
                 __syncwarp();
@@ -448,16 +466,16 @@ size_t signw_digit_bytes(int M, int K) {
 // first image that a layer writes, the kernel that wrote the chain's input.
 int launch_signw_digit(const RealGemmArgs& r, void* workspace, bool image_ready, void* out_image, int out_kind, int pos, int* clear,
                        int clear_words, cudaStream_t st) {
-    auto kern = signw_digit_kernel;
+    const bool digits_out = out_image && out_kind == 0;
+    auto kern = r.act == BNN_ACT_SIGMOID ? signw_digit_kernel<true> : signw_digit_kernel<false>;
     const int sms = device_sm_count();
     if (sms < 2 || !ensure_dynamic_smem(reinterpret_cast<const void*>(kern), SMEM_BYTES)) return BNN_ERR_CUDA;
     const TcStatus status = tc_status();
     if (!status.word) return BNN_ERR_CUDA;
     uint8_t* img = static_cast<uint8_t*>(workspace);
     uint8_t* out = static_cast<uint8_t*>(out_image);
-    const bool digits_out = out && out_kind == 0;
     const Image im(r.M, r.K, image_ready || digits_out);
-    auto sums = [&](uint8_t* base, int which) { return digits_out ? reinterpret_cast<uint32_t*>(base + im.sums(which)) : nullptr; };
+    auto sums = [&](uint8_t* base, int which) { return reinterpret_cast<uint32_t*>(base + im.sums(which)); };
     // (when the kernel before this one in the stream already wrote the image -- the layer that produced
     // these activations -- there is nothing to convert)
     if (!image_ready) {
@@ -466,14 +484,15 @@ int launch_signw_digit(const RealGemmArgs& r, void* workspace, bool image_ready,
         const size_t staged = (size_t)digit::GRAN * staged_pitch(r.K) * sizeof(float);
         const int blocks = ceil_div(r.M, digit::GRAN) + (digits_out ? 1 : 0);
         const Affine units{r.scale, r.shift, r.N};
-        uint32_t *first = sums(img, 0), *next = sums(out, 0);
+        uint32_t *first = digits_out ? sums(img, 0) : nullptr, *next = digits_out ? sums(out, 0) : nullptr;
         if (staged <= STAGED_MAX) x_digits_kernel<true><<<blocks, 256, staged, st>>>(x, img, first, next, units, clear, clear ? clear_words : 0);
         else x_digits_kernel<false><<<blocks, 256, 0, st>>>(x, img, first, next, units, clear, clear ? clear_words : 0);
     }
     const int steps = ceil_div(r.K, 32), pairs = sms / 2;
     const digit::Work w{r.N, r.M, digit::tile_rows(r.N, r.M, steps, pairs), 3, steps, 0};
-    const Args a{r.Bb, r.ldb, img, reinterpret_cast<const float*>(img + im.scales), sums(img, pos / 2), sums(img, pos / 2 + 1), r.scale, r.shift,
-                 Affine{r.next_scale, r.next_shift, r.next_N}, r.act, r.K, r.Y, r.ldy, out, out_kind, sums(out, (pos + 1) / 2)};
+    const Args a{r.Bb, r.ldb, img, reinterpret_cast<const float*>(img + im.scales), image_ready || digits_out ? sums(img, pos / 2) : nullptr,
+                 digits_out ? sums(img, pos / 2 + 1) : nullptr, r.scale, r.shift,
+                 Affine{r.next_scale, r.next_shift, r.next_N}, r.act == BNN_ACT_HARDTANH, r.K, r.Y, r.ldy, out, out_kind, digits_out ? sums(out, (pos + 1) / 2) : nullptr};
     CUtensorMap map;
     if (!encode_digit_map(&map, img + im.digits, im.rows, im.chunks, w.n / 2, digit::KB / 16)) return BNN_ERR_CUDA;
     const long long tiles = (long long)ceil_div(r.N, 2 * digit::ROWS) * ceil_div(r.M, w.n / 3);

@@ -232,3 +232,43 @@ def test_chained_layers_of_small_activations(env, widths, act, alpha, shift, fra
             top = (top * 1.0001).clamp(max=1.0)
             below = y.double()
     assert B.bnn_device_status() == 0
+
+
+@pytest.mark.parametrize("widths", [[50, 70, 300], [440, 1024, 700, 1024, 96]])
+@pytest.mark.parametrize("act", [2, 3])
+@pytest.mark.parametrize("full", [True, False])
+def test_chained_layers_carry_nans(env, widths, act, full):
+    """Frames with an infinity or a NaN come out as NaN behind Sigmoid units (a hardtanh unit turns them into -1), whether
+    the layers hand one another digits or fp32 rows, and a unit whose shift is a NaN spoils every frame from there on; the
+    other frames are what they are without."""
+    torch, B, model = env
+    frames, bad = 200, [3, 64, 199]
+    desc, plain = _chain(torch, B, model, widths, [0.1] * (len(widths) - 1), 0.1, act)
+    x = torch.randn((frames, widths[0]), generator=torch.Generator("cuda:0").manual_seed(2), device="cuda:0")
+    good = torch.ones(frames, dtype=torch.bool, device="cuda:0")
+    good[bad] = False
+    n = desc.workspace_bytes(frames) if full else desc.min_workspace_bytes(frames)
+
+    def run():
+        outs = [torch.empty((frames, w), device="cuda:0") for w in widths[1:]]
+        logp = torch.empty((frames, 70), device="cuda:0")
+        B.bnn_forward(desc, x, logp, torch.full((n,), 255, dtype=torch.uint8, device="cuda:0"), outs)
+        return outs + [logp]
+
+    clean = run()
+    x[3, 7], x[64, 0], x[199, 49] = float("inf"), float("nan"), float("-inf")
+    for a, b in zip(clean, run()):
+        assert torch.equal(a[good], b[good])
+        if act == B.ACT_SIGMOID:
+            assert bool(b[~good].isnan().all())
+        else:
+            assert not bool(b.isnan().any())
+    x[~good] = 0.0
+    plain[0][2][69] = float("nan")          # the last unit's shift in the first layer
+    spoilt = run()
+    if act == B.ACT_SIGMOID:
+        assert bool(spoilt[0][:, 69].isnan().all()) and not bool(spoilt[0][:, :69].isnan().any())
+        for b in spoilt[1:]:
+            assert bool(b.isnan().all())
+    else:
+        assert bool((spoilt[0][:, 69] == -1).all()) and not bool(spoilt[-1].isnan().any())
