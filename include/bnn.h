@@ -418,14 +418,12 @@ BNN_API int bnn_forward_events(const bnn_model* model, const float* X, int ldx, 
  *                        tiled tensor-core kernels (about 4x lower latency); 0 turns that off.
  *                        Integers and bits are identical; the fp32 sums differ by rounding order.
  *   BNN_OPT_XNOR_STACK : 1 (default) lets bnn_forward run consecutive binary hidden layers of one
- *                        shape with prepared weights (the loop over l of Algorithm 2's forward pass)
- *                        as ONE launch, in which a layer's frame tiles start as soon as the layer
+ *                        shape (with prepared weights beyond 16 frames; the loop over l of Algorithm 2's forward
+ *                        pass) as ONE launch, in which a layer's frame tiles start as soon as the layer
  *                        before has stored them; 0 launches one kernel per layer.  Same bits.  The CTAs
- *                        of such a launch wait for one another, so all of them (one per SM at most)
- *                        must be resident together: a caller that runs several forward passes on ONE
- *                        device at the same time (several streams or threads), whose kernels could share
- *                        the SMs between them, should set 0; otherwise such a launch may give up on a
- *                        bounded wait (status word set, see bnn_device_status) instead of finishing.
+ *                        of such a launch wait for one another; it is a cooperative launch, whose CTAs are
+ *                        placed together, so that several forward passes may run on one device at the
+ *                        same time (several streams or threads).
  *   BNN_OPT_SOFTMAX_FOLLOW: 1 (default) lets bnn_forward launch the log-softmax of a tensor-core top layer
  *                        on packed activations BEHIND that layer's kernel instead of after it: the
  *                        log-softmax kernel shares the SMs with the (tensor-pipe-bound) GEMM and takes every

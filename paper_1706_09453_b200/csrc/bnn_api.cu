@@ -585,8 +585,7 @@ int bnn_forward_events(const bnn_model* model, const float* X, int ldx, int M,
     const bool small = g_small_batch && M <= kSmallBatchMax;
     const int zo01 = model->act_values == BNN_VALUES_01;
     // The arrival counters of stacked binary layers are cleared before the first layer's kernels, not
-    // in front of the stacked launch itself: a memset between the first layer's kernel and that launch
-    // would take away its programmatic overlap with the first layer's tail.
+    // in front of the stacked launch itself, where the memset would take its time.
     // The same goes for the counters on which the log-softmax follows the top layer's kernel.
     int* top_done = nullptr;
     bool clear_pending = false, clear_by_first = false;
@@ -686,7 +685,7 @@ int bnn_forward_events(const bnn_model* model, const float* X, int ldx, int M,
                 if (int rc = check_packed(in, in_ld, y.K)) return rc;
                 const int ldob = bnn_packed_pitch(y.N);
                 if (int rc = launch_xnor_stack(static_cast<const uint32_t*>(in), in_ld, sl, n, M, y.N, y.K, ldob, zo01,
-                                               sync + sync_used, true, (cudaStream_t)stream))
+                                               sync + sync_used, (cudaStream_t)stream))
                     return rc;
                 sync_used += (int)(xnor_stack_sync_bytes(M, n) / sizeof(int));
                 in = sl[n - 1].out_bits;

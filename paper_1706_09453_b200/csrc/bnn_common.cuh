@@ -46,10 +46,10 @@ __device__ __forceinline__ uint4 ldg_nc_u4(const void* p) {
     return v;
 }
 
-// Programmatic dependent launch.  A kernel (that of the binary hidden layers, say) starts with
+// Programmatic dependent launch.  A kernel (that of the top layer, say) starts with
 // pdl_trigger() (the kernel after it in the stream may be scheduled as soon as all CTAs of this
 // one have got that far and SM resources free up), does what does not depend on the kernel
-// before it (set-up, the copy of its weight slice) and calls pdl_wait() before it reads that
+// before it (set-up) and calls pdl_wait() before it reads that
 // kernel's output: the wait returns once the kernel before it has completed and its writes are
 // visible.  A kernel of this kind cannot finish before its wait returns, so completion of one
 // implies completion of everything before it in the stream.  (The split passes and
@@ -70,6 +70,23 @@ inline cudaError_t launch_pdl(void (*kern)(KArgs...), dim3 grid, dim3 block, siz
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kern, static_cast<KArgs>(args)...);
+}
+
+// Cooperative launch, for kernels whose CTAs wait for one another: all of them are placed together or none, whatever runs
+// beside them on other streams.
+template <typename... KArgs, typename... Args>
+inline cudaError_t launch_cooperative(void (*kern)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, Args... args) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = block;
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeCooperative;
+    attr[0].val.cooperative = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
     return cudaLaunchKernelEx(&cfg, kern, static_cast<KArgs>(args)...);
@@ -111,8 +128,7 @@ int launch_xnor_res(const uint32_t* Ap, int ldap, const void* image, int M, int 
 // A run of consecutive fused Sign layers of one shape (N == K beyond the first) in ONE launch of that
 // kernel: layer l reads the bits layer l - 1 wrote (pitch ldob), layer 0 reads Ap.  `progress` points
 // to xnor_stack_sync_bytes(M, n_layers) bytes of ZEROED device memory (per frame tile and layer
-// boundary a counter of the epilogue warps that have stored their bits).  `chained`: the launch is part of a
-// forward pass (programmatic dependent launch on the layer kernel before it).
+// boundary a counter of the epilogue warps that have stored their bits).
 constexpr int kXnorStackMax = 8;
 struct XnorStackLayer {
     const void* image;
@@ -122,7 +138,7 @@ struct XnorStackLayer {
 };
 size_t xnor_stack_sync_bytes(int M, int n_layers);
 int launch_xnor_stack(const uint32_t* Ap, int ldap, const XnorStackLayer* layers, int n_layers, int M, int N, int K,
-                      int ldob, int zo, int* progress, bool chained, cudaStream_t st);
+                      int ldob, int zo, int* progress, cudaStream_t st);
 int launch_xnor_prepare(const uint32_t* Wp, int ldwp, int N, int K, void* image, cudaStream_t st);
 int launch_xnor_img(const uint32_t* Ap, int ldap, const void* image, int M, int N, int K,
                     int32_t* C, int ldc, const int32_t* thr, const uint32_t* flip,

@@ -311,28 +311,13 @@ int launch_small_signw(const float* X, int ldx, const uint32_t* Wp, int ldwp, in
     return launch_status();
 }
 
-// A cooperative launch where the CTAs wait for one another: all of them are placed together or none, whatever runs beside
-// them on other streams.  (It starts when the kernel before it has ended, which costs about 2 us against a
-// programmatic dependent launch.)  A single layer may start under the kernel before it.
+// The CTAs of a run wait for one another.  (Its launch starts when the kernel before it has ended, which costs about 2 us
+// against a programmatic dependent launch.)  A single layer may start under the kernel before it.
 template <typename Kern>
 static cudaError_t launch_run(Kern kern, int blocks, size_t smem, cudaStream_t st, const uint32_t* Ap, int ldap, const SmallRun& run,
                               int M, int N, int K, int ldob) {
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(blocks);
-    cfg.blockDim = dim3(THREADS);
-    cfg.dynamicSmemBytes = smem;
-    cfg.stream = st;
-    cudaLaunchAttribute attr;
-    if (run.n_layers > 1) {
-        attr.id = cudaLaunchAttributeCooperative;
-        attr.val.cooperative = 1;
-    } else {
-        attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
-        attr.val.programmaticStreamSerializationAllowed = 1;
-    }
-    cfg.attrs = &attr;
-    cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, kern, Ap, ldap, run, M, N, K, ldob);
+    return run.n_layers > 1 ? launch_cooperative(kern, dim3(blocks), dim3(THREADS), smem, st, Ap, ldap, run, M, N, K, ldob)
+                            : launch_pdl(kern, dim3(blocks), dim3(THREADS), smem, st, Ap, ldap, run, M, N, K, ldob);
 }
 
 int launch_small_xnor(const uint32_t* Ap, int ldap, const XnorSmallLayer* layers, int n_layers, int M, int N, int K,

@@ -257,9 +257,7 @@ xnor_res_kernel(const __grid_constant__ StackMaps maps, const __grid_constant__ 
     Control* ctl = reinterpret_cast<Control*>(smem + B_REGION + GROUPS * GROUP_BYTES);
     volatile int* abort_flag = &ctl->wait.abort;
 
-    // The kernel that follows in the stream may be scheduled as soon as this one's CTAs leave
-    // their SMs.  This kernel's own set-up and the copy of its weight slice need nothing the
-    // kernel before it writes; it waits (pdl_wait, below) before it touches the frames.
+    // The kernel that follows in the stream may be scheduled as soon as this one's CTAs leave their SMs.
     pdl_trigger();
 
     const int warp = warp_index(), lane = threadIdx.x & 31;
@@ -343,9 +341,6 @@ xnor_res_kernel(const __grid_constant__ StackMaps maps, const __grid_constant__ 
             const int ng = ceil_div(nks, 2);
             int gc = 0;   // groups issued so far, over all layers: slot gc % GROUPS, < GROUPS ahead of its consumers
             bool ok = true;
-            // the frames of layer 0 are the previous kernel's output: wait until that kernel has
-            // completed and its writes are visible (returns at once when there is no such dependency)
-            pdl_wait();
             for (int l = 0; l < L && ok; ++l)
                 for (int t = 0; t < share.count && ok; ++t) {
                     const int mt = share.first + t * share.step;
@@ -562,7 +557,7 @@ xnor_res_kernel(const __grid_constant__ StackMaps maps, const __grid_constant__ 
 
 template <int BN>
 int launch_bn(const uint32_t* Ap, int ldap, const XnorStackLayer* layers, int n_layers, int M, int N, int K, int ldob,
-              int zo, int* progress, bool chained, int sm_count, cudaStream_t st) {
+              int zo, int* progress, int sm_count, cudaStream_t st) {
     auto kern = xnor_res_kernel<BN>;
     if (!ensure_dynamic_smem(reinterpret_cast<const void*>(kern), SMEM_BYTES)) return BNN_ERR_CUDA;
     const long long tiles = (long long)ceil_div(M, BM) * ceil_div(N, BN);
@@ -579,12 +574,10 @@ int launch_bn(const uint32_t* Ap, int ldap, const XnorStackLayer* layers, int n_
         const uint32_t* in = l == 0 ? Ap : layers[l - 1].out_bits;
         if (!encode_packed_map(&maps.m[l], in, l == 0 ? ldap : ldob, M, K, BM)) return BNN_ERR_CUDA;
     }
-    // Programmatic dependent launch only inside a forward pass: there the kernel before this one is a
-    // layer's kernel and everything read before the wait (weights, thresholds) was complete before the
-    // forward pass started.  A stand-alone call may follow the kernel that wrote its thresholds or its
-    // weight image on the same stream, so it is launched the ordinary way.
-    if (chained) {
-        if (launch_pdl(kern, dim3(grid), dim3(THREADS), SMEM_BYTES, st, maps, a) != cudaSuccess) return BNN_ERR_CUDA;
+    // The CTAs of a run wait for one another.  (Launched so, it starts when the kernel before it has ended; as a programmatic
+    // dependent launch it would save 2 us, and two runs on two streams could each be placed in part and wait until they give up.)
+    if (n_layers > 1) {
+        if (launch_cooperative(kern, dim3(grid), dim3(THREADS), SMEM_BYTES, st, maps, a) != cudaSuccess) return BNN_ERR_CUDA;
     } else {
         kern<<<grid, THREADS, SMEM_BYTES, st>>>(maps, a);
     }
@@ -629,22 +622,22 @@ size_t xnor_stack_sync_bytes(int M, int n_layers) {
 }
 
 int launch_xnor_stack(const uint32_t* Ap, int ldap, const XnorStackLayer* layers, int n_layers, int M, int N, int K,
-                      int ldob, int zo, int* progress, bool chained, cudaStream_t st) {
+                      int ldob, int zo, int* progress, cudaStream_t st) {
     const int sms = sm_count_of_device();
     if (sms <= 0) return BNN_ERR_CUDA;
     if (n_layers < 1 || n_layers > kXnorStackMax || (n_layers > 1 && (N != K || !progress))) return BNN_ERR_UNSUPPORTED;
     const int bn = tile_units(M, N, K, sms);
-    if (bn == 192) return launch_bn<192>(Ap, ldap, layers, n_layers, M, N, K, ldob, zo, progress, chained, sms, st);
-    if (bn == 128) return launch_bn<128>(Ap, ldap, layers, n_layers, M, N, K, ldob, zo, progress, chained, sms, st);
-    if (bn == 96) return launch_bn<96>(Ap, ldap, layers, n_layers, M, N, K, ldob, zo, progress, chained, sms, st);
-    if (bn == 32) return launch_bn<32>(Ap, ldap, layers, n_layers, M, N, K, ldob, zo, progress, chained, sms, st);
+    if (bn == 192) return launch_bn<192>(Ap, ldap, layers, n_layers, M, N, K, ldob, zo, progress, sms, st);
+    if (bn == 128) return launch_bn<128>(Ap, ldap, layers, n_layers, M, N, K, ldob, zo, progress, sms, st);
+    if (bn == 96) return launch_bn<96>(Ap, ldap, layers, n_layers, M, N, K, ldob, zo, progress, sms, st);
+    if (bn == 32) return launch_bn<32>(Ap, ldap, layers, n_layers, M, N, K, ldob, zo, progress, sms, st);
     return BNN_ERR_UNSUPPORTED;
 }
 
 int launch_xnor_res(const uint32_t* Ap, int ldap, const void* image, int M, int N, int K,
                     const int32_t* thr, const uint32_t* flip, uint32_t* out_bits, int ldob, int zo, cudaStream_t st) {
     const XnorStackLayer one{image, thr, flip, out_bits};
-    return launch_xnor_stack(Ap, ldap, &one, 1, M, N, K, ldob, zo, nullptr, false, st);
+    return launch_xnor_stack(Ap, ldap, &one, 1, M, N, K, ldob, zo, nullptr, st);
 }
 
 }  // namespace bnn

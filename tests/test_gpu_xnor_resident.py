@@ -70,3 +70,26 @@ def test_resident_layer_decides_sums_of_zeros(env, k, n):
     bits = (out.unsqueeze(2) >> torch.arange(32, device="cuda:0", dtype=torch.int32)) & 1
     want = (thr <= 0).int().expand(m, n)
     assert torch.equal(bits.reshape(m, -1)[:, :n], want)
+
+
+@pytest.mark.parametrize("frames", [17, 100, 731, 3000])
+def test_several_streams_at_once(env, frames):
+    """Runs that do not fit the SMs side by side (32- to 192-unit tiles take 64 to 148 SMs each), on four streams."""
+    torch, B, model = env
+    cfg = dataclasses.replace(wl.CONFIGS["tiny"], hidden=2048, n_hidden=6, classes=500)
+    net = wl.make_model(cfg)
+    nets = [model.DeviceNet(net) for _ in range(4)]
+    X = model.to_dev(wl.make_frames(cfg, frames))
+    want = nets[0].forward(X).clone()
+    outs = [torch.empty_like(want) for _ in nets]
+    for dn in nets:
+        dn.workspace(frames)
+    torch.cuda.synchronize()
+    streams = [torch.cuda.Stream() for _ in nets]
+    for _ in range(30):
+        for dn, st, o in zip(nets, streams, outs):
+            with torch.cuda.stream(st):
+                dn.forward(X, o)
+    torch.cuda.synchronize()
+    assert all(torch.equal(o, want) for o in outs)
+    assert B.bnn_device_status() == 0
