@@ -267,7 +267,7 @@ BNN_API int bnn_output_prepare(const float* Wout, int ldw, int C, int H,
  *   |z - exact| <= H * 2^-23 * max_h |Wout[c][h]|  (2^-31 with four digits) + one fp32 rounding + the bias addition.
  * act_values : bnn_act_values of Hp.  H <= 2^15 (larger: BNN_ERR_UNSUPPORTED; use bnn_output_layer).
  * digits : device buffer, 256-byte aligned, at least bnn_output_digits_bytes(C, H) bytes.  In bnn_forward: the
- * `Wp` of a BNN_LAYER_REAL_OUT layer. */
+ * `Wp` of a BNN_LAYER_REAL_OUT layer whose `ldwp` is BNN_LDWP_DIGITS. */
 BNN_API size_t bnn_output_digits_bytes(int C, int H);
 BNN_API int bnn_output_prepare_digits(const float* Wout, int ldw, int C, int H,
                                       void* digits, size_t digits_bytes, void* stream);
@@ -286,11 +286,14 @@ typedef enum {
                               input layer the paper keeps real-valued in its best systems (Table 2) */
 } bnn_layer_kind;
 
+#define BNN_LDWP_DIGITS (-3)   /* no pitch: says what Wp of a REAL_OUT layer is */
+
 typedef struct bnn_layer {
     int kind;
     int K, N;              /* fan-in, fan-out */
-    const uint32_t* Wp;    /* SIGNW, XNOR: packed weights [N][ldwp]; REAL_OUT on packed activations:
-                              bnn_output_prepare_digits image of W (preferred to W_prepared), or NULL */
+    const uint32_t* Wp;    /* SIGNW, XNOR: packed weights [N][ldwp]; REAL_OUT: ignored, unless ldwp is
+                              BNN_LDWP_DIGITS: on packed activations the bnn_output_prepare_digits image of
+                              W (preferred to W_prepared), or NULL */
     int ldwp;
     const float* W;        /* REAL_OUT, REAL: fp32 weights [N][ldw] */
     int ldw;

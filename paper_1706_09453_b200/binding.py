@@ -421,7 +421,7 @@ class ModelDesc:
             wp, w = d.get("Wp"), d.get("W")
             a.Wp, a.ldwp = _ptr(wp, torch.int32), (_ld(wp) if wp is not None else 0)
             if d.get("W_digits") is not None:   # top layer: the digit image of W
-                a.Wp = _ptr(d["W_digits"])
+                a.Wp, a.ldwp = _ptr(d["W_digits"]), LDWP_DIGITS
             a.W, a.ldw = _ptr(w, torch.float32), (_ld(w) if w is not None else 0)
             a.W_prepared = _ptr(d.get("W_prepared"))
             a.scale, a.shift = _ptr(d.get("scale"), torch.float32), _ptr(d.get("shift"), torch.float32)
@@ -464,6 +464,7 @@ def bnn_forward_events(model: ModelDesc, X, logp, workspace, events, layer_out=N
 
 
 STATIC_WORKSPACE_BYTES = 8 << 20
+LDWP_DIGITS = -3         # ldwp of a top layer whose Wp is its digit image
 MAX_K_DIGITS = 1 << 15   # widest input of the kernels on byte digits
 
 

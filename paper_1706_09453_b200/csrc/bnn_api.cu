@@ -46,6 +46,9 @@ size_t layer_out_bytes(const bnn_layer& L, int M) {
     return (size_t)M * L.N * sizeof(float);
 }
 
+// The digit image of a top layer, or NULL.
+const void* digit_image(const bnn_layer& top) { return top.ldwp == BNN_LDWP_DIGITS ? top.Wp : nullptr; }
+
 int validate_model(const bnn_model* model) {
     if (!model || !model->layers) return BNN_ERR_NULL;
     const int L = model->n_layers;
@@ -87,7 +90,7 @@ int validate_model(const bnn_model* model) {
                 if (l != L - 1) return BNN_ERR_UNSUPPORTED;
                 if (!y.W) return BNN_ERR_NULL;
                 if (y.ldw < y.K) return BNN_ERR_SHAPE;
-                if (reinterpret_cast<uintptr_t>(y.Wp) & 255u) return BNN_ERR_ALIGN;   // the digit image, or NULL
+                if (reinterpret_cast<uintptr_t>(digit_image(y)) & 255u) return BNN_ERR_ALIGN;
                 break;
             default:
                 return BNN_ERR_UNSUPPORTED;
@@ -605,7 +608,7 @@ int bnn_forward_events(const bnn_model* model, const float* X, int ldx, int M,
         const bnn_layer& top = model->layers[L - 1];
         if (!small && g_softmax_follow && !events && lay.sync > lay.stack_sync && top.kind == BNN_LAYER_REAL_OUT && L > 1 &&
             model->layers[L - 2].act == BNN_ACT_SIGN_PACK &&
-            ((top.Wp && out_digit_can_be_followed(M, top.N, top.K)) || (top.W_prepared && out_tc_more_than_one_wave(M, top.N))))
+            ((digit_image(top) && out_digit_can_be_followed(M, top.N, top.K)) || (top.W_prepared && out_tc_more_than_one_wave(M, top.N))))
             top_done = sync + lay.stack_sync / sizeof(int);
         clear_pending = any || top_done;
         // When the first layer splits its input into an image, or is the small-batch kernel, that kernel clears them on its way (a memset
@@ -638,7 +641,7 @@ int bnn_forward_events(const bnn_model* model, const float* X, int ldx, int M,
         // (With more than four frames the digit kernel is the faster one: 2048 -> 3307, 8 frames 10 us against 20, 3 frames
         // 10 against 9; 1024 -> 2000, 8 frames 7 against 9.)
         if (y.kind == BNN_LAYER_REAL_OUT && small && in_bits && small_fits_out(y.K) &&
-            (M <= 4 || !y.Wp || y.K > kMaxKDigit || g_real_path == BNN_PATH_CUDA_CORE)) {
+            (M <= 4 || !digit_image(y) || y.K > kMaxKDigit || g_real_path == BNN_PATH_CUDA_CORE)) {
             if (int rc = check_packed(in, in_ld, y.K)) return rc;
             if (int rc = launch_small_out(static_cast<const uint32_t*>(in), in_ld, y.W, y.ldw, y.shift, M, y.N, y.K,
                                           logp, ldo, zo01, (cudaStream_t)stream)) return rc;
@@ -658,7 +661,7 @@ int bnn_forward_events(const bnn_model* model, const float* X, int ldx, int M,
                                        in_bits && model->act_values == BNN_VALUES_01,
                                        chain_in ? img + (size_t)chain_slot * img_half : img, chain_in ? img_half : img_bytes,
                                        model->log_prior, BNN_ACT_NONE, events ? events[L + 1] : nullptr, stream, chain_in,
-                                       in_bits ? top_done : nullptr, in_bits ? y.Wp : nullptr);
+                                       in_bits ? top_done : nullptr, in_bits ? digit_image(y) : nullptr);
             if (rc) return rc;
             if (events && events[L] &&
                 cudaEventRecord((cudaEvent_t)events[L], (cudaStream_t)stream) != cudaSuccess)

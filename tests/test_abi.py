@@ -132,6 +132,13 @@ def test_model_validation(lib):
     # fan-in mismatch
     bad, keep3 = model(layer(0, 440, 64, 1), layer(1, 32, 64, 1), layer(2, 64, 10))
     assert B.raw_call("bnn_forward", C.byref(bad), fake, 440, 8, fake, 10, fake, 1 << 20, None, None) == 2
+    # Wp of the top layer is ignored, wherever it points, unless ldwp says that it is the (256-byte aligned) digit image
+    top = layer(2, 64, 10)
+    top.Wp = fake + 4
+    old, keep6 = model(layer(0, 440, 64, 1), layer(1, 64, 64, 1), top)
+    assert lib.bnn_forward_workspace_bytes(C.byref(old), 8) == ws
+    old.layers[2].ldwp = B.LDWP_DIGITS
+    assert B.raw_call("bnn_forward", C.byref(old), fake, 440, 8, fake, 10, fake, 1 << 20, None, None) == 3
     # unknown activation values
     odd, keep5 = model(layer(0, 440, 64, 1), layer(1, 64, 64, 1), layer(2, 64, 10))
     odd.act_values = 7

@@ -272,3 +272,23 @@ def test_chained_layers_carry_nans(env, widths, act, full):
             assert bool(b.isnan().all())
     else:
         assert bool((spoilt[0][:, 69] == -1).all()) and not bool(spoilt[-1].isnan().any())
+
+
+def test_unmarked_packed_weights_of_the_top_layer_are_ignored(env):
+    """Whatever Wp of a top layer holds, the logits come from W and W_prepared unless ldwp marks a digit image."""
+    torch, B, model = env
+    cfg = wl.Config("wp", 4, 300, 100, 160, 2, 90)
+    dn = model.DeviceNet(wl.make_model(cfg))
+    x = model.to_dev(wl.make_frames(cfg))
+    img = torch.empty(B.bnn_output_prepared_bytes(90, 160), dtype=torch.uint8, device="cuda:0")
+    B.bnn_output_prepare(dn.Wout, img)
+    junk = torch.full((1 << 16,), 0x5A5A5A5A, dtype=torch.int32, device="cuda:0")
+    out = []
+    for wp in (None, junk.view(-1, 8)):
+        top = dict(dn.desc.layers[-1], W_prepared=img, W_digits=None, Wp=wp)
+        desc = B.ModelDesc(dn.desc.layers[:-1] + [top])
+        for frames in (8, 300):
+            logp = torch.empty((frames, 90), device="cuda:0")
+            ws = torch.empty(desc.workspace_bytes(frames), dtype=torch.uint8, device="cuda:0")
+            out.append(B.bnn_forward(desc, x[:frames], logp, ws))
+    assert torch.equal(out[0], out[2]) and torch.equal(out[1], out[3])
