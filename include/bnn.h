@@ -339,7 +339,7 @@ typedef struct bnn_model {
  * real-valued layer fed with fp32 activations (see bnn_output_layer_ws).
  * bnn_forward_min_workspace_bytes is the least it accepts (the two buffers and the counters;
  * sign-weight layers then keep their image in the rows of logp until the top layer writes those -- if they are
- * contiguous, ldo == C, and long enough -- or split their activations inside the GEMM, and hand on fp32 rows). */
+ * contiguous, ldo == C, long enough and apart from the layer's input and output -- or split their activations inside the GEMM, and hand on fp32 rows). */
 BNN_API size_t bnn_forward_workspace_bytes(const bnn_model* model, int M);
 BNN_API size_t bnn_forward_min_workspace_bytes(const bnn_model* model, int M);
 

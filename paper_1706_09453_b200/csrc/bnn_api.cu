@@ -46,6 +46,11 @@ size_t layer_out_bytes(const bnn_layer& L, int M) {
     return (size_t)M * L.N * sizeof(float);
 }
 
+bool overlap(const void* p, size_t n, const void* q, size_t m) {
+    const uintptr_t a = reinterpret_cast<uintptr_t>(p), b = reinterpret_cast<uintptr_t>(q);
+    return a < b + m && b < a + n;
+}
+
 // The digit image of a top layer, or NULL.
 const void* digit_image(const bnn_layer& top) { return top.ldwp == BNN_LDWP_DIGITS ? top.Wp : nullptr; }
 
@@ -762,10 +767,13 @@ int bnn_forward_events(const bnn_model* model, const float* X, int ldx, int M,
             if (!chain_in && !chain_out && !(l == 0 && splice_dim > 0) && ldo == model->layers[L - 1].N &&
                 img_in_bytes < signw_scratch_bytes(M, y.K, g_signw_terms, y.act)) {
                 // no room for the image in the workspace: the log-probabilities' own rows are free until the top
-                // layer writes them (contiguous rows only: what lies between rows is the caller's)
+                // layer writes them (contiguous rows only: what lies between rows is the caller's), unless the caller has
+                // this layer's input or output there too
                 const uintptr_t base = (reinterpret_cast<uintptr_t>(logp) + 255) & ~uintptr_t(255);
                 const uintptr_t end = reinterpret_cast<uintptr_t>(logp + (size_t)M * ldo);
-                if (end > base && end - base >= signw_scratch_bytes(M, y.K, g_signw_terms, y.act)) {
+                const bool apart = !overlap(logp, (size_t)M * ldo * sizeof(float), in, ((size_t)(M - 1) * in_ld + y.K) * sizeof(float)) &&
+                                   !overlap(logp, (size_t)M * ldo * sizeof(float), out, layer_out_bytes(y, M));
+                if (apart && end > base && end - base >= signw_scratch_bytes(M, y.K, g_signw_terms, y.act)) {
                     img_in = reinterpret_cast<char*>(base);
                     img_in_bytes = end - base;
                 }

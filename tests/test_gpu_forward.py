@@ -455,3 +455,27 @@ def test_forward_small_batch_other_topologies(env):
     mixed = dataclasses.replace(wl.CONFIGS["wsj_mixed"], hidden=512, classes=700, frames=7, n_hidden=4)
     run_mixed_net(env, mixed, 7)
     run_mixed_net(env, wl.CONFIGS["wsj_mixed"], 3)
+
+
+@pytest.mark.parametrize("act", [wl.ACT_SIGN, wl.ACT_HARDTANH])
+@pytest.mark.parametrize("at", ["start", "end"])
+def test_features_in_the_rows_of_the_output(env, act, at):
+    """X may lie in the buffer that logp is written to, also with the least workspace, where the first layer's image
+    would otherwise take that place: as with X elsewhere and a pitch that keeps the image out of logp.  (Later layers with
+    binary weights on real activations may use logp in the one pass and not in the other.)"""
+    torch, B, model = env
+    cfg = wl.Config("alias", 6, 700, 100, 256, 3, 1500, act, act == wl.ACT_HARDTANH)
+    dn = model.DeviceNet(wl.make_model(cfg))
+    x = model.to_dev(wl.make_frames(cfg))
+    n = dn.desc.min_workspace_bytes(700)
+    apart = torch.empty((700, 1504), device="cuda:0")[:, :1500]
+    B.bnn_forward(dn.desc, x, apart, torch.empty(n, dtype=torch.uint8, device="cuda:0"))
+    logp = torch.empty((700, 1500), device="cuda:0")
+    flat = logp.view(-1)
+    inside = (flat[:70000] if at == "start" else flat[-70000:]).view(700, 100)
+    inside.copy_(x)
+    B.bnn_forward(dn.desc, inside, logp, torch.empty(n, dtype=torch.uint8, device="cuda:0"))
+    if act == wl.ACT_SIGN:
+        assert torch.equal(logp, apart)
+    else:
+        assert float((logp - apart).abs().max()) <= LOGP_TOL
