@@ -188,7 +188,7 @@ BNN_API int bnn_signw_gemm(const float* X, int ldx, const uint32_t* Wp, int ldwp
  * in the order the tensor core reads it, which the GEMM streams: 2-5x faster than bnn_signw_gemm on the tensor
  * path.  With two terms (BNN_OPT_SIGNW_TERMS), K <= 2^15 and an activation other than SIGN_PACK the image holds every row of X as fixed-point numbers of a
  * power-of-two scale of its own in three byte digits, and the sums are exact integers:
- *   |y - exact| <= K * 2^-23 * max_k |x[m][k]| + one fp32 rounding (a row with an infinity or a NaN gives NaN);
+ *   |y - exact| <= K * 1.01 * 2^-23 * max_k |x[m][k]| + one fp32 rounding (a row with an infinity or a NaN gives NaN);
  * otherwise it holds bf16 terms, as bnn_signw_gemm.  Inside bnn_forward a layer writes the image of the next one of its kind
  * before a frame's largest output is known; max |x| is then replaced by a bound on it, min(1, max |scale| *
  * sqrt(K) |x'|_2 + max |shift|) for hardtanh units on inputs x', and likewise for Sigmoid.  Without workspace (NULL, or too small) it behaves exactly like
@@ -264,7 +264,8 @@ BNN_API int bnn_output_prepare(const float* Wout, int ldw, int C, int H,
  * row's mean magnitude), in the order the tensor core reads them; bnn_output_layer_digits multiplies the digits
  * with the activations' signs in integers, so that a logit is rounded once instead of at every step, and takes 3/4
  * of the tensor-core passes of bnn_output_layer's fp16 terms:
- *   |z - exact| <= H * 2^-23 * max_h |Wout[c][h]|  (2^-31 with four digits) + one fp32 rounding + the bias addition.
+ *   |z - exact| <= H * 1.01 * 2^-23 * max_h |Wout[c][h]|  (1.08 * 2^-31 with four digits) + one fp32 rounding + the bias
+ * addition.
  * act_values : bnn_act_values of Hp.  H <= 2^15 (larger: BNN_ERR_UNSUPPORTED; use bnn_output_layer).
  * digits : device buffer, 256-byte aligned, at least bnn_output_digits_bytes(C, H) bytes.  In bnn_forward: the
  * `Wp` of a BNN_LAYER_REAL_OUT layer whose `ldwp` is BNN_LDWP_DIGITS. */
@@ -333,7 +334,7 @@ typedef struct bnn_model {
 /* Bytes of scratch for M frames.  bnn_forward_workspace_bytes is what makes bnn_forward
  * fastest: two ping-pong activation buffers, the arrival counters of binary hidden layers that
  * run as one launch (a few bytes per 128 frames and layer) and of the log-softmax that follows the
- * top layer's kernel (4 bytes per 512 frames), and room for the split-activation
+ * top layer's kernel (4 bytes per 256 frames), and room for the split-activation
  * images: of the widest sign-weight layer (see bnn_signw_gemm_ws; two of them when such layers
  * follow one another, because each writes the next one's image while it reads its own) or of a
  * real-valued layer fed with fp32 activations (see bnn_output_layer_ws).
@@ -430,7 +431,7 @@ BNN_API int bnn_forward_events(const bnn_model* model, const float* X, int ldx, 
  *   BNN_OPT_SOFTMAX_FOLLOW: 1 (default) lets bnn_forward launch the log-softmax of a tensor-core top layer
  *                        on packed activations BEHIND that layer's kernel instead of after it: the
  *                        log-softmax kernel shares the SMs with the (tensor-pipe-bound) GEMM and takes every
- *                        512 frames as soon as all their logits are stored, so that only the last frames are
+ *                        256 or 512 frames (byte digits, fp16 terms) as soon as all their logits are stored, so that only the last frames are
  *                        left when the GEMM ends.  Same log-probabilities.  Its waits are bounded like all
  *                        others (BNN_OPT_WAIT_LIMIT_US).  0 runs the two kernels one after the other; so does
  *                        bnn_forward_events, whose per-layer events need them apart.

@@ -165,7 +165,7 @@ struct XnorSmallLayer {
     const uint32_t* flip;
     uint32_t* out_bits;
 };
-bool small_xnor_can_run(int N);   // more than one layer: every CTA of the launch needs an SM of its own
+bool small_xnor_can_run(int N);   // more than one layer: all CTAs of the launch (16 units each, two per SM) must be resident
 int launch_small_xnor(const uint32_t* Ap, int ldap, const XnorSmallLayer* layers, int n_layers, int M, int N, int K,
                       int ldob, int zo, int* arrived, cudaStream_t st);
 int launch_small_out(const uint32_t* Hp, int ldhp, const float* W, int ldw, const float* bias,

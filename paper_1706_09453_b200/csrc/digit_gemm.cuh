@@ -8,7 +8,7 @@
 // written in base 256 with balanced digits, v = d0 + 256 d1 + 65536 d2 (-128 <= d <= 127), i.e. three bytes per
 // element.  Bits widen to bytes, the tensor core multiplies bytes at twice the rate of half-precision numbers, and
 // its 32-bit sums are exact (K <= kMaxKDigit), so S is exact: the only rounding is that of v, at most
-// 2^-23 of the row's largest magnitude per element, and one rounding of the result to fp32.  Three digit
+// 1.01 * 2^-23 of the row's largest magnitude per element (1 / 0x7F7F7F, see scale_exponent), and one rounding of the result to fp32.  Three digit
 // passes at the byte rate cost 1.5 half-precision passes, where two half-precision terms cost 2 and add up
 // in fp32 with a rounding per step; the operand's image is three bytes per element instead of four.
 //

@@ -4,7 +4,7 @@
 // The weights are static, so they are prepared once (bnn_output_prepare_digits): fixed-point numbers of a
 // power-of-two scale of each class's own, written as byte digits in the order the tensor core reads shared memory
 // (digit_gemm.cuh).  Three digits (about 23 bits relative to the class's largest weight) as long as every class's
-// largest weight is at most 16 times its mean magnitude -- then even if all H roundings, each at most 2^-23 of
+// largest weight is at most 16 times its mean magnitude -- then even if all H roundings, each at most 1.01 * 2^-23 of
 // the largest weight, add up, a logit is within 2^-19 of sum |w| -- and four digits (31 bits) for the whole
 // matrix otherwise.  The choice is made on the device and read from the image by the GEMM.
 //

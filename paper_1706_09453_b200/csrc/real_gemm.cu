@@ -374,9 +374,9 @@ log_softmax_rows_reg_kernel(float* __restrict__ Z, int ldz, int M, int C, const 
 // claimed kFollowRows at a time, in order, from one counter (done[groups], zero at launch), so a CTA that starts
 // late goes straight to the rows that are left.  Every wait is bounded: after status.limit clocks the
 // CTA sets the status word and returns.
-// The CTA is small -- four warps, one per scheduler of an SM -- because that is what fits beside the 17 warps
-// of 72 registers of the kernel it follows: the busiest scheduler's register file has room for one more
-// warp of up to 152 registers.
+// The CTA is small -- four warps, one per scheduler of an SM -- because that is what fits beside the kernel it follows:
+// five warps of at most 80 registers on each scheduler (out_digit_tc.cu) leave 112 of its 512 registers a lane for one
+// more warp (17 warps of 72, out_gemm_tc.cu: 152).
 constexpr int kFollowRows = 2, kFollowThreads = 128;
 template <int V, bool EVEN>
 __global__ void __launch_bounds__(kFollowThreads, 5)     // at most 96 registers: more were not resident beside it

@@ -18,7 +18,7 @@
 // six layers, 98 -> 100 us.)
 // The fp16 image of the real-valued layer on fp32 activations (out_gemm_f32_tc.cu) is written the same way.
 //
-// |result - exact| <= K * 2^-23 * max_k |x[m][k]| at worst (every rounding of a frame at its largest and of one
+// |result - exact| <= K * 1.01 * 2^-23 * max_k |x[m][k]| at worst (every rounding of a frame at its largest and of one
 // sign; typically sqrt(K) 2^-25), plus one rounding to fp32.  Two bf16 terms, which this path used before, keep 2^-17 of
 // each |x| and round the sums at every step.
 //

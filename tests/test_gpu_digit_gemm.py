@@ -38,13 +38,12 @@ def test_output_layer_digits(env, m, h, c, outlier, values):
     B.bnn_output_layer_digits(model.to_dev(hp), digits, model.to_dev(b), z[:, :c], h, log_softmax=False, values=values)
     a = np.unpackbits(hp.view(np.uint8), axis=1, bitorder="little")[:, :h].astype(np.float64)
     want = (a if values else 2 * a - 1) @ w.astype(np.float64).T + b
-    # every weight is off by at most half a unit of its row's fixed-point scale: 2^-22 of the largest weight when three
-    # digits are taken (the library's criterion; the scale may lose a bit to the power of two), 2^-30 with four;
-    # then two roundings of the result and one of the bias addition
+    # every weight is off by at most half a unit of its row's fixed-point scale, the finest power of two at which the largest
+    # weight stays within 0x7F7F7F when three digits are taken (the library's criterion), within 2e9 with four; then two roundings of the result and one of the bias addition
     mx, sm = np.abs(w).max(1).astype(np.float64), np.abs(w).sum(1, dtype=np.float64)
     four = bool((h * mx > 16 * sm).any())
     assert four or not outlier or h < 64
-    bound = h * mx * (2.0 ** -30 if four else 2.0 ** -22) / 2 + 3 * 2.0 ** -24 * (np.abs(want) + np.abs(b))
+    bound = h * mx / (2e9 if four else 0x7F7F7F) + 3 * 2.0 ** -24 * (np.abs(want) + np.abs(b))
     got = z.cpu().numpy()
     assert (np.abs(got[:, :c] - want) <= bound).all(), (np.abs(got[:, :c] - want) / bound).max()
     np.testing.assert_array_equal(got[:, c], 9.0)
@@ -69,9 +68,9 @@ def test_signw_gemm_digits(env, m, n, k, act):
     ref, _ = o.signw_gemm(x, wp, k)
     mx = np.abs(x).max(1).astype(np.float64)[:, None]
     pre = sc.astype(np.float64) * ref + sh
-    # every value is off by at most half a unit of its row's fixed-point scale (2^-22 of the largest); the sum, the
+    # every value is off by at most half a unit of its row's fixed-point scale (see above); the sum, the
     # scale and the affine round once each
-    bound = np.abs(sc) * (k * mx * 2.0 ** -22 / 2 + 2.0 ** -23 * np.abs(ref)) + 2.0 ** -23 * (np.abs(pre) + np.abs(sh))
+    bound = np.abs(sc) * (k * mx / 0x7F7F7F + 2.0 ** -23 * np.abs(ref)) + 2.0 ** -23 * (np.abs(pre) + np.abs(sh))
     got = y.cpu().numpy()
     np.testing.assert_array_equal(got[:, n], 9.0)
     if act == B.ACT_HARDTANH:
@@ -123,7 +122,7 @@ def test_output_layer_digits_many_tiles(env, m, h, c, outlier, values):
     a = torch.from_numpy(np.unpackbits(hp.view(np.uint8), axis=1, bitorder="little")[:, :h]).cuda().double()
     want = (a if values else 2 * a - 1) @ wd.double().T
     # as above: half a unit of the row's scale per weight, then two roundings of the result
-    bound = h * wd.abs().amax(1).double() * (2.0 ** -30 if outlier else 2.0 ** -22) / 2 + 2.0 ** -23 * want.abs()
+    bound = h * wd.abs().amax(1).double() / (2e9 if outlier else 0x7F7F7F) + 2.0 ** -23 * want.abs()
     z = torch.empty((m, c), dtype=torch.float32, device="cuda:0")
     hpd = model.to_dev(hp)
     for _ in range(4):
@@ -140,7 +139,7 @@ def test_signw_gemm_digits_many_tiles(env, m, n, k):
     wp = wl.make_bit_planes(n, k, 0.5, 3 + m + n, B.packed_pitch(k))
     w = 2 * torch.from_numpy(np.unpackbits(wp.view(np.uint8), axis=1, bitorder="little")[:, :k]).cuda().double() - 1
     want = x.double() @ w.T
-    bound = k * x.abs().amax(1).double()[:, None] * 2.0 ** -22 / 2 + 2.0 ** -23 * want.abs()     # as above
+    bound = k * x.abs().amax(1).double()[:, None] / 0x7F7F7F + 2.0 ** -23 * want.abs()     # as above
     ws = torch.empty(B.bnn_signw_workspace_bytes(m, k), dtype=torch.uint8, device="cuda:0")
     y = torch.empty((m, n), dtype=torch.float32, device="cuda:0")
     wd = model.to_dev(wp)
@@ -166,9 +165,9 @@ def test_chained_digit_layers_many_tiles(env):
             w = torch.from_numpy(np.where(np.asarray(net.W[l]) < 0, -1.0, 1.0)).cuda()
             sc, sh = (torch.from_numpy(np.array(v, dtype=np.float64)).cuda() for v in (net.scale[l], net.shift[l]))
             dot = below.double() @ w.T
-            # half a unit of the scale per value: 2^-22 of the frame's largest in the first layer, of 1 behind a hardtanh
+            # half a unit of the scale per value: of the frame's largest in the first layer, of 1 at most behind a hardtanh
             unit = below.abs().amax(1).double()[:, None] if l == 0 else 1.0
-            bound = sc.abs() * (w.shape[1] * unit * 2.0 ** -22 / 2 + 2.0 ** -23 * dot.abs()) + 2.0 ** -23 * (sc * dot + sh).abs()
+            bound = sc.abs() * (w.shape[1] * unit / 0x7F7F7F + 2.0 ** -23 * dot.abs()) + 2.0 ** -23 * (sc * dot + sh).abs()
             err = (outs[l].double() - (sc * dot + sh).clamp(-1, 1)).abs()
             assert bool((err <= bound).all()), (l, float((err / bound).max()))
             below = outs[l]

@@ -27,8 +27,9 @@ def env():
     return torch, binding, model
 
 
-def run_binary_net(env, cfg, frames, mode=0, sample=None, prepare_xnor=True, values=0, minimal_workspace=False):
-    """Runs bnn_forward on `frames` frames; compares the frames in `sample` (all if None)."""
+def run_binary_net(env, cfg, frames, mode=0, sample=None, prepare_xnor=True, values=0, minimal_workspace=False, pad=0):
+    """Runs bnn_forward on `frames` frames; compares the frames in `sample` (all if None).  pad: columns between the rows of
+    the output (minimal workspace)."""
     torch, B, model = env
     net = wl.make_model(cfg)
     X = wl.make_frames(cfg, frames)
@@ -37,7 +38,7 @@ def run_binary_net(env, cfg, frames, mode=0, sample=None, prepare_xnor=True, val
     if minimal_workspace:
         small = torch.empty(dn.desc.min_workspace_bytes(frames), dtype=torch.uint8, device="cuda:0")
         assert small.numel() < dn.desc.workspace_bytes(frames)
-        logp = torch.empty((frames, cfg.classes), dtype=torch.float32, device="cuda:0")
+        logp = torch.empty((frames, cfg.classes + pad), dtype=torch.float32, device="cuda:0")[:, :cfg.classes]
         B.bnn_forward(dn.desc, model.to_dev(X), logp, small, layer_out=outs)
     else:
         logp = dn.forward(model.to_dev(X), layer_out=outs)
@@ -158,10 +159,12 @@ def test_forward_stacked_hidden_layers_edge_shapes(env, hidden, n_hidden, frames
     (2561, 3400, 0, True),    # one frame in the last group
     (2100, 4100, 0, False),   # more classes than the following kernel holds in registers: the kernels run one after the other
 ])
-def test_forward_log_softmax_following_the_top_layer(env, frames, classes, values, with_prior):
-    """The log-softmax launched behind the top layer's kernel, taking each group of 512 frames as soon as
-    its logits are complete (default when the top layer has more than one wave of tiles), against the
-    oracle, against the two kernels run one after the other, and repeated into the same workspace."""
+@pytest.mark.parametrize("form", ["digits", "halves"])
+def test_forward_log_softmax_following_the_top_layer(env, frames, classes, values, with_prior, form):
+    """The log-softmax launched behind the top layer's kernel, taking each group of frames (256 on byte digits of the
+    weights, 512 on their fp16 terms) as soon as its logits are complete (default when the top layer has more than one
+    wave of tiles), against the oracle, against the two kernels run one after the other, and repeated into the same
+    workspace."""
     import dataclasses
     torch, B, model = env
     cfg = dataclasses.replace(wl.CONFIGS["tiny"], hidden=256, n_hidden=2, classes=classes)
@@ -170,6 +173,11 @@ def test_forward_log_softmax_following_the_top_layer(env, frames, classes, value
     rng = np.random.default_rng(frames)
     log_prior = np.log(rng.dirichlet(np.ones(classes) * 5.0)).astype(np.float32) if with_prior else None
     dn = model.DeviceNet(net, act_values=values, log_prior=log_prior)
+    if form == "halves":      # a caller who prepares the top layer's weights as fp16 terms only
+        img = torch.empty(B.bnn_output_prepared_bytes(classes, cfg.hidden), dtype=torch.uint8, device="cuda:0")
+        B.bnn_output_prepare(dn.Wout, img)
+        dn.desc = B.ModelDesc(dn.desc.layers[:-1] + [dict(dn.desc.layers[-1], W_digits=None, W_prepared=img)],
+                              act_values=values, log_prior=dn.log_prior)
     outs = dn.layer_out_buffers(frames)
     Xd = model.to_dev(X)
     a = dn.forward(Xd, layer_out=outs).clone()
@@ -187,7 +195,7 @@ def test_forward_log_softmax_following_the_top_layer(env, frames, classes, value
     assert (a - b).abs().max().item() <= 1e-5
     for _ in range(3):   # the counters are cleared by every call
         assert torch.equal(dn.forward(Xd), a)
-    # rows of the output that are not 16-byte aligned: the following kernel does not apply, same result
+    # rows of the output that are not 16-byte aligned: the following kernel takes their edges word by word, same result
     wide = torch.full((frames, classes + 3), 7.0, dtype=torch.float32, device="cuda:0")
     c = dn.forward(Xd, logp=wide[:, :classes])
     assert (c - a).abs().max().item() <= 1e-5
@@ -213,10 +221,12 @@ def test_forward_ami_config_full_batch_sampled_frames(env):
     run_binary_net(env, cfg, cfg.frames, sample=sample)
 
 
-def test_forward_minimal_workspace_against_the_oracle(env):
-    """With only the minimal scratch the first layer runs without the split-activation image (its
-    kernel splits inside the GEMM): the same procedure against the oracle as with the full scratch."""
-    run_binary_net(env, wl.CONFIGS["tiny"], 200, minimal_workspace=True)
+@pytest.mark.parametrize("pad", [0, 4])
+def test_forward_minimal_workspace_against_the_oracle(env, pad):
+    """With only the minimal scratch the first layer keeps its split-activation image in the rows of the output, or, where
+    these are not contiguous, runs without one (its kernel splits inside the GEMM): the same procedure against the
+    oracle as with the full scratch."""
+    run_binary_net(env, wl.CONFIGS["tiny"], 200, minimal_workspace=True, pad=pad)
     assert env[1].bnn_device_status() == 0
 
 
