@@ -186,8 +186,9 @@ BNN_API int bnn_signw_gemm(const float* X, int ldx, const uint32_t* Wp, int ldwp
 /* bnn_signw_gemm with scratch.  With `workspace` (device, 256-byte aligned, at least
  * bnn_signw_workspace_bytes(M, K) bytes) the real operand is written once per call as an image laid out
  * in the order the tensor core reads it, which the GEMM streams: 2-5x faster than bnn_signw_gemm on the tensor
- * path.  With two terms (BNN_OPT_SIGNW_TERMS), K <= 2^15 and an activation other than SIGN_PACK the image holds every row of X as fixed-point numbers of a
- * power-of-two scale of its own in three byte digits, and the sums are exact integers:
+ * path.  With two terms (BNN_OPT_SIGNW_TERMS), K <= 2^15 and an activation other than SIGN_PACK the image holds the sums and
+ * differences of the pairs (k, k + 16) of every row of X as fixed-point numbers of a scale of the row's own in three byte digits, and the sums of
+ * these are exact integers:
  *   |y - exact| <= K * 1.01 * 2^-23 * max_k |x[m][k]| + one fp32 rounding (a row with an infinity or a NaN gives NaN);
  * otherwise it holds bf16 terms, as bnn_signw_gemm.  Inside bnn_forward a layer writes the image of the next one of its kind
  * before a frame's largest output is known; max |x| is then replaced by a bound on it, min(1, max |scale| *
@@ -258,12 +259,12 @@ BNN_API size_t bnn_output_prepared_bytes(int C, int H);
 BNN_API int bnn_output_prepare(const float* Wout, int ldw, int C, int H,
                                void* prepared, size_t prepared_bytes, void* stream);
 
-/* The top layer on packed activations with exact sums.  bnn_output_prepare_digits writes each class row once as
- * fixed-point numbers of a power-of-two scale of its own, in three byte digits (about 23 bits relative to the row's
+/* The top layer on packed activations with exact sums.  bnn_output_prepare_digits writes the sums and differences of the pairs
+ * (h, h + 16) of each class row once as fixed-point numbers of a scale of the row's own, in three byte digits (about 23 bits relative to the row's
  * largest weight; four digits, 31 bits, for the whole matrix when some row's largest weight exceeds 16 times the
  * row's mean magnitude), in the order the tensor core reads them; bnn_output_layer_digits multiplies the digits
- * with the activations' signs in integers, so that a logit is rounded once instead of at every step, and takes 3/4
- * of the tensor-core passes of bnn_output_layer's fp16 terms:
+ * with the activations' signs in integers (of a sum and a difference a pair of signs meets one: 2:4 sparsity), so that a logit is rounded once instead of at every step, and takes 3/8
+ * of the tensor-core time of bnn_output_layer's fp16 terms:
  *   |z - exact| <= H * 1.01 * 2^-23 * max_h |Wout[c][h]|  (1.08 * 2^-31 with four digits) + one fp32 rounding + the bias
  * addition.
  * act_values : bnn_act_values of Hp.  H <= 2^15 (larger: BNN_ERR_UNSUPPORTED; use bnn_output_layer).

@@ -1,37 +1,48 @@
 // Products of a real-valued operand with packed sign bits as exact integer products on the tensor cores
-// (tcgen05 kind::i8), on CTA pairs: the engine of the top layer on packed activations (out_gemm_tc.cu) and of
+// (tcgen05 kind::i8, 2:4 sparse), on CTA pairs: the engine of the top layer on packed activations (out_digit_tc.cu) and of
 // the layers with binary weights on real-valued input (signw_digit_tc.cu).
 //
-//   S[a][b] = sum_k sigma[a][k] * v[b][k],    sigma in {-1, +1} (or {0, 1}),  v = round(real[b][k] * 2^e_b)
+// Two signs times two numbers are one sign times one number: s1 v1 + s2 v2 = s1 (v1 + v2) where s1 = s2 and s1 (v1 - v2)
+// elsewhere.  With the digits operand holding the sum and the difference of every pair (k, k + 16) in place of the two values,
+// a row of signs has exactly one +-1 and one 0 for each pair: the 2:4 sparsity of the tensor core, which takes 64
+// positions in the time of 32 (measured on B200, 256 x 192 outputs per CTA pair: 96 clocks either way).
 //
-// Every row of the real operand is scaled by a power of two of its own to a fixed-point number of about 23 bits and
-// written in base 256 with balanced digits, v = d0 + 256 d1 + 65536 d2 (-128 <= d <= 127), i.e. three bytes per
-// element.  Bits widen to bytes, the tensor core multiplies bytes at twice the rate of half-precision numbers, and
+//   S[a][b] = sum over pairs of sigma[a][k] * v[b][pair, choice],    v = round((real[b][k] +- real[b][k + 16]) / r_b)
+//
+// Every row of the real operand has a scale r_b of its own, such that its largest pair comes close to 0x7F7F7F, and is written in
+// base 256 with balanced digits, v = d0 + 256 d1 + 65536 d2 (-128 <= d <= 127), i.e. three bytes per
+// element.  The tensor core multiplies bytes at twice the rate of half-precision numbers, and
 // its 32-bit sums are exact (K <= kMaxKDigit), so S is exact: the only rounding is that of v, at most
-// 1.01 * 2^-23 of the row's largest magnitude per element (1 / 0x7F7F7F, see scale_exponent), and one rounding of the result to fp32.  Three digit
-// passes at the byte rate cost 1.5 half-precision passes, where two half-precision terms cost 2 and add up
-// in fp32 with a rounding per step; the operand's image is three bytes per element instead of four.
+// r_b / 2 <= 1.01 * 2^-23 of the row's largest magnitude per pair, and one rounding of the result to fp32.  (A power of two for a
+// scale would cost a pair's sum the bit that it has more than its two values; half as many roundings and scales that use
+// the whole range make the error smaller than that of rounding every value to a power of two: on N(0, 1) rows of 440 / 2048 / 3072,
+// rms error of a sum over sum |x| 9.0e-9 -> 7.3e-9 / 4.6e-9 -> 3.7e-9 / 4.0e-9 -> 3.1e-9.)
 //
 // Layout: the bits are the M operand, the digits the N operand.  A pair of CTAs (cluster of two, one per SM of
-// a TPC) works on a tile of 256 bit rows x N digit rows; each CTA widens its own 128 bit rows into its
-// tensor memory (the MMA reads its A operand from there, so the widened bits cost the shared memory nothing) and
+// a TPC) works on a tile of 256 bit rows x two parts of N digit rows; each CTA widens its own 128 bit rows into its
+// tensor memory (the MMA reads its A operand and its metadata from there, so the widened bits cost the shared memory nothing) and
 // loads half of the digit rows into its shared memory.  The digits of 8 consecutive b are one granule of 8 ND
 // digit rows, row = (b / 8) 8 ND + q 8 + b % 8, so a thread of the epilogue finds the ND sums of an output in its own
-// tensor-memory lane.  The image is [K / 16][rows][16 bytes]; inside a group of 32 positions of K byte 4 t + j
-// belongs to k = t + 8 j, which makes widening a shift, an AND and a multiply-add per four positions.
-// N is a launch argument, 192 or 96 (64 or 32 b with three digits): the narrow tile fills more SMs when
-// the batch is small (tile_rows).
+// tensor-memory lane.  The image is [K / 16][rows][16 bytes]; which byte of a group of 64 positions belongs to which
+// pair is chosen so that widening is cheap (widen_pairs, image_byte).
+// N is a launch argument, 192, 96 or 48 (64, 32 or 16 b with three digits): narrow tiles fill more SMs when the batch is small
+// (tile_rows).  Both parts meet the same widened bits: what widening costs (some 60 instructions per thread and 128
+// positions, and shifts and logic operations share a pipe of half the rate) is spread over 384 digit rows.  The other
+// way to share, two blocks of 256 bit rows on one part of digits, halves the bytes from L2 instead, but widens twice as much:
+// 8192 x 3400 x 2048, 84 us.
 //
 // Roles in a CTA of 20 warps:
-//   warps 0-7    epilogue (the kernel's own), two warps per tensor-memory lane quarter; two accumulators, so the
-//                epilogue of a tile overlaps the MMAs of the next
-//   warps 8, 9   rank 0: issue the MMAs of the pair and the commits, which arrive in both CTAs.  The two warps
-//                take blocks of 256 positions in turn; the sums are exact, so their order does not matter
+//   warps 0-7    epilogue (the kernel's own), two warps per tensor-memory lane quarter
+//   warps 8, 9   rank 0: issue the MMAs of the pair and the commits, which arrive in both CTAs.  Each warp has a part with its
+//                accumulator; since the epilogue reads one accumulator after the other, one part runs ahead and its
+//                epilogue is hidden behind the other's MMAs.
 //   warp 10      one thread issues the TMA loads of the digit image
-//   warps 12-19  two teams of four warps widen the bit rows, thread = one row; each team one half of every stage
-// A stage is complete when rank 0's barrier has the arrivals (or bytes) of BOTH CTAs; the partner arrives there
+//   warps 12-19  widen the bit rows, thread = one row; two teams of four warps, each one half of every stage
+// A stage, 256 positions of K, is one barrier: it is complete when rank 0's has the arrivals and bytes of BOTH CTAs; the partner arrives there
 // directly.  (Measured on B200: a thread of rank 1 that waits for its own CTA's stage and passes it on with a
-// cluster-scope release costs 1200 clocks per stage, whatever its size.)
+// cluster-scope release costs 1200 clocks per stage, whatever its size.  A wait costs an issuing warp some 180 clocks even when it
+// succeeds at once, beside 16 warps that compute: one wait for the bits and one for the digits, of 128 positions each, left
+// the tensor pipe idle half of the time.)
 // Every wait is bounded; a wait that runs out sets the CTA's abort flag, all roles of both CTAs fall through
 // to the common teardown (the partner's waits run out too) and the device status word is set.
 #pragma once
@@ -47,11 +58,12 @@ using namespace tc;
 constexpr int ROWS = 128;                     // bit rows per CTA
 constexpr int GRAN = 8;                       // b per granule
 constexpr int KB = 256;                       // positions of K per stage
-constexpr uint32_t A_COLS = KB / 4;           // 32-bit tensor-memory columns per stage of bits
+constexpr int GROUP = 64;                     // positions per MMA
+constexpr uint32_t TEAM_COLS = KB / GROUP / 2 * 10, STAGE_COLS = 2 * TEAM_COLS;    // 32-bit tensor-memory columns: 8 of signs and 2 of metadata per group
+constexpr int PARTS = 2;                      // of a tile: accumulators, issuing warps
 constexpr int MAX_N = 192;
-constexpr int B_STAGE = MAX_N / 2 * KB;       // 24 KB: shared memory of a stage of digits (half of it used when N = 96)
-constexpr int B_STAGES = 7, MAX_B_STAGES = 14, MAX_A_STAGES = 4;
-constexpr int RING_BYTES = B_STAGES * B_STAGE;
+constexpr int MAX_STAGES = 8;
+constexpr int RING_BYTES = 7 * 96 * KB;       // 168 KB of digits: 3 stages of N = 192, 7 of 96, 8 of 48
 constexpr int EPI_WARPS = 8, MMA_WARP = 8, MMA_WARP2 = 9, COPY_WARP = 10, PROD_WARP0 = 12, TEAM_WARPS = 4, TEAMS = 2;
 constexpr int THREADS = (PROD_WARP0 + TEAMS * TEAM_WARPS) * 32;
 // What the kernels declare as their largest block: caps them at 80 registers a thread, which leaves room on the SM for
@@ -60,26 +72,32 @@ constexpr int REG_THREADS = 768;
 constexpr uint32_t TMEM_COLS = 512;
 
 struct Bars {
-    uint64_t full_a[2 * MAX_A_STAGES], empty_a[2 * MAX_A_STAGES];      // per half of a stage (one team's share)
-    uint64_t full_b[MAX_B_STAGES], empty_b[MAX_B_STAGES];
-    uint64_t acc_full[2], acc_empty[2], started[2];
+    uint64_t full[MAX_STAGES], empty[MAX_STAGES];
+    uint64_t acc_full[PARTS], acc_empty[PARTS];
     uint32_t tmem_base;
     WaitState wait;
 };
 
-// The tiles of a launch: 256 bit rows x `n` digit rows; consecutive tiles share the bit rows (b_fast) or the digits.
+// The tiles of a launch: 256 bit rows x 2 parts of `n` digit rows; consecutive tiles share the bit rows (b_fast) or the digits.
 struct Work {
     int a_rows, b_rows;        // rows of the two operands
-    int n, nd;                 // digit rows per tile, digits per element
-    int steps;                 // groups of 32 positions of K
+    int n, nd;                 // digit rows per part, digits per element
+    int steps, half_tail;      // groups of 64 positions of K; whether the last one has 32 at most
     int b_fast;
-    __device__ __forceinline__ int nb() const { return n / nd; }                            // b per tile
+    __device__ __forceinline__ int grans() const { return n / (GRAN * nd); }                // granules per part (the rows left over are not used)
+    __device__ __forceinline__ int part_b() const { return grans() * GRAN; }
     __device__ __forceinline__ int a_tiles() const { return (a_rows + 2 * ROWS - 1) / (2 * ROWS); }
-    __device__ __forceinline__ int b_tiles() const { return (b_rows + nb() - 1) / nb(); }
-    __device__ __forceinline__ int a_stages() const { return n == MAX_N ? 2 : MAX_A_STAGES; }
-    __device__ __forceinline__ int b_stages() const { return n == MAX_N ? B_STAGES : MAX_B_STAGES; }
-    __device__ __forceinline__ uint32_t b_stage_bytes() const { return (uint32_t)(n / 2 * KB); }
-    __device__ __forceinline__ uint32_t a_col() const { return 2u * (uint32_t)n; }          // bits start after the two accumulators
+    __device__ __forceinline__ int b_tiles() const { return (b_rows + PARTS * part_b() - 1) / (PARTS * part_b()); }
+    __device__ __forceinline__ int ring() const { return n == MAX_N ? 3 : n == MAX_N / 2 ? 7 : MAX_STAGES; }
+    __device__ __forceinline__ uint32_t stage_bytes() const { return (uint32_t)(n * KB); }  // digits of both parts in one CTA
+    __device__ __forceinline__ int stages() const { return (steps + KB / GROUP - 1) / (KB / GROUP); }          // of a tile
+    __device__ __forceinline__ uint32_t a_col() const { return (uint32_t)(PARTS * n); }     // bits start after the accumulators
+    // Epilogue warps 0-3 and 4-7 halve every part (of 192 digit rows), or have a part each: 32 b per warp with three digits, so
+    // that a row of its stores is 128 bytes (64 take twice as many sectors at odd offsets: 731 frames x 3307 classes, 89 us
+    // a pass against 85).
+    __device__ __forceinline__ bool halved() const { return n == MAX_N; }
+    // Whether a part of a tile lies beyond the digits; such a part is left out.
+    __device__ __forceinline__ bool beyond(int tile_b, int part) const { return (tile_b * PARTS + part) * part_b() >= b_rows; }
 };
 // The tiles of this CTA pair in order.  Integer divisions only here, once per role: one per tile, let alone per stage,
 // costs the producers more than the widening itself.
@@ -110,20 +128,15 @@ private:
 };
 
 // Common set-up; returns the tensor-memory base.  Called by all threads of both CTAs.
-__device__ __forceinline__ uint32_t set_up(Bars* bars, const TcStatus& status, int warp) {
+__device__ __forceinline__ uint32_t set_up(Bars* bars, const TcStatus& status, int warp, bool halved) {
     if (threadIdx.x == 0) {
-        for (int s = 0; s < 2 * MAX_A_STAGES; ++s) {
-            mbar_init(smem_u32(&bars->full_a[s]), 2 * TEAM_WARPS);     // rank 0: the widening warps of both CTAs
-            mbar_init(smem_u32(&bars->empty_a[s]), 1);
+        for (int s = 0; s < MAX_STAGES; ++s) {
+            mbar_init(smem_u32(&bars->full[s]), 2 * TEAMS * TEAM_WARPS + 1);  // rank 0: the widening warps of both CTAs, its copying thread (+ bytes of both CTAs)
+            mbar_init(smem_u32(&bars->empty[s]), PARTS);               // a commit of each issuing warp
         }
-        for (int s = 0; s < MAX_B_STAGES; ++s) {
-            mbar_init(smem_u32(&bars->full_b[s]), 1);                  // rank 0: its copying thread (+ bytes of both CTAs)
-            mbar_init(smem_u32(&bars->empty_b[s]), 1);
-        }
-        for (int b = 0; b < 2; ++b) {
-            mbar_init(smem_u32(&bars->acc_full[b]), 2);                // one commit of each issuing warp
-            mbar_init(smem_u32(&bars->acc_empty[b]), 2 * EPI_WARPS);   // rank 0: the epilogue warps of both CTAs
-            mbar_init(smem_u32(&bars->started[b]), 1);
+        for (int b = 0; b < PARTS; ++b) {
+            mbar_init(smem_u32(&bars->acc_full[b]), 1);
+            mbar_init(smem_u32(&bars->acc_empty[b]), halved ? 2 * EPI_WARPS : EPI_WARPS);   // rank 0: the epilogue warps of both CTAs that read it
         }
         wait_state_init(&bars->wait, status);
         mbar_init_fence();
@@ -152,163 +165,173 @@ __device__ __forceinline__ void tear_down(Bars* bars, const TcStatus& status, in
 // digit rows x 16.  What lies beyond the image reads as zeros.
 __device__ __forceinline__ void copy_digits(const Work& w, const CUtensorMap* map, uint32_t ring, Bars* bars, int rank) {
     volatile int* abort_flag = &bars->wait.abort;
-    const int stages = w.b_stages();
-    const uint32_t bytes = w.b_stage_bytes();
+    const int ring_stages = w.ring(), stages = w.stages(), part_rows = w.part_b() * w.nd;
+    const uint32_t bytes = w.stage_bytes();
     int s = 0;
     uint32_t ph = 1;          // parity to wait for on `empty`: a fresh barrier passes parity 1
     for (Tiles t(w); t.left > 0; t.next()) {
-        const int row0 = t.b * w.n + rank * (w.n / 2);
-        for (int k = 0; k < w.steps; k += KB / 32) {
-            if (!mbar_wait(smem_u32(&bars->empty_b[s]), ph, abort_flag)) return;
-            const uint32_t bar = smem_u32(&bars->full_b[s]);
+        const int row0 = t.b * PARTS * part_rows + rank * (w.n / 2);
+        for (int kb = 0; kb < stages; ++kb) {
+            if (!mbar_wait(smem_u32(&bars->empty[s]), ph, abort_flag)) return;
+            const uint32_t bar = smem_u32(&bars->full[s]), bar0 = peer_addr(bar, 0), dst = ring + s * bytes;
             if (rank == 0) mbar_arrive_expect_tx(bar, 2 * bytes);
-            tma_load_2d_pair(ring + s * bytes, map, row0 * 2, k * 2, peer_addr(bar, 0));
-            if (++s == stages) { s = 0; ph ^= 1u; }
+            tma_load_2d_pair(dst, map, row0 * 2, kb * (KB / 16), bar0);
+            tma_load_2d_pair(dst + (bytes >> 1), map, (row0 + part_rows) * 2, kb * (KB / 16), bar0);
+            if (++s == ring_stages) { s = 0; ph ^= 1u; }
         }
     }
 }
 
-// Eight words of four bytes: word t holds bits t, t + 8, t + 16, t + 24 as +64 / -64 (or 64 / 0): 64 and -64
-// differ in the top bit of the byte alone, so that a word is a shift and one three-input logic operation (+1 / -1 would
-// take a third).  The sums come out 64 times as large.
-template <bool ZO>
-__device__ __forceinline__ void widen_bytes(uint32_t word, uint32_t* o) {
+// A group of 64 positions, two packed words.  Its 32 pairs are bit i of `sign` (position i of w0's lower half, or of w1's) and bit i
+// of `other` (16 positions on); the pair takes the difference where the two differ.  Compressed byte 4 j + q is pair
+// t(j) + 8 q, t(j) = 4 (j / 2 % 2) + 2 (j % 2) + j / 4, so that
+//   - a word of signs, o[j], is a shift and one three-input logic operation: 64 and -64 differ in the top bit of the byte alone (+1 / -1
+//     would take a third; the sums come out 64 times as large);
+//   - the metadata, o[8] and o[9], are the choices with two pairs of bits of the bit index exchanged (16 with 4, 8 with 2).  The
+//     indices of compressed bytes 2 c and 2 c + 1, positions 0 or 1 and 2 or 3 of group c of four, are 0 + choice and 2 + choice.
+__device__ __forceinline__ void widen_pairs(uint32_t w0, uint32_t w1, uint32_t* signs, uint32_t* meta) {
+    const uint32_t sign = __byte_perm(w0, w1, 0x5410), other = __byte_perm(w0, w1, 0x7632);
 #pragma unroll
-    for (int t = 0; t < 8; ++t) {
-        if (ZO) o[t] = (t < 7 ? word << (6 - (t < 7 ? t : 6)) : word >> 1) & 0x40404040u;
-        else o[t] = (~(word << (7 - t)) & 0x80808080u) ^ 0x40404040u;
+    for (int j = 0; j < 8; ++j) {
+        const int t = 4 * ((j >> 1) & 1) + 2 * (j & 1) + (j >> 2);
+        signs[j] = (~(sign << (7 - t)) & 0x80808080u) ^ 0x40404040u;
     }
+    uint32_t x = sign ^ other, y = ((x >> 12) ^ x) & 0x0000F0F0u;
+    x ^= y ^ (y << 12);
+    y = ((x >> 6) ^ x) & 0x00CC00CCu;
+    x ^= y ^ (y << 6);
+    meta[0] = (x & 0x55555555u) | 0x88888888u;
+    meta[1] = ((x >> 1) & 0x55555555u) | 0x88888888u;
+}
+// The other side of it: where in the 64 bytes of a group the digits of pair (k, k + 16) lie, k = 32 w + t + 8 q (w, q = 0, 1; t < 8):
+// the sum at image_byte, the difference behind it.  A last group that is one word (`half`) has its 16 pairs in its first two
+// chunks of 16 bytes, and the image ends there; w = 0.
+__host__ __device__ __forceinline__ constexpr int image_byte(bool half, int w, int t, int q) {
+    return half ? 8 * (t & 3) + 4 * (t >> 2) + 2 * q : 32 * (t & 1) + 16 * (t >> 2) + 8 * ((t >> 1) & 1) + 4 * w + 2 * q;
+}
+// The bits of such a word, spread over the two words of a whole group: bit t + 8 q of either half goes to bit 16 (t / 4) + 8 q + 2 (t % 4)
+// of `sign` or `other`.
+__device__ __forceinline__ uint32_t spread_pairs(uint32_t x) {
+    x = (x & 0x0F0Fu) | ((x & 0xF0F0u) << 12);
+    x = (x | (x << 2)) & 0x33333333u;
+    return (x | (x << 1)) & 0x55555555u;
+}
+__device__ __forceinline__ void spread_half_group(uint32_t& w0, uint32_t& w1) {
+    const uint32_t sign = spread_pairs(w0 & 0xFFFFu), other = spread_pairs(w0 >> 16);
+    w0 = __byte_perm(sign, other, 0x5410);
+    w1 = __byte_perm(sign, other, 0x7632);
 }
 
 // Warps PROD_WARP0 ..: thread = one bit row of this CTA; each team takes 128 positions of every stage.  The packed row is
-// read 16 bytes (the team's share of a stage) at a time, two stages ahead of use.  Bits at positions >= K may
-// hold anything: the digits are zero there.
-template <bool ZO>
+// read 16 bytes (the team's share of a stage) at a time, two stages ahead of use.
+// Bits at positions >= K may hold anything: a pair's sum and difference are the same number where its second position is
+// beyond K, and zero where both are.
 __device__ __forceinline__ void widen_bits(const Work& w, const uint32_t* __restrict__ P, int ldp, Bars* bars, uint32_t tmem,
                                            int rank, int warp, int lane) {
     volatile int* abort_flag = &bars->wait.abort;
     Tiles t(w);
-    const int total_tiles = t.left;
     const int team = (warp - PROD_WARP0) / TEAM_WARPS;
-    const int r = (warp & 3) * 32 + lane;                   // a warp may only touch the lanes of its quarter
-    const uint32_t tdst = tmem + ((uint32_t)((warp & 3) * 32) << 16) + w.a_col() + (uint32_t)team * (A_COLS / 2);
-    const int groups = (w.steps + 3) >> 2, blocks = (w.steps + 7) >> 3;     // 128-position groups and stages per tile
-    const int a_stages = w.a_stages();
-    int pf_g = team;                                        // the next group to fetch, of the tile `t` is at
-    auto row_of = [&]() {
-        const int row = t.a * (2 * ROWS) + rank * ROWS + r;
-        return t.left > 0 && row < w.a_rows ? reinterpret_cast<const uint4*>(P + (size_t)row * ldp) : nullptr;
+    const int r = rank * ROWS + (warp & 3) * 32 + lane;         // (a warp may only touch the lanes of its quarter)
+    const uint32_t tdst = tmem + ((uint32_t)((warp & 3) * 32) << 16) + w.a_col() + (uint32_t)team * TEAM_COLS;
+    const int words4 = (w.steps + 1) >> 1;                      // 16-byte pieces of a row
+    const int stages = w.stages();
+    const int missing = (stages - 1) * TEAMS + team >= words4 ? 1 : 0;           // of this team's pieces, in the last stage
+    // of the stages of a tile, counted down: the one whose last group is half a group
+    const int tail = w.half_tail && ((words4 - 1) & 1) == team ? 1 + missing : -1;
+    const bool tail_high = !(w.steps & 1);
+    const uint4* next_piece = nullptr;
+    int pieces = 0;                                             // left of the tile that is being fetched
+    int left = t.left * stages;                                 // stages still to be filled
+    auto next_tile = [&]() {
+        const int row = t.left > 0 ? t.a * (2 * ROWS) + r : 0;
+        next_piece = reinterpret_cast<const uint4*>(P + (size_t)(row < w.a_rows ? row : 0) * ldp) + team;    // (rows beyond go nowhere)
+        pieces = stages;
+        t.next();
     };
-    const uint4* pf_row = row_of();
+    next_tile();
     auto fetch = [&]() {
         uint4 o = make_uint4(0u, 0u, 0u, 0u);
-        if (pf_row && pf_g < groups) o = ldg_nc_u4(pf_row + pf_g);
-        pf_g += TEAMS;
-        if (pf_g >= 2 * blocks) { pf_g = team; t.next(); pf_row = row_of(); }
+        if (pieces > missing) o = ldg_nc_u4(next_piece);
+        next_piece += TEAMS;
+        if (--pieces == 0) next_tile();
         return o;
     };
-    int s = 0;
+    const uint32_t end = tdst + (uint32_t)w.ring() * STAGE_COLS;
+    uint32_t dst = tdst, empty = smem_u32(&bars->empty[0]), full = smem_u32(&bars->full[0]);
+    if (rank != 0) full = peer_addr(full, 0);
     uint32_t ph = 1;
-    const int total = total_tiles * blocks;
     uint4 cur = fetch(), nxt = fetch();
-    uint32_t o[32];
-    auto widen = [&](const uint4& v) {
-        widen_bytes<ZO>(v.x, o); widen_bytes<ZO>(v.y, o + 8); widen_bytes<ZO>(v.z, o + 16); widen_bytes<ZO>(v.w, o + 24);
+    uint32_t o[20];
+    int at = stages;                                            // stages left of the tile that is being widened
+    auto widen = [&](uint4 v) {
+        if (at == tail) {
+            if (tail_high) spread_half_group(v.z, v.w);
+            else spread_half_group(v.x, v.y);
+        }
+        if (--at == 0) at = stages;
+        widen_pairs(v.x, v.y, o, o + 16);
+        widen_pairs(v.z, v.w, o + 8, o + 18);
     };
     widen(cur);
-    for (int it = 0; it < total; ++it) {
-        // what lies between a free slot and a full one is kept short: the row was widened before the wait
-        if (!warp_wait(smem_u32(&bars->empty_a[2 * s + team]), ph, abort_flag, lane)) return;
-        tmem_st32(tdst + s * A_COLS, o);
+    for (; left > 0; --left) {
+        // what lies between a free stage and a full one is kept short: the row was widened before the wait
+        if (!warp_wait(empty, ph, abort_flag, lane)) return;
+        tmem_st16(dst, o);
+        tmem_st4(dst + 16, o + 16);
         cur = nxt;
         nxt = fetch();
         tmem_st_wait();
         tc_fence_before_sync();
         __syncwarp();
         if (lane == 0) {
-            const uint32_t bar = smem_u32(&bars->full_a[2 * s + team]);
-            if (rank == 0) mbar_arrive(bar);
-            else mbar_arrive_cluster(peer_addr(bar, 0));
+            if (rank == 0) mbar_arrive(full);
+            else mbar_arrive_cluster(full);
         }
-        if (++s == a_stages) { s = 0; ph ^= 1u; }
+        dst += STAGE_COLS; empty += 8; full += 8;
+        if (dst == end) {
+            dst = tdst; empty -= 8 * (uint32_t)w.ring(); full -= 8 * (uint32_t)w.ring();
+            ph ^= 1u;
+        }
         widen(cur);
     }
 }
 
-// Both barriers of a stage: polled together first, so that a stage that is ready costs one round trip.
-__device__ __forceinline__ bool warp_wait_both(uint32_t bar0, uint32_t par0, uint32_t bar1, uint32_t par1, volatile int* abort_flag) {
-    const bool r0 = mbar_try_wait(bar0, par0), r1 = mbar_try_wait(bar1, par1);
-    if (__all_sync(0xFFFFFFFFu, r0 && r1)) return true;
-    return warp_wait(bar0, par0, abort_flag, 0) && warp_wait(bar1, par1, abort_flag, 0);
-}
-
-// Warps MMA_WARP and MMA_WARP2 of rank 0, converged; they take the stages of a tile in turn.  What an issuing
-// warp does besides its MMAs (waits about 100 clocks each even when they succeed, commits) is time that only the
-// other warp's MMAs can fill.  The bits of a stage come and go in two halves: tensor memory holds only two stages
-// beside the accumulators, and a half that is handed back after its four MMAs has the time of twelve to be refilled.
-__device__ __forceinline__ void issue(const Work& w, uint32_t ring, Bars* bars, uint32_t tmem, int which) {
+// Warps MMA_WARP and MMA_WARP2 of rank 0, converged, each with its part of every tile.  What an issuing warp does besides its MMAs is
+// time that only the other warp's MMAs can fill.
+__device__ __forceinline__ void issue(const Work& w, uint32_t ring, Bars* bars, uint32_t tmem, int part) {
     volatile int* abort_flag = &bars->wait.abort;
-    const int tiles = Tiles(w).left;
-    const uint32_t idesc = instr_desc(kAccS32, kFmtS8, kFmtS8, 2 * ROWS, w.n);
-    const int a_stages = w.a_stages(), b_stages = w.b_stages();
+    const uint32_t idesc = instr_desc(kAccS32, kFmtS8, kFmtS8, 2 * ROWS, w.n) | kSparse;
+    const int ring_stages = w.ring(), stages = w.stages();
     const uint32_t chunk16 = (uint32_t)(w.n / 2);            // 16-byte units between chunks of 16 positions
-    const uint32_t stage16 = w.b_stage_bytes() >> 4;
-    const uint64_t desc = smem_desc_kmajor(ring, chunk16 * 16u, 128);
-    const uint32_t desc_lo = (uint32_t)desc, desc_hi = (uint32_t)(desc >> 32), step16 = 2 * chunk16;   // an MMA takes two chunks
-    const uint32_t ta0 = tmem + w.a_col();
-    const int blocks = (w.steps + 7) >> 3;
-    int sa = 0, sb = 0;
-    uint32_t pa = 0, pb = 0;
-    for (int tl = 0; tl < tiles; ++tl) {
-        const int b = tl & 1;
-        if (!warp_wait(smem_u32(&bars->acc_empty[b]), (uint32_t)(((tl >> 1) & 1) ^ 1), abort_flag, 0)) return;
-        tc_fence_after_sync();
-        const uint32_t d = tmem + (uint32_t)(b * w.n);
-        for (int kb = 0; kb < blocks; ++kb) {
-            if ((kb & 1) == which) {
-                // The MMA that overwrites the accumulator has to come first.  This wait also stands before those for the
-                // stage, because a wait on a parity holds only for one who knows that the phase before it is over.  With
-                // an odd number of stages per tile the other warp takes two in a row, the last of a tile and the first
-                // of the next; when there are two slots the former had this stage's.  `started` says that the other
-                // warp has issued the latter, so it has found the former full.
-                if (kb == 1 && !warp_wait(smem_u32(&bars->started[b]), (uint32_t)((tl >> 1) & 1), abort_flag, 0)) return;
-                if (!warp_wait_both(smem_u32(&bars->full_b[sb]), pb, smem_u32(&bars->full_a[2 * sa]), pa, abort_flag)) return;
-                tc_fence_after_sync();
-                // the address field (16-byte units) is advanced by plain additions: the ring lies below 2^14 * 16 bytes
-                const uint32_t db = desc_lo + (uint32_t)sb * stage16;
-                const uint32_t ta = ta0 + (uint32_t)sa * A_COLS;
-                const int n_mma = w.steps - 8 * kb;           // 8 but for the last stage
-                if (elect_one()) {
-                    mma_i8_ts_pair(d, ta, db, desc_hi, idesc, kb != 0);
-                    if (kb == 0) mma_commit_pair(smem_u32(&bars->started[b]));
-                    if (n_mma >= 4) {
-                        mma_i8_ts_pair(d, ta + 8, db + step16, desc_hi, idesc, 1u);
-                        mma_i8_ts_pair(d, ta + 16, db + 2 * step16, desc_hi, idesc, 1u);
-                        mma_i8_ts_pair(d, ta + 24, db + 3 * step16, desc_hi, idesc, 1u);
-                    } else {
-                        for (int j = 1; j < n_mma; ++j) mma_i8_ts_pair(d, ta + 8 * j, db + j * step16, desc_hi, idesc, 1u);
-                    }
-                    mma_commit_pair(smem_u32(&bars->empty_a[2 * sa]));
-                }
-                if (!warp_wait(smem_u32(&bars->full_a[2 * sa + 1]), pa, abort_flag, 0)) return;
-                tc_fence_after_sync();
-                if (elect_one()) {
-                    if (n_mma >= 8) {
-                        mma_i8_ts_pair(d, ta + 32, db + 4 * step16, desc_hi, idesc, 1u);
-                        mma_i8_ts_pair(d, ta + 40, db + 5 * step16, desc_hi, idesc, 1u);
-                        mma_i8_ts_pair(d, ta + 48, db + 6 * step16, desc_hi, idesc, 1u);
-                        mma_i8_ts_pair(d, ta + 56, db + 7 * step16, desc_hi, idesc, 1u);
-                    } else {
-                        for (int j = 4; j < n_mma; ++j) mma_i8_ts_pair(d, ta + 8 * j, db + j * step16, desc_hi, idesc, 1u);
-                    }
-                    mma_commit_pair(smem_u32(&bars->empty_a[2 * sa + 1]));
-                    mma_commit_pair(smem_u32(&bars->empty_b[sb]));
-                }
-            }
-            if (++sa == a_stages) { sa = 0; pa ^= 1u; }
-            if (++sb == b_stages) { sb = 0; pb ^= 1u; }
+    const uint32_t stage16 = w.stage_bytes() >> 4;
+    const uint64_t desc = smem_desc_kmajor(ring + (uint32_t)part * (w.stage_bytes() >> 1), chunk16 * 16u, 128);
+    const uint32_t desc_lo = (uint32_t)desc, desc_hi = (uint32_t)(desc >> 32), step16 = 4 * chunk16;   // an MMA takes four chunks
+    const uint32_t d = tmem + (uint32_t)(part * w.n), ta0 = tmem + w.a_col();
+    int s = 0;
+    uint32_t ph = 0, pacc = 1;
+    for (Tiles t(w); t.left > 0; t.next()) {
+        const bool beyond = w.beyond(t.b, part);
+        if (!beyond) {
+            if (!warp_wait(smem_u32(&bars->acc_empty[part]), pacc, abort_flag, 0)) return;
+            tc_fence_after_sync();
+            pacc ^= 1u;
         }
-        if (elect_one()) mma_commit_pair(smem_u32(&bars->acc_full[b]));
+        for (int kb = 0; kb < stages; ++kb) {
+            if (!warp_wait(smem_u32(&bars->full[s]), ph, abort_flag, 0)) return;
+            tc_fence_after_sync();
+            // the address field (16-byte units) is advanced by plain additions: the ring lies below 2^14 * 16 bytes
+            const uint32_t db = desc_lo + (uint32_t)s * stage16, ta = ta0 + (uint32_t)s * STAGE_COLS;
+            const int left = beyond ? 0 : w.steps - 4 * kb;   // groups: 4 but for the last stage
+            if (elect_one()) {
+                if (left > 0) mma_i8_sp_ts_pair(d, ta, ta + 16, db, desc_hi, idesc, kb != 0);
+                if (left > 1) mma_i8_sp_ts_pair(d, ta + 8, ta + 18, db + step16, desc_hi, idesc, 1u);
+                if (left > 2) mma_i8_sp_ts_pair(d, ta + TEAM_COLS, ta + TEAM_COLS + 16, db + 2 * step16, desc_hi, idesc, 1u);
+                if (left > 3) mma_i8_sp_ts_pair(d, ta + TEAM_COLS + 8, ta + TEAM_COLS + 18, db + 3 * step16, desc_hi, idesc, 1u);
+                mma_commit_pair(smem_u32(&bars->empty[s]));
+                if (kb + 1 == stages && !beyond) mma_commit_pair(smem_u32(&bars->acc_full[part]));
+            }
+            if (++s == ring_stages) { s = 0; ph ^= 1u; }
+        }
     }
 }
 
@@ -319,7 +342,7 @@ __device__ __forceinline__ void release_acc(Bars* bars, int b, int lane) {
     if (lane == 0) mbar_arrive_cluster(peer_addr(smem_u32(&bars->acc_empty[b]), 0));
 }
 
-// The sums S of one granule (8 outputs of this thread's bit row) in fp32.  With three digits the two low sums are
+// The sums S of one granule (8 outputs of this thread's bit row) in fp32: with three digits the two low sums are
 // joined exactly as an integer (below 2^24, i.e. an exact float, unless a row's middle digits add up almost
 // without cancelling; then the rounding is still below the row's quantisation steps); with four, digit sums are carried
 // into one another first.
@@ -329,74 +352,57 @@ __device__ __forceinline__ void load_granule(uint32_t taddr, int nd, uint32_t (&
     tmem_ld8(taddr + 16, d[2]);
     if (nd == 4) tmem_ld8(taddr + 24, d[3]);
 }
-__device__ __forceinline__ void join_granule(const uint32_t (&d)[4][8], int nd, float (&S)[8]) {
-    if (nd == 4) {
-#pragma unroll
-        for (int i = 0; i < 8; ++i) {
-            const int d0 = (int)d[0][i] >> 6;
-            const int d1 = ((int)d[1][i] >> 6) + (d0 >> 8);
-            const int d2 = ((int)d[2][i] >> 6) + (d1 >> 8);
-            const int low = ((d2 & 255) << 16) | ((d1 & 255) << 8) | (d0 & 255);
-            S[i] = fmaf((float)(((int)d[3][i] >> 6) + (d2 >> 8)), 16777216.0f, (float)low);
-        }
-    } else {
-#pragma unroll
-        for (int i = 0; i < 8; ++i) {
-            // the high sum is below 2^22: adding 1.5 * 2^23 as an integer to its bits makes it a float without the
-            // conversion unit, which the other conversion of every output already keeps busy
-            const float high = __int_as_float(((int)d[2][i] >> 6) + 0x4B400000) - 12582912.0f;
-            S[i] = fmaf(high, 65536.0f, (float)((int)d[1][i] * 4 + ((int)d[0][i] >> 6)));
-        }
-    }
+__device__ __forceinline__ float join4(int s0, int s1, int s2, int s3) {
+    const int d0 = s0 >> 6;
+    const int d1 = (s1 >> 6) + (d0 >> 8);
+    const int d2 = (s2 >> 6) + (d1 >> 8);
+    const int low = ((d2 & 255) << 16) | ((d1 & 255) << 8) | (d0 & 255);
+    return fmaf((float)((s3 >> 6) + (d2 >> 8)), 16777216.0f, (float)low);
 }
-// `n` consecutive granules, handed to `use(g, S)` one by one; with three digits the next one is on its way meanwhile.
-template <typename F>
-__device__ __forceinline__ void granules(uint32_t taddr, int n, int nd, F use) {
-    uint32_t d[4][8];
-    float S[8];
-    if (nd == 4) {
-#pragma unroll 1
-        for (int g = 0; g < n; ++g) {
-            load_granule(taddr + (uint32_t)g * 32, 4, d);
-            tmem_ld_wait();
-            join_granule(d, 4, S);
-            use(g, S);
-        }
-        return;
-    }
-    load_granule(taddr, 3, d);
-#pragma unroll 1
-    for (int g = 0; g < n; ++g) {
-        tmem_ld_wait();
-        join_granule(d, 3, S);
-        if (g + 1 < n) load_granule(taddr + (uint32_t)(g + 1) * 24, 3, d);
-        use(g, S);
-    }
-}
-
+// low + 65536 high, the two parts of a sum of three digits.
+__device__ __forceinline__ float low_part(int s0, int s1) { return (float)(s1 * 4 + (s0 >> 6)); }
+// The high sum is below 2^22: adding 1.5 * 2^23 as an integer to its bits makes it a float without the
+// conversion unit, which the other conversion of every output already keeps busy.
+__device__ __forceinline__ float high_part(int s2) { return __int_as_float((s2 >> 6) + 0x4B400000) - 12582912.0f; }
 // 2^h for -126 <= h <= 127.
 __device__ __forceinline__ float power_of_two(int h) { return __int_as_float((127 + h) << 23); }
-// Largest e (up to 140) such that mx * 2^e is a balanced number of nd digits: at most 127 * (65536 + 256 + 1) =
-// 0x7F7F7F with three, and somewhat below 127 * 2^24 with four (2e9).  mx >= 0; its exponent and fraction fields
-// are compared with those of the limit.
-__device__ __forceinline__ int scale_exponent(float mx, int nd) {
+// Largest e (up to 140) such that mx * 2^e is a balanced number of three digits: at most 127 * (65536 + 256 + 1) = 0x7F7F7F.
+// mx >= 0; its exponent and fraction fields are compared with those of the limit.
+__device__ __forceinline__ int scale_exponent(float mx) {
     const int bits = __float_as_int(mx);
     if (bits == 0) return 0;
-    const int over = (bits & 0x7FFFFF) > (nd == 4 ? 7236393 : 0x7EFEFE) ? 1 : 0;     // 2e9 / 2^30, 0x7F7F7F / 2^22
-    const int e = (nd == 4 ? 30 : 22) + 127 - (bits >> 23) - over;
+    const int e = 22 + 127 - (bits >> 23) - ((bits & 0x7FFFFF) > 0x7EFEFE ? 1 : 0);     // 0x7F7F7F / 2^22
     return e > 140 ? 140 : e;
 }
-// 2^-e, or NaN for a row that holds an infinity or a NaN.
-__device__ __forceinline__ float inverse_scale(float mx, int nd) {
-    const int e = scale_exponent(mx, nd), h = e >> 1;
-    return __float_as_int(mx) < 0x7F800000 ? power_of_two(-h) * power_of_two(h - e) : __int_as_float(0x7FC00000);
-}
-// x * 2^e rounded to an integer; 2^e comes as two powers of two (e may be beyond the exponent range of one).
+// The scale of a row, from half of the largest |x1| + |x2| of its pairs (half, because a pair's sum may be beyond the largest float).
+constexpr float kTopValue = 8355700.0f;       // somewhat below 0x7F7F7F: room for roundings
 struct Scale {
     float a, b;
-    __device__ __forceinline__ explicit Scale(int e) : a(power_of_two(e >> 1)), b(power_of_two(e - (e >> 1))) {}
-    __device__ __forceinline__ int fixed_point(float x) const { return __float2int_rn(x * a * b); }
+    float inverse;                            // what a unit stands for
+    __device__ __forceinline__ explicit Scale(float half_top) {
+        if (half_top >= 0x1p-100f) {
+            a = 1.0f;
+            b = __fdiv_rn(kTopValue, half_top);
+            inverse = __fdiv_rn(2.0f, b);
+        } else {                              // (1 / scale may be beyond the largest float)
+            const int e = half_top > 0.f ? scale_exponent(half_top) - 1 : 0, h = e >> 1;
+            a = power_of_two(h + 1);
+            b = power_of_two(e - h);
+            inverse = power_of_two(-h) * power_of_two(h - e);
+        }
+    }
+    // The numbers of a pair.  Its two products are rounded to integers and fractions, which are added apart: a float of more than
+    // 2^22 has no more than one bit of fraction left, and the sum is better rounded once.
+    __device__ __forceinline__ void pair(float x1, float x2, int& sum, int& difference) const {
+        const float p1 = x1 * a * (0.5f * b), p2 = x2 * a * (0.5f * b);
+        const int i1 = __float2int_rn(p1), i2 = __float2int_rn(p2);
+        const float f1 = p1 - (float)i1, f2 = p2 - (float)i2;
+        sum = i1 + i2 + __float2int_rn(f1 + f2);
+        difference = i1 - i2 + __float2int_rn(f1 - f2);
+    }
 };
+// Half of |x1| + |x2|.
+__device__ __forceinline__ float half_sum(float x1, float x2) { return fmaf(0.5f, x1, 0.5f * x2); }
 // The balanced base-256 digits of v in the bytes of a word: the sum of 128 at every place turns them into ordinary
 // bytes (no borrows), and the exclusive or takes 128 off each byte again.
 __device__ __forceinline__ uint32_t digits3(int v) { return ((uint32_t)v + 0x00808080u) ^ 0x00808080u; }
@@ -408,15 +414,19 @@ __device__ __forceinline__ uint32_t gather_bytes(uint32_t a, uint32_t b, uint32_
     return __byte_perm(__byte_perm(a, b, lo), __byte_perm(c, d, lo), 0x5410);
 }
 
-// Digit rows per tile (192 or 96) for `a_rows` x `b_rows` outputs on `pairs` CTA pairs: the one with the least
-// estimated time.  An MMA of 32 positions takes N / 2 clocks in the tensor pipe but not less than about 70, the
-// rate at which it can be issued; a launch takes ceil(tiles / pairs) turns.
+// Digit rows per part of a tile (192, 96 or 48).
+inline long long tile_count(int a_rows, int b_rows, int n) { return (long long)ceil_div(a_rows, 2 * ROWS) * ceil_div(b_rows, PARTS * n / 3); }
+// For `a_rows` x `b_rows` outputs of `steps` groups of 64 positions on `pairs` CTA pairs: the width with the least
+// estimated time.  A launch takes ceil(tiles / pairs) turns.
 inline int tile_rows(int a_rows, int b_rows, int steps, int pairs) {
-    auto cost = [&](int n, int clocks) {
-        const long long tiles = (long long)ceil_div(a_rows, 2 * ROWS) * ceil_div(b_rows, n / 3);
-        return (tiles + pairs - 1) / pairs * ((long long)steps * clocks + 800);
-    };
-    return cost(96, 70) < cost(192, 100) ? 96 : 192;
+    constexpr struct { int n, clocks; } widths[] = {{192, 290}, {96, 170}, {48, 110}};
+    int best = 0;
+    long long least = -1;
+    for (const auto& s : widths) {
+        const long long cost = (tile_count(a_rows, b_rows, s.n) + pairs - 1) / pairs * ((long long)steps * s.clocks + 1200);
+        if (least < 0 || cost < least) { least = cost; best = s.n; }
+    }
+    return best;
 }
 
 }  // namespace digit

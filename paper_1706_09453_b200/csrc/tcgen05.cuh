@@ -168,6 +168,11 @@ __device__ __forceinline__ void tma_store_2d(const CUtensorMap* map, int x, int 
     asm volatile("cp.async.bulk.tensor.2d.global.shared::cta.tile.bulk_group [%0, {%1, %2}], [%3];"
                  ::"l"(map), "r"(x), "r"(y), "r"(src) : "memory");
 }
+// The same with an L2 cache policy.
+__device__ __forceinline__ void tma_store_2d_hint(const CUtensorMap* map, int x, int y, uint32_t src, uint64_t policy) {
+    asm volatile("cp.async.bulk.tensor.2d.global.shared::cta.tile.bulk_group.L2::cache_hint [%0, {%1, %2}], [%3], %4;"
+                 ::"l"(map), "r"(x), "r"(y), "r"(src), "l"(policy) : "memory");
+}
 __device__ __forceinline__ void bulk_commit() { asm volatile("cp.async.bulk.commit_group;" ::: "memory"); }
 // all but the N latest groups have read their shared memory / are complete
 template <int N> __device__ __forceinline__ void bulk_wait_read() { asm volatile("cp.async.bulk.wait_group.read %0;" ::"n"(N) : "memory"); }
@@ -320,14 +325,20 @@ __device__ __forceinline__ void tmem_alloc_pair(uint32_t slot_smem, uint32_t nco
 __device__ __forceinline__ void tmem_dealloc_pair(uint32_t taddr, uint32_t ncols) {
     asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(taddr), "r"(ncols) : "memory");
 }
-// D[256 x N] (+)= A[256 x 32] * B[N x 32]^T on bytes, 32-bit integer sums; A in the tensor memory of both CTAs.  B's
-// descriptor comes as two words, so that stepping through a stage is 32-bit arithmetic.
-__device__ __forceinline__ void mma_i8_ts_pair(uint32_t tmem_d, uint32_t tmem_a, uint32_t db_lo, uint32_t db_hi, uint32_t idesc, uint32_t accumulate) {
+// D[256 x N] (+)= A[256 x 64] * B[N x 64]^T on bytes, 32-bit integer sums; A in the tensor memory of both CTAs.  B's
+// descriptor comes as two words, so that stepping through a stage is 32-bit arithmetic.  A is 2:4 sparse, and half of it is stored: of every
+// four consecutive positions two, in ascending order (32 bytes per row,
+// 8 columns), and which ones in the metadata, two 2-bit indices per four positions, the lower one in the lower
+// bits.  The metadata of a row of A lie in that row's lane, eight groups of four positions per column, the first in the lowest
+// bits (two columns).  idesc: kSparse added.
+constexpr uint32_t kSparse = 1u << 2;
+__device__ __forceinline__ void mma_i8_sp_ts_pair(uint32_t tmem_d, uint32_t tmem_a, uint32_t tmem_meta, uint32_t db_lo, uint32_t db_hi, uint32_t idesc,
+                                                  uint32_t accumulate) {
     asm volatile(
         "{\n\t.reg .pred p;\n\t.reg .b64 b;\n\t"
-        "setp.ne.b32 p, %5, 0;\n\tmov.b64 b, {%2, %3};\n\t"
-        "tcgen05.mma.cta_group::2.kind::i8 [%0], [%1], b, %4, p;\n\t}"
-        ::"r"(tmem_d), "r"(tmem_a), "r"(db_lo), "r"(db_hi), "r"(idesc), "r"(accumulate) : "memory");
+        "setp.ne.b32 p, %6, 0;\n\tmov.b64 b, {%3, %4};\n\t"
+        "tcgen05.mma.sp.cta_group::2.kind::i8 [%0], [%1], b, [%2], %5, p;\n\t}"
+        ::"r"(tmem_d), "r"(tmem_a), "r"(tmem_meta), "r"(db_lo), "r"(db_hi), "r"(idesc), "r"(accumulate) : "memory");
 }
 // Arrive on the barrier at this offset in BOTH CTAs once every MMA issued so far by this thread has completed.
 __device__ __forceinline__ void mma_commit_pair(uint32_t bar) {
@@ -371,6 +382,19 @@ __device__ __forceinline__ void tmem_st32(uint32_t taddr, const uint32_t (&r)[32
           "r"(r[16]), "r"(r[17]), "r"(r[18]), "r"(r[19]), "r"(r[20]), "r"(r[21]), "r"(r[22]), "r"(r[23]),
           "r"(r[24]), "r"(r[25]), "r"(r[26]), "r"(r[27]), "r"(r[28]), "r"(r[29]), "r"(r[30]), "r"(r[31])
         : "memory");
+}
+// The same, 16 and 4 columns.
+__device__ __forceinline__ void tmem_st16(uint32_t taddr, const uint32_t* r) {
+    asm volatile(
+        "tcgen05.st.sync.aligned.32x32b.x16.b32 [%0], "
+        "{%1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, %16};"
+        ::"r"(taddr), "r"(r[0]), "r"(r[1]), "r"(r[2]), "r"(r[3]), "r"(r[4]), "r"(r[5]), "r"(r[6]), "r"(r[7]),
+          "r"(r[8]), "r"(r[9]), "r"(r[10]), "r"(r[11]), "r"(r[12]), "r"(r[13]), "r"(r[14]), "r"(r[15])
+        : "memory");
+}
+__device__ __forceinline__ void tmem_st4(uint32_t taddr, const uint32_t* r) {
+    asm volatile("tcgen05.st.sync.aligned.32x32b.x4.b32 [%0], {%1, %2, %3, %4};"
+                 ::"r"(taddr), "r"(r[0]), "r"(r[1]), "r"(r[2]), "r"(r[3]) : "memory");
 }
 __device__ __forceinline__ void tmem_st_wait() {
     asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
