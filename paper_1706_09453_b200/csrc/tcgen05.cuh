@@ -340,6 +340,15 @@ __device__ __forceinline__ void mma_i8_sp_ts_pair(uint32_t tmem_d, uint32_t tmem
         "tcgen05.mma.sp.cta_group::2.kind::i8 [%0], [%1], b, [%2], %5, p;\n\t}"
         ::"r"(tmem_d), "r"(tmem_a), "r"(tmem_meta), "r"(db_lo), "r"(db_hi), "r"(idesc), "r"(accumulate) : "memory");
 }
+// D[256 x N] (+)= A[256 x 64] * B[N x 64]^T on 4-bit operands (mma_mxf4_ts above on a pair); A and the scales in the tensor
+// memory of both CTAs.
+__device__ __forceinline__ void mma_mxf4_ts_pair(uint32_t tmem_d, uint32_t tmem_a, uint32_t db_lo, uint32_t db_hi, uint32_t idesc,
+                                                 uint32_t sfa, uint32_t sfb, uint32_t accumulate) {
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t.reg .b64 b;\n\tsetp.ne.b32 p, %5, 0;\n\tmov.b64 b, {%2, %3};\n\t"
+        "tcgen05.mma.cta_group::2.kind::mxf4.block_scale.block32 [%0], [%1], b, %4, [%6], [%7], p;\n\t}"
+        ::"r"(tmem_d), "r"(tmem_a), "r"(db_lo), "r"(db_hi), "r"(idesc), "r"(accumulate), "r"(sfa), "r"(sfb) : "memory");
+}
 // Arrive on the barrier at this offset in BOTH CTAs once every MMA issued so far by this thread has completed.
 __device__ __forceinline__ void mma_commit_pair(uint32_t bar) {
     asm volatile("tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;"

@@ -19,22 +19,26 @@
 // w holds, in nibble i, bit 4i + t of w:   ((w << (3 - t)) & 0x88888888) ^ 0xAAAAAAAA
 // (sign bit = NOT the input bit, exponent field = 01).
 //
-// Roles in a CTA of 27 warps (persistent, one CTA per SM, tiles of 128 frames x 192 units):
-//   warp 26      one thread issues 2-D TMA tile loads of the packed rows (64 bytes per row =
+// A pair of CTAs (cluster of two, one per SM of a TPC) works on a tile of 256 frames x two parts of 128 units: each CTA widens
+// its own 128 frames and half of the units, where a CTA by itself would widen all of them.  Roles in a CTA of 28 warps
+// (persistent, one CTA per SM):
+//   warp 27      one thread issues 2-D TMA tile loads of the packed rows (64 bytes per row =
 //                two stages) into a staging ring (64-byte swizzle, no multicast)
-//   warps 6-13   two teams widen the frame rows, thread = one row, 32 bytes -> 128 bytes per stage,
+//   warps 10-17  two teams widen the frame rows, thread = one row, 32 bytes -> 128 bytes per stage,
 //                written to tensor memory (the MMA reads its A operand from there); they take alternate stages
-//   warps 14-25  two teams widen the unit rows the same way into shared memory, two stages per iteration
-//   warps 4, 5   issue the MMAs (4 per stage, K = 64 each) and the commits; the two warps take the stages in turn
-//   warps 0-3    epilogue: accumulator -> Sign/threshold -> repacked bits (or int32 output);
-//                two accumulators in tensor memory, so it overlaps the next tile's MMAs
-// Every wait is bounded; a wait that runs out sets the CTA's abort flag, all roles fall
+//   warps 18-25  two teams widen the unit rows the same way into shared memory
+//   warps 8, 9   rank 0: issue the MMAs (4 per stage and part, K = 64 each) and the commits, which arrive in both CTAs; a warp has a part
+//                with its accumulator.  The epilogue reads one accumulator after the other, so one part runs ahead (by
+//                up to the ring's six stages) and its epilogue is hidden behind the other's MMAs.
+//   warps 0-7    epilogue: accumulator -> Sign/threshold -> repacked bits (or int32 output), two warps per tensor-memory lane quarter
+// A stage of both operands is one barrier of rank 0, on which the widening warps of both CTAs arrive.
+// Every wait is bounded; a wait that runs out sets the CTA's abort flag, all roles of both CTAs fall
 // through to the common teardown and the device status word is set.
 //
-// What bounds it, measured on B200: the widening (two teams per operand; a stage takes about 720 clocks against 384
-// of MMA; with one team per operand, one issuing thread and the int32 tile written out by the epilogue warps it took
-// about 1000).  65536 x 4096 x 4096, int32 out, 647 -> 472 us; 4096 x 2048 x 4096 31 -> 23 us (its tiles have 8
-// stages, so the int32 epilogue counts there).
+// What bounds it, measured on B200: the widening (about 600 clocks per stage of 256 x 256 outputs against 512 of MMA).  A CTA that
+// widened 128 frames and 192 units by itself took 720 clocks per stage of 128 x 192 outputs (384 of MMA).  65536 x 4096 x 4096, int32 out,
+// 483 -> 394 us; 4096 x 2048 x 4096 24.0 -> 22.2 us (its tiles have 8 stages, so the int32 epilogue counts there, and 256
+// tiles are 3.5 turns of 74 pairs).
 #include "bnn_common.cuh"
 #include "tcgen05.cuh"
 #include "xnor_widen.cuh"
@@ -45,24 +49,21 @@ namespace {
 
 using namespace tc;
 
-constexpr int BM = 128, BN = 192;
+constexpr int BM = 128;                                   // frames per CTA
+constexpr int PARTS = 2, PN = 128, BN = PARTS * PN;       // units per part and tile
+constexpr int BR = BN / 2;                                // unit rows per CTA: half of each part
 constexpr int BK = 256;                                   // bits of K per stage = nibbles per widened row
 constexpr int ROW_BYTES = BK / 2;                         // widened bytes per row and stage (128)
-constexpr int B_BYTES = BN * ROW_BYTES, STAGE_BYTES = B_BYTES;   // only the unit operand lives in shared memory
-constexpr int A_STAGES = 3, B_STAGES = 4;               // rings of the frame operand (tensor memory) and the unit operand
-// A stage `it` of the CTA's sequence has barrier it % A_BARS, an even number, so that a barrier always belongs to the same
-// team and issuing warp (a wait on a parity holds only for one who has seen every phase before it).
-constexpr int A_BARS = 2 * A_STAGES;
-static_assert(B_STAGES % 2 == 0, "a stage of units always belongs to the same issuing warp");
-constexpr int EPI_WARPS = 4, MMA_WARP = 4, MMA_WARP2 = 5, PROD_WARP0 = 6, TEAMS = 2, A_WARPS = BM / 32, B_WARPS = BN / 32;
-constexpr int PROD_WARPS = TEAMS * (A_WARPS + B_WARPS);
-constexpr int TMA_WARP = PROD_WARP0 + PROD_WARPS;
-constexpr int THREADS = (TMA_WARP + 1) * 32;              // 864
-constexpr int GROUPS = 4;                                 // staging ring: groups of two stages (an odd last stage has an empty partner)
-constexpr int GA_BYTES = BM * 64, GB_BYTES = BN * 64, GROUP_BYTES = GA_BYTES + GB_BYTES;
-constexpr uint32_t TMEM_A_COL = 2 * BN;                   // A stages start after the two accumulators
+constexpr int PART_BYTES = PN / 2 * ROW_BYTES, STAGE_BYTES = PARTS * PART_BYTES;   // only the unit operand lives in shared memory
+constexpr int STAGES = 6;                                 // even: a stage always belongs to the same team of producers
+constexpr int EPI_WARPS = 8, MMA_WARP = 8, PROD_WARP0 = 10, TEAMS = 2, A_WARPS = BM / 32, B_WARPS = BR / 32;
+constexpr int TMA_WARP = PROD_WARP0 + TEAMS * (A_WARPS + B_WARPS);
+constexpr int THREADS = (TMA_WARP + 1) * 32;
+constexpr int GROUPS = 3;                                 // staging ring: groups of two stages (an odd last stage has an empty partner)
+constexpr int GA_BYTES = BM * 64, GB_BYTES = BR * 64, GROUP_BYTES = GA_BYTES + GB_BYTES;
+constexpr uint32_t TMEM_A_COL = BN;                       // A stages start after the two accumulators
 constexpr uint32_t A_COLS = ROW_BYTES / 4;                // 32-bit columns per A stage
-constexpr uint32_t TMEM_SF_COL = TMEM_A_COL + A_STAGES * A_COLS, SF_COLS = 32;   // block scales: 16 columns per operand
+constexpr uint32_t TMEM_SF_COL = TMEM_A_COL + STAGES * A_COLS, SF_COLS = 32;   // block scales: 16 columns per operand
 constexpr uint32_t TMEM_COLS = 512;
 
 // With int32 output each epilogue warp needs two staging blocks of 32 rows x 128 bytes (1024-byte aligned).
@@ -71,15 +72,14 @@ template <bool STORE_C> struct Cfg {
 };
 
 struct Control {
-    int T[BN];               // per unit: threshold + kMagicBits (Sign epilogue only)
-    uint32_t flipw[BN / 32];
-    uint64_t full_a[A_BARS], empty_a[A_BARS], full_b[B_STAGES], empty_b[B_STAGES], acc_full[2], acc_empty[2], started[2];
+    int T[EPI_WARPS][PN / 2];        // per epilogue warp: threshold + kMagicBits of its units (Sign epilogue only)
+    uint64_t full[STAGES], empty[STAGES], acc_full[PARTS], acc_empty[PARTS];
     uint64_t group_full[GROUPS], group_empty[GROUPS];
     uint32_t tmem_base;
     WaitState wait;
 };
 template <bool STORE_C> constexpr int smem_bytes() {
-    return B_STAGES * STAGE_BYTES + GROUPS * GROUP_BYTES + (int)sizeof(Control) + Cfg<STORE_C>::CSTAGE_BYTES + 1024;
+    return STAGES * STAGE_BYTES + GROUPS * GROUP_BYTES + (int)sizeof(Control) + Cfg<STORE_C>::CSTAGE_BYTES + 1024;
 }
 static_assert(smem_bytes<false>() <= 232448 && smem_bytes<true>() <= 232448, "shared memory of one CTA");
 static_assert(TMEM_SF_COL + SF_COLS <= TMEM_COLS, "tensor memory columns");
@@ -89,24 +89,19 @@ struct ProducerArgs {
     uint32_t tmem;        // base of the tensor-memory allocation
     Control* ctl;
     volatile int* abort_flag;
-    int tiles, nks, kw;
+    int total;            // stages of all tiles of this pair
+    int nks, kw;
     uint32_t tmask;
-    int lane;
+    int rank, lane;
 };
 
 // The eight 16-byte chunks of one widened row and stage; `ks` is the stage's index in the row.
-// ZO: the row's bits stand for (0,1) instead of (-1,+1); RAGGED: the last stage has positions >= K.
+// ZO: the row's bits stand for (0,1) instead of (-1,+1); RAGGED: the last stage has positions >= K, whose nibbles are set to +0 (in the
+// unit rows; what the frame rows hold there then does not matter).
 template <bool ZO, bool RAGGED>
 __device__ __forceinline__ void widen_stage(const ProducerArgs& a, int ks, const uint4& v0, const uint4& v1, uint4 (&o)[8]) {
     const uint32_t w[8] = {v0.x, v0.y, v0.z, v0.w, v1.x, v1.y, v1.z, v1.w};
-    if (ZO) {
-#pragma unroll
-        for (int c = 0; c < 8; ++c) {
-            const int g = 8 * ks + c;   // index of the word in the row
-            const uint32_t valid = (!RAGGED || g < a.kw - 1) ? 0xFFFFFFFFu : (g == a.kw - 1 ? a.tmask : 0u);
-            o[c] = widen01_masked(w[c], valid);
-        }
-    } else if (RAGGED && ks == a.nks - 1) {
+    if (RAGGED && ks == a.nks - 1) {
 #pragma unroll
         for (int c = 0; c < 8; ++c) {
             const int g = 8 * ks + c;   // index of the word in the row
@@ -115,47 +110,54 @@ __device__ __forceinline__ void widen_stage(const ProducerArgs& a, int ks, const
         }
     } else {
 #pragma unroll
-        for (int c = 0; c < 8; ++c) o[c] = widen(w[c]);
+        for (int c = 0; c < 8; ++c) o[c] = ZO ? widen01(w[c]) : widen(w[c]);
     }
 }
 
-// Producer of the frame operand: thread = row `r` of every tile of this CTA; team `team` takes one of the two stages of every
-// group, widened rows written to tensor memory.
+// Producer of an operand: thread = row `r` of every tile of this CTA's half; team `team` takes one of the two stages of every
+// staging group.  FRAMES: widened rows go to tensor memory, else (unit rows) to shared memory.
 // Template arguments say what the loops of the producers have to deal with: code that is there for another case costs this
 // one, though it is not executed.
-template <bool ZO, bool RAGGED>
-__device__ __forceinline__ void produce_a(const ProducerArgs& a, int r, int team) {
+template <bool FRAMES, bool ZO, bool RAGGED>
+__device__ __forceinline__ void produce(const ProducerArgs& a, int r, int team) {
     Control* ctl = a.ctl;
-    const int my_tiles = (a.tiles - 1 - (int)blockIdx.x) / (int)gridDim.x + 1;
-    const int ng = ceil_div(a.nks, 2), total = 2 * my_tiles * ng;
     // TMEM lane of this thread's frame row: a warp may only touch lanes 32*(warp%4)..+31
     const uint32_t tdst0 = a.tmem + ((uint32_t)(r & ~31) << 16) + TMEM_A_COL;
+    // rows of a part in shared memory: K-major core matrices, chunk c of 16 bytes PN / 2 rows apart
+    const uint32_t bdst0 = a.smem + (r / (PN / 2)) * PART_BYTES + (r % (PN / 2)) * 16;
     // this row inside a staging group: 64 bytes per row, 16-byte chunk c stored at c ^ ((r/2)%4)
     const uint32_t sw = (uint32_t)(r >> 1) & 3u;
-    const uint32_t stg0 = a.smem + B_STAGES * STAGE_BYTES + r * 64 + (((2u * team) ^ (sw & 2u)) << 4);
+    const uint32_t stg0 = a.smem + STAGES * STAGE_BYTES + (FRAMES ? 0 : GA_BYTES) + r * 64 + (((2u * team) ^ (sw & 2u)) << 4);
     const uint32_t lo = (sw & 1u) << 4;
-    int ks = team;
-    for (int it = team; it < total; it += TEAMS) {
-        const int g = it >> 1, gslot = g % GROUPS;
-        if (!warp_wait(smem_u32(&ctl->group_full[gslot]), (uint32_t)((g / GROUPS) & 1), a.abort_flag, a.lane)) break;
+    const uint32_t full0 = a.rank == 0 ? smem_u32(&ctl->full[0]) : peer_addr(smem_u32(&ctl->full[0]), 0);
+    int ks = team, gslot = 0, s = team;
+    uint32_t gph = 0, ph = 1;                  // parities to wait for (a fresh barrier passes 1)
+    for (int it = team; it < a.total; it += TEAMS) {
+        if (!warp_wait(smem_u32(&ctl->group_full[gslot]), gph, a.abort_flag, a.lane)) return;
         const uint32_t src = stg0 + gslot * GROUP_BYTES;
         const uint4 v0 = lds128u(src + lo), v1 = lds128u(src + (lo ^ 16u));
-        const int s = it % A_STAGES;
-        const int e = it + A_BARS - A_STAGES;          // the stage that had this slot; a fresh barrier passes parity 1
-        if (!warp_wait(smem_u32(&ctl->empty_a[e % A_BARS]), (uint32_t)(((e / A_BARS) & 1) ^ 1), a.abort_flag, a.lane)) break;
         uint4 o[8];
         widen_stage<ZO, RAGGED>(a, ks, v0, v1, o);
-        // 32-bit column 4c + t of the stage = word t of chunk c: the byte order of the
-        // K-major shared-memory layout of the other operand
-        uint32_t wr[32];
+        if (!warp_wait(smem_u32(&ctl->empty[s]), ph, a.abort_flag, a.lane)) return;
+        if (FRAMES) {
+            // 32-bit column 4c + t of the stage = word t of chunk c: the byte order of the
+            // K-major shared-memory layout of the other operand
+            uint32_t wr[32];
 #pragma unroll
-        for (int c = 0; c < 8; ++c) { wr[4 * c] = o[c].x; wr[4 * c + 1] = o[c].y; wr[4 * c + 2] = o[c].z; wr[4 * c + 3] = o[c].w; }
-        tmem_st32(tdst0 + s * A_COLS, wr);
-        tmem_st_wait();
-        tc_fence_before_sync();
+            for (int c = 0; c < 8; ++c) { wr[4 * c] = o[c].x; wr[4 * c + 1] = o[c].y; wr[4 * c + 2] = o[c].z; wr[4 * c + 3] = o[c].w; }
+            tmem_st32(tdst0 + s * A_COLS, wr);
+            tmem_st_wait();
+            tc_fence_before_sync();
+        } else {
+            const uint32_t dst = bdst0 + s * STAGE_BYTES;
+#pragma unroll
+            for (int c = 0; c < 8; ++c) sts128(dst + c * (PN / 2 * 16), o[c].x, o[c].y, o[c].z, o[c].w);
+            fence_proxy_async_smem();
+        }
         __syncwarp();
         if (a.lane == 0) {
-            mbar_arrive(smem_u32(&ctl->full_a[it % A_BARS]));
+            if (a.rank == 0) mbar_arrive(full0 + 8u * s);
+            else mbar_arrive_cluster(full0 + 8u * s);
             // The staging slot is handed back only here, after the stores that consumed the loaded
             // words: a shared-memory load that has merely been issued does not hold back the TMA
             // write that refills the slot (that write belongs to the async proxy; only the data
@@ -163,54 +165,14 @@ __device__ __forceinline__ void produce_a(const ProducerArgs& a, int r, int team
             mbar_arrive(smem_u32(&ctl->group_empty[gslot]));
         }
         ks += TEAMS;
-        if (ks >= 2 * ng) ks = team;
-    }
-}
-
-// Producer of the unit operand: thread = row `r`; the teams take the staging groups in turn, two stages per
-// iteration, so the fixed costs of an iteration (group wait, proxy fence, warp barrier, release) are paid once per
-// two stages; widened rows go to shared memory, each team to its half of the ring.
-template <bool RAGGED>
-__device__ __forceinline__ void produce_b(const ProducerArgs& a, int r, int team) {
-    Control* ctl = a.ctl;
-    const int my_tiles = (a.tiles - 1 - (int)blockIdx.x) / (int)gridDim.x + 1;
-    const int ng = ceil_div(a.nks, 2), total = my_tiles * ng;
-    const int s = 2 * team;
-    const uint32_t dst0 = a.smem + s * STAGE_BYTES + r * 16;
-    const uint32_t stg0 = a.smem + B_STAGES * STAGE_BYTES + GA_BYTES + r * 64;
-    const uint32_t sw = (uint32_t)(r >> 1) & 3u;
-    uint32_t ph = 1;
-    int kg = team;
-    for (int g = team; g < total; g += TEAMS) {
-        while (kg >= ng) kg -= ng;
-        const int gslot = g % GROUPS;
-        if (!warp_wait(smem_u32(&ctl->group_full[gslot]), (uint32_t)((g / GROUPS) & 1), a.abort_flag, a.lane)) break;
-        const uint32_t src = stg0 + gslot * GROUP_BYTES;
-        const uint4 v0 = lds128u(src + ((0u ^ sw) << 4)), v1 = lds128u(src + ((1u ^ sw) << 4));
-        const uint4 v2 = lds128u(src + ((2u ^ sw) << 4)), v3 = lds128u(src + ((3u ^ sw) << 4));
-        if (!warp_wait(smem_u32(&ctl->empty_b[s]), ph, a.abort_flag, a.lane)) break;
-        uint4 o[8];
-        widen_stage<false, RAGGED>(a, 2 * kg, v0, v1, o);
-#pragma unroll
-        for (int c = 0; c < 8; ++c) sts128(dst0 + c * (BN * 16), o[c].x, o[c].y, o[c].z, o[c].w);
-        if (!warp_wait(smem_u32(&ctl->empty_b[s + 1]), ph, a.abort_flag, a.lane)) break;
-        widen_stage<false, RAGGED>(a, 2 * kg + 1, v2, v3, o);
-#pragma unroll
-        for (int c = 0; c < 8; ++c) sts128(dst0 + STAGE_BYTES + c * (BN * 16), o[c].x, o[c].y, o[c].z, o[c].w);
-        fence_proxy_async_smem();
-        __syncwarp();
-        if (a.lane == 0) {
-            mbar_arrive(smem_u32(&ctl->full_b[s]));
-            mbar_arrive(smem_u32(&ctl->full_b[s + 1]));
-            mbar_arrive(smem_u32(&ctl->group_empty[gslot]));   // after the stores that consumed the loaded words (see produce_a)
-        }
-        ph ^= 1u;
-        kg += TEAMS;
+        if (ks >= 2 * ceil_div(a.nks, 2)) ks = team;
+        if (++gslot == GROUPS) { gslot = 0; gph ^= 1u; }
+        if ((s += TEAMS) >= STAGES) { s = team; ph ^= 1u; }
     }
 }
 
 template <bool STORE_C, bool SIGN_PACK>
-__global__ void __launch_bounds__(THREADS, 1)
+__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(THREADS, 1)
 xnor_tc_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CUtensorMap mapB,
                 const __grid_constant__ CUtensorMap mapC, int tma_c,
                 int M, int N, int K, int32_t* __restrict__ C, int ldc,
@@ -218,50 +180,43 @@ xnor_tc_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_constant__
                 uint32_t* __restrict__ out_bits, int ldob, int zo, TcStatus status) {
     extern __shared__ uint8_t smem_raw[];
     uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
-    const uint32_t cstage = smem_u32(smem) + B_STAGES * STAGE_BYTES + GROUPS * GROUP_BYTES;
-    Control* ctl = reinterpret_cast<Control*>(smem + B_STAGES * STAGE_BYTES + GROUPS * GROUP_BYTES + Cfg<STORE_C>::CSTAGE_BYTES);
+    const uint32_t cstage = smem_u32(smem) + STAGES * STAGE_BYTES + GROUPS * GROUP_BYTES;
+    Control* ctl = reinterpret_cast<Control*>(smem + STAGES * STAGE_BYTES + GROUPS * GROUP_BYTES + Cfg<STORE_C>::CSTAGE_BYTES);
     volatile int* abort_flag = &ctl->wait.abort;
 
-    const int warp = warp_index(), lane = threadIdx.x & 31;
+    const int warp = warp_index(), lane = threadIdx.x & 31, rank = (int)cluster_rank();
     const int kw = words_for(K);
     const int nks = ceil_div(K, BK);
-    const int m_tiles = ceil_div(M, BM), n_tiles = ceil_div(N, BN);
-    const int tiles = m_tiles * n_tiles;
+    const int n_tiles = ceil_div(N, BN), tiles = ceil_div(M, 2 * BM) * n_tiles;
+    const int pair = (int)blockIdx.x >> 1, pairs = (int)gridDim.x >> 1;      // tiles pair, pair + pairs, ..; unit tiles vary fastest
 
     if (threadIdx.x == 0) {
-        for (int s = 0; s < A_BARS; ++s) {
-            mbar_init(smem_u32(&ctl->full_a[s]), A_WARPS);
-            mbar_init(smem_u32(&ctl->empty_a[s]), 1);
+        for (int s = 0; s < STAGES; ++s) {
+            mbar_init(smem_u32(&ctl->full[s]), 2 * (A_WARPS + B_WARPS));     // rank 0: the widening warps of both CTAs
+            mbar_init(smem_u32(&ctl->empty[s]), PARTS);                      // a commit of each issuing warp
         }
-        for (int s = 0; s < B_STAGES; ++s) {
-            mbar_init(smem_u32(&ctl->full_b[s]), B_WARPS);
-            mbar_init(smem_u32(&ctl->empty_b[s]), 1);
-        }
-        for (int b = 0; b < 2; ++b) {
-            mbar_init(smem_u32(&ctl->acc_full[b]), 2);       // one commit of each issuing warp
-            mbar_init(smem_u32(&ctl->started[b]), 1);
-            mbar_init(smem_u32(&ctl->acc_empty[b]), EPI_WARPS);
+        for (int b = 0; b < PARTS; ++b) {
+            mbar_init(smem_u32(&ctl->acc_full[b]), 1);
+            mbar_init(smem_u32(&ctl->acc_empty[b]), 2 * EPI_WARPS);          // rank 0: the epilogue warps of both CTAs
         }
         for (int b = 0; b < GROUPS; ++b) {
             mbar_init(smem_u32(&ctl->group_full[b]), 1);            // the issuing thread (+ bytes)
-            mbar_init(smem_u32(&ctl->group_empty[b]), TEAMS * A_WARPS + B_WARPS);  // every warp that reads it
+            mbar_init(smem_u32(&ctl->group_empty[b]), TEAMS * (A_WARPS + B_WARPS));  // every warp that reads it
         }
         wait_state_init(&ctl->wait, status);
         mbar_init_fence();
     }
-    if (warp == MMA_WARP) {
-        tmem_alloc(smem_u32(&ctl->tmem_base), TMEM_COLS);
-        tmem_relinquish();
-    }
+    __syncwarp();
+    if (warp == MMA_WARP) tmem_alloc_pair(smem_u32(&ctl->tmem_base), TMEM_COLS);
     tc_fence_before_sync();
-    __syncthreads();
+    cluster_sync();           // barriers of both CTAs initialised, tensor memory of both allocated
     tc_fence_after_sync();
     const uint32_t tmem = ctl->tmem_base;
     pdl_trigger();
     // The set-up above overlaps the end of the kernel before this one (products of one size in a row, us: 4096 x 2048 x 4096
     // 26.5 -> 23.7, 700 x 1024 x 1024 9.7 -> 7.2).
     pdl_wait();
-    if (warp < EPI_WARPS) {
+    if (warp < 4) {
         // Block scales of both operands: every byte 127, the ue8m0 code of 2^0.  The whole
         // region is filled, so the values do not depend on how the scales are laid out in it.
         uint32_t ones[32];
@@ -271,208 +226,189 @@ xnor_tc_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_constant__
         tmem_st_wait();
     }
     tc_fence_before_sync();
-    __syncthreads();
+    cluster_sync();
     tc_fence_after_sync();
 
     if (warp >= PROD_WARP0) {
-        ProducerArgs pa{smem_u32(smem), tmem, ctl, abort_flag, tiles, nks, kw, tail_mask(K), lane};
+        const int my_tiles = pair < tiles ? (tiles - 1 - pair) / pairs + 1 : 0;
+        const ProducerArgs pa{smem_u32(smem), tmem, ctl, abort_flag, my_tiles * 2 * ceil_div(nks, 2), nks, kw, tail_mask(K), rank, lane};
         const bool ragged = (kw % 8 != 0) || pa.tmask != 0xFFFFFFFFu;   // the last stage has positions >= K
         if (warp == TMA_WARP) {
             // ---------------- one thread feeds the staging ring, a group of two stages at a time
             if (lane == 0) {
-                const uint32_t stg = smem_u32(smem) + B_STAGES * STAGE_BYTES;
+                const uint32_t stg = smem_u32(smem) + STAGES * STAGE_BYTES;
                 const int ng = ceil_div(nks, 2);
-                int gc = 0;
+                int slot = 0;
+                uint32_t ph = 1;
                 bool ok = true;
-                for (int tile = blockIdx.x; tile < tiles && ok; tile += gridDim.x) {
-                    const int n0 = (tile % n_tiles) * BN, m0 = (tile / n_tiles) * BM;   // unit tiles vary fastest
-                    for (int g = 0; g < ng; ++g, ++gc) {
-                        const int slot = gc % GROUPS;
-                        if (gc >= GROUPS) {
-                            ok = mbar_wait_relaxed(smem_u32(&ctl->group_empty[slot]), (uint32_t)(((gc / GROUPS) - 1) & 1), abort_flag);
-                            if (!ok) break;
-                        }
-                        const uint32_t bar = smem_u32(&ctl->group_full[slot]);
+                for (int tile = pair; tile < tiles && ok; tile += pairs) {
+                    const int n0 = (tile % n_tiles) * BN + rank * (PN / 2), m0 = (tile / n_tiles) * (2 * BM) + rank * BM;
+                    for (int g = 0; g < ng; ++g) {
+                        ok = mbar_wait_relaxed(smem_u32(&ctl->group_empty[slot]), ph, abort_flag);
+                        if (!ok) break;
+                        const uint32_t bar = smem_u32(&ctl->group_full[slot]), dst = stg + slot * GROUP_BYTES;
                         mbar_arrive_expect_tx(bar, GROUP_BYTES);
-                        tma_load_2d(stg + slot * GROUP_BYTES, &mapA, g * 16, m0, bar);
-                        tma_load_2d(stg + slot * GROUP_BYTES + GA_BYTES, &mapB, g * 16, n0, bar);
+                        tma_load_2d(dst, &mapA, g * 16, m0, bar);
+                        tma_load_2d(dst + GA_BYTES, &mapB, g * 16, n0, bar);
+                        tma_load_2d(dst + GA_BYTES + GB_BYTES / 2, &mapB, g * 16, n0 + PN, bar);
+                        if (++slot == GROUPS) { slot = 0; ph ^= 1u; }
                     }
                 }
             }
             __syncwarp();
         } else if (warp < PROD_WARP0 + TEAMS * A_WARPS) {
             const int row = (warp & 3) * 32 + lane, team = (warp - PROD_WARP0) / A_WARPS;
-            if (zo) ragged ? produce_a<true, true>(pa, row, team) : produce_a<true, false>(pa, row, team);
-            else ragged ? produce_a<false, true>(pa, row, team) : produce_a<false, false>(pa, row, team);
+            if (zo) produce<true, true, false>(pa, row, team);
+            else produce<true, false, false>(pa, row, team);
         } else {
             const int pw = warp - PROD_WARP0 - TEAMS * A_WARPS, team = pw / B_WARPS, row = (pw - team * B_WARPS) * 32 + lane;
-            ragged ? produce_b<true>(pa, row, team) : produce_b<false>(pa, row, team);
+            ragged ? produce<false, false, true>(pa, row, team) : produce<false, false, false>(pa, row, team);
         }
-    } else if (warp == MMA_WARP || warp == MMA_WARP2) {
-        // ---------------- MMA issue: two converged warps, which take the CTA's stages in turn and accumulate into the
-        // same accumulator (the sums are exact integers, so their order does not matter; only the stage that
-        // overwrites the accumulator has to come first, see `started`).  What an issuing warp does besides its
-        // MMAs (waits, commits) is time the tensor pipe idles unless the other warp fills it.
-        const int w = warp - MMA_WARP;
-        constexpr uint32_t idesc = instr_desc_mxf4(BM, BN);
+    } else if (warp >= EPI_WARPS) {
+        // ---------------- MMA issue: two converged warps of rank 0, each with its part of every tile.  What an issuing warp does
+        // besides its MMAs (waits, commits) is time the tensor pipe idles unless the other warp fills it.
+        const int part = warp - MMA_WARP;
+        constexpr uint32_t idesc = instr_desc_mxf4(2 * BM, PN);
         const uint32_t sfa = tmem + TMEM_SF_COL, sfb = tmem + TMEM_SF_COL + SF_COLS / 2;
-        const uint64_t desc = smem_desc_kmajor(smem_u32(smem), BN * 16, 128);
+        const uint64_t desc = smem_desc_kmajor(smem_u32(smem) + part * PART_BYTES, PN / 2 * 16, 128);
         const uint32_t desc_lo = (uint32_t)desc, desc_hi = (uint32_t)(desc >> 32);
-        constexpr uint32_t kStepJ = (2 * BN * 16) >> 4, kStepS = STAGE_BYTES >> 4;
-        int sa = w, ba = w, sb = w;     // this warp's next stage: slot of the A ring, its barrier, slot of the B ring
-        uint32_t pa = 0, pb = 0;        // ... and the parities the `full` barriers show next
-        int tl = 0;
-        bool ok = true;
-        for (int tile = blockIdx.x; tile < tiles && ok; tile += gridDim.x, ++tl) {
-            const int b = tl & 1;
-            ok = warp_wait(smem_u32(&ctl->acc_empty[b]), (uint32_t)(((tl >> 1) & 1) ^ 1), abort_flag, lane);
+        constexpr uint32_t kStepJ = (2 * (PN / 2) * 16) >> 4, kStepS = STAGE_BYTES >> 4;
+        const uint32_t d = tmem + (uint32_t)(part * PN);
+        int s = 0;
+        uint32_t ph = 0, pacc = 1;
+        bool ok = rank == 0;
+        for (int tile = pair; tile < tiles && ok; tile += pairs) {
+            ok = warp_wait(smem_u32(&ctl->acc_empty[part]), pacc, abort_flag, lane);
             if (!ok) break;
+            pacc ^= 1u;
             tc_fence_after_sync();
-            const uint32_t d = tmem + (uint32_t)(b * BN);
-            for (int ks = w; ks < 2 * ceil_div(nks, 2); ks += 2) {
-                ok = warp_wait(smem_u32(&ctl->full_b[sb]), pb, abort_flag, lane) && warp_wait(smem_u32(&ctl->full_a[ba]), pa, abort_flag, lane) &&
-                     (ks != 1 || warp_wait(smem_u32(&ctl->started[b]), (uint32_t)((tl >> 1) & 1), abort_flag, lane));
+            const bool beyond = (tile % n_tiles) * BN + part * PN >= N;      // no such units: nothing to multiply
+            for (int ks = 0; ks < 2 * ceil_div(nks, 2); ++ks) {
+                ok = warp_wait(smem_u32(&ctl->full[s]), ph, abort_flag, lane);
                 if (!ok) break;
                 tc_fence_after_sync();
                 // the address field (16-byte units) is advanced by plain additions: the ring lies below 2^14 * 16
                 // bytes.  An MMA takes 64 positions of K = 32 bytes: 8 columns of A, two 16-byte chunks of B
-                const uint32_t db = desc_lo + (uint32_t)sb * kStepS;
-                const uint32_t ta = tmem + TMEM_A_COL + sa * A_COLS;
-                if (ks == nks) {        // the empty partner of an odd last stage
-                    if (elect_one()) {
-                        mma_commit(smem_u32(&ctl->empty_a[ba]));
-                        mma_commit(smem_u32(&ctl->empty_b[sb]));
+                const uint32_t db = desc_lo + (uint32_t)s * kStepS;
+                const uint32_t ta = tmem + TMEM_A_COL + s * A_COLS;
+                if (elect_one()) {
+                    if (ks < nks && !beyond) {        // (not the empty partner of an odd last stage)
+                        mma_mxf4_ts_pair(d, ta, db, desc_hi, idesc, sfa, sfb, ks != 0);
+                        mma_mxf4_ts_pair(d, ta + 8, db + kStepJ, desc_hi, idesc, sfa, sfb, 1u);
+                        mma_mxf4_ts_pair(d, ta + 16, db + 2 * kStepJ, desc_hi, idesc, sfa, sfb, 1u);
+                        mma_mxf4_ts_pair(d, ta + 24, db + 3 * kStepJ, desc_hi, idesc, sfa, sfb, 1u);
                     }
-                } else if (elect_one()) {
-                    mma_mxf4_ts(d, ta, db, desc_hi, idesc, sfa, sfb, ks != 0);
-                    if (ks == 0) mma_commit(smem_u32(&ctl->started[b]));
-                    mma_mxf4_ts(d, ta + 8, db + kStepJ, desc_hi, idesc, sfa, sfb, 1u);
-                    mma_mxf4_ts(d, ta + 16, db + 2 * kStepJ, desc_hi, idesc, sfa, sfb, 1u);
-                    mma_mxf4_ts(d, ta + 24, db + 3 * kStepJ, desc_hi, idesc, sfa, sfb, 1u);
-                    mma_commit(smem_u32(&ctl->empty_a[ba]));
-                    mma_commit(smem_u32(&ctl->empty_b[sb]));
+                    mma_commit_pair(smem_u32(&ctl->empty[s]));
                 }
-                if ((sa += 2) >= A_STAGES) sa -= A_STAGES;
-                if ((ba += 2) >= A_BARS) { ba -= A_BARS; pa ^= 1u; }
-                if ((sb += 2) >= B_STAGES) { sb -= B_STAGES; pb ^= 1u; }
+                if (++s == STAGES) { s = 0; ph ^= 1u; }
             }
-            if (ok && elect_one()) mma_commit(smem_u32(&ctl->acc_full[b]));
+            if (ok && elect_one()) mma_commit_pair(smem_u32(&ctl->acc_full[part]));
         }
         __syncwarp();
     } else {
-        // ---------------- epilogue: 128 threads, thread = one frame (TMEM lane)
-        const int row_in_tile = warp * 32 + lane;
+        // ---------------- epilogue: thread = one frame (TMEM lane); of a part's units warps 0-3 take the first half, warps 4-7 the second
+        const int half = warp >> 2, quarter = warp & 3;
         const float magic = __int_as_float(kMagicBits);
-        int tl = 0;
+        uint32_t par = 0;
         bool ok = true;
-        for (int tile = blockIdx.x; tile < tiles && ok; tile += gridDim.x, ++tl) {
-            const int n0 = (tile % n_tiles) * BN, m0 = (tile / n_tiles) * BM;   // unit tiles vary fastest
-            const int m = m0 + row_in_tile;
-            if (SIGN_PACK) {
-                epi_bar_sync();  // previous tile's readers of T are done
+        for (int tile = pair; tile < tiles && ok; tile += pairs, par ^= 1u) {
+            const int m0 = (tile / n_tiles) * (2 * BM) + rank * BM + quarter * 32, m = m0 + lane;
+            for (int part = 0; part < PARTS; ++part) {
+                const int n0 = (tile % n_tiles) * BN + part * PN + half * (PN / 2);       // the first of this warp's 64 units
+                if (SIGN_PACK) {
 #pragma unroll
-                for (int h = 0; h < 2; ++h) {
-                    const int nl = row_in_tile + h * 128, n = n0 + nl;
-                    if (nl < BN) ctl->T[nl] = kMagicBits + (n < N ? thr[n] : 0);
-                }
-                if (row_in_tile < BN / 32) {
-                    const int wi = (n0 >> 5) + row_in_tile;
-                    ctl->flipw[row_in_tile] = wi < words_for(N) ? flip[wi] : 0u;
-                }
-                epi_bar_sync();
-            }
-            const int b = tl & 1;
-            // all four epilogue warps take the same decision, so none is left at a barrier
-            ok = epi_all(warp_wait_relaxed(smem_u32(&ctl->acc_full[b]), (uint32_t)((tl >> 1) & 1), abort_flag, lane));
-            if (!ok) break;
-            tc_fence_after_sync();
-            const uint32_t taddr = tmem + ((uint32_t)(warp * 32) << 16) + (uint32_t)(b * BN);
-            uint32_t words[BN / 32];
-#pragma unroll
-            for (int g = 0; g < BN / 32; ++g) {
-                uint32_t acc[32];
-                tmem_ld32(taddr + g * 32, acc);
-                tmem_ld_wait();
-                if (g + 1 == BN / 32) {
-                    // the accumulator is read: the MMA warps may start the tile after the next on it
-                    tc_fence_before_sync();
+                    for (int h = 0; h < PN / 64; ++h) ctl->T[warp][h * 32 + lane] = kMagicBits + (n0 + h * 32 + lane < N ? thr[n0 + h * 32 + lane] : 0);
                     __syncwarp();
-                    if (lane == 0) mbar_arrive(smem_u32(&ctl->acc_empty[b]));
                 }
-                const int nb = n0 + g * 32;
-                // The accumulator holds the integer dot product as a float; adding 1.5 * 2^23
-                // leaves that integer, offset by kMagicBits, in the bit pattern of the sum.
-                int q[32];
+                ok = warp_wait_relaxed(smem_u32(&ctl->acc_full[part]), par, abort_flag, lane);
+                if (!ok) break;
+                tc_fence_after_sync();
+                const uint32_t taddr = tmem + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(part * PN + half * (PN / 2));
+                uint32_t words[PN / 64];
 #pragma unroll
-                for (int j = 0; j < 32; ++j) q[j] = __float_as_int(__uint_as_float(acc[j]) + magic);
-                if (STORE_C) {
-                    // Each thread parks its 32 integers (128 bytes of one output row) in shared memory, 16-byte
-                    // chunk i at i ^ (row % 8).  One thread then has the 32 x 128-byte block stored, which goes on while
-                    // the warp turns to the next 32 columns.  (Measured on B200: written by the warp with 16-byte stores,
-                    // 8 lanes to a row, the epilogue took as long as 16 stages of MMAs.)
-                    // A tile store clips a row to 16 bytes, not to elements, and wants an aligned pitch.  Elsewhere the
-                    // warp writes the block a row at a time, and each row from the 32-byte sector its first
-                    // column lies in (from the block before) to the one of its last column, which is left to the next
-                    // block: every store but those at the tile's edges then covers whole sectors.  (4096 x 2048 x
-                    // 4095, microseconds: a thread a row 102, rows of 32 columns 68, whole sectors 57; 4096 columns 29.)
-                    const bool whole = tma_c && (nb + 31 < N || N % 4 == 0);
-                    const uint32_t blk = cstage + (uint32_t)((warp * 2 + (g & 1)) * 4096);
-                    if (lane == 0) bulk_wait_read<1>();      // the block's store of two rounds ago has read it
-                    __syncwarp();
+                for (int g = 0; g < PN / 64; ++g) {
+                    uint32_t acc[32];
+                    tmem_ld32(taddr + g * 32, acc);
+                    tmem_ld_wait();
+                    if (g + 1 == PN / 64) {
+                        // the accumulator is read: the part's next tile may start on it
+                        tc_fence_before_sync();
+                        __syncwarp();
+                        if (lane == 0) mbar_arrive_cluster(peer_addr(smem_u32(&ctl->acc_empty[part]), 0));
+                    }
+                    const int nb = n0 + g * 32;
+                    // The accumulator holds the integer dot product as a float; adding 1.5 * 2^23
+                    // leaves that integer, offset by kMagicBits, in the bit pattern of the sum.
+                    int q[32];
 #pragma unroll
-                    for (int i = 0; i < 8; ++i)
-                        sts128(blk + lane * 128 + ((i ^ (lane & 7)) << 4), (uint32_t)(q[4 * i] - kMagicBits), (uint32_t)(q[4 * i + 1] - kMagicBits),
-                               (uint32_t)(q[4 * i + 2] - kMagicBits), (uint32_t)(q[4 * i + 3] - kMagicBits));
-                    if (whole) fence_proxy_async_smem();
-                    __syncwarp();
-                    if (whole) {
-                        if (lane == 0 && nb < N && m0 + warp * 32 < M) tma_store_2d(&mapC, nb, m0 + warp * 32, blk);
-                    } else if (nb < N) {
-                        const int rows = M - (m0 + warp * 32) < 32 ? M - (m0 + warp * 32) : 32;
-                        const bool tail = g + 1 == BN / 32 || nb + 32 >= N;     // the last block of the tile's row
-                        int32_t* dst = C + (size_t)(m0 + warp * 32) * ldc + nb;
-                        uint32_t at = (uint32_t)(reinterpret_cast<uintptr_t>(dst) >> 2);   // in words; its low bits count
-                        const uint32_t both = cstage + (uint32_t)(warp * 8192);
+                    for (int j = 0; j < 32; ++j) q[j] = __float_as_int(__uint_as_float(acc[j]) + magic);
+                    if (STORE_C) {
+                        // Each thread parks its 32 integers (128 bytes of one output row) in shared memory, 16-byte
+                        // chunk i at i ^ (row % 8).  One thread then has the 32 x 128-byte block stored, which goes on while
+                        // the warp turns to the next 32 columns.  (Measured on B200: written by the warp with 16-byte stores,
+                        // 8 lanes to a row, the epilogue took as long as 16 stages of MMAs.)
+                        // A tile store clips a row to 16 bytes, not to elements, and wants an aligned pitch.  Elsewhere the
+                        // warp writes the block a row at a time, and each row from the 32-byte sector its first
+                        // column lies in (from the block before) to the one of its last column, which is left to the next
+                        // block: every store but those at the tile's edges then covers whole sectors.  (4096 x 2048 x
+                        // 4095, microseconds: a thread a row 102, rows of 32 columns 68, whole sectors 57; 4096 columns 29.)
+                        const bool whole = tma_c && (nb + 31 < N || N % 4 == 0);
+                        const uint32_t blk = cstage + (uint32_t)((warp * 2 + (g & 1)) * 4096);
+                        if (lane == 0) bulk_wait_read<1>();      // the block's store of two rounds ago has read it
+                        __syncwarp();
+#pragma unroll
+                        for (int i = 0; i < 8; ++i)
+                            sts128(blk + lane * 128 + ((i ^ (lane & 7)) << 4), (uint32_t)(q[4 * i] - kMagicBits), (uint32_t)(q[4 * i + 1] - kMagicBits),
+                                   (uint32_t)(q[4 * i + 2] - kMagicBits), (uint32_t)(q[4 * i + 3] - kMagicBits));
+                        if (whole) fence_proxy_async_smem();
+                        __syncwarp();
+                        if (whole) {
+                            if (lane == 0 && nb < N && m0 < M) tma_store_2d(&mapC, nb, m0, blk);
+                        } else if (nb < N) {
+                            const int rows = M - m0 < 32 ? M - m0 : 32;
+                            const bool tail = g + 1 == PN / 64 || nb + 32 >= N;     // the last block of this warp's row
+                            int32_t* dst = C + (size_t)m0 * ldc + nb;
+                            uint32_t at = (uint32_t)(reinterpret_cast<uintptr_t>(dst) >> 2);   // in words; its low bits count
+                            const uint32_t both = cstage + (uint32_t)(warp * 8192);
 #pragma unroll 4
-                        for (int r = 0; r < rows; ++r, dst += ldc, at += (uint32_t)ldc) {
-                            const int back = g == 0 ? 0 : (int)(at & 7u);       // columns of the block before that this store takes along
-                            const int lead = (int)(at & 7u) - back;             // the tile's first block starts inside a sector
-                            const int col = lane - back - lead;                 // from -7 to 31
-                            const uint32_t buf = both + (uint32_t)(((g & 1) ^ (col < 0)) * 4096) + r * 128;
-                            const uint32_t v = lds32u(buf + ((((uint32_t)col >> 2) & 7u) ^ ((uint32_t)r & 7u)) * 16 + (col & 3) * 4);
-                            if (col >= -back && nb + col < N) dst[col] = (int32_t)v;
-                            if (tail) {
-                                const int rest = col + 32;                      // the columns that stay over
-                                const uint32_t t = lds32u(both + (uint32_t)((g & 1) * 4096) + r * 128 + ((((uint32_t)rest >> 2) & 7u) ^ ((uint32_t)r & 7u)) * 16 + (rest & 3) * 4);
-                                if (rest < 32 && nb + rest < N) dst[rest] = (int32_t)t;
+                            for (int r = 0; r < rows; ++r, dst += ldc, at += (uint32_t)ldc) {
+                                const int back = g == 0 ? 0 : (int)(at & 7u);       // columns of the block before that this store takes along
+                                const int lead = (int)(at & 7u) - back;             // the warp's first block starts inside a sector
+                                const int col = lane - back - lead;                 // from -7 to 31
+                                const uint32_t buf = both + (uint32_t)(((g & 1) ^ (col < 0)) * 4096) + r * 128;
+                                const uint32_t v = lds32u(buf + ((((uint32_t)col >> 2) & 7u) ^ ((uint32_t)r & 7u)) * 16 + (col & 3) * 4);
+                                if (col >= -back && nb + col < N) dst[col] = (int32_t)v;
+                                if (tail) {
+                                    const int rest = col + 32;                      // the columns that stay over
+                                    const uint32_t t = lds32u(both + (uint32_t)((g & 1) * 4096) + r * 128 + ((((uint32_t)rest >> 2) & 7u) ^ ((uint32_t)r & 7u)) * 16 + (rest & 3) * 4);
+                                    if (rest < 32 && nb + rest < N) dst[rest] = (int32_t)t;
+                                }
                             }
                         }
+                        if (lane == 0) bulk_commit();            // (an empty group keeps the count)
                     }
-                    if (lane == 0) bulk_commit();            // (an empty group keeps the count)
+                    if (SIGN_PACK) {
+                        // bit = (dot - thr >= 0); the sign bits are shifted in from the top, element 31
+                        // first, so element j ends up in bit j, inverted.
+                        uint32_t wd = 0u;
+#pragma unroll
+                        for (int j = 31; j >= 0; --j)
+                            wd = __funnelshift_l((uint32_t)(q[j] - ctl->T[warp][g * 32 + j]), wd, 1);
+                        const int valid = N - nb;  // columns of this word that exist
+                        words[g] = valid > 0 ? (~wd ^ __ldg(flip + (nb >> 5))) & (valid < 32 ? (1u << valid) - 1u : 0xFFFFFFFFu) : 0u;
+                    }
                 }
                 if (SIGN_PACK) {
-                    // bit = (dot - thr >= 0); the sign bits are shifted in from the top, element 31
-                    // first, so element j ends up in bit j, inverted.
-                    uint32_t wd = 0u;
-#pragma unroll
-                    for (int j = 31; j >= 0; --j)
-                        wd = __funnelshift_l((uint32_t)(q[j] - ctl->T[g * 32 + j]), wd, 1);
-                    words[g] = ~wd ^ ctl->flipw[g];
-                    const int valid = N - nb;  // columns of this word that exist
-                    if (valid < 32) words[g] = valid > 0 ? (words[g] & ((1u << valid) - 1u)) : 0u;
-                }
-            }
-            if (SIGN_PACK && m < M) {
-                const int nw = words_for(N), w0 = n0 >> 5;
-                uint32_t* dst = out_bits + (size_t)m * ldob + w0;
-                if (w0 + BN / 32 <= nw) {   // 6 words; rows are 16-byte aligned, n0/32 is a multiple of 6
-#pragma unroll
-                    for (int i = 0; i < BN / 64; ++i)
-                        reinterpret_cast<uint2*>(dst)[i] = make_uint2(words[2 * i], words[2 * i + 1]);
-                } else {
-#pragma unroll
-                    for (int g = 0; g < BN / 32; ++g)
-                        if (w0 + g < nw) dst[g] = words[g];
+                    if (m < M) {
+                        const int nw = words_for(N), w0 = n0 >> 5;
+                        uint32_t* dst = out_bits + (size_t)m * ldob + w0;
+                        if (w0 + PN / 64 <= nw) {   // 2 words; rows are 16-byte aligned, n0/32 is even
+                            *reinterpret_cast<uint2*>(dst) = make_uint2(words[0], words[1]);
+                        } else if (w0 < nw) {
+                            dst[0] = words[0];
+                        }
+                    }
+                    __syncwarp();           // T is read
                 }
             }
         }
@@ -480,11 +416,12 @@ xnor_tc_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_constant__
     }
 
     // ---------------- teardown: every thread arrives here, also after an aborted wait
+    __syncwarp();
     tc_fence_before_sync();
-    __syncthreads();
+    cluster_sync();           // nobody reads the partner's shared or tensor memory any more
     if (warp == MMA_WARP) {
         tc_fence_after_sync();
-        tmem_dealloc(tmem, TMEM_COLS);
+        tmem_dealloc_pair(tmem, TMEM_COLS);
     }
     if (threadIdx.x == 0 && ctl->wait.abort) atomicExch(status.word, 1);
 }
@@ -496,15 +433,15 @@ int launch_variant(const uint32_t* Ap, int ldap, const uint32_t* Wp, int ldwp, i
     auto kern = xnor_tc_kernel<STORE_C, SIGN_PACK>;
     constexpr int SMEM = smem_bytes<STORE_C>();
     const int sm_count = device_sm_count();
-    if (sm_count <= 0 || !ensure_dynamic_smem(reinterpret_cast<const void*>(kern), SMEM)) return BNN_ERR_CUDA;
-    const int tiles = ceil_div(M, BM) * ceil_div(N, BN);
-    const int grid = tiles < sm_count ? tiles : sm_count;
+    if (sm_count < 2 || !ensure_dynamic_smem(reinterpret_cast<const void*>(kern), SMEM)) return BNN_ERR_CUDA;
+    const long long tiles = (long long)ceil_div(M, 2 * BM) * ceil_div(N, BN);
+    const int grid = 2 * (int)(tiles < sm_count / 2 ? tiles : sm_count / 2);
     const TcStatus status = tc_status();
     if (!status.word) return BNN_ERR_CUDA;
     // tensor maps of the two packed operands: [rows][ceil(K/32) words] with the caller's pitch;
-    // boxes of 16 words x (128 | 192) rows; whatever lies outside the tensor reads as zero
+    // boxes of 16 words x (128 | 64) rows; whatever lies outside the tensor reads as zero
     CUtensorMap mapA, mapB;
-    if (!encode_packed_map(&mapA, Ap, ldap, M, K, BM) || !encode_packed_map(&mapB, Wp, ldwp, N, K, BN))
+    if (!encode_packed_map(&mapA, Ap, ldap, M, K, BM) || !encode_packed_map(&mapB, Wp, ldwp, N, K, PN / 2))
         return BNN_ERR_CUDA;
     const int tma_c = C && ldc % 4 == 0 && (reinterpret_cast<uintptr_t>(C) & 15) == 0;
     CUtensorMap mapC{};
