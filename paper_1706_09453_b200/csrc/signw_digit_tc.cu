@@ -25,6 +25,8 @@
 // Bound by the epilogue for large batches (the sparse MMAs of a tile take 6 thousand clocks, its epilogue 8), by launch latency for small ones.  Measured on
 // B200 against dense MMAs on one digit per value, whole passes of six layers 2048 wide and their top layer: 8192 frames 728 -> 712 us, 517 frames
 // 101 -> 98.6; 8192 x 440 -> 2048 by itself, with its fp32 results, 64 -> 48 us.
+#include <cuda_fp16.h>
+
 #include "bnn_common.cuh"
 #include "digit_gemm.cuh"
 #include "tcgen05.cuh"

@@ -20,9 +20,9 @@
 // (sign bit = NOT the input bit, exponent field = 01).
 //
 // A pair of CTAs (cluster of two, one per SM of a TPC) works on a tile of 256 frames x two parts of 128 units: each CTA widens
-// its own 128 frames and half of the units, where a CTA by itself would widen all of them.  Roles in a CTA of 28 warps
+// its own 128 frames and half of the units, where a CTA by itself would widen all of them.  Roles in a CTA of 27 warps
 // (persistent, one CTA per SM):
-//   warp 27      one thread issues 2-D TMA tile loads of the packed rows (64 bytes per row =
+//   warp 26      one thread issues 2-D TMA tile loads of the packed rows (64 bytes per row =
 //                two stages) into a staging ring (64-byte swizzle, no multicast)
 //   warps 10-17  two teams widen the frame rows, thread = one row, 32 bytes -> 128 bytes per stage,
 //                written to tensor memory (the MMA reads its A operand from there); they take alternate stages
