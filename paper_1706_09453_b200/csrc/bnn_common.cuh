@@ -139,6 +139,10 @@ struct XnorStackLayer {
 size_t xnor_stack_sync_bytes(int M, int n_layers);
 int launch_xnor_stack(const uint32_t* Ap, int ldap, const XnorStackLayer* layers, int n_layers, int M, int N, int K,
                       int ldob, int zo, int* progress, cudaStream_t st);
+// The same on CTA pairs (xnor_gemm_pair.cu), and the clocks that it is estimated to take per layer (0: not for this shape).
+long long xnor_pair_clocks(int M, int N, int K, int sm_count);
+int launch_xnor_pair(const uint32_t* Ap, int ldap, const XnorStackLayer* layers, int n_layers, int M, int N, int K,
+                     int ldob, int zo, int* progress, cudaStream_t st);
 int launch_xnor_prepare(const uint32_t* Wp, int ldwp, int N, int K, void* image, cudaStream_t st);
 int launch_xnor_img(const uint32_t* Ap, int ldap, const void* image, int M, int N, int K,
                     int32_t* C, int ldc, const int32_t* thr, const uint32_t* flip,

@@ -42,8 +42,7 @@
 // kernel and the first MMA of the next.)
 //
 // What bounds it, measured on B200: 65536 frames x 3072 the widening of the frame rows (2 teams, about 430 clocks per
-// stage against 256 of MMA; five layers 1.18 ms, 1.51 before the issue from one elected lane and the lean producer
-// loop); 8192 x 2048 MMA (384 clocks per stage of 192 units), epilogue and the fill of a layer's pipeline in like parts
+// stage against 256 of MMA; five layers 1.18 ms: such runs go to pairs of CTAs, xnor_gemm_pair.cu); 8192 x 2048 MMA (384 clocks per stage of 192 units), epilogue and the fill of a layer's pipeline in like parts
 // (five layers 76 us, 91 before); a layer of one frame tile per CTA the chain store - count - load - widen -
 // MMA - decide, about 7 us (731 frames 36 us, 50 before, when all tiles were 192 wide).
 #include <type_traits>
@@ -593,13 +592,13 @@ int launch_bn(const uint32_t* Ap, int ldap, const XnorStackLayer* layers, int n_
 // narrow ones where there are too few frame tiles for all SMs.  Measured on B200, four 2048-wide layers, microseconds with
 // 192 / 128 / 96 / 32 units: 100 frames 29.5 / 27.3 / 27.0 / 25.5, 731 frames 30.4 / 28.5 / 28.8 / 33.5, 2000 frames
 // 35.4 / 33.8 / 37.3 / 71, 4000 frames 43 / 47 / 62 / 128.
-static int tile_units(int M, int N, int K, int sm_count) {
+static int tile_units(int M, int N, int K, int sm_count, long long& best_cost) {
     const int nks = ceil_div(K, BK), m_tiles = ceil_div(M, BM);
     if (nks > Cfg<128>::SLOTS) return 0;
     struct Candidate { int bn, slots, stage; };
     const Candidate all[] = {{192, Cfg<192>::SLOTS, 480}, {128, Cfg<128>::SLOTS, 460}, {96, Cfg<96>::SLOTS, 450}, {32, Cfg<32>::SLOTS, 400}};
     int best = 0;
-    long long best_cost = 0;
+    best_cost = 0;
     for (const Candidate& c : all) {
         const int n_tiles = ceil_div(N, c.bn);
         if (nks > c.slots || n_tiles > sm_count) continue;
@@ -614,7 +613,8 @@ static int sm_count_of_device() { return device_sm_count(); }
 
 bool xnor_res_applicable(int N, int K) {
     const int sms = sm_count_of_device();
-    return sms > 0 && tile_units(BM, N, K, sms) != 0;
+    long long cost;
+    return sms > 0 && tile_units(BM, N, K, sms, cost) != 0;
 }
 
 size_t xnor_stack_sync_bytes(int M, int n_layers) {
@@ -626,7 +626,14 @@ int launch_xnor_stack(const uint32_t* Ap, int ldap, const XnorStackLayer* layers
     const int sms = sm_count_of_device();
     if (sms <= 0) return BNN_ERR_CUDA;
     if (n_layers < 1 || n_layers > kXnorStackMax || (n_layers > 1 && (N != K || !progress))) return BNN_ERR_UNSUPPORTED;
-    const int bn = tile_units(M, N, K, sms);
+    long long cost;
+    const int bn = tile_units(M, N, K, sms, cost);
+    // Pairs of CTAs where they are estimated to be a tenth faster: large batches of fan-ins above 2048, whose weights leave a CTA
+    // 128 units (five 3072-wide layers of 65536 frames: a pass 3156 -> 2934 us).  Elsewhere tiles of 256 frames x 256 units leave
+    // more of the last turn empty than they save (8192 x 2048: a pass 237 -> 240 us; 731 frames 84 -> 91).
+    const long long pair_cost = xnor_pair_clocks(M, N, K, sms);
+    if (bn != 0 && K > 2048 && pair_cost > 0 && pair_cost + pair_cost / 10 < cost)
+        return launch_xnor_pair(Ap, ldap, layers, n_layers, M, N, K, ldob, zo, progress, st);
     if (bn == 192) return launch_bn<192>(Ap, ldap, layers, n_layers, M, N, K, ldob, zo, progress, sms, st);
     if (bn == 128) return launch_bn<128>(Ap, ldap, layers, n_layers, M, N, K, ldob, zo, progress, sms, st);
     if (bn == 96) return launch_bn<96>(Ap, ldap, layers, n_layers, M, N, K, ldob, zo, progress, sms, st);
