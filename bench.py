@@ -244,8 +244,13 @@ def layer_table(cfg, frames, peaks, sm_mhz, xnor_path="tensor", real_path="tenso
             # back once; the widened frame operand goes to tensor memory instead).
             tiles_m, tiles_n = -(-frames // 128), -(-cfg.hidden // 192)
             kpad = -(-k // 256) * 256
-            smem_bytes = tiles_m * tiles_n * kpad * (192 * (0.5 + 0.5 + 0.125 + 0.125) + 128 * (0.125 + 0.125))
+            # xnor_tc_kernel: tiles of 256 x 256 on CTA pairs, 128 rows of either operand per CTA
+            pair_tiles = 2 * -(-frames // 256) * -(-cfg.hidden // 256)
+            smem_bytes = pair_tiles * kpad * (128 * (0.5 + 0.5 + 0.125 + 0.125) + 128 * (0.125 + 0.125))
             kern = xnor_kernel_name(k, xnor_path, prepared, stacked and cfg.n_hidden > 2)
+            if kern == "xnor_res_kernel" and 2048 < k <= 3072 and frames >= 9000:     # a run of such layers
+                kern = "xnor_pair_kernel"
+                smem_bytes = pair_tiles * kpad * (128 * 0.5 + 128 * (0.125 + 0.125)) + SMS * kpad * 128 * 0.5
             if kern == "xnor_img_kernel":
                 # weights prepared once: their widened image arrives by bulk copies (4 bits written,
                 # 4 bits read by the tensor core per weight bit and tile visit); nothing else
@@ -271,18 +276,18 @@ def layer_table(cfg, frames, peaks, sm_mhz, xnor_path="tensor", real_path="tenso
                 rows.append(dict(name="signw_%d" % (l + 1), kernel="x_split_kernel+signw_img_kernel",
                                  work=work, unit="TFLOP/s", bound="tensor", peak=peaks["bf16"], passes=2))
             else:
-                # three byte digits of the activations, exact integer MMAs at twice the half-precision rate
+                # three byte digits of the activations, exact 2:4 sparse integer MMAs at four times the half-precision rate
                 rows.append(dict(name="signw_%d" % (l + 1), kernel="signw_digit_kernel" if chained else "x_digits_kernel+signw_digit_kernel",
-                                 work=work, unit="TFLOP/s", bound="tensor", peak=2.0 * peaks["bf16"], passes=3))
+                                 work=work, unit="TFLOP/s", bound="tensor", peak=4.0 * peaks["bf16"], passes=3))
         else:
             rows.append(dict(name="signw_%d" % (l + 1), kernel="real_gemm_kernel", work=work, unit="TFLOP/s",
                              bound="alu", peak=fp32_peak))
         k = cfg.hidden
     owork = 2.0 * frames * cfg.classes * cfg.hidden
     if real_path == "tensor" and cfg.act == 1 and not mixed:
-        # three byte digits of the weights, exact integer MMAs at twice the half-precision rate
+        # three byte digits of the weights, exact 2:4 sparse integer MMAs at four times the half-precision rate
         rows.append(dict(name="output_gemm", kernel="out_digit_kernel", work=owork, unit="TFLOP/s", bound="tensor",
-                         peak=2.0 * peaks["bf16"], passes=3))
+                         peak=4.0 * peaks["bf16"], passes=3))
     elif real_path == "tensor":
         # fp32 activations: both operands in two fp16 terms, three MMAs per step
         # (its fp16 activation image comes from the epilogue of the layer before: no split launch)
@@ -525,7 +530,7 @@ def run_ours(args):
     if not args.no_stack and frames > 16:
         merged = []
         for r in rows:
-            if (merged and r["kernel"] == "xnor_res_kernel" and merged[-1]["kernel"] == "xnor_res_kernel"
+            if (merged and r["kernel"] in ("xnor_res_kernel", "xnor_pair_kernel") and merged[-1]["kernel"] == r["kernel"]
                     and r["work"] == merged[-1]["work_per_layer"]):
                 m = merged[-1]
                 m["ms"] += r["ms"]; m["work"] += r["work"]; m["layers"] += 1
@@ -555,7 +560,7 @@ def run_ours(args):
     dk, dg = max(groups.items(), key=lambda kv: kv[1]["ms"])
     dom = dg["row"]
     achieved = dg["work"] / (dg["ms"] * 1e-3) / dom.get("scale", 1e12)
-    if dk in ("xnor_tc_kernel", "xnor_img_kernel", "xnor_res_kernel"):
+    if dk in ("xnor_tc_kernel", "xnor_img_kernel", "xnor_res_kernel", "xnor_pair_kernel"):
         peak_source = ("rate of a bare kind::mxf4 MMA loop measured in this run (%.0f Tbop/s); 4 x the %s bf16 figure of "
                        "MEASURED_PEAKS.json (%s) would be %.0f; of measured" % (peaks["mxf4"], regime, peaks["source"], 4 * bf16_peak))
     elif dom["bound"] == "tensor":
