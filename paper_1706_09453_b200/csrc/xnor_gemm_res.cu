@@ -628,11 +628,11 @@ int launch_xnor_stack(const uint32_t* Ap, int ldap, const XnorStackLayer* layers
     if (n_layers < 1 || n_layers > kXnorStackMax || (n_layers > 1 && (N != K || !progress))) return BNN_ERR_UNSUPPORTED;
     long long cost;
     const int bn = tile_units(M, N, K, sms, cost);
-    // Pairs of CTAs where they are estimated to be a tenth faster: large batches of fan-ins above 2048, whose weights leave a CTA
-    // 128 units (five 3072-wide layers of 65536 frames: a pass 3156 -> 2934 us).  Elsewhere tiles of 256 frames x 256 units leave
+    // Pairs of CTAs for fan-ins above 2048, whose weights leave a CTA 128 units, where they are estimated to be faster (passes of six layers, us: 65536 frames of
+    // 3072 units 3156 -> 2934, 16384 448 -> 384, 8192 239 -> 214, 2500 112 -> 98; 9000 of 2900 258 -> 216; 5000 of 2560 138 -> 120).  Elsewhere tiles of 256 frames x 256 units leave
     // more of the last turn empty than they save (8192 x 2048: a pass 237 -> 240 us; 731 frames 84 -> 91).
     const long long pair_cost = xnor_pair_clocks(M, N, K, sms);
-    if (bn != 0 && K > 2048 && pair_cost > 0 && pair_cost + pair_cost / 10 < cost)
+    if (bn != 0 && K > 2048 && pair_cost > 0 && pair_cost < cost)
         return launch_xnor_pair(Ap, ldap, layers, n_layers, M, N, K, ldob, zo, progress, st);
     if (bn == 192) return launch_bn<192>(Ap, ldap, layers, n_layers, M, N, K, ldob, zo, progress, sms, st);
     if (bn == 128) return launch_bn<128>(Ap, ldap, layers, n_layers, M, N, K, ldob, zo, progress, sms, st);

@@ -19,7 +19,7 @@
 // w holds, in nibble i, bit 4i + t of w:   ((w << (3 - t)) & 0x88888888) ^ 0xAAAAAAAA
 // (sign bit = NOT the input bit, exponent field = 01).
 //
-// A pair of CTAs (cluster of two, one per SM of a TPC) works on a tile of 256 frames x two parts of 128 units: each CTA widens
+// A pair of CTAs (cluster of two, one per SM of a TPC) works on a tile of 256 frames x two parts of 128 units (64 where that fills more SMs, part_units): each CTA widens
 // its own 128 frames and half of the units, where a CTA by itself would widen all of them.  Roles in a CTA of 27 warps
 // (persistent, one CTA per SM):
 //   warp 26      one thread issues 2-D TMA tile loads of the packed rows (64 bytes per row =
@@ -50,21 +50,26 @@ namespace {
 using namespace tc;
 
 constexpr int BM = 128;                                   // frames per CTA
-constexpr int PARTS = 2, PN = 128, BN = PARTS * PN;       // units per part and tile
-constexpr int BR = BN / 2;                                // unit rows per CTA: half of each part
+constexpr int PARTS = 2;
 constexpr int BK = 256;                                   // bits of K per stage = nibbles per widened row
 constexpr int ROW_BYTES = BK / 2;                         // widened bytes per row and stage (128)
-constexpr int PART_BYTES = PN / 2 * ROW_BYTES, STAGE_BYTES = PARTS * PART_BYTES;   // only the unit operand lives in shared memory
 constexpr int STAGES = 6;                                 // even: a stage always belongs to the same team of producers
-constexpr int EPI_WARPS = 8, MMA_WARP = 8, PROD_WARP0 = 10, TEAMS = 2, A_WARPS = BM / 32, B_WARPS = BR / 32;
-constexpr int TMA_WARP = PROD_WARP0 + TEAMS * (A_WARPS + B_WARPS);
-constexpr int THREADS = (TMA_WARP + 1) * 32;
+constexpr int EPI_WARPS = 8, MMA_WARP = 8, PROD_WARP0 = 10, TEAMS = 2, A_WARPS = BM / 32;
 constexpr int GROUPS = 3;                                 // staging ring: groups of two stages (an odd last stage has an empty partner)
-constexpr int GA_BYTES = BM * 64, GB_BYTES = BR * 64, GROUP_BYTES = GA_BYTES + GB_BYTES;
-constexpr uint32_t TMEM_A_COL = BN;                       // A stages start after the two accumulators
+constexpr int GA_BYTES = BM * 64;
 constexpr uint32_t A_COLS = ROW_BYTES / 4;                // 32-bit columns per A stage
-constexpr uint32_t TMEM_SF_COL = TMEM_A_COL + STAGES * A_COLS, SF_COLS = 32;   // block scales: 16 columns per operand
-constexpr uint32_t TMEM_COLS = 512;
+constexpr uint32_t SF_COLS = 32, TMEM_COLS = 512;
+
+// PN: units per part, 128 or 64.
+template <int PN> struct Tile {
+    static constexpr int BN = PARTS * PN, BR = BN / 2, B_WARPS = BR / 32;              // units per tile; unit rows per CTA: half of each part
+    static constexpr int PART_BYTES = PN / 2 * ROW_BYTES, STAGE_BYTES = PARTS * PART_BYTES;   // only the unit operand lives in shared memory
+    static constexpr int TMA_WARP = PROD_WARP0 + TEAMS * (A_WARPS + B_WARPS), THREADS = (TMA_WARP + 1) * 32;
+    static constexpr int GB_BYTES = BR * 64, GROUP_BYTES = GA_BYTES + GB_BYTES;
+    static constexpr uint32_t TMEM_A_COL = BN;                                          // A stages start after the two accumulators
+    static constexpr uint32_t TMEM_SF_COL = TMEM_A_COL + STAGES * A_COLS;               // block scales: 16 columns per operand
+    static_assert(TMEM_SF_COL + SF_COLS <= TMEM_COLS, "tensor memory columns");
+};
 
 // With int32 output each epilogue warp needs two staging blocks of 32 rows x 128 bytes (1024-byte aligned).
 template <bool STORE_C> struct Cfg {
@@ -72,17 +77,16 @@ template <bool STORE_C> struct Cfg {
 };
 
 struct Control {
-    int T[EPI_WARPS][PN / 2];        // per epilogue warp: threshold + kMagicBits of its units (Sign epilogue only)
+    int T[EPI_WARPS][64];            // per epilogue warp: threshold + kMagicBits of its units (Sign epilogue only)
     uint64_t full[STAGES], empty[STAGES], acc_full[PARTS], acc_empty[PARTS];
     uint64_t group_full[GROUPS], group_empty[GROUPS];
     uint32_t tmem_base;
     WaitState wait;
 };
-template <bool STORE_C> constexpr int smem_bytes() {
-    return STAGES * STAGE_BYTES + GROUPS * GROUP_BYTES + (int)sizeof(Control) + Cfg<STORE_C>::CSTAGE_BYTES + 1024;
+template <bool STORE_C, int PN> constexpr int smem_bytes() {
+    return STAGES * Tile<PN>::STAGE_BYTES + GROUPS * Tile<PN>::GROUP_BYTES + (int)sizeof(Control) + Cfg<STORE_C>::CSTAGE_BYTES + 1024;
 }
-static_assert(smem_bytes<false>() <= 232448 && smem_bytes<true>() <= 232448, "shared memory of one CTA");
-static_assert(TMEM_SF_COL + SF_COLS <= TMEM_COLS, "tensor memory columns");
+static_assert(smem_bytes<false, 128>() <= 232448 && smem_bytes<true, 128>() <= 232448, "shared memory of one CTA");
 
 struct ProducerArgs {
     uint32_t smem;        // shared-space address of stage 0
@@ -118,8 +122,11 @@ __device__ __forceinline__ void widen_stage(const ProducerArgs& a, int ks, const
 // staging group.  FRAMES: widened rows go to tensor memory, else (unit rows) to shared memory.
 // Template arguments say what the loops of the producers have to deal with: code that is there for another case costs this
 // one, though it is not executed.
-template <bool FRAMES, bool ZO, bool RAGGED>
+template <int PN, bool FRAMES, bool ZO, bool RAGGED>
 __device__ __forceinline__ void produce(const ProducerArgs& a, int r, int team) {
+    using T = Tile<PN>;
+    constexpr int STAGE_BYTES = T::STAGE_BYTES, PART_BYTES = T::PART_BYTES, GROUP_BYTES = T::GROUP_BYTES;
+    constexpr uint32_t TMEM_A_COL = T::TMEM_A_COL;
     Control* ctl = a.ctl;
     // TMEM lane of this thread's frame row: a warp may only touch lanes 32*(warp%4)..+31
     const uint32_t tdst0 = a.tmem + ((uint32_t)(r & ~31) << 16) + TMEM_A_COL;
@@ -171,13 +178,17 @@ __device__ __forceinline__ void produce(const ProducerArgs& a, int r, int team) 
     }
 }
 
-template <bool STORE_C, bool SIGN_PACK>
-__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(THREADS, 1)
+template <int PN, bool STORE_C, bool SIGN_PACK>
+__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(Tile<PN>::THREADS, 1)
 xnor_tc_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CUtensorMap mapB,
                 const __grid_constant__ CUtensorMap mapC, int tma_c,
                 int M, int N, int K, int32_t* __restrict__ C, int ldc,
                 const int32_t* __restrict__ thr, const uint32_t* __restrict__ flip,
                 uint32_t* __restrict__ out_bits, int ldob, int zo, TcStatus status) {
+    using Tl = Tile<PN>;
+    constexpr int BN = Tl::BN, B_WARPS = Tl::B_WARPS, TMA_WARP = Tl::TMA_WARP, STAGE_BYTES = Tl::STAGE_BYTES, PART_BYTES = Tl::PART_BYTES;
+    constexpr int GB_BYTES = Tl::GB_BYTES, GROUP_BYTES = Tl::GROUP_BYTES;
+    constexpr uint32_t TMEM_A_COL = Tl::TMEM_A_COL, TMEM_SF_COL = Tl::TMEM_SF_COL;
     extern __shared__ uint8_t smem_raw[];
     uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
     const uint32_t cstage = smem_u32(smem) + STAGES * STAGE_BYTES + GROUPS * GROUP_BYTES;
@@ -258,11 +269,11 @@ xnor_tc_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_constant__
             __syncwarp();
         } else if (warp < PROD_WARP0 + TEAMS * A_WARPS) {
             const int row = (warp & 3) * 32 + lane, team = (warp - PROD_WARP0) / A_WARPS;
-            if (zo) produce<true, true, false>(pa, row, team);
-            else produce<true, false, false>(pa, row, team);
+            if (zo) produce<PN, true, true, false>(pa, row, team);
+            else produce<PN, true, false, false>(pa, row, team);
         } else {
             const int pw = warp - PROD_WARP0 - TEAMS * A_WARPS, team = pw / B_WARPS, row = (pw - team * B_WARPS) * 32 + lane;
-            ragged ? produce<false, false, true>(pa, row, team) : produce<false, false, false>(pa, row, team);
+            ragged ? produce<PN, false, false, true>(pa, row, team) : produce<PN, false, false, false>(pa, row, team);
         }
     } else if (warp >= EPI_WARPS) {
         // ---------------- MMA issue: two converged warps of rank 0, each with its part of every tile.  What an issuing warp does
@@ -353,7 +364,8 @@ xnor_tc_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_constant__
                         // block: every store but those at the tile's edges then covers whole sectors.  (4096 x 2048 x
                         // 4095, microseconds: a thread a row 102, rows of 32 columns 68, whole sectors 57; 4096 columns 29.)
                         const bool whole = tma_c && (nb + 31 < N || N % 4 == 0);
-                        const uint32_t blk = cstage + (uint32_t)((warp * 2 + (g & 1)) * 4096);
+                        const int which = PN == 64 ? part : g & 1;       // of the warp's two blocks, in turn
+                        const uint32_t blk = cstage + (uint32_t)((warp * 2 + which) * 4096);
                         if (lane == 0) bulk_wait_read<1>();      // the block's store of two rounds ago has read it
                         __syncwarp();
 #pragma unroll
@@ -375,12 +387,12 @@ xnor_tc_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_constant__
                                 const int back = g == 0 ? 0 : (int)(at & 7u);       // columns of the block before that this store takes along
                                 const int lead = (int)(at & 7u) - back;             // the warp's first block starts inside a sector
                                 const int col = lane - back - lead;                 // from -7 to 31
-                                const uint32_t buf = both + (uint32_t)(((g & 1) ^ (col < 0)) * 4096) + r * 128;
+                                const uint32_t buf = both + (uint32_t)((which ^ (col < 0)) * 4096) + r * 128;
                                 const uint32_t v = lds32u(buf + ((((uint32_t)col >> 2) & 7u) ^ ((uint32_t)r & 7u)) * 16 + (col & 3) * 4);
                                 if (col >= -back && nb + col < N) dst[col] = (int32_t)v;
                                 if (tail) {
                                     const int rest = col + 32;                      // the columns that stay over
-                                    const uint32_t t = lds32u(both + (uint32_t)((g & 1) * 4096) + r * 128 + ((((uint32_t)rest >> 2) & 7u) ^ ((uint32_t)r & 7u)) * 16 + (rest & 3) * 4);
+                                    const uint32_t t = lds32u(both + (uint32_t)(which * 4096) + r * 128 + ((((uint32_t)rest >> 2) & 7u) ^ ((uint32_t)r & 7u)) * 16 + (rest & 3) * 4);
                                     if (rest < 32 && nb + rest < N) dst[rest] = (int32_t)t;
                                 }
                             }
@@ -402,8 +414,8 @@ xnor_tc_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_constant__
                     if (m < M) {
                         const int nw = words_for(N), w0 = n0 >> 5;
                         uint32_t* dst = out_bits + (size_t)m * ldob + w0;
-                        if (w0 + PN / 64 <= nw) {   // 2 words; rows are 16-byte aligned, n0/32 is even
-                            *reinterpret_cast<uint2*>(dst) = make_uint2(words[0], words[1]);
+                        if (PN == 128 && w0 + 2 <= nw) {   // rows are 16-byte aligned, n0/32 is even
+                            *reinterpret_cast<uint2*>(dst) = make_uint2(words[0], words[PN / 64 - 1]);
                         } else if (w0 < nw) {
                             dst[0] = words[0];
                         }
@@ -426,27 +438,38 @@ xnor_tc_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_constant__
     if (threadIdx.x == 0 && ctl->wait.abort) atomicExch(status.word, 1);
 }
 
-template <bool STORE_C, bool SIGN_PACK>
+// Units per part.  A launch takes ceil(tiles / pairs) turns of nks stages and an epilogue; a stage of 64 + 64 units takes more than half the
+// clocks of one of 128 + 128, because the frames are widened all the same.  Measured on B200, us, 128 / 64 units: 300 x 8000 x 1501 24.4 / 18.5,
+// 2500 x 2000 x 2503 24.8 / 22.1, 5000 x 1500 x 1203 23.5 / 20.5.
+int part_units(int M, int N, int K, int pairs) {
+    auto clocks = [&](int pn, int stage) {
+        const long long tiles = (long long)ceil_div(M, 2 * BM) * ceil_div(N, PARTS * pn);
+        return (tiles + pairs - 1) / pairs * ((long long)ceil_div(K, BK) * stage + 24 * pn);
+    };
+    return clocks(64, 400) < clocks(128, 600) ? 64 : 128;
+}
+
+template <int PN, bool STORE_C, bool SIGN_PACK>
 int launch_variant(const uint32_t* Ap, int ldap, const uint32_t* Wp, int ldwp, int M, int N, int K,
                    int32_t* C, int ldc, const int32_t* thr, const uint32_t* flip,
                    uint32_t* out_bits, int ldob, int zo, cudaStream_t st) {
-    auto kern = xnor_tc_kernel<STORE_C, SIGN_PACK>;
-    constexpr int SMEM = smem_bytes<STORE_C>();
+    auto kern = xnor_tc_kernel<PN, STORE_C, SIGN_PACK>;
+    constexpr int SMEM = smem_bytes<STORE_C, PN>();
     const int sm_count = device_sm_count();
     if (sm_count < 2 || !ensure_dynamic_smem(reinterpret_cast<const void*>(kern), SMEM)) return BNN_ERR_CUDA;
-    const long long tiles = (long long)ceil_div(M, 2 * BM) * ceil_div(N, BN);
+    const long long tiles = (long long)ceil_div(M, 2 * BM) * ceil_div(N, Tile<PN>::BN);
     const int grid = 2 * (int)(tiles < sm_count / 2 ? tiles : sm_count / 2);
     const TcStatus status = tc_status();
     if (!status.word) return BNN_ERR_CUDA;
     // tensor maps of the two packed operands: [rows][ceil(K/32) words] with the caller's pitch;
-    // boxes of 16 words x (128 | 64) rows; whatever lies outside the tensor reads as zero
+    // boxes of 16 words x (128 | PN / 2) rows; whatever lies outside the tensor reads as zero
     CUtensorMap mapA, mapB;
     if (!encode_packed_map(&mapA, Ap, ldap, M, K, BM) || !encode_packed_map(&mapB, Wp, ldwp, N, K, PN / 2))
         return BNN_ERR_CUDA;
     const int tma_c = C && ldc % 4 == 0 && (reinterpret_cast<uintptr_t>(C) & 15) == 0;
     CUtensorMap mapC{};
     if (tma_c && !encode_int32_map(&mapC, C, ldc, M, N)) return BNN_ERR_CUDA;
-    const cudaError_t e = launch_pdl(kern, dim3(grid), dim3(THREADS), SMEM, st, mapA, mapB, mapC, tma_c, M, N, K, C, ldc, thr, flip, out_bits, ldob, zo, status);
+    const cudaError_t e = launch_pdl(kern, dim3(grid), dim3(Tile<PN>::THREADS), SMEM, st, mapA, mapB, mapC, tma_c, M, N, K, C, ldc, thr, flip, out_bits, ldob, zo, status);
     return e == cudaSuccess ? launch_status() : BNN_ERR_CUDA;
 }
 
@@ -456,9 +479,10 @@ int launch_xnor_tc(const uint32_t* Ap, int ldap, const uint32_t* Wp, int ldwp, i
                    int K, int32_t* C, int ldc, const int32_t* thr, const uint32_t* flip,
                    uint32_t* out_bits, int ldob, int zo, cudaStream_t st) {
     const bool sp = out_bits != nullptr;
-    if (C && sp) return launch_variant<true, true>(Ap, ldap, Wp, ldwp, M, N, K, C, ldc, thr, flip, out_bits, ldob, zo, st);
-    if (C) return launch_variant<true, false>(Ap, ldap, Wp, ldwp, M, N, K, C, ldc, thr, flip, out_bits, ldob, zo, st);
-    return launch_variant<false, true>(Ap, ldap, Wp, ldwp, M, N, K, C, ldc, thr, flip, out_bits, ldob, zo, st);
+    auto go = [&](auto wide, auto narrow) { return (part_units(M, N, K, device_sm_count() / 2) == 64 ? narrow : wide)(Ap, ldap, Wp, ldwp, M, N, K, C, ldc, thr, flip, out_bits, ldob, zo, st); };
+    if (C && sp) return go(launch_variant<128, true, true>, launch_variant<64, true, true>);
+    if (C) return go(launch_variant<128, true, false>, launch_variant<64, true, false>);
+    return go(launch_variant<128, false, true>, launch_variant<64, false, true>);
 }
 
 }  // namespace bnn
