@@ -52,7 +52,8 @@ constexpr int STAGING_PITCH = 33;
 constexpr int BLOCK = 32 * 32 * 4, CONSTS = 2 * 32 * 4;
 constexpr int STAGING = digit::EPI_WARPS * (BLOCK + CONSTS);
 static_assert(STAGING >= digit::EPI_WARPS * 32 * STAGING_PITCH * 4, "either use fits");
-constexpr int SMEM_BYTES = digit::RING_BYTES + STAGING + (int)sizeof(digit::Bars) + 1024;
+constexpr int TOTALS = 4 * 32 * 4;       // of each epilogue warp, behind the staging: the digit sums of its classes, for activations in (0,1)
+constexpr int SMEM_BYTES = digit::RING_BYTES + STAGING + digit::EPI_WARPS * TOTALS + (int)sizeof(digit::Bars) + 1024;
 constexpr int kFollowGroupMin = 2 * digit::ROWS;
 static_assert(SMEM_BYTES <= 232448, "shared memory of one CTA");
 
@@ -140,12 +141,11 @@ __global__ void out_digits_kernel(const float* __restrict__ W, int ldw, int C, i
 }
 
 // ---- the GEMM ---------------------------------------------------------------------------
-// The digit sums of a granule's classes over all pairs (the last granule's beyond it).
-__device__ __forceinline__ void add_totals(uint32_t (&d)[4][8], const int* totals, int gran, int last) {
-    const int4* tot = reinterpret_cast<const int4*>(totals + (gran < last ? gran : last) * 4 * digit::GRAN);
+// The digit sums over all pairs of the 8 classes of granule g of this warp (shared-space address: [4 digits][32 classes]).
+__device__ __forceinline__ void add_totals(uint32_t (&d)[4][8], uint32_t totals, int g) {
 #pragma unroll
     for (int q = 0; q < 4; ++q) {
-        const int4 lo = __ldg(tot + 2 * q), hi = __ldg(tot + 2 * q + 1);
+        const uint4 lo = lds128u(totals + q * 128 + g * 32), hi = lds128u(totals + q * 128 + g * 32 + 16);
         d[q][0] += lo.x; d[q][1] += lo.y; d[q][2] += lo.z; d[q][3] += lo.w;
         d[q][4] += hi.x; d[q][5] += hi.y; d[q][6] += hi.z; d[q][7] += hi.w;
     }
@@ -163,7 +163,7 @@ out_digit_kernel(const __grid_constant__ CUtensorMap map, const __grid_constant_
     pdl_trigger();
     uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
     uint8_t* staging = smem + digit::RING_BYTES;
-    digit::Bars* bars = reinterpret_cast<digit::Bars*>(staging + STAGING);
+    digit::Bars* bars = reinterpret_cast<digit::Bars*>(staging + STAGING + digit::EPI_WARPS * TOTALS);
     volatile int* abort_flag = &bars->wait.abort;
     const int warp = warp_index(), lane = threadIdx.x & 31, rank = (int)cluster_rank();
     const uint32_t ring = smem_u32(smem);
@@ -194,6 +194,7 @@ out_digit_kernel(const __grid_constant__ CUtensorMap map, const __grid_constant_
         asm volatile("createpolicy.fractional.L2::evict_last.b64 %0, 1.0;" : "=l"(pol));
         by_blocks = by_blocks && w.nd == 3;
         const uint32_t block_smem = smem_u32(staging) + warp * BLOCK, consts = smem_u32(staging) + digit::EPI_WARPS * BLOCK + warp * CONSTS;
+        const uint32_t tot_smem = smem_u32(staging) + STAGING + warp * TOTALS;
         uint32_t parities = 0u;                                 // to wait for, of the parts
         bool ok = true;
         for (digit::Tiles t(w); ok && t.left > 0; t.next()) {
@@ -202,6 +203,17 @@ out_digit_kernel(const __grid_constant__ CUtensorMap map, const __grid_constant_
                 const bool has = cl < ncls && c < C;
                 const float rs = has ? __ldg(scales + c) * (ZO ? 0.5f : 1.0f) : 0.f;
                 const float bia = (bias && has) ? __ldg(bias + c) : 0.f;
+                if (ZO) {
+                    // before the wait for the accumulator, which then is read without waiting for these (8192 x 3400 x 2048 on
+                    // (0,1) activations 89 -> 80 us, 3401 classes 124 -> 100; dense digits took 101)
+                    const int cls = (part_gran + g0) * digit::GRAN + lane;
+                    const int* t0 = totals + (cls / digit::GRAN) * 4 * digit::GRAN + cls % digit::GRAN;
+                    int* mine_totals = reinterpret_cast<int*>(staging + STAGING + warp * TOTALS);
+                    __syncwarp();
+#pragma unroll
+                    for (int q = 0; q < 4; ++q) mine_totals[q * 32 + lane] = lane < ncls && cls < C ? __ldg(t0 + q * digit::GRAN) : 0;
+                    __syncwarp();
+                }
                 if (by_blocks) {
                     float* mine_consts = reinterpret_cast<float*>(staging + digit::EPI_WARPS * BLOCK + warp * CONSTS);
                     mine_consts[lane] = rs;
@@ -223,7 +235,7 @@ out_digit_kernel(const __grid_constant__ CUtensorMap map, const __grid_constant_
 #pragma unroll
                     for (int g = 0; g < 4; ++g) {
                         tmem_ld_wait();
-                        if (ZO) add_totals(d, totals, part_gran + g0 + g, (C - 1) / digit::GRAN);
+                        if (ZO) add_totals(d, tot_smem, g);
                         float z[8];
 #pragma unroll
                         for (int i = 0; i < 8; ++i) z[i] = fmaf(digit::high_part((int)d[2][i]), 65536.0f, digit::low_part((int)d[0][i], (int)d[1][i]));
@@ -262,7 +274,7 @@ out_digit_kernel(const __grid_constant__ CUtensorMap map, const __grid_constant_
 #pragma unroll 1
                     for (int g = 0; g < g1 - g0; ++g) {
                         tmem_ld_wait();
-                        if (ZO) add_totals(d, totals, part_gran + g0 + g, (C - 1) / digit::GRAN);
+                        if (ZO) add_totals(d, tot_smem, g);
                         float* dst = row + g * digit::GRAN;
                         if (w.nd == 4) {
 #pragma unroll
