@@ -276,6 +276,7 @@ __device__ __forceinline__ void widen_bits(const Work& w, const uint32_t* __rest
     for (; left > 0; --left) {
         // what lies between a free stage and a full one is kept short: the row was widened before the wait
         if (!warp_wait(empty, ph, abort_flag, lane)) return;
+        tc_fence_after_sync();          // the MMAs that read these columns come first
         tmem_st16(dst, o);
         tmem_st4(dst + 16, o + 16);
         cur = nxt;

@@ -125,6 +125,7 @@ __device__ __forceinline__ void produce(uint32_t staging, uint32_t tmem, Control
             wr[4 * c] = o.x; wr[4 * c + 1] = o.y; wr[4 * c + 2] = o.z; wr[4 * c + 3] = o.w;
         }
         if (!warp_wait(smem_u32(&ctl->empty_a[s]), ph, abort_flag, lane)) return;
+        tc_fence_after_sync();          // the MMAs that read these columns come first
         tmem_st32(tdst0 + s * A_COLS, wr);
         tmem_st_wait();
         tc_fence_before_sync();

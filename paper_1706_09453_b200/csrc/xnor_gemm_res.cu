@@ -192,6 +192,7 @@ __device__ __forceinline__ void produce_a(const ProducerArgs& a, int r, int team
                 wr[4 * c] = o.x; wr[4 * c + 1] = o.y; wr[4 * c + 2] = o.z; wr[4 * c + 3] = o.w;
             }
         }
+        tc_fence_after_sync();          // the MMAs that read these columns come first
         tmem_st32(tdst0 + s * A_COLS, wr);
         tmem_st_wait();
         tc_fence_before_sync();

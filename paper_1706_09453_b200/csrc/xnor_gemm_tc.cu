@@ -152,6 +152,7 @@ __device__ __forceinline__ void produce(const ProducerArgs& a, int r, int team) 
             uint32_t wr[32];
 #pragma unroll
             for (int c = 0; c < 8; ++c) { wr[4 * c] = o[c].x; wr[4 * c + 1] = o[c].y; wr[4 * c + 2] = o[c].z; wr[4 * c + 3] = o[c].w; }
+            tc_fence_after_sync();      // the MMAs that read these columns come first
             tmem_st32(tdst0 + s * A_COLS, wr);
             tmem_st_wait();
             tc_fence_before_sync();
