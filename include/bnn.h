@@ -186,10 +186,9 @@ BNN_API int bnn_signw_gemm(const float* X, int ldx, const uint32_t* Wp, int ldwp
 /* bnn_signw_gemm with scratch.  With `workspace` (device, 256-byte aligned, at least
  * bnn_signw_workspace_bytes(M, K) bytes) the real operand is written once per call as an image laid out
  * in the order the tensor core reads it, which the GEMM streams: 2-5x faster than bnn_signw_gemm on the tensor
- * path.  With two terms (BNN_OPT_SIGNW_TERMS), K <= 2^15 and an activation other than SIGN_PACK the image holds the sums and
- * differences of the pairs (k, k + 16) of every row of X as fixed-point numbers of a scale of the row's own in three byte digits, and the sums of
- * these are exact integers:
- *   |y - exact| <= K * 1.01 * 2^-23 * max_k |x[m][k]| + one fp32 rounding (a row with an infinity or a NaN gives NaN);
+ * path.  With two terms (BNN_OPT_SIGNW_TERMS), K <= 2^15 and an activation other than SIGN_PACK the image holds every row of X as fixed-point numbers of a
+ * power-of-two scale of its own in three byte digits, and the sums are exact integers:
+ *   |y - exact| <= K * 1.01 * 2^-23 * max_k |x[m][k]|, and the sum and the affine round to fp32 once each (a row with an infinity or a NaN gives NaN);
  * otherwise it holds bf16 terms, as bnn_signw_gemm.  Inside bnn_forward a layer writes the image of the next one of its kind
  * before a frame's largest output is known; max |x| is then replaced by a bound on it, min(1, max |scale| *
  * sqrt(K) |x'|_2 + max |shift|) for hardtanh units on inputs x', and likewise for Sigmoid.  Without workspace (NULL, or too small) it behaves exactly like

@@ -1,6 +1,6 @@
 // Products of a real-valued operand with packed sign bits as exact integer products on the tensor cores
-// (tcgen05 kind::i8, 2:4 sparse), on CTA pairs: the engine of the top layer on packed activations (out_digit_tc.cu) and of
-// the layers with binary weights on real-valued input (signw_digit_tc.cu).
+// (tcgen05 kind::i8, 2:4 sparse), on CTA pairs: the engine of the top layer on packed activations (out_digit_tc.cu), and what it
+// shares with that of the layers with binary weights on real-valued input (digit_dense.cuh).
 //
 // Two signs times two numbers are one sign times one number: s1 v1 + s2 v2 = s1 (v1 + v2) where s1 = s2 and s1 (v1 - v2)
 // elsewhere.  With the digits operand holding the sum and the difference of every pair (k, k + 16) in place of the two values,
@@ -104,7 +104,8 @@ struct Work {
 struct Tiles {
     int a, b;                  // coordinates of the current tile
     int left;                  // tiles from the current one on
-    __device__ __forceinline__ explicit Tiles(const Work& w) {
+    template <typename W>
+    __device__ __forceinline__ explicit Tiles(const W& w) {
         const int pairs = (int)gridDim.x >> 1, first = (int)blockIdx.x >> 1;
         const int na = w.a_tiles(), nb = w.b_tiles(), count = na * nb;
         left = first < count ? (count - 1 - first) / pairs + 1 : 0;
@@ -127,6 +128,20 @@ private:
     __device__ __forceinline__ void set(int fast, int slow) { a = b_fast_ ? slow : fast; b = b_fast_ ? fast : slow; }
 };
 
+// The end of the set-up: thread 0 has initialised the barriers of `bars`.  Returns the tensor-memory base.
+template <typename B>
+__device__ __forceinline__ uint32_t finish_set_up(B* bars, const TcStatus& status, int warp) {
+    if (threadIdx.x == 0) {
+        wait_state_init(&bars->wait, status);
+        mbar_init_fence();
+    }
+    __syncwarp();
+    if (warp == MMA_WARP) tmem_alloc_pair(smem_u32(&bars->tmem_base), TMEM_COLS);
+    tc_fence_before_sync();
+    cluster_sync();           // barriers of both CTAs initialised, tensor memory of both allocated
+    tc_fence_after_sync();
+    return bars->tmem_base;
+}
 // Common set-up; returns the tensor-memory base.  Called by all threads of both CTAs.
 __device__ __forceinline__ uint32_t set_up(Bars* bars, const TcStatus& status, int warp, bool halved) {
     if (threadIdx.x == 0) {
@@ -138,19 +153,13 @@ __device__ __forceinline__ uint32_t set_up(Bars* bars, const TcStatus& status, i
             mbar_init(smem_u32(&bars->acc_full[b]), 1);
             mbar_init(smem_u32(&bars->acc_empty[b]), halved ? 2 * EPI_WARPS : EPI_WARPS);   // rank 0: the epilogue warps of both CTAs that read it
         }
-        wait_state_init(&bars->wait, status);
-        mbar_init_fence();
     }
-    __syncwarp();
-    if (warp == MMA_WARP) tmem_alloc_pair(smem_u32(&bars->tmem_base), TMEM_COLS);
-    tc_fence_before_sync();
-    cluster_sync();           // barriers of both CTAs initialised, tensor memory of both allocated
-    tc_fence_after_sync();
-    return bars->tmem_base;
+    return finish_set_up(bars, status, warp);
 }
 
 // Common teardown; every thread of both CTAs arrives here, also after an aborted wait.
-__device__ __forceinline__ void tear_down(Bars* bars, const TcStatus& status, int warp, uint32_t tmem) {
+template <typename B>
+__device__ __forceinline__ void tear_down(B* bars, const TcStatus& status, int warp, uint32_t tmem) {
     __syncwarp();
     tc_fence_before_sync();
     cluster_sync();           // nobody reads the partner's shared or tensor memory any more
@@ -337,7 +346,8 @@ __device__ __forceinline__ void issue(const Work& w, uint32_t ring, Bars* bars, 
 }
 
 // Epilogue warps: this warp has read its share of the tile's accumulator.
-__device__ __forceinline__ void release_acc(Bars* bars, int b, int lane) {
+template <typename B>
+__device__ __forceinline__ void release_acc(B* bars, int b, int lane) {
     tc_fence_before_sync();
     __syncwarp();
     if (lane == 0) mbar_arrive_cluster(peer_addr(smem_u32(&bars->acc_empty[b]), 0));
@@ -365,8 +375,6 @@ __device__ __forceinline__ float low_part(int s0, int s1) { return (float)(s1 * 
 // The high sum is below 2^22: adding 1.5 * 2^23 as an integer to its bits makes it a float without the
 // conversion unit, which the other conversion of every output already keeps busy.
 __device__ __forceinline__ float high_part(int s2) { return __int_as_float((s2 >> 6) + 0x4B400000) - 12582912.0f; }
-// 2^h for -126 <= h <= 127.
-__device__ __forceinline__ float power_of_two(int h) { return __int_as_float((127 + h) << 23); }
 // Largest e (up to 140) such that mx * 2^e is a balanced number of three digits: at most 127 * (65536 + 256 + 1) = 0x7F7F7F.
 // mx >= 0; its exponent and fraction fields are compared with those of the limit.
 __device__ __forceinline__ int scale_exponent(float mx) {
@@ -375,33 +383,6 @@ __device__ __forceinline__ int scale_exponent(float mx) {
     const int e = 22 + 127 - (bits >> 23) - ((bits & 0x7FFFFF) > 0x7EFEFE ? 1 : 0);     // 0x7F7F7F / 2^22
     return e > 140 ? 140 : e;
 }
-// The scale of a row, from half of the largest |x1| + |x2| of its pairs (half, because a pair's sum may be beyond the largest float).
-constexpr float kTopValue = 8355700.0f;       // somewhat below 0x7F7F7F: room for roundings
-struct Scale {
-    float a, b;
-    float inverse;                            // what a unit stands for
-    __device__ __forceinline__ explicit Scale(float half_top) {
-        if (half_top >= 0x1p-100f) {
-            a = 1.0f;
-            b = __fdiv_rn(kTopValue, half_top);
-            inverse = __fdiv_rn(2.0f, b);
-        } else {                              // (1 / scale may be beyond the largest float)
-            const int e = half_top > 0.f ? scale_exponent(half_top) - 1 : 0, h = e >> 1;
-            a = power_of_two(h + 1);
-            b = power_of_two(e - h);
-            inverse = power_of_two(-h) * power_of_two(h - e);
-        }
-    }
-    // The numbers of a pair.  Its two products are rounded to integers and fractions, which are added apart: a float of more than
-    // 2^22 has no more than one bit of fraction left, and the sum is better rounded once.
-    __device__ __forceinline__ void pair(float x1, float x2, int& sum, int& difference) const {
-        const float p1 = x1 * a * (0.5f * b), p2 = x2 * a * (0.5f * b);
-        const int i1 = __float2int_rn(p1), i2 = __float2int_rn(p2);
-        const float f1 = p1 - (float)i1, f2 = p2 - (float)i2;
-        sum = i1 + i2 + __float2int_rn(f1 + f2);
-        difference = i1 - i2 + __float2int_rn(f1 - f2);
-    }
-};
 // Half of |x1| + |x2|.
 __device__ __forceinline__ float half_sum(float x1, float x2) { return fmaf(0.5f, x1, 0.5f * x2); }
 // The balanced base-256 digits of v in the bytes of a word: the sum of 128 at every place turns them into ordinary

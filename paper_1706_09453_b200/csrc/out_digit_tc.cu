@@ -85,12 +85,13 @@ __global__ void out_range_kernel(const float* __restrict__ W, int ldw, int C, in
     }
 }
 
+constexpr float kTopValue = 8355700.0f;       // somewhat below 0x7F7F7F, the largest balanced number of three digits: room for roundings
 // What a unit of a class's fixed-point numbers stands for.  With three digits any fp32 number will do, because the numbers are prepared in
 // double precision, and the smallest that keeps the largest pair within range is the most precise.  (The margin is that of the
 // rounding of `half`.)  With four, where the rounding of the result is all that counts, a power of two, which costs none.
 __device__ __forceinline__ float class_scale(float half, int nd) {
     if (!(half > 0.f)) return half == 0.f ? 1.0f : half;      // no weights; a NaN
-    if (nd == 3) return __double2float_ru(2.0 * (double)half / (double)digit::kTopValue);
+    if (nd == 3) return __double2float_ru(2.0 * (double)half / (double)kTopValue);
     int e;
     frexp(2.0 * (double)half / 2e9, &e);
     return (float)ldexp(1.0, e > -149 ? e : -149);

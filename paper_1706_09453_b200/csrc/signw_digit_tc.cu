@@ -1,9 +1,9 @@
-// Binary weights x real-valued activations on the tensor cores with exact integer sums (digit_gemm.cuh):
+// Binary weights x real-valued activations on the tensor cores with exact integer sums (digit_dense.cuh):
 //
-//   1. x_digits_kernel writes the sums and differences of the pairs of every frame once per call as fixed-point numbers of a
-//      scale of the frame's own, in three byte digits, in the order the tensor core reads shared memory (an image in scratch);
+//   1. x_digits_kernel writes every frame once per call as fixed-point numbers of a power-of-two scale of its own, in
+//      three byte digits, in the order the tensor core reads shared memory (an image in scratch);
 //   2. signw_digit_kernel multiplies the digits with the packed +-1 weights: units on the M side (tensor-memory
-//      lane = unit), frame digits on the N side, 256 units x 128 (64, 32) frames per tile and CTA pair.
+//      lane = unit), frame digits on the N side, 256 units x 64 (or 32) frames per tile and CTA pair.
 //
 // For layers that hand on real values.  (A layer with Sign units keeps the bf16 terms of signw_img_tc.cu: there a
 // pre-activation near zero turns any change of rounding into another bit, so its sums stay what they were.)
@@ -11,24 +11,26 @@
 // bytes.  When the layer that consumes the outputs is again of this kind (a network with binary weights and real
 // activations, Algorithm 1), the epilogue also writes them as that layer's image.  A frame's scale then has to be chosen before
 // its largest output is known: from a bound on its outputs, min(1, max |scale| * sum |x| + max |shift|) for hardtanh and
-// likewise for Sigmoid, with sum |x| <= sqrt(K sum x^2) and 2 (x1^2 + x2^2) = (x1 + x2)^2 + (x1 - x2)^2, for which every kernel of
-// such a chain adds up the squares of each frame's high digits as it writes them (one instruction per four).  A scale for outputs up to 1 would do in most
+// likewise for Sigmoid, with sum |x| <= sqrt(K sum x^2), for which every kernel of such a chain adds up the squares of each
+// frame's high digits as it writes them (one instruction per four units).  A scale for outputs up to 1 would do in most
 // networks, but loses outputs that are all small: six layers of 2048 units with scale 0.001, relative error of the last
 // one's outputs 0.75 with it, 6e-6 with scales from the bound, 1.3e-5 with two bf16 terms.  (What the bound costs: 517 frames,
 // six layers, 98 -> 100 us.)
 // The fp16 image of the real-valued layer on fp32 activations (out_gemm_f32_tc.cu) is written the same way.
 //
-// |result - exact| <= K / 2 * 1.01 * 2^-22 * max_k |x[m][k]| at worst (every rounding of a frame at its largest and of one
-// sign; typically sqrt(K) 2^-25), plus the rounding to fp32.  Two bf16 terms, which this path used before, keep 2^-17 of
+// |result - exact| <= K * 1.01 * 2^-23 * max_k |x[m][k]| at worst (every rounding of a frame at its largest and of one
+// sign; typically sqrt(K) 2^-25), plus one rounding to fp32.  Two bf16 terms, which this path used before, keep 2^-17 of
 // each |x| and round the sums at every step.
 //
-// Bound by the epilogue for large batches (the sparse MMAs of a tile take 6 thousand clocks, its epilogue 8), by launch latency for small ones.  Measured on
-// B200 against dense MMAs on one digit per value, whole passes of six layers 2048 wide and their top layer: 8192 frames 728 -> 712 us, 517 frames
-// 101 -> 98.6; 8192 x 440 -> 2048 by itself, with its fp32 results, 64 -> 48 us.
+// Bound by the tensor pipe and the board's power for large batches, by launch latency for small ones.  Measured on
+// B200 against two bf16 terms on tiles of 128 frames x 512 units, 2048 -> 2048 units chained: 8192 frames 112 -> 63 us,
+// 517 frames 56 -> 11 us; largest error of a sum 2^-17 -> 3e-7 of sum |x|.
+#include <cfloat>
+
 #include <cuda_fp16.h>
 
 #include "bnn_common.cuh"
-#include "digit_gemm.cuh"
+#include "digit_dense.cuh"
 #include "tcgen05.cuh"
 
 namespace bnn {
@@ -36,11 +38,12 @@ namespace bnn {
 namespace {
 
 using namespace tc;
+namespace dense = digit::dense;
 
 // Staging per epilogue warp: 32 frame scales of the input, then 32 of the output and 32 x 8 sums, or 32 frames x two fp16
 // terms of 32 units.
 constexpr int STAGING = 128 + 4096;
-constexpr int SMEM_BYTES = digit::RING_BYTES + digit::EPI_WARPS * STAGING + (int)sizeof(digit::Bars) + 1024;
+constexpr int SMEM_BYTES = dense::RING_BYTES + digit::EPI_WARPS * STAGING + (int)sizeof(dense::Bars) + 1024;
 constexpr int BOUNDS_WARP = digit::COPY_WARP + 1;
 static_assert(SMEM_BYTES <= 232448, "shared memory of one CTA");
 
@@ -97,17 +100,16 @@ struct UnitBounds {
         scale = v.x; shift = v.y; top_shift = v.z;
     }
     __device__ __forceinline__ void store(uint8_t* img) const { *reinterpret_cast<uint4*>(img) = make_uint4(scale, shift, top_shift, 0u); }
-    // Exponent of the scale of a frame whose inputs' magnitudes add up to at most `sum`: outputs are written as multiples of
-    // 256 / 127 * 2^-e, so that twice the largest one (a pair's sum) is at most 127 * 65536 and an output of 1 is written exactly.  (Up to
-    // 101: beyond, 2^-e leaves the range of numbers that keep their precision.)
+    // Exponent of the scale of a frame whose inputs' magnitudes add up to at most `sum`.  (Up to 100: beyond, 2^-e leaves the
+    // range of numbers that keep their precision.)
     __device__ __forceinline__ int exponent(float sum, bool sigmoid) const {
         const float d = __uint_as_float(scale) * sum, sh = __uint_as_float(shift);
         const float top = __uint_as_float(top_shift & kTop ? top_shift & ~kTop : ~top_shift);
         // roundings of the sums, the affine and the activation stay far below the margins
         float b = sigmoid ? expf(d + top + 1e-6f * (d + sh)) : d + sh;
         b *= 1.0001f;
-        const int e = digit::scale_exponent(0.9922f * (max(scale, shift) < kInf && b < 1.0f ? b : 1.0f));
-        return e > 101 ? 101 : e;
+        const int e = digit::scale_exponent(max(scale, shift) < kInf && b < 1.0f ? b : 1.0f);
+        return e > 100 ? 100 : e;
     }
 };
 
@@ -143,25 +145,16 @@ struct Frames {
     }
 };
 
-// Outputs are written as multiples of 1 / (kOutputUnits 2^e), see UnitBounds::exponent.
-constexpr float kOutputUnits = 127.0f / 256.0f;
-// A NaN among a layer's outputs is handed on as the number below all others, of which the high digit, -128, alone is not zero (the others
-// have high digits of -127 and more), and a part of a frame's sum of squares (at most 8 * 4 * 127^2 together) is replaced by one that
-// shows in the sum.
+// A NaN among a layer's outputs is handed on as the number below all others, of which the high digit alone is not zero.  The
+// outputs of Sigmoid units are not negative, so their high digits with the top bit set are NaNs, and a part of a frame's
+// sum of squares (at most 8 * 4 * 127^2 together) is replaced by one that shows in the sum.
 constexpr float kNaNDigits = -8388608.0f;
 constexpr int kNaNSquare = 1 << 27;
-// Whether one of the four digits is -128.
-__device__ __forceinline__ bool has_nan_digit(uint32_t x) {
-    const uint32_t y = x ^ 0x80808080u;
-    return ((y - 0x01010101u) & ~y & 0x80808080u) != 0u;
-}
 constexpr uint32_t kNaNOutput = 0x80000000u;     // in a frame's sum
 
-// At least sum_k |x|, given the scale and the sum of the squares of the high digits of all sums and differences: |x1| + |x2| of a pair is
-// the larger of its two, each at most 65536 |high| + 32896 units.
-__device__ __forceinline__ int pair_count(int K) { return (K >> 5) * 16 + ((K & 31) < 16 ? K & 31 : 16); }
+// At least sum_k |v| * 2^-e, given 2^-e and the sum of the squares of the high digits (|v| <= 65536 |high| + 32896).
 __device__ __forceinline__ float magnitude_bound(float inv_scale, uint32_t squares, int K) {
-    const float root = sqrtf((float)pair_count(K));
+    const float root = sqrtf((float)K);
     return inv_scale * root * fmaf(65536.0f, sqrtf((float)squares), 32896.0f * root);
 }
 
@@ -174,11 +167,11 @@ __host__ __device__ __forceinline__ int staged_pitch(int K) { return ((K + 3) & 
 // sums, next_sums (a chain of layers) or nullptr: this image's sums are written, those of the image that the layer behind
 // this kernel writes are cleared; one more block finds the bounds of that layer, `units`.
 template <bool STAGED>
-__global__ void __launch_bounds__(256, 4)
+__global__ void __launch_bounds__(256, 8)
 x_digits_kernel(Frames x, uint8_t* __restrict__ img, uint32_t* __restrict__ sums, uint32_t* __restrict__ next_sums,
                 Affine units, int* __restrict__ clear, int clear_words) {
     extern __shared__ float rows[];
-    __shared__ float tops[digit::GRAN];
+    __shared__ int exps[digit::GRAN];
     __shared__ uint32_t parts[3];
     pdl_trigger();   // the GEMM may be scheduled as SMs free up; it waits before it reads the image
     // As the first kernel of a forward pass this one also clears the pass's counters (a few hundred
@@ -200,91 +193,63 @@ x_digits_kernel(Frames x, uint8_t* __restrict__ img, uint32_t* __restrict__ sums
         return;
     }
     const int m0 = blockIdx.x * digit::GRAN, pitch = staged_pitch(x.K);
-    {   // largest magnitude of each frame as bits (orders NaN above infinity above every number) and largest pair: a warp per frame
+    {   // largest magnitude of each frame as bits (orders NaN above infinity above every number): a warp per frame
         const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
         uint32_t top = 0u;
-        float all = 0.f, half = 0.f;
+        float all = 0.f;
 #pragma unroll 4
-        for (int k0 = 0; k0 < x.K; k0 += 128) {
-            const int k = k0 + 4 * lane;
+        for (int k = 4 * lane; k < x.K; k += 128) {
             const float4 v = x.four(m0 + warp, k);
-            if (STAGED && k < x.K) *reinterpret_cast<float4*>(rows + warp * pitch + k) = v;
-            const float4 a = make_float4(fabsf(v.x), fabsf(v.y), fabsf(v.z), fabsf(v.w));
-            top = max(max(top, __float_as_uint(a.x)), __float_as_uint(a.y));
-            top = max(max(top, __float_as_uint(a.z)), __float_as_uint(a.w));
-            all += (a.x + a.y) + (a.z + a.w);
-            half = fmaxf(half, fmaxf(digit::half_sum(a.x, __shfl_xor_sync(0xFFFFFFFFu, a.x, 4)), digit::half_sum(a.y, __shfl_xor_sync(0xFFFFFFFFu, a.y, 4))));
-            half = fmaxf(half, fmaxf(digit::half_sum(a.z, __shfl_xor_sync(0xFFFFFFFFu, a.z, 4)), digit::half_sum(a.w, __shfl_xor_sync(0xFFFFFFFFu, a.w, 4))));
+            if (STAGED) *reinterpret_cast<float4*>(rows + warp * pitch + k) = v;
+            top = max(max(top, __float_as_uint(fabsf(v.x))), __float_as_uint(fabsf(v.y)));
+            top = max(max(top, __float_as_uint(fabsf(v.z))), __float_as_uint(fabsf(v.w)));
+            all += (fabsf(v.x) + fabsf(v.y)) + (fabsf(v.z) + fabsf(v.w));
         }
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) {
             top = max(top, __shfl_xor_sync(0xFFFFFFFFu, top, o));
-            half = fmaxf(half, __shfl_xor_sync(0xFFFFFFFFu, half, o));
             all += __shfl_xor_sync(0xFFFFFFFFu, all, o);
         }
         if (lane == 0) {
-            const bool finite = top < 0x7F800000u;
-            const digit::Scale scale(finite ? half : 0.f);
-            tops[warp] = finite ? half : 0.f;
-            reinterpret_cast<float*>(img + im.scales)[m0 + warp] = finite ? scale.inverse : __int_as_float(0x7FC00000);
+            const float mx = __uint_as_float(top);
+            exps[warp] = digit::scale_exponent(mx);
+            reinterpret_cast<float*>(img + im.scales)[m0 + warp] = top < 0x7F800000u ? dense::inverse_scale(exps[warp]) : __int_as_float(0x7FC00000);
             if (sums) {
                 // what gives magnitude_bound() the sum of the magnitudes itself; roundings stay far below 0.001
-                const float t = 0.5f * all * scale.a * scale.b * (1.001f / 65536.0f);
-                sums[m0 + warp] = (uint32_t)(t * t / (float)pair_count(x.K)) + 1u;
+                const dense::Scale scale(exps[warp]);
+                const float t = all * scale.a * scale.b * (1.001f / 65536.0f);
+                sums[m0 + warp] = (uint32_t)(t * t / (float)x.K) + 1u;
                 next_sums[m0 + warp] = 0u;
             }
         }
     }
     __syncthreads();
-    // thread -> frame i, half hh of a group of 64 positions: positions t + 8 j of it with t / 4 = hh, i.e. 16 pairs, in two chunks of
-    // each digit row (digit::image_byte)
+    // thread -> frame i, half hh of a group of 32 positions: 16 values, one chunk of each digit row
     const int i = threadIdx.x & 7, hh = (threadIdx.x >> 3) & 1;
-    const digit::Scale scale(tops[i]);
+    const dense::Scale scale(exps[i]);
     uint8_t* dst0 = img + im.digits + ((size_t)blockIdx.x * (3 * digit::GRAN) + i) * 16;
-    for (int g = threadIdx.x >> 4; 4 * g < im.chunks; g += 16) {
-        const bool half = 4 * g + 2 == im.chunks;
-        float4 f[8];
+    for (int g = threadIdx.x >> 4; g < im.chunks / 2; g += 16) {
+        float4 f[4];
 #pragma unroll
-        for (int j = 0; j < 8; ++j) {
-            const int k = 64 * g + 8 * j + 4 * hh;
+        for (int j = 0; j < 4; ++j) {
+            const int k = 32 * g + 8 * j + 4 * hh;
             if (STAGED) f[j] = k < x.K ? *reinterpret_cast<const float4*>(rows + i * pitch + k) : make_float4(0.f, 0.f, 0.f, 0.f);
             else f[j] = x.four(m0 + i, k);
         }
+        uint32_t d[3][4];
 #pragma unroll
-        for (int u = 0; u < 2; ++u) {              // chunk 2 u + hh: t % 2 = u
-            uint32_t d[3][4];
+        for (int t = 0; t < 4; ++t) {
+            uint32_t v[4];
 #pragma unroll
-            for (int y = 0; y < 4; ++y) {          // word y: t / 2 % 2 = y / 2, word y % 2 of the group, two pairs
-                uint32_t v[4];
-#pragma unroll
-                for (int q = 0; q < 2; ++q) {
-                    const int c = u + 2 * (y >> 1), j = 4 * (y & 1) + q;
-                    const float4 lo = f[j], hi = f[j + 2];
-                    const float x1 = c == 0 ? lo.x : c == 1 ? lo.y : c == 2 ? lo.z : lo.w;
-                    const float x2 = c == 0 ? hi.x : c == 1 ? hi.y : c == 2 ? hi.z : hi.w;
-                    int sum, difference;
-                    scale.pair(x1, x2, sum, difference);
-                    v[2 * q] = digit::digits3(sum);
-                    v[2 * q + 1] = digit::digits3(difference);
-                }
-                d[0][y] = digit::gather_bytes<0>(v[0], v[1], v[2], v[3]);
-                d[1][y] = digit::gather_bytes<1>(v[0], v[1], v[2], v[3]);
-                d[2][y] = digit::gather_bytes<2>(v[0], v[1], v[2], v[3]);
-            }
-            if (!half) {
-                uint8_t* dst = dst0 + (size_t)(4 * g + 2 * u + hh) * im.rows * 16;
-#pragma unroll
-                for (int q = 0; q < 3; ++q)
-                    *reinterpret_cast<uint4*>(dst + q * digit::GRAN * 16) = make_uint4(d[q][0], d[q][1], d[q][2], d[q][3]);
-            } else {                               // t % 4 = u and u + 2
-#pragma unroll
-                for (int y = 0; y < 4; y += 2) {
-                    uint8_t* dst = dst0 + (size_t)(4 * g + (y >> 1)) * im.rows * 16 + 8 * u + 4 * hh;
-#pragma unroll
-                    for (int q = 0; q < 3; ++q) *reinterpret_cast<uint32_t*>(dst + q * digit::GRAN * 16) = d[q][y];
-                }
-            }
+            for (int j = 0; j < 4; ++j) v[j] = digit::digits3(scale.fixed_point(t == 0 ? f[j].x : t == 1 ? f[j].y : t == 2 ? f[j].z : f[j].w));
+            d[0][t] = digit::gather_bytes<0>(v[0], v[1], v[2], v[3]);
+            d[1][t] = digit::gather_bytes<1>(v[0], v[1], v[2], v[3]);
+            d[2][t] = digit::gather_bytes<2>(v[0], v[1], v[2], v[3]);
         }
+        uint8_t* dst = dst0 + (size_t)(2 * g + hh) * im.rows * 16;
+#pragma unroll
+        for (int q = 0; q < 3; ++q)
+            *reinterpret_cast<uint4*>(dst + q * digit::GRAN * 16) = make_uint4(d[q][0], d[q][1], d[q][2], d[q][3]);
     }
 }
 
@@ -309,40 +274,40 @@ struct Args {
 // launch to the next; 517 frames, six layers, 100.2 us, with a kernel per kind 101.6.)
 template <bool SIGMOID>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(digit::THREADS, 1)
-signw_digit_kernel(const __grid_constant__ CUtensorMap map, const __grid_constant__ digit::Work w, const __grid_constant__ Args g,
+signw_digit_kernel(const __grid_constant__ CUtensorMap map, const __grid_constant__ dense::Work w, const __grid_constant__ Args g,
                    TcStatus status) {
     extern __shared__ uint8_t smem_raw[];
     uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
-    uint8_t* staging = smem + digit::RING_BYTES;
-    digit::Bars* bars = reinterpret_cast<digit::Bars*>(staging + digit::EPI_WARPS * STAGING);
+    uint8_t* staging = smem + dense::RING_BYTES;
+    dense::Bars* bars = reinterpret_cast<dense::Bars*>(staging + digit::EPI_WARPS * STAGING);
     volatile int* abort_flag = &bars->wait.abort;
     const int warp = warp_index(), lane = threadIdx.x & 31, rank = (int)cluster_rank();
     const bool digits_out = g.img_out && g.img_out_kind == 0;
     const uint32_t ring = smem_u32(smem);
-    const uint32_t tmem = digit::set_up(bars, status, warp, w.halved());
+    const uint32_t tmem = dense::set_up(bars, status, warp);
 
     if (warp >= digit::PROD_WARP0) {
-        digit::widen_bits(w, g.Wp, g.ldwp, bars, tmem, rank, warp, lane);
+        dense::widen_bits(w, g.Wp, g.ldwp, bars, tmem, rank, warp, lane);
     } else if (warp == digit::COPY_WARP) {
         // the image is the output of the kernel before this one in the stream: wait until that kernel has
         // completed and its writes are visible (the weights do not depend on it)
         pdl_wait();
-        if (lane == 0) digit::copy_digits(w, &map, ring, bars, rank);
+        if (lane == 0) dense::copy_digits(w, &map, ring, bars, rank);
     } else if (warp == BOUNDS_WARP) {
         if (digits_out && blockIdx.x == 0) {
             const UnitBounds b(g.next, lane, 32);
             if (lane == 0) b.store(g.img_out);
         }
     } else if (warp >= digit::EPI_WARPS) {
-        if (rank == 0 && warp <= digit::MMA_WARP2) digit::issue(w, ring, bars, tmem, warp - digit::MMA_WARP);
+        if (rank == 0 && warp <= digit::MMA_WARP2) dense::issue(w, ring, bars, tmem, warp - digit::MMA_WARP);
     } else {
-        // ---------------- epilogue: thread = one unit (tensor-memory lane); of a tile's frames, or of either part's, warps 0-3 take the
+        // ---------------- epilogue: thread = one unit (tensor-memory lane); of a tile's frames warps 0-3 take the
         // first half, warps 4-7 the second
         pdl_wait();
         const int M = w.b_rows, N = w.a_rows;
-        const bool halved = w.halved();
-        const int grans = w.grans(), per = halved ? (grans + 1) >> 1 : grans;
-        const int g0 = halved ? (warp >> 2) * per : 0, ng = grans - g0 < per ? grans - g0 : per;
+        const int grans = w.n / (3 * digit::GRAN), per = (grans + 1) >> 1;
+        const int g0 = (warp >> 2) * per, ng = grans - g0 < per ? grans - g0 : per;
+        const int nb = w.nb();
         uint8_t* mine = staging + warp * STAGING;
         float* rs = reinterpret_cast<float*>(mine);      // frame scales of the input (2^-e) ...
         float* os = rs + 32;                             // ... and of the digits handed on (2^e)
@@ -350,158 +315,148 @@ signw_digit_kernel(const __grid_constant__ CUtensorMap map, const __grid_constan
         const Image im(M, N, true);                      // of the digits handed on
         const UnitBounds bounds = digits_out ? UnitBounds(g.img) : UnitBounds{0u, 0u, 0u};
         const int half_off = ((lane & 15) >> 2) * 16 + (lane & 3) * 4 + (lane >> 4) * 2;     // of this unit in the fp16 image
-        // byte transpose between the lanes l, l + 16, l + 8, l + 24 (sum and difference of a pair, then of the next): selectors of
-        // the two exchanges
-        const uint32_t sel16 = lane & 16 ? 0x3276u : 0x5410u, sel8 = lane & 8 ? 0x3175u : 0x6420u;
-        const float second = lane & 16 ? -1.0f : 1.0f;
-        uint32_t parities = 0u;                          // to wait for, of the parts
-        bool ok = true;
-        for (digit::Tiles t(w); ok && t.left > 0; t.next()) {
+        // byte transpose between the lanes l, l + 8, l + 16, l + 24: selectors of the two exchanges
+        const uint32_t sel16 = lane & 16 ? 0x3276u : 0x5410u, sel8 = lane & 8 ? 0x3715u : 0x6240u;
+        int tl = 0;
+        for (digit::Tiles t(w); t.left > 0; t.next(), ++tl) {
             const int n0 = t.a * (2 * digit::ROWS) + rank * digit::ROWS + (warp & 3) * 32, n = n0 + lane;
+            const int f0 = t.b * nb + g0 * digit::GRAN;
             const bool unit = n < N;
             const float sc = (g.scale && unit) ? __ldg(g.scale + n) : 1.0f;
             const float sh = (g.shift && unit) ? __ldg(g.shift + n) : 0.0f;
-            for (int part = halved ? 0 : warp >> 2; part < (halved ? digit::PARTS : (warp >> 2) + 1) && !w.beyond(t.b, part); ++part) {
-                const int f0 = ((t.b * digit::PARTS + part) * grans + g0) * digit::GRAN;
-                __syncwarp();
-                // the scale of the first frame and that of its digits; these serve all frames of this warp when they have the
-                // same scales, as they have in a chain whose outputs are not all small
-                float r0, o0;
-                bool same_in, same_out;
-                {
-                    const int f = f0 + lane;
-                    const bool one = n0 == 0 && f < M && lane < ng * digit::GRAN;     // of all warps that work on a frame
-                    float r = f < M ? __ldcg(g.in_scales + f) : 0.f, o = 0.f;
-                    const uint32_t word = g.in_sums && f < M ? __ldcg(g.in_sums + f) : 0u;
-                    if (word & kNaNOutput) r = __int_as_float(0x7FC00000);
-                    rs[lane] = r;
-                    if (digits_out) {
-                        const int e = bounds.exponent(magnitude_bound(r, word & ~kNaNOutput, g.K), SIGMOID);
-                        o = digit::power_of_two(e) * kOutputUnits;
-                        os[lane] = o;
-                        if (one) {
-                            reinterpret_cast<float*>(g.img_out + im.scales)[f] = digit::power_of_two(-e) * (1.0f / kOutputUnits);
-                            g.spare_sums[f] = 0u;
-                        }
+            __syncwarp();
+            // sc and the scale of the first frame, the scale of its digits; these serve all frames of this warp when they have the
+            // same scales, as they have in a chain whose outputs are not all small
+            float scr, o0;
+            bool same_in, same_out;
+            {
+                const int f = f0 + lane;
+                const bool one = n0 == 0 && f < M && lane < ng * digit::GRAN;     // of all warps that work on a frame
+                float r = f < M ? __ldcg(g.in_scales + f) : 0.f, o = 0.f;
+                const uint32_t word = g.in_sums && f < M ? __ldcg(g.in_sums + f) : 0u;
+                if (word & kNaNOutput) r = __int_as_float(0x7FC00000);
+                rs[lane] = r;
+                if (digits_out) {
+                    const int e = bounds.exponent(magnitude_bound(r, word & ~kNaNOutput, g.K), SIGMOID);
+                    o = dense::power_of_two(e);
+                    os[lane] = o;
+                    if (one) {
+                        reinterpret_cast<float*>(g.img_out + im.scales)[f] = dense::power_of_two(-e);
+                        g.spare_sums[f] = 0u;
                     }
-                    r0 = __shfl_sync(0xFFFFFFFFu, r, 0);
-                    o0 = __shfl_sync(0xFFFFFFFFu, o, 0);
-                    const bool none = f >= M || lane >= ng * digit::GRAN;
-                    same_in = __all_sync(0xFFFFFFFFu, none || r == r0);
-                    same_out = __all_sync(0xFFFFFFFFu, none || o == o0);
                 }
-                __syncwarp();
-                ok = warp_wait_relaxed(smem_u32(&bars->acc_full[part]), (parities >> part) & 1u, abort_flag, lane);
-                parities ^= 1u << part;
-                if (!ok) break;
-                tc_fence_after_sync();
-                const uint32_t taddr = tmem + ((uint32_t)((warp & 3) * 32) << 16) + (uint32_t)(part * w.n + g0 * 3 * digit::GRAN);
-                const bool any = f0 < M && n0 < N;                      // uniform over the warp
-                if (any) {
-                    uint32_t d[4][8];
-                    digit::load_granule(taddr, 3, d);
+                const float r0 = __shfl_sync(0xFFFFFFFFu, r, 0);
+                o0 = __shfl_sync(0xFFFFFFFFu, o, 0);
+                scr = sc * r0;                           // fma(sc, S r, sh) = fma(sc r, S, sh) as long as sc r is exact
+                const bool exact = sc == 0.f || (fabsf(scr) >= FLT_MIN && fabsf(scr) <= FLT_MAX);
+                const bool none = f >= M || lane >= ng * digit::GRAN;
+                same_in = __all_sync(0xFFFFFFFFu, exact && (none || r == r0));
+                same_out = __all_sync(0xFFFFFFFFu, none || o == o0);
+            }
+            __syncwarp();
+            const int b = tl & 1;
+            if (!warp_wait_relaxed(smem_u32(&bars->acc_full[b]), (uint32_t)((tl >> 1) & 1), abort_flag, lane)) break;
+            tc_fence_after_sync();
+            const uint32_t taddr = tmem + ((uint32_t)((warp & 3) * 32) << 16) + (uint32_t)(b * w.n + g0 * 3 * digit::GRAN);
+            const bool any = f0 < M && n0 < N;                      // uniform over the warp
+            if (any) {
+                uint32_t d[4][8];
+                digit::load_granule(taddr, 3, d);
 #pragma unroll 1
-                    for (int gi = 0; gi < ng; ++gi) {
-                        tmem_ld_wait();
-                        // S r = 65536 r high + r low: the scale costs no rounding of its own
-                        float y[8];
-                        if (same_in) {
-                            const float r16 = 65536.0f * r0;
+                for (int gi = 0; gi < ng; ++gi) {
+                    tmem_ld_wait();
+                    float S[8], y[8];
 #pragma unroll
-                            for (int i = 0; i < 8; ++i) y[i] = fmaf(digit::high_part((int)d[2][i]), r16, digit::low_part((int)d[0][i], (int)d[1][i]) * r0);
+                    for (int i = 0; i < 8; ++i) S[i] = fmaf(digit::high_part((int)d[2][i]), 65536.0f, digit::low_part((int)d[0][i], (int)d[1][i]));
+                    if (gi + 1 < ng) digit::load_granule(taddr + (uint32_t)(gi + 1) * 24, 3, d);
+                    if (same_in) {
+#pragma unroll
+                        for (int i = 0; i < 8; ++i) y[i] = fmaf(scr, S[i], sh);
+                    } else {
+                        const float4 ra = reinterpret_cast<const float4*>(rs)[2 * gi], rb = reinterpret_cast<const float4*>(rs)[2 * gi + 1];
+                        const float r[8] = {ra.x, ra.y, ra.z, ra.w, rb.x, rb.y, rb.z, rb.w};
+#pragma unroll
+                        for (int i = 0; i < 8; ++i) y[i] = fmaf(sc, S[i] * r[i], sh);
+                    }
+                    if (SIGMOID) {
+#pragma unroll
+                        for (int i = 0; i < 8; ++i) y[i] = 1.0f / (1.0f + expf(-y[i]));
+                    } else if (g.hardtanh) {
+#pragma unroll
+                        for (int i = 0; i < 8; ++i) y[i] = fminf(fmaxf(y[i], -1.0f), 1.0f);
+                    }
+                    const int f = f0 + gi * digit::GRAN;
+                    if (g.Y && unit) {
+                        float* dst = g.Y + (size_t)f * g.ldy + n;
+#pragma unroll
+                        for (int i = 0; i < 8; ++i, dst += g.ldy)
+                            if (f + i < M) *dst = y[i];
+                    }
+                    if (digits_out && f < M) {
+                        // digits of the 8 frames, byte q of word i; four frames at a time: bytes gathered per digit,
+                        // transposed over the four lanes whose units are neighbours in the image, stored as words
+                        uint32_t v[8];
+                        if (same_out) {
+#pragma unroll
+                            for (int i = 0; i < 8; ++i) y[i] *= o0;
                         } else {
-                            const float4 ra = reinterpret_cast<const float4*>(rs)[2 * gi], rb = reinterpret_cast<const float4*>(rs)[2 * gi + 1];
-                            const float r[8] = {ra.x, ra.y, ra.z, ra.w, rb.x, rb.y, rb.z, rb.w};
+                            const float4 oa = reinterpret_cast<const float4*>(os)[2 * gi], ob = reinterpret_cast<const float4*>(os)[2 * gi + 1];
+                            const float o[8] = {oa.x, oa.y, oa.z, oa.w, ob.x, ob.y, ob.z, ob.w};
 #pragma unroll
-                            for (int i = 0; i < 8; ++i) y[i] = fmaf(digit::high_part((int)d[2][i]), 65536.0f * r[i], digit::low_part((int)d[0][i], (int)d[1][i]) * r[i]);
+                            for (int i = 0; i < 8; ++i) y[i] *= o[i];
                         }
-                        if (gi + 1 < ng) digit::load_granule(taddr + (uint32_t)(gi + 1) * 24, 3, d);
 #pragma unroll
-                        for (int i = 0; i < 8; ++i) y[i] = fmaf(sc, y[i], sh);
-                        if (SIGMOID) {
-#pragma unroll
-                            for (int i = 0; i < 8; ++i) y[i] = 1.0f / (1.0f + expf(-y[i]));
-                        } else if (g.hardtanh) {
-#pragma unroll
-                            for (int i = 0; i < 8; ++i) y[i] = fminf(fmaxf(y[i], -1.0f), 1.0f);
+                        for (int i = 0; i < 8; ++i) {
+                            if (SIGMOID) y[i] = fmaxf(y[i], kNaNDigits);      // (a hardtanh unit gives -1 for a NaN)
+                            v[i] = unit ? digit::digits3(__float2int_rn(y[i])) : 0u;
                         }
-                        const int f = f0 + gi * digit::GRAN;
-                        if (g.Y && unit) {
-                            float* dst = g.Y + (size_t)f * g.ldy + n;
+                        uint8_t* dst = g.img_out + im.digits + ((size_t)(2 * (n0 >> 5) + ((lane >> 2) & 1)) * im.rows + (size_t)(f / digit::GRAN) * 24 + (lane >> 3)) * 16 + (lane & 3) * 4;
 #pragma unroll
-                            for (int i = 0; i < 8; ++i, dst += g.ldy)
-                                if (f + i < M) *dst = y[i];
-                        }
-                        if (digits_out && f < M) {
-                            // digits of the 8 frames, byte q of word i: the lower 16 lanes write the sums of the pairs (unit, unit + 16),
-                            // the upper ones the differences; four frames at a time: bytes gathered per digit,
-                            // transposed over the four lanes that are neighbours in the image, stored as words
-                            uint32_t v[8];
-                            if (same_out) {
+                        for (int h = 0; h < 2; ++h)
 #pragma unroll
-                                for (int i = 0; i < 8; ++i) y[i] *= o0;
-                            } else {
-                                const float4 oa = reinterpret_cast<const float4*>(os)[2 * gi], ob = reinterpret_cast<const float4*>(os)[2 * gi + 1];
-                                const float o[8] = {oa.x, oa.y, oa.z, oa.w, ob.x, ob.y, ob.z, ob.w};
-#pragma unroll
-                                for (int i = 0; i < 8; ++i) y[i] *= o[i];
+                            for (int q = 0; q < 3; ++q) {
+                                uint32_t x = q == 0 ? digit::gather_bytes<0>(v[4 * h], v[4 * h + 1], v[4 * h + 2], v[4 * h + 3])
+                                           : q == 1 ? digit::gather_bytes<1>(v[4 * h], v[4 * h + 1], v[4 * h + 2], v[4 * h + 3])
+                                                    : digit::gather_bytes<2>(v[4 * h], v[4 * h + 1], v[4 * h + 2], v[4 * h + 3]);
+                                x = __byte_perm(x, __shfl_xor_sync(0xFFFFFFFFu, x, 16), sel16);
+                                x = __byte_perm(x, __shfl_xor_sync(0xFFFFFFFFu, x, 8), sel8);
+                                *reinterpret_cast<uint32_t*>(dst + (q * 8 + h * 4) * 16) = x;
+                                if (q == 2) squares[gi * 64 + h * 32 + lane] = SIGMOID && (x & 0x80808080u) ? kNaNSquare : __dp4a((int)x, (int)x, 0);     // frame 4 h + lane / 8
                             }
+                    } else if (g.img_out && !digits_out) {
 #pragma unroll
-                            for (int i = 0; i < 8; ++i) {
-                                const float mine_y = unit ? y[i] : 0.f;
-                                float z = fmaf(second, mine_y, __shfl_xor_sync(0xFFFFFFFFu, mine_y, 16));
-                                if (SIGMOID && !(z == z)) z = kNaNDigits;      // (a hardtanh unit gives -1 for a NaN)
-                                v[i] = digit::digits3(__float2int_rn(z));
-                            }
-                            const int byte = digit::image_byte(4 * (n0 >> 6) + 2 == im.chunks, (n0 >> 5) & 1, lane & 7, 0);
-                            uint8_t* dst = g.img_out + im.digits + ((size_t)(4 * (n0 >> 6) + (byte >> 4)) * im.rows + (size_t)(f / digit::GRAN) * 24 + (lane >> 3)) * 16 + (byte & 15);
-#pragma unroll
-                            for (int h = 0; h < 2; ++h)
-#pragma unroll
-                                for (int q = 0; q < 3; ++q) {
-                                    uint32_t x = q == 0 ? digit::gather_bytes<0>(v[4 * h], v[4 * h + 1], v[4 * h + 2], v[4 * h + 3])
-                                               : q == 1 ? digit::gather_bytes<1>(v[4 * h], v[4 * h + 1], v[4 * h + 2], v[4 * h + 3])
-                                                        : digit::gather_bytes<2>(v[4 * h], v[4 * h + 1], v[4 * h + 2], v[4 * h + 3]);
-                                    x = __byte_perm(x, __shfl_xor_sync(0xFFFFFFFFu, x, 16), sel16);
-                                    x = __byte_perm(x, __shfl_xor_sync(0xFFFFFFFFu, x, 8), sel8);
-                                    *reinterpret_cast<uint32_t*>(dst + (q * 8 + h * 4) * 16) = x;
-                                    if (q == 2) squares[gi * 64 + h * 32 + lane] = SIGMOID && has_nan_digit(x) ? kNaNSquare : __dp4a((int)x, (int)x, 0);     // frame 4 h + lane / 8
-                                }
-                        } else if (g.img_out && !digits_out) {
-#pragma unroll
-                            for (int i = 0; i < 8; ++i) {
-                                const float v = unit ? y[i] : 0.f;
-                                const __half hi = __float2half_rn(v), lo = __float2half_rn(v - __half2float(hi));
-                                uint8_t* p = mine + 128 + (gi * digit::GRAN + i) * 64 + half_off;
-                                *reinterpret_cast<__half*>(p) = hi;
-                                *reinterpret_cast<__half*>(p + 2048) = lo;
-                            }
+                        for (int i = 0; i < 8; ++i) {
+                            const float v = unit ? y[i] : 0.f;
+                            const __half hi = __float2half_rn(v), lo = __float2half_rn(v - __half2float(hi));
+                            uint8_t* p = mine + 128 + (gi * digit::GRAN + i) * 64 + half_off;
+                            *reinterpret_cast<__half*>(p) = hi;
+                            *reinterpret_cast<__half*>(p + 2048) = lo;
                         }
                     }
                 }
-                digit::release_acc(bars, part, lane);
-                if (digits_out && any) {
-                    // of the eight parts of a frame's sum
-                    __syncwarp();
-                    const int4 a = reinterpret_cast<const int4*>(squares)[2 * lane], c = reinterpret_cast<const int4*>(squares)[2 * lane + 1];
-                    const int sum = (a.x + a.y) + (a.z + a.w) + (c.x + c.y) + (c.z + c.w);
-                    if (lane < ng * digit::GRAN && f0 + lane < M) {
-                        if (sum >= kNaNSquare) atomicOr(g.out_sums + f0 + lane, kNaNOutput);
-                        else atomicAdd(g.out_sums + f0 + lane, (uint32_t)sum);
-                    }
+            }
+            digit::release_acc(bars, b, lane);
+            if (digits_out && any) {
+                // of the eight parts of a frame's sum
+                __syncwarp();
+                const int4 a = reinterpret_cast<const int4*>(squares)[2 * lane], c = reinterpret_cast<const int4*>(squares)[2 * lane + 1];
+                const int sum = (a.x + a.y) + (a.z + a.w) + (c.x + c.y) + (c.z + c.w);
+                if (lane < ng * digit::GRAN && f0 + lane < M) {
+                    if (sum >= kNaNSquare) atomicOr(g.out_sums + f0 + lane, kNaNOutput);
+                    else atomicAdd(g.out_sums + f0 + lane, (uint32_t)sum);
                 }
-                if (any && g.img_out && !digits_out) {
-                    __syncwarp();
-                    if (lane < ng * digit::GRAN && f0 + lane < M) {
-                        const int f = f0 + lane;
-                        uint8_t* dst = g.img_out + ((size_t)(f >> 8) * words_for(N) + (n0 >> 5)) * 32768u + (size_t)(f & 255) * 16;
-                        const uint8_t* src = mine + 128 + lane * 64;
+            }
+            if (any && g.img_out && !digits_out) {
+                __syncwarp();
+                if (lane < ng * digit::GRAN && f0 + lane < M) {
+                    const int f = f0 + lane;
+                    uint8_t* dst = g.img_out + ((size_t)(f >> 8) * words_for(N) + (n0 >> 5)) * 32768u + (size_t)(f & 255) * 16;
+                    const uint8_t* src = mine + 128 + lane * 64;
 #pragma unroll
-                        for (int q = 0; q < 8; ++q)       // term q / 4, chunk q % 4
-                            *reinterpret_cast<uint4*>(dst + q * 4096) = *reinterpret_cast<const uint4*>(src + (q >> 2) * 2048 + (q & 3) * 16);
-                    }
-                    __syncwarp();
+                    for (int q = 0; q < 8; ++q)       // term q / 4, chunk q % 4
+                        *reinterpret_cast<uint4*>(dst + q * 4096) = *reinterpret_cast<const uint4*>(src + (q >> 2) * 2048 + (q & 3) * 16);
                 }
+                __syncwarp();
             }
         }
     }
@@ -542,14 +497,14 @@ int launch_signw_digit(const RealGemmArgs& r, void* workspace, bool image_ready,
         if (staged <= STAGED_MAX) x_digits_kernel<true><<<blocks, 256, staged, st>>>(x, img, first, next, units, clear, clear ? clear_words : 0);
         else x_digits_kernel<false><<<blocks, 256, 0, st>>>(x, img, first, next, units, clear, clear ? clear_words : 0);
     }
-    const int steps = ceil_div(r.K, digit::GROUP), pairs = sms / 2;
-    const digit::Work w{r.N, r.M, digit::tile_rows(r.N, r.M, steps, pairs), 3, steps, ceil_div(r.K, 32) & 1, 0};
+    const int steps = ceil_div(r.K, 32), pairs = sms / 2;
+    const dense::Work w{r.N, r.M, dense::tile_rows(r.N, r.M, steps, pairs), steps, 0};
     const Args a{r.Bb, r.ldb, img, reinterpret_cast<const float*>(img + im.scales), image_ready || digits_out ? sums(img, pos / 2) : nullptr,
                  digits_out ? sums(img, pos / 2 + 1) : nullptr, r.scale, r.shift,
                  Affine{r.next_scale, r.next_shift, r.next_N}, r.act == BNN_ACT_HARDTANH, r.K, r.Y, r.ldy, out, out_kind, digits_out ? sums(out, (pos + 1) / 2) : nullptr};
     CUtensorMap map;
     if (!encode_digit_map(&map, img + im.digits, im.rows, im.chunks, w.n / 2, digit::KB / 16)) return BNN_ERR_CUDA;
-    const long long tiles = digit::tile_count(r.N, r.M, w.n);
+    const long long tiles = dense::tile_count(r.N, r.M, w.n);
     if (launch_pdl(kern, dim3(2 * (int)(tiles < pairs ? tiles : pairs)), dim3(digit::THREADS), SMEM_BYTES, st, map, w, a, status) != cudaSuccess)
         return BNN_ERR_CUDA;
     return launch_status();

@@ -325,8 +325,16 @@ __device__ __forceinline__ void tmem_alloc_pair(uint32_t slot_smem, uint32_t nco
 __device__ __forceinline__ void tmem_dealloc_pair(uint32_t taddr, uint32_t ncols) {
     asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(taddr), "r"(ncols) : "memory");
 }
-// D[256 x N] (+)= A[256 x 64] * B[N x 64]^T on bytes, 32-bit integer sums; A in the tensor memory of both CTAs.  B's
-// descriptor comes as two words, so that stepping through a stage is 32-bit arithmetic.  A is 2:4 sparse, and half of it is stored: of every
+// D[256 x N] (+)= A[256 x 32] * B[N x 32]^T on bytes, 32-bit integer sums; A in the tensor memory of both CTAs.  B's
+// descriptor comes as two words, so that stepping through a stage is 32-bit arithmetic.
+__device__ __forceinline__ void mma_i8_ts_pair(uint32_t tmem_d, uint32_t tmem_a, uint32_t db_lo, uint32_t db_hi, uint32_t idesc, uint32_t accumulate) {
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t.reg .b64 b;\n\t"
+        "setp.ne.b32 p, %5, 0;\n\tmov.b64 b, {%2, %3};\n\t"
+        "tcgen05.mma.cta_group::2.kind::i8 [%0], [%1], b, %4, p;\n\t}"
+        ::"r"(tmem_d), "r"(tmem_a), "r"(db_lo), "r"(db_hi), "r"(idesc), "r"(accumulate) : "memory");
+}
+// D[256 x N] (+)= A[256 x 64] * B[N x 64]^T on bytes.  A is 2:4 sparse, and half of it is stored: of every
 // four consecutive positions two, in ascending order (32 bytes per row,
 // 8 columns), and which ones in the metadata, two 2-bit indices per four positions, the lower one in the lower
 // bits.  The metadata of a row of A lie in that row's lane, eight groups of four positions per column, the first in the lowest
