@@ -176,6 +176,26 @@ class ClockSampler:
 
 
 # ------------------------------------------------------------------ roofline bookkeeping
+def hidden_run_tile(frames, n, k):
+    """The kernel and units per tile that a run of binary hidden layers takes: the least of the library's estimates of the clocks
+    per layer (tile_units in xnor_gemm_res.cu, xnor_pair_clocks in xnor_gemm_pair.cu)."""
+    def up(a, b):
+        return -(-a // b)
+
+    nks, best = up(k, 256), None
+    for bn, slots, stage in ((192, 8, 480), (128, 12, 460), (96, 16, 450), (32, 48, 400)):
+        if nks <= slots and up(n, bn) <= SMS:
+            cost = up(up(frames, 128), SMS // up(n, bn)) * nks * stage + (0 if 2 * nks <= slots else bn * nks * 2 // 3)
+            if best is None or cost < best[0]:
+                best = (cost, "xnor_res_kernel", bn)
+    pairs = SMS // 2
+    if best and k > 2048 and nks <= 12 and up(n, 256) <= pairs:
+        cost = up(up(frames, 256), pairs // up(n, 256)) * nks * 660 + (max(2 * nks - 12, 0) * 540)
+        if cost < best[0]:
+            best = (cost, "xnor_pair_kernel", 256)
+    return best[1:] if best else (None, None)
+
+
 def xnor_kernel_name(k, xnor_path, prepared, stacked=True):
     """The kernel bnn_forward runs for a binary hidden layer of fan-in k (see bnn_api.cu); `stacked`: the
     layer is one of a run of equal layers that goes out as one launch."""
@@ -248,8 +268,10 @@ def layer_table(cfg, frames, peaks, sm_mhz, xnor_path="tensor", real_path="tenso
             pair_tiles = 2 * -(-frames // 256) * -(-cfg.hidden // 256)
             smem_bytes = pair_tiles * kpad * (128 * (0.5 + 0.5 + 0.125 + 0.125) + 128 * (0.125 + 0.125))
             kern = xnor_kernel_name(k, xnor_path, prepared, stacked and cfg.n_hidden > 2)
-            if kern == "xnor_res_kernel" and 2048 < k <= 3072 and frames >= 9000:     # a run of such layers
-                kern = "xnor_pair_kernel"
+            bn = 192
+            if kern == "xnor_res_kernel":
+                kern, bn = hidden_run_tile(frames, cfg.hidden, k)
+            if kern == "xnor_pair_kernel":
                 smem_bytes = pair_tiles * kpad * (128 * 0.5 + 128 * (0.125 + 0.125)) + SMS * kpad * 128 * 0.5
             if kern == "xnor_img_kernel":
                 # weights prepared once: their widened image arrives by bulk copies (4 bits written,
@@ -257,7 +279,6 @@ def layer_table(cfg, frames, peaks, sm_mhz, xnor_path="tensor", real_path="tenso
                 smem_bytes = tiles_m * tiles_n * kpad * (192 * (0.5 + 0.5) + 128 * (0.125 + 0.125))
             elif kern == "xnor_res_kernel":
                 # weights resident: written once per CTA, read by the tensor core on every tile visit
-                bn = 192 if k <= 2048 else 128
                 tiles_n = -(-cfg.hidden // bn)
                 smem_bytes = tiles_m * tiles_n * kpad * (bn * 0.5 + 128 * (0.125 + 0.125)) + SMS * kpad * bn * 0.5
             rows.append(dict(name="xnor_%d" % (l + 1), kernel=kern, work=work, unit="Tbop/s",
@@ -276,9 +297,9 @@ def layer_table(cfg, frames, peaks, sm_mhz, xnor_path="tensor", real_path="tenso
                 rows.append(dict(name="signw_%d" % (l + 1), kernel="x_split_kernel+signw_img_kernel",
                                  work=work, unit="TFLOP/s", bound="tensor", peak=peaks["bf16"], passes=2))
             else:
-                # three byte digits of the activations, exact 2:4 sparse integer MMAs at four times the half-precision rate
+                # three byte digits of the activations, exact integer MMAs at twice the half-precision rate
                 rows.append(dict(name="signw_%d" % (l + 1), kernel="signw_digit_kernel" if chained else "x_digits_kernel+signw_digit_kernel",
-                                 work=work, unit="TFLOP/s", bound="tensor", peak=4.0 * peaks["bf16"], passes=3))
+                                 work=work, unit="TFLOP/s", bound="tensor", peak=2.0 * peaks["bf16"], passes=3))
         else:
             rows.append(dict(name="signw_%d" % (l + 1), kernel="real_gemm_kernel", work=work, unit="TFLOP/s",
                              bound="alu", peak=fp32_peak))

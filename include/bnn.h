@@ -258,13 +258,15 @@ BNN_API size_t bnn_output_prepared_bytes(int C, int H);
 BNN_API int bnn_output_prepare(const float* Wout, int ldw, int C, int H,
                                void* prepared, size_t prepared_bytes, void* stream);
 
-/* The top layer on packed activations with exact sums.  bnn_output_prepare_digits writes the sums and differences of the pairs
- * (h, h + 16) of each class row once as fixed-point numbers of a scale of the row's own, in three byte digits (about 23 bits relative to the row's
- * largest weight; four digits, 31 bits, for the whole matrix when some row's largest weight exceeds 16 times the
- * row's mean magnitude), in the order the tensor core reads them; bnn_output_layer_digits multiplies the digits
- * with the activations' signs in integers (of a sum and a difference a pair of signs meets one: 2:4 sparsity), so that a logit is rounded once instead of at every step, and takes 3/8
+/* The top layer on packed activations with exact sums.  bnn_output_prepare_digits writes each class row once as fixed-point numbers
+ * of a scale of the row's own, in byte digits, in the order the tensor core reads them: sums and differences of the pairs (h, h + 16) in three digits, of
+ * which a pair of signs meets one (2:4 sparsity); or, for matrices of which that is less precise than single weights rounded to a power of two (their
+ * weights fill their range evenly, just below a power of two), single weights in three digits (about 23 bits relative to the row's
+ * largest weight); or single weights in four (31 bits) when some row's largest weight exceeds 16 times the
+ * row's mean magnitude.  bnn_output_layer_digits multiplies the digits
+ * with the activations' signs in integers, so that a logit is rounded once instead of at every step, and takes 3/8 (single weights: 3/4, 1)
  * of the tensor-core time of bnn_output_layer's fp16 terms:
- *   |z - exact| <= H * 1.01 * 2^-23 * max_h |Wout[c][h]|  (1.08 * 2^-31 with four digits) + one fp32 rounding + the bias
+ *   |z - exact| <= H * 1.01 * 2^-24 * max_h |Wout[c][h]|  (1.08 * 2^-31 with four digits) + one fp32 rounding + with a bias one more, of its
  * addition.
  * act_values : bnn_act_values of Hp.  H <= 2^15 (larger: BNN_ERR_UNSUPPORTED; use bnn_output_layer).
  * digits : device buffer, 256-byte aligned, at least bnn_output_digits_bytes(C, H) bytes.  In bnn_forward: the

@@ -258,12 +258,12 @@ size_t out_prepared_bytes(int C, int H);
 int launch_out_prepare(const float* W, int ldw, int C, int H, void* prepared, cudaStream_t st);
 // A top-layer kernel that is followed by the log-softmax gets `done` (out_done_bytes(M) zeroed bytes): one counter
 // per group_rows frames, then the row counter of the kernel that follows; every epilogue warp adds 1 to a group's
-// counter once its share of a tile of that group is stored; `need` (need4 where flag is given and *flag is set)
+// counter once its share of a tile of that group is stored; need[*form] (need[0] where no form is given)
 // arrivals complete a group.  launch_log_softmax_rows_follow, launched right behind, consumes the groups in order.
 struct FollowArgs {
     int* done;
-    int need, need4;
-    const int* flag;
+    int need[3];
+    const int* form;
     int group_rows;
 };
 constexpr int kFollowGroupRows = 256;    // the smallest group

@@ -1,9 +1,9 @@
-// The layers with binary weights on real-valued input (signw_digit_tc.cu): every number by itself in byte digits (digit_gemm.cuh has
-// the products of sums and differences of pairs), exact integer products with packed sign bits on the tensor cores (tcgen05 kind::i8), on CTA pairs.
+// The layers with binary weights on real-valued input (signw_digit_tc.cu), and top layers whose weights lose as pairs (out_digit_tc.cu): every number by itself in
+// byte digits (digit_gemm.cuh has the products of sums and differences of pairs), exact integer products with packed sign bits on the tensor cores (tcgen05 kind::i8), on CTA pairs.
 //
-//   S[a][b] = sum_k sigma[a][k] * v[b][k],    sigma in {-1, +1},  v = round(real[b][k] * 2^e_b)
+//   S[a][b] = sum_k sigma[a][k] * v[b][k],    sigma in {-1, +1} (or {0, 1}),  v = round(real[b][k] * 2^e_b)
 //
-// Every row of the real operand is scaled by a power of two of its own to a fixed-point number of about 23 bits and
+// Every row of the real operand is scaled by a power of two (out_digit_tc.cu: by any number) of its own to a fixed-point number of about 23 bits (or, with four digits, 31) and
 // written in base 256 with balanced digits, v = d0 + 256 d1 + 65536 d2 (-128 <= d <= 127), i.e. three bytes per
 // element; the 32-bit sums are exact (K <= kMaxKDigit), so the only rounding is that of v, at most
 // 1.01 * 2^-23 of the row's largest magnitude per element (1 / 0x7F7F7F, see scale_exponent), and those of the result.
@@ -52,10 +52,11 @@ struct Bars {
 // The tiles of a launch: 256 bit rows x `n` digit rows.
 struct Work {
     int a_rows, b_rows;        // rows of the two operands
-    int n;                     // digit rows per tile
+    int n, nd;                 // digit rows per tile, digits per element
     int steps;                 // groups of 32 positions of K
     int b_fast;
-    __device__ __forceinline__ int nb() const { return n / 3; }                             // b per tile
+    __device__ __forceinline__ int grans() const { return n / (GRAN * nd); }                // granules per tile
+    __device__ __forceinline__ int nb() const { return grans() * GRAN; }                    // b per tile
     __device__ __forceinline__ int a_tiles() const { return (a_rows + 2 * ROWS - 1) / (2 * ROWS); }
     __device__ __forceinline__ int b_tiles() const { return (b_rows + nb() - 1) / nb(); }
     __device__ __forceinline__ int a_stages() const { return n == MAX_N ? 2 : MAX_A_STAGES; }
@@ -64,23 +65,25 @@ struct Work {
     __device__ __forceinline__ uint32_t a_col() const { return 2u * (uint32_t)n; }          // bits start after the two accumulators
 };
 
+// By one thread, or every `step`th barrier of a kind by each of `step` threads (one thread takes half a microsecond).
+__device__ __forceinline__ void init_bars(Bars* bars, int first = 0, int step = 1) {
+    for (int s = first; s < 2 * MAX_A_STAGES; s += step) {
+        mbar_init(smem_u32(&bars->full_a[s]), 2 * TEAM_WARPS);     // rank 0: the widening warps of both CTAs
+        mbar_init(smem_u32(&bars->empty_a[s]), 1);
+    }
+    for (int s = first; s < MAX_B_STAGES; s += step) {
+        mbar_init(smem_u32(&bars->full_b[s]), 1);                  // rank 0: its copying thread (+ bytes of both CTAs)
+        mbar_init(smem_u32(&bars->empty_b[s]), 1);
+    }
+    for (int b = first; b < 2; b += step) {
+        mbar_init(smem_u32(&bars->acc_full[b]), 2);                // one commit of each issuing warp
+        mbar_init(smem_u32(&bars->acc_empty[b]), 2 * EPI_WARPS);   // rank 0: the epilogue warps of both CTAs
+        mbar_init(smem_u32(&bars->started[b]), 1);
+    }
+}
 // Common set-up; returns the tensor-memory base.  Called by all threads of both CTAs.
 __device__ __forceinline__ uint32_t set_up(Bars* bars, const TcStatus& status, int warp) {
-    if (threadIdx.x == 0) {
-        for (int s = 0; s < 2 * MAX_A_STAGES; ++s) {
-            mbar_init(smem_u32(&bars->full_a[s]), 2 * TEAM_WARPS);     // rank 0: the widening warps of both CTAs
-            mbar_init(smem_u32(&bars->empty_a[s]), 1);
-        }
-        for (int s = 0; s < MAX_B_STAGES; ++s) {
-            mbar_init(smem_u32(&bars->full_b[s]), 1);                  // rank 0: its copying thread (+ bytes of both CTAs)
-            mbar_init(smem_u32(&bars->empty_b[s]), 1);
-        }
-        for (int b = 0; b < 2; ++b) {
-            mbar_init(smem_u32(&bars->acc_full[b]), 2);                // one commit of each issuing warp
-            mbar_init(smem_u32(&bars->acc_empty[b]), 2 * EPI_WARPS);   // rank 0: the epilogue warps of both CTAs
-            mbar_init(smem_u32(&bars->started[b]), 1);
-        }
-    }
+    if (threadIdx.x == 0) init_bars(bars);
     return finish_set_up(bars, status, warp);
 }
 
@@ -93,7 +96,7 @@ __device__ __forceinline__ void copy_digits(const Work& w, const CUtensorMap* ma
     int s = 0;
     uint32_t ph = 1;          // parity to wait for on `empty`: a fresh barrier passes parity 1
     for (Tiles t(w); t.left > 0; t.next()) {
-        const int row0 = t.b * w.n + rank * (w.n / 2);
+        const int row0 = t.b * w.nb() * w.nd + rank * (w.n / 2);
         for (int k = 0; k < w.steps; k += KB / 32) {
             if (!mbar_wait(smem_u32(&bars->empty_b[s]), ph, abort_flag)) return;
             const uint32_t bar = smem_u32(&bars->full_b[s]);
@@ -104,17 +107,22 @@ __device__ __forceinline__ void copy_digits(const Work& w, const CUtensorMap* ma
     }
 }
 
-// Eight words of four bytes: word t holds bits t, t + 8, t + 16, t + 24 as +64 / -64: these
+// Eight words of four bytes: word t holds bits t, t + 8, t + 16, t + 24 as +64 / -64 (or, ZO, 64 / 0): 64 and -64
 // differ in the top bit of the byte alone, so that a word is a shift and one three-input logic operation (+1 / -1 would
 // take a third).  The sums come out 64 times as large.
+template <bool ZO>
 __device__ __forceinline__ void widen_bytes(uint32_t word, uint32_t* o) {
 #pragma unroll
-    for (int t = 0; t < 8; ++t) o[t] = (~(word << (7 - t)) & 0x80808080u) ^ 0x40404040u;
+    for (int t = 0; t < 8; ++t) {
+        if (ZO) o[t] = (t < 7 ? word << (6 - (t < 7 ? t : 6)) : word >> 1) & 0x40404040u;
+        else o[t] = (~(word << (7 - t)) & 0x80808080u) ^ 0x40404040u;
+    }
 }
 
 // Warps PROD_WARP0 ..: thread = one bit row of this CTA; each team takes 128 positions of every stage.  The packed row is
 // read 16 bytes (the team's share of a stage) at a time, two stages ahead of use.  Bits at positions >= K may
 // hold anything: the digits are zero there.
+template <bool ZO>
 __device__ __forceinline__ void widen_bits(const Work& w, const uint32_t* __restrict__ P, int ldp, Bars* bars, uint32_t tmem,
                                            int rank, int warp, int lane) {
     volatile int* abort_flag = &bars->wait.abort;
@@ -144,7 +152,7 @@ __device__ __forceinline__ void widen_bits(const Work& w, const uint32_t* __rest
     uint4 cur = fetch(), nxt = fetch();
     uint32_t o[32];
     auto widen = [&](const uint4& v) {
-        widen_bytes(v.x, o); widen_bytes(v.y, o + 8); widen_bytes(v.z, o + 16); widen_bytes(v.w, o + 24);
+        widen_bytes<ZO>(v.x, o); widen_bytes<ZO>(v.y, o + 8); widen_bytes<ZO>(v.z, o + 16); widen_bytes<ZO>(v.w, o + 24);
     };
     widen(cur);
     for (int it = 0; it < total; ++it) {

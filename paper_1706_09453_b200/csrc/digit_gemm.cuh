@@ -374,7 +374,7 @@ __device__ __forceinline__ float join4(int s0, int s1, int s2, int s3) {
 __device__ __forceinline__ float low_part(int s0, int s1) { return (float)(s1 * 4 + (s0 >> 6)); }
 // The high sum is below 2^22: adding 1.5 * 2^23 as an integer to its bits makes it a float without the
 // conversion unit, which the other conversion of every output already keeps busy.
-__device__ __forceinline__ float high_part(int s2) { return __int_as_float((s2 >> 6) + 0x4B400000) - 12582912.0f; }
+__device__ __forceinline__ float high_part(int s2, int more = 0) { return __int_as_float((s2 >> 6) + more + 0x4B400000) - 12582912.0f; }
 // Largest e (up to 140) such that mx * 2^e is a balanced number of three digits: at most 127 * (65536 + 256 + 1) = 0x7F7F7F.
 // mx >= 0; its exponent and fraction fields are compared with those of the limit.
 __device__ __forceinline__ int scale_exponent(float mx) {

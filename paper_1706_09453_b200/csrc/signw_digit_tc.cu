@@ -287,7 +287,7 @@ signw_digit_kernel(const __grid_constant__ CUtensorMap map, const __grid_constan
     const uint32_t tmem = dense::set_up(bars, status, warp);
 
     if (warp >= digit::PROD_WARP0) {
-        dense::widen_bits(w, g.Wp, g.ldwp, bars, tmem, rank, warp, lane);
+        dense::widen_bits<false>(w, g.Wp, g.ldwp, bars, tmem, rank, warp, lane);
     } else if (warp == digit::COPY_WARP) {
         // the image is the output of the kernel before this one in the stream: wait until that kernel has
         // completed and its writes are visible (the weights do not depend on it)
@@ -498,7 +498,7 @@ int launch_signw_digit(const RealGemmArgs& r, void* workspace, bool image_ready,
         else x_digits_kernel<false><<<blocks, 256, 0, st>>>(x, img, first, next, units, clear, clear ? clear_words : 0);
     }
     const int steps = ceil_div(r.K, 32), pairs = sms / 2;
-    const dense::Work w{r.N, r.M, dense::tile_rows(r.N, r.M, steps, pairs), steps, 0};
+    const dense::Work w{r.N, r.M, dense::tile_rows(r.N, r.M, steps, pairs), 3, steps, 0};
     const Args a{r.Bb, r.ldb, img, reinterpret_cast<const float*>(img + im.scales), image_ready || digits_out ? sums(img, pos / 2) : nullptr,
                  digits_out ? sums(img, pos / 2 + 1) : nullptr, r.scale, r.shift,
                  Affine{r.next_scale, r.next_shift, r.next_N}, r.act == BNN_ACT_HARDTANH, r.K, r.Y, r.ldy, out, out_kind, digits_out ? sums(out, (pos + 1) / 2) : nullptr};

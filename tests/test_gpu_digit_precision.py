@@ -49,6 +49,27 @@ KINDS = ["normal", "uniform 0.7", "uniform 0.99", "uniform 0.033", "positive", "
 
 
 @pytest.mark.parametrize("kind", KINDS)
+@pytest.mark.parametrize("h", [440, 2048])
+@pytest.mark.parametrize("values", [0, 1])
+def test_top_layer(env, kind, h, values):
+    torch, B, model = env
+    m, c = 500, 1000
+    w = rows(torch, kind, c, h)
+    hp = wl.make_bit_planes(m, h, 0.5, h, B.packed_pitch(h))
+    digits = torch.empty(B.bnn_output_digits_bytes(c, h), dtype=torch.uint8, device="cuda:0")
+    B.bnn_output_prepare_digits(w, digits)
+    z = torch.empty((m, c), device="cuda:0")
+    B.bnn_output_layer_digits(model.to_dev(hp), digits, None, z, h, log_softmax=False, values=values)
+    a = signs(torch, hp, h)
+    if values:
+        a = (a + 1) / 2
+    want = a @ w.double().T
+    ref = (a @ powers_of_two(torch, w, w.abs().amax(1)).T).float().double()
+    assert rms(z.double() - want) <= MARGIN * rms(ref - want)
+    assert B.bnn_device_status() == 0
+
+
+@pytest.mark.parametrize("kind", KINDS)
 @pytest.mark.parametrize("k", [440, 2048])
 @pytest.mark.parametrize("magnitude", [1.0, 1e-34])
 def test_binary_weights(env, kind, k, magnitude):
