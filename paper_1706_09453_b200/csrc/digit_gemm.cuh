@@ -399,13 +399,15 @@ __device__ __forceinline__ uint32_t gather_bytes(uint32_t a, uint32_t b, uint32_
 // Digit rows per part of a tile (192, 96 or 48).
 inline long long tile_count(int a_rows, int b_rows, int n) { return (long long)ceil_div(a_rows, 2 * ROWS) * ceil_div(b_rows, PARTS * n / 3); }
 // For `a_rows` x `b_rows` outputs of `steps` groups of 64 positions on `pairs` CTA pairs: the width with the least
-// estimated time.  A launch takes ceil(tiles / pairs) turns.
-inline int tile_rows(int a_rows, int b_rows, int steps, int pairs) {
-    constexpr struct { int n, clocks; } widths[] = {{192, 290}, {96, 170}, {48, 110}};
+// estimated time.  A launch takes ceil(tiles / pairs) turns of so many clocks per group and for an epilogue, by rows or (not of 48) by blocks; fitted to
+// 74 launches of each width on B200 (16 .. 16384 rows x 500 .. 6000, 5 .. 56 groups), of which the choice takes 0.2 % more than the best width on the mean, 3 % at most.
+// us, 192 / 96 / 48: 1461 x 1823, 7 groups 12.4 / 10.3 / 12.0; 4844 x 678, 8 groups 12.5 / 11.1 / 14.3; 8192 x 3400, 32 groups 74 / 88 / 158.
+inline int tile_rows(int a_rows, int b_rows, int steps, int pairs, bool blocks) {
+    constexpr struct { int n, clocks, by_rows, by_blocks; } widths[] = {{192, 215, 6300, 3300}, {96, 155, 3150, 1650}, {48, 142, 1900, 1900}};
     int best = 0;
     long long least = -1;
     for (const auto& s : widths) {
-        const long long cost = (tile_count(a_rows, b_rows, s.n) + pairs - 1) / pairs * ((long long)steps * s.clocks + 1200);
+        const long long cost = (tile_count(a_rows, b_rows, s.n) + pairs - 1) / pairs * ((long long)steps * s.clocks + (blocks ? s.by_blocks : s.by_rows));
         if (least < 0 || cost < least) { least = cost; best = s.n; }
     }
     return best;

@@ -460,7 +460,7 @@ out_digit_kernel(const __grid_constant__ CUtensorMap map, const __grid_constant_
 }
 
 int out_tile_rows(int M, int C, int H) {
-    return digit::tile_rows(M, C, ceil_div(H, digit::GROUP), device_sm_count() / 2);
+    return digit::tile_rows(M, C, ceil_div(H, digit::GROUP), device_sm_count() / 2, C % 4 == 0);
 }
 int single_tile_rows(int M, int C, int H) {
     return dense::tile_rows(M, C, ceil_div(H, 32), device_sm_count() / 2);
