@@ -262,7 +262,7 @@ int launch_out_prepare(const float* W, int ldw, int C, int H, void* prepared, cu
 // arrivals complete a group.  launch_log_softmax_rows_follow, launched right behind, consumes the groups in order.
 struct FollowArgs {
     int* done;
-    int need[3];
+    int need[4];
     const int* form;
     int group_rows;
 };

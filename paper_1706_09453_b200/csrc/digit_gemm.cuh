@@ -363,12 +363,13 @@ __device__ __forceinline__ void load_granule(uint32_t taddr, int nd, uint32_t (&
     tmem_ld8(taddr + 16, d[2]);
     if (nd == 4) tmem_ld8(taddr + 24, d[3]);
 }
-__device__ __forceinline__ float join4(int s0, int s1, int s2, int s3) {
+// (2^24 high + more is added)
+__device__ __forceinline__ float join4(int s0, int s1, int s2, int s3, int high = 0, int more = 0) {
     const int d0 = s0 >> 6;
     const int d1 = (s1 >> 6) + (d0 >> 8);
     const int d2 = (s2 >> 6) + (d1 >> 8);
     const int low = ((d2 & 255) << 16) | ((d1 & 255) << 8) | (d0 & 255);
-    return fmaf((float)((s3 >> 6) + (d2 >> 8)), 16777216.0f, (float)low);
+    return fmaf((float)((s3 >> 6) + (d2 >> 8) + high), 16777216.0f, (float)(low + more));
 }
 // low + 65536 high, the two parts of a sum of three digits.
 __device__ __forceinline__ float low_part(int s0, int s1) { return (float)(s1 * 4 + (s0 >> 6)); }

@@ -2,12 +2,14 @@
 //   z[m][c] = sum_h Wout[c][h] * a[m][h] + b[c].
 //
 // The weights are static, so they are prepared once (bnn_output_prepare_digits): as fixed-point numbers of a scale of each class's
-// own, written as byte digits in the order the tensor core reads shared memory.  Three forms, of which the device chooses one for the whole matrix
+// own, written as byte digits in the order the tensor core reads shared memory.  Four forms, of which the device chooses one for the whole matrix
 // (out_range_kernel) and the GEMM reads the choice from the image:
 //   pairs   sums and differences of pairs of weights in three digits (digit_gemm.cuh): half the tensor-core time of the others, for matrices of which it is as precise;
 //   three   every weight in three digits (digit_dense.cuh), about 23 bits relative to the class's largest weight;
 //   four    every weight in four digits (31 bits), where some class's largest weight is more than 16 times its mean magnitude.  Up to that,
-//           even if all H roundings of three digits, each at most 1.01 * 2^-24 of the largest weight, add up, a logit is within 1.01 * 2^-20 of sum |w|.
+//           even if all H roundings of three digits, each at most 1.01 * 2^-24 of the largest weight, add up, a logit is within 1.01 * 2^-20 of sum |w|;
+//   pairs, four   the same on pairs, for 2000 and more units, where the tensor core counts: single weights -> pairs, us, 16384 x 4000 x 3072 517 -> 431, 8192 x 3400 x 2048
+//           138 -> 120; but 8336 x 1370 x 416 33 -> 36, 4844 x 678 x 492 14 -> 18.
 //
 // The GEMM runs on CTA pairs, frames on the M side (tensor-memory lane = frame), class digits on the N side: a tile
 // is 256 frames x 128 (64, 32) classes on pairs, x 64 or 32 (48, 24) else.  The epilogue transposes through shared memory so that a store covers
@@ -30,7 +32,10 @@ namespace {
 using namespace tc;
 namespace dense = digit::dense;
 
-enum Form { kPairs = 0, kFour = 1, kThree = 2 };
+enum Form { kPairs = 0, kFour = 1, kThree = 2, kPairsFour = 3 };
+constexpr int kPairsFourMin = 2000;      // units
+__host__ __device__ constexpr bool in_pairs(int form) { return form == kPairs || form == kPairsFour; }
+__host__ __device__ constexpr int digits_of(int form) { return form == kFour || form == kPairsFour ? 4 : 3; }
 
 // The image: [Header, 256 bytes][largest magnitude per class][half of the largest |w1| + |w2| per class][scale per class][sum over all pairs per class][digits].
 struct Header {
@@ -60,8 +65,8 @@ DigitImage digit_image(int C, int H) {
 
 constexpr int STAGING_PITCH = 33;
 // Staging of the epilogue warps: 32 x 33 logits of each, or a block of 32 x 32 of each (1 KB aligned); then of each the scales and biases of its 32 classes and, for activations in (0,1),
-// the high parts of their sums over all pairs.
-constexpr int BLOCK = 32 * 32 * 4, ROWS_BYTES = 32 * STAGING_PITCH * 4, CONSTS = 3 * 32 * 4;
+// the high and low parts of their sums over all pairs.
+constexpr int BLOCK = 32 * 32 * 4, ROWS_BYTES = 32 * STAGING_PITCH * 4, CONSTS = 4 * 32 * 4;
 constexpr int STAGING = digit::EPI_WARPS * (ROWS_BYTES + CONSTS);
 static_assert(dense::RING_BYTES == digit::RING_BYTES, "either ring fits");
 constexpr int SMEM_BYTES = digit::RING_BYTES + STAGING + (int)sizeof(digit::Bars) + (int)sizeof(dense::Bars) + 1024;
@@ -74,11 +79,11 @@ constexpr double kTop = 8355711.0;       // 0x7F7F7F, the largest balanced numbe
 // double precision, and the smallest that keeps the largest within range is the most precise.  (Pairs: the margin is that of the
 // rounding of `half`.)  With four, where the rounding of the result is all that counts, a power of two, which costs none.
 __device__ __forceinline__ float class_scale(int form, float mx, float half) {
-    const float top = form == kPairs ? half : mx;
-    if (!(top > 0.f)) return top == 0.f ? 1.0f : top;         // no weights; a NaN
-    if (form != kFour) return __double2float_ru(form == kPairs ? 2.0 * (double)half / (kTop - 11.0) : (double)mx / kTop);
+    const double top = in_pairs(form) ? 2.0 * (double)half : (double)mx;
+    if (!(top > 0.0)) return (float)(top == 0.0 ? 1.0 : top);         // no weights; a NaN
+    if (digits_of(form) == 3) return __double2float_ru(top / (form == kPairs ? kTop - 11.0 : kTop));
     int e;
-    frexp((double)mx / 2e9, &e);
+    frexp(top / 2e9, &e);
     return (float)ldexp(1.0, e > -149 ? e : -149);
 }
 
@@ -128,7 +133,7 @@ __global__ void out_range_kernel(const float* __restrict__ W, int ldw, int C, in
 __global__ void out_digits_kernel(const float* __restrict__ W, int ldw, int C, int H, int Cpad8, int rows, int chunks,
                                   const float* __restrict__ mx, const float* __restrict__ tops, Header* head, float* __restrict__ scales,
                                   unsigned long long* __restrict__ totals, uint8_t* __restrict__ img) {
-    const int form = head->outlier ? kFour : head->balance > 0 ? kThree : kPairs, nd = form == kFour ? 4 : 3;
+    const int form = head->outlier ? (H >= kPairsFourMin ? kPairsFour : kFour) : head->balance > 0 ? kThree : kPairs, nd = digits_of(form);
     const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= (long long)chunks * Cpad8) return;
     if (i == 0) head->form = form;
@@ -146,7 +151,7 @@ __global__ void out_digits_kernel(const float* __restrict__ W, int ldw, int C, i
 #pragma unroll
     for (int x = 0; x < 4; ++x) {                // word x of the chunk
         uint32_t v[4];
-        if (form == kPairs) {                    // two pairs
+        if (in_pairs(form)) {                    // two pairs
 #pragma unroll
             for (int y = 0; y < 2; ++y) {
                 // the t, w and q = y of digit::image_byte(half, w, t, q) = 16 (ch % 4) + 4 x + 2 y
@@ -191,19 +196,22 @@ __device__ __forceinline__ void count_in(int* done, int tile) {
 }
 
 // What a class's sums are multiplied by, and what is added.  PAIRS01: pairs on activations in (0,1), where the class's sum over all pairs comes in, as
-// 65536 high + low: the high part is added to that of the products, which costs nothing; the low part goes with the bias.
+// 65536 high + low: the high part is added to that of the products, which costs nothing; the low part goes with the bias.  (Four digits: 2^24 high + low, which is
+// added to the low part.)
 template <bool PAIRS01>
 struct Class {
     float scale, bias;
-    int high;
-    __device__ __forceinline__ Class(const Logits& o, int c, bool some) : high(0) {
+    int high, low;
+    __device__ __forceinline__ Class(const Logits& o, int c, bool some, int nd) : high(0), low(0) {
         some = some && c < o.C;
         scale = some ? __ldg(o.scales + c) * (PAIRS01 ? 0.5f : 1.0f) : 0.f;
         bias = o.bias && some ? __ldg(o.bias + c) : 0.f;
         if (PAIRS01) {
             const long long total = some ? __ldg(o.totals + c) : 0;
-            high = (int)((total + 32768) >> 16);
-            bias = fmaf((float)(int)(total - ((long long)high << 16)), scale, bias);
+            const int bits = nd == 3 ? 16 : 24;
+            high = (int)((total + (1ll << (bits - 1))) >> bits);
+            low = (int)(total - ((long long)high << bits));
+            if (nd == 3) bias = fmaf((float)low, scale, bias);
         }
     }
 };
@@ -213,7 +221,7 @@ struct Classes {
     uint32_t smem;
     __device__ __forceinline__ Classes(uint8_t* staging, int warp)
         : consts(reinterpret_cast<float*>(staging + digit::EPI_WARPS * ROWS_BYTES + warp * CONSTS)), smem(smem_u32(consts)) {}
-    // `all`, or the high parts only.
+    // `all`, or the sums only.
     template <bool PAIRS01>
     __device__ __forceinline__ void put(const Class<PAIRS01>& c, bool all) {
         const int lane = threadIdx.x & 31;
@@ -222,7 +230,10 @@ struct Classes {
             consts[lane] = c.scale;
             consts[32 + lane] = c.bias;
         }
-        if (PAIRS01) reinterpret_cast<int*>(consts)[64 + lane] = c.high;
+        if (PAIRS01) {
+            reinterpret_cast<int*>(consts)[64 + lane] = c.high;
+            reinterpret_cast<int*>(consts)[96 + lane] = c.low;
+        }
         __syncwarp();
     }
     __device__ __forceinline__ static void get(uint32_t at, float (&v)[8]) {
@@ -237,6 +248,17 @@ struct Classes {
         if (PAIRS01) get(smem + 256 + g * 32, t);
 #pragma unroll
         for (int i = 0; i < 8; ++i) z[i] = fmaf(digit::high_part((int)d[2][i], __float_as_int(t[i])), 65536.0f, digit::low_part((int)d[0][i], (int)d[1][i]));
+    }
+    // The same with four digits.
+    template <bool PAIRS01>
+    __device__ __forceinline__ void sums4(const uint32_t (&d)[4][8], int g, float (&z)[8]) const {
+        float t[8] = {}, u[8] = {};
+        if (PAIRS01) {
+            get(smem + 256 + g * 32, t);
+            get(smem + 384 + g * 32, u);
+        }
+#pragma unroll
+        for (int i = 0; i < 8; ++i) z[i] = digit::join4((int)d[0][i], (int)d[1][i], (int)d[2][i], (int)d[3][i], __float_as_int(t[i]), __float_as_int(u[i]));
     }
     // Its logits, scale * (65536 high + low) + bias, of which the low part and the bias are rounded first, and the sum once.
     template <bool PAIRS01>
@@ -306,7 +328,7 @@ __device__ __forceinline__ uint64_t keep_policy() {
 }
 
 // Pairs, epilogue: thread = one frame (tensor-memory lane); of a tile's classes, or of either part's, warps 0-3 take
-// the first half, warps 4-7 the second.  by_blocks: the logits leave by tile stores (out_map).
+// the first half, warps 4-7 the second.  by_blocks (three digits): the logits leave by tile stores (out_map).
 template <bool ZO>
 __device__ __forceinline__ void pairs_epilogue(const digit::Work& w, const Logits& o, const CUtensorMap* out_map, bool by_blocks, uint8_t* staging,
                                                digit::Bars* bars, uint32_t tmem, int rank, int warp, int lane) {
@@ -324,8 +346,8 @@ __device__ __forceinline__ void pairs_epilogue(const digit::Work& w, const Logit
             const int c0 = ((t.b * digit::PARTS + part) * grans + g0) * digit::GRAN;
             const int n = g1 - g0, cl = store_lane(n);
             // before the wait for the accumulator, which then is read without waiting for these
-            const Class<ZO> y(o, c0 + lane, lane < n * digit::GRAN);
-            const bool scaled = by_blocks || !o.bias;
+            const Class<ZO> y(o, c0 + lane, lane < n * digit::GRAN, w.nd);
+            const bool scaled = by_blocks || (!o.bias && w.nd == 3);       // (with four digits the scale is a power of two)
             if (ZO || scaled) classes.put(y, scaled);
             const float scale = __shfl_sync(0xFFFFFFFFu, y.scale, cl), bias = __shfl_sync(0xFFFFFFFFu, y.bias, cl);
             const int f0 = t.a * (2 * digit::ROWS) + rank * digit::ROWS + (warp & 3) * 32;
@@ -333,7 +355,7 @@ __device__ __forceinline__ void pairs_epilogue(const digit::Work& w, const Logit
             parities ^= 1u << part;
             if (!ok) return;
             tc_fence_after_sync();
-            const uint32_t taddr = tmem + ((uint32_t)((warp & 3) * 32) << 16) + (uint32_t)(part * w.n) + (uint32_t)g0 * 24;
+            const uint32_t taddr = tmem + ((uint32_t)((warp & 3) * 32) << 16) + (uint32_t)(part * w.n + g0 * digit::GRAN * w.nd);
             if (by_blocks) {
                 // 32 frames x 32 classes: a tile store, which drops what lies outside
                 uint32_t d[4][8];
@@ -367,7 +389,8 @@ __device__ __forceinline__ void pairs_epilogue(const digit::Work& w, const Logit
             } else {
                 auto released = [&] { digit::release_acc(bars, part, lane); };
                 if (scaled) store_rows<true>(o, mine, taddr, n, 3, f0, c0, scale, bias, pol, [&](const uint32_t (&d)[4][8], int g, float (&z)[8]) { classes.logits3<ZO>(d, g, z); }, released);
-                else store_rows<false>(o, mine, taddr, n, 3, f0, c0, scale, bias, pol, [&](const uint32_t (&d)[4][8], int g, float (&z)[8]) { classes.sums3<ZO>(d, g, z); }, released);
+                else if (w.nd == 3) store_rows<false>(o, mine, taddr, n, 3, f0, c0, scale, bias, pol, [&](const uint32_t (&d)[4][8], int g, float (&z)[8]) { classes.sums3<ZO>(d, g, z); }, released);
+                else store_rows<false>(o, mine, taddr, n, 4, f0, c0, scale, bias, pol, [&](const uint32_t (&d)[4][8], int g, float (&z)[8]) { classes.sums4<ZO>(d, g, z); }, released);
                 if (o.done) count_in(o.done, t.a);
             }
         }
@@ -396,8 +419,8 @@ __device__ __forceinline__ void single_weights(const dense::Work& w, const Logit
         for (digit::Tiles t(w); t.left > 0; t.next(), ++tl) {
             const int c0 = t.b * w.nb() + g0 * digit::GRAN, b = tl & 1;
             const int n = g1 - g0, cl = store_lane(n);
-            const Class<false> y(o, c0 + lane, lane < n * digit::GRAN);
-            const bool scaled = !o.bias && w.nd == 3;        // (with four digits the scale is a power of two)
+            const Class<false> y(o, c0 + lane, lane < n * digit::GRAN, w.nd);
+            const bool scaled = !o.bias && w.nd == 3;        // as above
             if (scaled) classes.put(y, true);
             const float scale = __shfl_sync(0xFFFFFFFFu, y.scale, cl), bias = __shfl_sync(0xFFFFFFFFu, y.bias, cl);
             const int f0 = t.a * (2 * digit::ROWS) + rank * digit::ROWS + (warp & 3) * 32;
@@ -407,11 +430,7 @@ __device__ __forceinline__ void single_weights(const dense::Work& w, const Logit
             auto released = [&] { digit::release_acc(bars, b, lane); };
             if (scaled) store_rows<true>(o, mine, taddr, n, 3, f0, c0, scale, bias, pol, [&](const uint32_t (&d)[4][8], int g, float (&z)[8]) { classes.logits3<false>(d, g, z); }, released);
             else if (w.nd == 3) store_rows<false>(o, mine, taddr, n, 3, f0, c0, scale, bias, pol, [&](const uint32_t (&d)[4][8], int g, float (&z)[8]) { classes.sums3<false>(d, g, z); }, released);
-            else
-                store_rows<false>(o, mine, taddr, n, 4, f0, c0, scale, bias, pol, [&](const uint32_t (&d)[4][8], int, float (&z)[8]) {
-#pragma unroll
-                    for (int i = 0; i < 8; ++i) z[i] = digit::join4((int)d[0][i], (int)d[1][i], (int)d[2][i], (int)d[3][i]);
-                }, released);
+            else store_rows<false>(o, mine, taddr, n, 4, f0, c0, scale, bias, pol, [&](const uint32_t (&d)[4][8], int g, float (&z)[8]) { classes.sums4<false>(d, g, z); }, released);
             if (o.done) count_in(o.done, t.a);
         }
     }
@@ -421,7 +440,7 @@ __device__ __forceinline__ void single_weights(const dense::Work& w, const Logit
 template <bool ZO>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(digit::REG_THREADS, 1)
 out_digit_kernel(const __grid_constant__ CUtensorMap map, const __grid_constant__ CUtensorMap single_map, const __grid_constant__ CUtensorMap out_map, int by_blocks,
-                 const uint32_t* __restrict__ Hp, int ldhp, const int* __restrict__ form, const __grid_constant__ digit::Work w, dense::Work single, const __grid_constant__ Logits o,
+                 const uint32_t* __restrict__ Hp, int ldhp, const int* __restrict__ form, digit::Work w, dense::Work single, const __grid_constant__ Logits o,
                  TcStatus status) {
     extern __shared__ uint8_t smem_raw[];
     // A kernel launched behind this one with programmatic stream serialisation (the log-softmax that
@@ -443,8 +462,8 @@ out_digit_kernel(const __grid_constant__ CUtensorMap map, const __grid_constant_
                      // this one: 2 us of 35 on 256 frames of the small network
     const int f = __ldg(form);
 
-    if (f != kPairs) {
-        single.nd = f == kFour ? 4 : 3;
+    w.nd = single.nd = digits_of(f);
+    if (!in_pairs(f)) {
         single_weights<ZO>(single, o, &single_map, Hp, ldhp, ring, staging, more, tmem, rank, warp, lane);
         if (more->wait.abort) bars->wait.abort = 1;
     } else if (warp >= digit::PROD_WARP0) {
@@ -454,7 +473,7 @@ out_digit_kernel(const __grid_constant__ CUtensorMap map, const __grid_constant_
     } else if (warp >= digit::EPI_WARPS) {
         if (rank == 0 && warp <= digit::MMA_WARP2) digit::issue(w, ring, bars, tmem, warp - digit::MMA_WARP);
     } else {
-        pairs_epilogue<ZO>(w, o, &out_map, by_blocks != 0, staging, bars, tmem, rank, warp, lane);
+        pairs_epilogue<ZO>(w, o, &out_map, by_blocks && w.nd == 3, staging, bars, tmem, rank, warp, lane);
     }
     digit::tear_down(bars, status, warp, tmem);
 }
@@ -493,9 +512,10 @@ bool out_digit_can_be_followed(int M, int C, int H) {
 }
 FollowArgs out_digit_follow(const void* image, int M, int C, int H, int* done) {
     const int n = out_tile_rows(M, C, H);
-    // the epilogue warps of every tile (and part)
-    auto single = [&](int nd) { return ceil_div(C, single_tile_rows(M, C, H) / (digit::GRAN * nd) * digit::GRAN) * 2 * digit::EPI_WARPS; };
-    return FollowArgs{done, {ceil_div(C, n / 3) * (n == digit::MAX_N ? 2 : 1) * digit::EPI_WARPS, single(4), single(3)},
+    // the epilogue warps of every tile or part, by Form
+    auto parts = [&](int rows, int nd) { return ceil_div(C, rows / (digit::GRAN * nd) * digit::GRAN) * digit::EPI_WARPS; };
+    const int per = n == digit::MAX_N ? 2 : 1, s = single_tile_rows(M, C, H);
+    return FollowArgs{done, {parts(n, 3) * per, parts(s, 4) * 2, parts(s, 3) * 2, parts(n, 4) * per},
                       &static_cast<const Header*>(image)->form, 2 * digit::ROWS};
 }
 

@@ -354,7 +354,7 @@ int launch_out_prepare(const float* W, int ldw, int C, int H, void* prepared, cu
 
 FollowArgs out_tc_follow(int C, int* done) {
     const int need = ceil_div(C, BC) * EPI_WARPS;
-    return FollowArgs{done, {need, need, need}, nullptr, FN};
+    return FollowArgs{done, {need, need, need, need}, nullptr, FN};
 }
 // With no more tiles than SMs every tile ends at about the same time: nothing for a following kernel to
 // overlap with (measured: 1-2 % slower than two launches in a row on 256 frames).

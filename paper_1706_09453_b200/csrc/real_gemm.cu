@@ -387,7 +387,7 @@ log_softmax_rows_follow_kernel(float* __restrict__ Z, int ldz, int M, int C, con
     __shared__ int claim;
     int* const done = follow.done;
     const int form = follow.form ? __ldg(follow.form) : 0;
-    const int group_rows = follow.group_rows, need = form == 0 ? follow.need[0] : form == 1 ? follow.need[1] : follow.need[2];
+    const int group_rows = follow.group_rows, need = form == 0 ? follow.need[0] : form == 1 ? follow.need[1] : form == 2 ? follow.need[2] : follow.need[3];
     int* next_row = done + ceil_div(M, group_rows);
     int pending = 0, ready_group = -1;   // thread 0: the claim in flight; the last group seen complete
     int par = 0;
