@@ -115,6 +115,10 @@ constexpr int kMaxKDigit = 1 << 15;
 int launch_xnor_tc(const uint32_t* Ap, int ldap, const uint32_t* Wp, int ldwp, int M, int N,
                    int K, int32_t* C, int ldc, const int32_t* thr, const uint32_t* flip,
                    uint32_t* out_bits, int ldob, int zo, cudaStream_t st);
+// The same on single CTAs (xnor_gemm_cta.cu).
+int launch_xnor_cta(const uint32_t* Ap, int ldap, const uint32_t* Wp, int ldwp, int M, int N,
+                   int K, int32_t* C, int ldc, const int32_t* thr, const uint32_t* flip,
+                   uint32_t* out_bits, int ldob, int zo, cudaStream_t st);
 // The same product with the unit operand given as the image launch_xnor_prepare built from the
 // packed weights (xnor_gemm_img.cu): xnor_image_bytes(N, K) bytes, 256-byte aligned.
 size_t xnor_image_bytes(int N, int K);

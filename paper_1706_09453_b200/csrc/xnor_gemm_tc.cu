@@ -19,14 +19,14 @@
 // w holds, in nibble i, bit 4i + t of w:   ((w << (3 - t)) & 0x88888888) ^ 0xAAAAAAAA
 // (sign bit = NOT the input bit, exponent field = 01).
 //
-// A pair of CTAs (cluster of two, one per SM of a TPC) works on a tile of 256 frames x two parts of 128 units (64 where that fills more SMs, part_units): each CTA widens
-// its own 128 frames and half of the units, where a CTA by itself would widen all of them.  Roles in a CTA of 27 warps
+// A pair of CTAs (cluster of two, one per SM of a TPC) works on a tile of 256 frames x two parts of 128 units (64 where that fills more SMs, launch_xnor_tc): each CTA widens
+// its own 128 frames and half of the units, where a CTA by itself (xnor_gemm_cta.cu) widens all of them.  Roles in a CTA of 27 warps, with parts of 64 units 23
 // (persistent, one CTA per SM):
-//   warp 26      one thread issues 2-D TMA tile loads of the packed rows (64 bytes per row =
+//   the last     one thread issues 2-D TMA tile loads of the packed rows (64 bytes per row =
 //                two stages) into a staging ring (64-byte swizzle, no multicast)
 //   warps 10-17  two teams widen the frame rows, thread = one row, 32 bytes -> 128 bytes per stage,
 //                written to tensor memory (the MMA reads its A operand from there); they take alternate stages
-//   warps 18-25  two teams widen the unit rows the same way into shared memory
+//   warps 18-25  (18-21) two teams widen the unit rows the same way into shared memory
 //   warps 8, 9   rank 0: issue the MMAs (4 per stage and part, K = 64 each) and the commits, which arrive in both CTAs; a warp has a part
 //                with its accumulator.  The epilogue reads one accumulator after the other, so one part runs ahead (by
 //                up to the ring's six stages) and its epilogue is hidden behind the other's MMAs.
@@ -41,7 +41,7 @@
 // tiles are 3.5 turns of 74 pairs).
 #include "bnn_common.cuh"
 #include "tcgen05.cuh"
-#include "xnor_widen.cuh"
+#include "xnor_both.cuh"
 
 namespace bnn {
 
@@ -94,29 +94,9 @@ struct ProducerArgs {
     Control* ctl;
     volatile int* abort_flag;
     int total;            // stages of all tiles of this pair
-    int nks, kw;
-    uint32_t tmask;
+    both::Rows rows;
     int rank, lane;
 };
-
-// The eight 16-byte chunks of one widened row and stage; `ks` is the stage's index in the row.
-// ZO: the row's bits stand for (0,1) instead of (-1,+1); RAGGED: the last stage has positions >= K, whose nibbles are set to +0 (in the
-// unit rows; what the frame rows hold there then does not matter).
-template <bool ZO, bool RAGGED>
-__device__ __forceinline__ void widen_stage(const ProducerArgs& a, int ks, const uint4& v0, const uint4& v1, uint4 (&o)[8]) {
-    const uint32_t w[8] = {v0.x, v0.y, v0.z, v0.w, v1.x, v1.y, v1.z, v1.w};
-    if (RAGGED && ks == a.nks - 1) {
-#pragma unroll
-        for (int c = 0; c < 8; ++c) {
-            const int g = 8 * ks + c;   // index of the word in the row
-            const uint32_t valid = g < a.kw - 1 ? 0xFFFFFFFFu : (g == a.kw - 1 ? a.tmask : 0u);
-            o[c] = widen_masked(w[c], valid);
-        }
-    } else {
-#pragma unroll
-        for (int c = 0; c < 8; ++c) o[c] = ZO ? widen01(w[c]) : widen(w[c]);
-    }
-}
 
 // Producer of an operand: thread = row `r` of every tile of this CTA's half; team `team` takes one of the two stages of every
 // staging group.  FRAMES: widened rows go to tensor memory, else (unit rows) to shared memory.
@@ -144,7 +124,7 @@ __device__ __forceinline__ void produce(const ProducerArgs& a, int r, int team) 
         const uint32_t src = stg0 + gslot * GROUP_BYTES;
         const uint4 v0 = lds128u(src + lo), v1 = lds128u(src + (lo ^ 16u));
         uint4 o[8];
-        widen_stage<ZO, RAGGED>(a, ks, v0, v1, o);
+        both::widen_stage<ZO, RAGGED>(a.rows, ks, v0, v1, o);
         if (!warp_wait(smem_u32(&ctl->empty[s]), ph, a.abort_flag, a.lane)) return;
         if (FRAMES) {
             // 32-bit column 4c + t of the stage = word t of chunk c: the byte order of the
@@ -173,7 +153,7 @@ __device__ __forceinline__ void produce(const ProducerArgs& a, int r, int team) 
             mbar_arrive(smem_u32(&ctl->group_empty[gslot]));
         }
         ks += TEAMS;
-        if (ks >= 2 * ceil_div(a.nks, 2)) ks = team;
+        if (ks >= 2 * a.rows.groups()) ks = team;
         if (++gslot == GROUPS) { gslot = 0; gph ^= 1u; }
         if ((s += TEAMS) >= STAGES) { s = team; ph ^= 1u; }
     }
@@ -197,8 +177,8 @@ xnor_tc_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_constant__
     volatile int* abort_flag = &ctl->wait.abort;
 
     const int warp = warp_index(), lane = threadIdx.x & 31, rank = (int)cluster_rank();
-    const int kw = words_for(K);
-    const int nks = ceil_div(K, BK);
+    const both::Rows rows(K);
+    const int nks = rows.nks;
     const int n_tiles = ceil_div(N, BN), tiles = ceil_div(M, 2 * BM) * n_tiles;
     const int pair = (int)blockIdx.x >> 1, pairs = (int)gridDim.x >> 1;      // tiles pair, pair + pairs, ..; unit tiles vary fastest
 
@@ -243,13 +223,12 @@ xnor_tc_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_constant__
 
     if (warp >= PROD_WARP0) {
         const int my_tiles = pair < tiles ? (tiles - 1 - pair) / pairs + 1 : 0;
-        const ProducerArgs pa{smem_u32(smem), tmem, ctl, abort_flag, my_tiles * 2 * ceil_div(nks, 2), nks, kw, tail_mask(K), rank, lane};
-        const bool ragged = (kw % 8 != 0) || pa.tmask != 0xFFFFFFFFu;   // the last stage has positions >= K
+        const ProducerArgs pa{smem_u32(smem), tmem, ctl, abort_flag, my_tiles * 2 * rows.groups(), rows, rank, lane};
         if (warp == TMA_WARP) {
             // ---------------- one thread feeds the staging ring, a group of two stages at a time
             if (lane == 0) {
                 const uint32_t stg = smem_u32(smem) + STAGES * STAGE_BYTES;
-                const int ng = ceil_div(nks, 2);
+                const int ng = rows.groups();
                 int slot = 0;
                 uint32_t ph = 1;
                 bool ok = true;
@@ -274,7 +253,7 @@ xnor_tc_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_constant__
             else produce<PN, true, false, false>(pa, row, team);
         } else {
             const int pw = warp - PROD_WARP0 - TEAMS * A_WARPS, team = pw / B_WARPS, row = (pw - team * B_WARPS) * 32 + lane;
-            ragged ? produce<PN, false, false, true>(pa, row, team) : produce<PN, false, false, false>(pa, row, team);
+            rows.ragged() ? produce<PN, false, false, true>(pa, row, team) : produce<PN, false, false, false>(pa, row, team);
         }
     } else if (warp >= EPI_WARPS) {
         // ---------------- MMA issue: two converged warps of rank 0, each with its part of every tile.  What an issuing warp does
@@ -295,7 +274,7 @@ xnor_tc_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_constant__
             pacc ^= 1u;
             tc_fence_after_sync();
             const bool beyond = (tile % n_tiles) * BN + part * PN >= N;      // no such units: nothing to multiply
-            for (int ks = 0; ks < 2 * ceil_div(nks, 2); ++ks) {
+            for (int ks = 0; ks < 2 * rows.groups(); ++ks) {
                 ok = warp_wait(smem_u32(&ctl->full[s]), ph, abort_flag, lane);
                 if (!ok) break;
                 tc_fence_after_sync();
@@ -326,7 +305,7 @@ xnor_tc_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_constant__
         for (int tile = pair; tile < tiles && ok; tile += pairs, par ^= 1u) {
             const int m0 = (tile / n_tiles) * (2 * BM) + rank * BM + quarter * 32, m = m0 + lane;
             for (int part = 0; part < PARTS; ++part) {
-                const int n0 = (tile % n_tiles) * BN + part * PN + half * (PN / 2);       // the first of this warp's 64 units
+                const int n0 = (tile % n_tiles) * BN + part * PN + half * (PN / 2);       // the first of this warp's PN / 2 units
                 if (SIGN_PACK) {
 #pragma unroll
                     for (int h = 0; h < PN / 64; ++h) ctl->T[warp][h * 32 + lane] = kMagicBits + (n0 + h * 32 + lane < N ? thr[n0 + h * 32 + lane] : 0);
@@ -354,61 +333,12 @@ xnor_tc_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_constant__
                     int q[32];
 #pragma unroll
                     for (int j = 0; j < 32; ++j) q[j] = __float_as_int(__uint_as_float(acc[j]) + magic);
-                    if (STORE_C) {
-                        // Each thread parks its 32 integers (128 bytes of one output row) in shared memory, 16-byte
-                        // chunk i at i ^ (row % 8).  One thread then has the 32 x 128-byte block stored, which goes on while
-                        // the warp turns to the next 32 columns.  (Measured on B200: written by the warp with 16-byte stores,
-                        // 8 lanes to a row, the epilogue took as long as 16 stages of MMAs.)
-                        // A tile store clips a row to 16 bytes, not to elements, and wants an aligned pitch.  Elsewhere the
-                        // warp writes the block a row at a time, and each row from the 32-byte sector its first
-                        // column lies in (from the block before) to the one of its last column, which is left to the next
-                        // block: every store but those at the tile's edges then covers whole sectors.  (4096 x 2048 x
-                        // 4095, microseconds: a thread a row 102, rows of 32 columns 68, whole sectors 57; 4096 columns 29.)
-                        const bool whole = tma_c && (nb + 31 < N || N % 4 == 0);
-                        const int which = PN == 64 ? part : g & 1;       // of the warp's two blocks, in turn
-                        const uint32_t blk = cstage + (uint32_t)((warp * 2 + which) * 4096);
-                        if (lane == 0) bulk_wait_read<1>();      // the block's store of two rounds ago has read it
-                        __syncwarp();
-#pragma unroll
-                        for (int i = 0; i < 8; ++i)
-                            sts128(blk + lane * 128 + ((i ^ (lane & 7)) << 4), (uint32_t)(q[4 * i] - kMagicBits), (uint32_t)(q[4 * i + 1] - kMagicBits),
-                                   (uint32_t)(q[4 * i + 2] - kMagicBits), (uint32_t)(q[4 * i + 3] - kMagicBits));
-                        if (whole) fence_proxy_async_smem();
-                        __syncwarp();
-                        if (whole) {
-                            if (lane == 0 && nb < N && m0 < M) tma_store_2d(&mapC, nb, m0, blk);
-                        } else if (nb < N) {
-                            const int rows = M - m0 < 32 ? M - m0 : 32;
-                            const bool tail = g + 1 == PN / 64 || nb + 32 >= N;     // the last block of this warp's row
-                            int32_t* dst = C + (size_t)m0 * ldc + nb;
-                            uint32_t at = (uint32_t)(reinterpret_cast<uintptr_t>(dst) >> 2);   // in words; its low bits count
-                            const uint32_t both = cstage + (uint32_t)(warp * 8192);
-#pragma unroll 4
-                            for (int r = 0; r < rows; ++r, dst += ldc, at += (uint32_t)ldc) {
-                                const int back = g == 0 ? 0 : (int)(at & 7u);       // columns of the block before that this store takes along
-                                const int lead = (int)(at & 7u) - back;             // the warp's first block starts inside a sector
-                                const int col = lane - back - lead;                 // from -7 to 31
-                                const uint32_t buf = both + (uint32_t)((which ^ (col < 0)) * 4096) + r * 128;
-                                const uint32_t v = lds32u(buf + ((((uint32_t)col >> 2) & 7u) ^ ((uint32_t)r & 7u)) * 16 + (col & 3) * 4);
-                                if (col >= -back && nb + col < N) dst[col] = (int32_t)v;
-                                if (tail) {
-                                    const int rest = col + 32;                      // the columns that stay over
-                                    const uint32_t t = lds32u(both + (uint32_t)(which * 4096) + r * 128 + ((((uint32_t)rest >> 2) & 7u) ^ ((uint32_t)r & 7u)) * 16 + (rest & 3) * 4);
-                                    if (rest < 32 && nb + rest < N) dst[rest] = (int32_t)t;
-                                }
-                            }
-                        }
-                        if (lane == 0) bulk_commit();            // (an empty group keeps the count)
-                    }
+                    if (STORE_C)
+                        both::store_block(cstage + (uint32_t)(warp * 8192), PN == 64 ? part : g & 1, g == 0, g + 1 == PN / 64, q, &mapC, tma_c, C, ldc, M, N,
+                                          m0, nb, lane);
                     if (SIGN_PACK) {
-                        // bit = (dot - thr >= 0); the sign bits are shifted in from the top, element 31
-                        // first, so element j ends up in bit j, inverted.
-                        uint32_t wd = 0u;
-#pragma unroll
-                        for (int j = 31; j >= 0; --j)
-                            wd = __funnelshift_l((uint32_t)(q[j] - ctl->T[warp][g * 32 + j]), wd, 1);
                         const int valid = N - nb;  // columns of this word that exist
-                        words[g] = valid > 0 ? (~wd ^ __ldg(flip + (nb >> 5))) & (valid < 32 ? (1u << valid) - 1u : 0xFFFFFFFFu) : 0u;
+                        words[g] = valid > 0 ? (both::sign_word(q, ctl->T[warp] + g * 32) ^ __ldg(flip + (nb >> 5))) & (valid < 32 ? (1u << valid) - 1u : 0xFFFFFFFFu) : 0u;
                     }
                 }
                 if (SIGN_PACK) {
@@ -439,17 +369,6 @@ xnor_tc_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_constant__
     if (threadIdx.x == 0 && ctl->wait.abort) atomicExch(status.word, 1);
 }
 
-// Units per part.  A launch takes ceil(tiles / pairs) turns of nks stages and an epilogue; a stage of 64 + 64 units takes more than half the
-// clocks of one of 128 + 128, because the frames are widened all the same.  Measured on B200, us, 128 / 64 units: 300 x 8000 x 1501 24.4 / 18.5,
-// 2500 x 2000 x 2503 24.8 / 22.1, 5000 x 1500 x 1203 23.5 / 20.5.
-int part_units(int M, int N, int K, int pairs) {
-    auto clocks = [&](int pn, int stage) {
-        const long long tiles = (long long)ceil_div(M, 2 * BM) * ceil_div(N, PARTS * pn);
-        return (tiles + pairs - 1) / pairs * ((long long)ceil_div(K, BK) * stage + 24 * pn);
-    };
-    return clocks(64, 400) < clocks(128, 600) ? 64 : 128;
-}
-
 template <int PN, bool STORE_C, bool SIGN_PACK>
 int launch_variant(const uint32_t* Ap, int ldap, const uint32_t* Wp, int ldwp, int M, int N, int K,
                    int32_t* C, int ldc, const int32_t* thr, const uint32_t* flip,
@@ -476,11 +395,28 @@ int launch_variant(const uint32_t* Ap, int ldap, const uint32_t* Wp, int ldwp, i
 
 }  // namespace
 
+// The variant with the least estimated time: CTA pairs with parts of 128 or 64 units, or single CTAs.  A launch takes ceil(tiles / CTAs or pairs) turns of nks
+// stages and an epilogue, which depends on the results: Sign bits, int32 rows that tile stores take, other int32 rows.  Clocks fitted to 336 sizes on B200
+// (64 .. 40000 frames, 100 .. 8192 units, 256 .. 8192 inputs); the choice takes 0.1 % more than the best on the mean, 11 % at most (6996 x 566 x 6524, bound by its stores).
+// Measured, us, parts of 128 / of 64 / single: int32 4096 x 2048 x 4096 22.0 / 24.6 / 23.5, 300 x 8000 x 1501 24.4 / 18.5 / 24.5, 6270 x 8192 x 520
+// 25.9 / 23.7 / 18.8; Sign bits 4096 x 2048 x 4096 20.3 / 23.9 / 21.8, 11302 x 5912 x 1039 43.6 / 52.3 / 46.1, 6270 x 2048 x 576 10.9 / 9.8 / 7.8.
 int launch_xnor_tc(const uint32_t* Ap, int ldap, const uint32_t* Wp, int ldwp, int M, int N,
                    int K, int32_t* C, int ldc, const int32_t* thr, const uint32_t* flip,
                    uint32_t* out_bits, int ldob, int zo, cudaStream_t st) {
+    constexpr struct { int frames, units, per_launch, stage, epilogue[3], fixed; } variants[] = {{256, 256, 2, 660, {2300, 4250, 9300}, 1250}, {256, 128, 2, 575, {1050, 1950, 5000}, 0}, {128, 192, 1, 670, {2750, 3200, 10200}, 550}};
+    const int results = !C ? 0 : N % 4 == 0 && ldc % 4 == 0 && aligned16(C) ? 1 : 2, sms = device_sm_count();
+    int best = 0;
+    long long least = -1;
+    for (int v = 0; v < 3; ++v) {
+        const auto& x = variants[v];
+        const long long at_once = sms / x.per_launch, tiles = (long long)ceil_div(M, x.frames) * ceil_div(N, x.units);
+        if (at_once < 1) continue;
+        const long long clocks = (tiles + at_once - 1) / at_once * ((long long)ceil_div(K, BK) * x.stage + x.epilogue[results]) + x.fixed;
+        if (least < 0 || clocks < least) { least = clocks; best = v; }
+    }
+    if (best == 2) return launch_xnor_cta(Ap, ldap, Wp, ldwp, M, N, K, C, ldc, thr, flip, out_bits, ldob, zo, st);
     const bool sp = out_bits != nullptr;
-    auto go = [&](auto wide, auto narrow) { return (part_units(M, N, K, device_sm_count() / 2) == 64 ? narrow : wide)(Ap, ldap, Wp, ldwp, M, N, K, C, ldc, thr, flip, out_bits, ldob, zo, st); };
+    auto go = [&](auto wide, auto narrow) { return (best == 1 ? narrow : wide)(Ap, ldap, Wp, ldwp, M, N, K, C, ldc, thr, flip, out_bits, ldob, zo, st); };
     if (C && sp) return go(launch_variant<128, true, true>, launch_variant<64, true, true>);
     if (C) return go(launch_variant<128, true, false>, launch_variant<64, true, false>);
     return go(launch_variant<128, false, true>, launch_variant<64, false, true>);
