@@ -218,7 +218,7 @@ x_digits_kernel(Frames x, uint8_t* __restrict__ img, uint32_t* __restrict__ sums
                 // what gives magnitude_bound() the sum of the magnitudes itself; roundings stay far below 0.001
                 const dense::Scale scale(exps[warp]);
                 const float t = all * scale.a * scale.b * (1.001f / 65536.0f);
-                sums[m0 + warp] = (uint32_t)(t * t / (float)x.K) + 1u;
+                sums[m0 + warp] = (uint32_t)fminf(t * t / (float)x.K, 0x1p29f) + 1u;     // (the magnitudes may add up to infinity)
                 next_sums[m0 + warp] = 0u;
             }
         }

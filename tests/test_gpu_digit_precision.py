@@ -122,3 +122,27 @@ def test_rows_handed_on(env, kind, top, act):
     # (one row of numbers here, so the mean is over 500 sums of 2048 roundings: 5 % or so)
     assert rms(outs[1].double() - want) <= 1.1 * rms(ref - want)
     assert B.bnn_device_status() == 0
+
+
+def test_magnitudes_that_add_up_to_infinity(env):
+    """The scale of the outputs comes from a bound on the sums; a row of finite numbers whose magnitudes overflow has none below one."""
+    torch, B, model = env
+    m, k, n = 40, 440, 300
+    front, wp = (wl.make_bit_planes(r, c, 0.5, c, B.packed_pitch(c)) for r, c in ((n, k), (n, n)))
+    w3 = torch.randn((3, n), device="cuda:0")
+    img = torch.empty(B.bnn_output_prepared_bytes(3, n), dtype=torch.uint8, device="cuda:0")
+    B.bnn_output_prepare(w3, img)
+    small, scale = torch.full((n,), 1.2e-38, device="cuda:0"), torch.full((n,), 1 / 1024, device="cuda:0")
+    desc = B.ModelDesc([dict(kind=B.LAYER_SIGNW, K=k, N=n, Wp=model.to_dev(front), scale=small, shift=None, act=B.ACT_HARDTANH),
+                        dict(kind=B.LAYER_SIGNW, K=n, N=n, Wp=model.to_dev(wp), scale=scale, shift=None, act=B.ACT_HARDTANH),
+                        dict(kind=B.LAYER_REAL_OUT, K=n, N=3, W=w3, W_prepared=img)])
+    x = (0.5 + torch.rand((m, k), generator=torch.Generator("cuda:0").manual_seed(3), device="cuda:0")) * 1e37
+    outs = [torch.empty((m, n), device="cuda:0") for _ in range(2)]
+    B.bnn_forward(desc, x, torch.empty((m, 3), device="cuda:0"), torch.empty(desc.workspace_bytes(m), dtype=torch.uint8, device="cuda:0"), outs)
+    assert bool(x.abs().sum(1).isinf().all())
+    want = (x.double() @ signs(torch, front, k).T * small.double()).clamp(-1, 1)
+    assert float(want.abs().max()) > 0.5 and float((outs[0].double() - want).abs().max()) < 1e-5
+    want = outs[0].double() @ signs(torch, wp, n).T / 1024
+    # half a unit per value, 1.01 * 2^-23 of one at most
+    assert float((outs[1].double() - want).abs().max()) < n / 1024 * 1.01 * 2.0 ** -23 + 2.0 ** -22
+    assert B.bnn_device_status() == 0
