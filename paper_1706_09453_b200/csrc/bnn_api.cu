@@ -108,9 +108,9 @@ int validate_model(const bnn_model* model) {
 }
 
 // Whether hidden layer l can be part of a run launched as one kernel: a fused Sign layer on packed
-// input with prepared weights, of a shape the resident-weights kernel takes (fan-in up to 3072).  As
-// ONE launch of several layers that kernel also wins on its narrow tiles (fan-in above 2048: AMI-scale
-// hidden layers 1.70 ms for five against 5 x 0.39 for the kernel that widens both operands on the fly);
+// input with prepared weights, of a shape the resident-weights kernels take (fan-in up to 3072).  As
+// ONE launch of several layers these also win above a fan-in of 2048, where a CTA holds the weights of 128 units and a pair of
+// CTAs those of 256 (AMI-scale hidden layers, 65536 frames: 0.96 ms for five);
 // a single such layer is left to bnn_xnor_gemm_prepared's own choice.
 bool stackable(const bnn_model* model, int l) {
     const bnn_layer& y = model->layers[l];
@@ -239,10 +239,9 @@ static int xnor_gemm_impl(const uint32_t* Ap, int ldap, const uint32_t* Wp, int 
     }
     if (!C && !ob) return BNN_ERR_NULL;
     if (image) {
-        // Fused Sign layer: the kernel that keeps a unit tile's weights in shared memory where
-        // measurement favours it (K <= 2048, tiles of 192 units; with K <= 3072 its tiles shrink
-        // to 128 units and the kernel that widens packed weights on the fly is faster, so that
-        // one runs when the packed weights are at hand).  int32 output and the remaining shapes:
+        // Fused Sign layer: the kernels that keep a unit tile's weights in shared memory for K <= 2048,
+        // and up to 3072 where the packed weights are not at hand (tiles of 128 units, or of 256 on CTA pairs).  A single layer of such a fan-in goes to the
+        // kernel that widens packed weights on the fly: 0.7 to 1.0 times as long on B200, but 1.08 for 27296 x 1390 x 2290.  int32 output and the remaining shapes:
         // the kernel that streams the image.
         const bool fused = !C && g_xnor_prepared != BNN_PREPARED_STREAM && xnor_res_applicable(N, K);
         const bool wide_tiles = K <= 2048;

@@ -12,11 +12,12 @@
 // Every row of the real operand has a scale r_b of its own, such that its largest pair comes close to 0x7F7F7F, and is written in
 // base 256 with balanced digits, v = d0 + 256 d1 + 65536 d2 (-128 <= d <= 127), i.e. three bytes per
 // element.  The tensor core multiplies bytes at twice the rate of half-precision numbers, and
-// its 32-bit sums are exact (K <= kMaxKDigit), so S is exact: the only rounding is that of v, at most
-// r_b / 2 <= 1.01 * 2^-23 of the row's largest magnitude per pair, and one rounding of the result to fp32.  (A power of two for a
-// scale would cost a pair's sum the bit that it has more than its two values; half as many roundings and scales that use
-// the whole range make the error smaller than that of rounding every value to a power of two: on N(0, 1) rows of 440 / 2048 / 3072,
-// rms error of a sum over sum |x| 9.0e-9 -> 7.3e-9 / 4.6e-9 -> 3.7e-9 / 4.0e-9 -> 3.1e-9.)
+// its 32-bit sums are exact (K <= kMaxKDigit), so S is exact: the only roundings are that of v, at most
+// r_b / 2 <= 1.01 * 2^-23 of the row's largest magnitude per pair (v is formed in double precision), and those of the result to fp32.  A pair's sum
+// has a bit more than its two values.  Half as many roundings and scales that use
+// the whole range make up for it unless a row fills its range evenly just below a power of two: rms error of a sum, over that of rounding every value
+// to a power of two, 440 / 2048 values: N(0, 1) 0.74 - 0.80, uniform in +-0.7 0.88, in +-0.033 0.72, but in +-0.99 1.21 - 1.23, of 0.9 .. 1 1.15.  Such matrices go
+// to digit_dense.cuh (out_digit_tc.cu).
 //
 // Layout: the bits are the M operand, the digits the N operand.  A pair of CTAs (cluster of two, one per SM of
 // a TPC) works on a tile of 256 bit rows x two parts of N digit rows; each CTA widens its own 128 bit rows into its

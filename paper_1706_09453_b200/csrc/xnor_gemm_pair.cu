@@ -1,5 +1,5 @@
-// Runs of binary hidden layers of large batches: the layers of xnor_gemm_res.cu (weights resident in shared memory, one launch for a
-// run, frame tiles handed from layer to layer through counters) on CTA pairs.
+// Binary hidden layers with fan-ins above 2048, in runs or by themselves, where that is estimated to be faster (xnor_pair_clocks): the layers of xnor_gemm_res.cu
+// (weights resident in shared memory, one launch for a run, frame tiles handed from layer to layer through counters) on CTA pairs.
 //
 // There a CTA widens its frames for 192 units, or for 128 where the fan-in is above 2048, because the weights of more would not fit its shared
 // memory; with 128 units a stage takes 430 clocks of widening for 256 of MMA.  Here a pair of CTAs (cluster of two, one per
@@ -16,7 +16,7 @@
 //   warp 11      one thread issues the TMA loads of the weight stages of all layers, round a ring of twelve
 //   warps 12-19  two teams of four warps widen the frame rows into tensor memory; the teams take alternate stages
 // What bounds it, measured on B200: 65536 frames x 3072, about 660 clocks per stage against 512 of MMA; a pass of the network of five
-// such layers 3156 -> 2934 us.
+// such layers 3156 -> 2934 us.  (Its 640 threads have 96 registers each; the epilogue spills 72 bytes.)
 // Every wait is bounded; a wait that runs out sets the CTA's abort flag, all roles of both CTAs fall
 // through to the common teardown and the device status word is set.
 #include "bnn_common.cuh"

@@ -1,5 +1,5 @@
 """Products of packed signs with real-valued rows as exact integer products of byte digits, at the sizes where the
-kernels can go wrong: edges of the 256-row x 64- (or 32-) column tiles, fan-ins around 32 / 128 / 256 positions, one
+kernels can go wrong: edges of the 256-row tiles, of 128, 64 or 32 columns on pairs and 64 or 32 on single numbers, fan-ins around 32 / 128 / 256 positions, one
 row, several turns of the persistent grid, and rows that need a fourth digit."""
 import numpy as np
 import pytest

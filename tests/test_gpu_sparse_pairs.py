@@ -1,5 +1,5 @@
-"""Signs times numbers as signs times sums and differences of pairs (2:4 sparse products of byte digits), at the sizes where the
-layout of the pairs can go wrong: fan-ins that end inside a pair, a word, a group of 64 or a stage of 256 positions, in
+"""Signs times numbers as byte digits: the top layer's as signs times sums and differences of pairs (2:4 sparse products), and layers with
+binary weights, whose numbers stand by themselves, at the sizes where the layout of the digits can go wrong: fan-ins that end inside a pair, a word, a group of 64 or a stage of 256 positions, in
 tiles of every width; and pairs whose sums are the largest numbers of their rows."""
 import numpy as np
 import pytest
@@ -87,7 +87,7 @@ def test_binary_weights_fan_ins(env, m, n):
         outs = [torch.empty((m, k), device="cuda:0"), torch.empty((m, n), device="cuda:0")]
         B.bnn_forward(desc, x0, torch.empty((m, 3), device="cuda:0"), torch.empty(desc.workspace_bytes(m), dtype=torch.uint8, device="cuda:0"), outs)
         dot = outs[0].double() @ w.T
-        # outputs of a hardtanh are written in units of 256 / 127 / 2^23 at most
+        # outputs of a hardtanh are written in units of 2^-22 at most
         bound = 0.5 * ((k + 16) / 2 * 128 / 127 * 2.0 ** -22 / 1.0 + 2.0 ** -22 * dot.abs()) + 2.0 ** -23
         err = (outs[1].double() - (0.5 * dot).clamp(-1, 1)).abs()
         assert bool((err <= bound).all()), (k, float((err / bound).max()))
