@@ -16,8 +16,8 @@
 // 32 consecutive classes of a frame.  With (0,1) activations, h = (1 + sigma) / 2: the sum over all pairs of a class,
 // prepared with the image, is added.
 //
-// Bound by what L2 delivers (at the full rate of the sparse MMAs a CTA would take 64 bytes of digits per clock; it gets about
-// 39) and by the epilogue's reads of the accumulators.  Measured on B200, single weights in three digits -> pairs, 3400 classes x 2048 units:
+// Bound by what L2 delivers (at the full rate of the sparse MMAs a CTA would take 64 bytes of digits per clock; 8192 x 3400 x 2048 takes 740 MB,
+// 35 bytes per clock and SM) and by the epilogue's reads of the accumulators.  Measured on B200, single weights in three digits -> pairs, 3400 classes x 2048 units:
 // 8192 frames 109 -> 73 us (the MMAs take 40), in (0,1) 102 -> 76, 20 frames 9.2 -> 7.7; 3401 classes 110 -> 86; 731 frames x 3307 19 -> 16.4;
 // 16384 x 4000 x 3072 360 -> 250.
 #include "bnn_common.cuh"
